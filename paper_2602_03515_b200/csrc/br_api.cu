@@ -219,7 +219,8 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
     if (L.right) h->tcq_bytes = std::max(h->tcq_bytes, qr_tc_scratch_bytes(L.d.n));
   }
   if (max_k) {
-    int want_big = br_handle::kBigLanes;
+    // an order that one cluster factorises leaves most of the GPU to others: every lane holds the largest
+    int want_big = qr_one_launch((int64_t)max_k) ? br_handle::kMaxLanes : br_handle::kBigLanes;
     // tuning aid: BR_REFRESH_LANES=1..6 sets the number of concurrent full-size refresh lanes
     if (const char* env = std::getenv("BR_REFRESH_LANES")) {
       const int v = std::atoi(env);
@@ -422,31 +423,36 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
   QrTc* tcq = nullptr;
   if (L.use_tc && (h->cond_known[ci] & 1) && !complete)
     for (QrTc* t : ln.tcq) if (qr_tc_order(t) == k) tcq = t;
+  // a small order is factorised in one launch of one cluster; with the smallest the product goes along
+  const bool one = qr_one_launch(k);
+  const bool fold = one && k <= kOrthFoldedProduct && L.d.src == BR_SRC_SECOND && !complete;
+  const float* F = left_side ? L.L : L.R;
   for (int it = 0; it < h->hp.power_iters; ++it) {
-    if (L.d.src == BR_SRC_SECOND) {
-      const float* F = left_side ? L.L : L.R;
-      // widen once, then fp64 products (the products of fp32 values are exact either way)
-      BR_CUDA(h, f32_to_f64(F, ln.rF, k * k, s));
-      BR_CUDA(h, f32_to_f64(Q, ln.rQ, k * k, s));
-      count(h, 2);
+    if (!one) { BR_CUDA(h, f32_to_f64(Q, ln.rQ, k * k, s)); count(h); }       // the current basis, for the product and its completion
+    if (fold) {
+      // inside the launch below
+    } else if (L.d.src == BR_SRC_SECOND) {
       if (tcq) {
+        // widen once, then fp64 products (the products of fp32 values are exact either way)
+        BR_CUDA(h, f32_to_f64(F, ln.rF, k * k, s));
+        count(h);
         br_status st = deflated_power(h, ln, tcq, k, s);
         if (st != BR_OK) return st;
-      } else {
-        BR_CUDA(h, dgemm(0, 0, k, k, k, 1.0, ln.rF, k, ln.rQ, k, 0.0, ln.rA, k, s));
+      } else if (one) {
+        BR_CUDA(h, sdgemm(0, 0, k, k, k, 1.0, F, k, Q, k, 0.0, ln.rA, k, s));
         count(h); h->stats.gemm_flops += 2.0 * k * k * k;
+      } else {
+        BR_CUDA(h, f32_to_f64(F, ln.rF, k * k, s));
+        BR_CUDA(h, dgemm(0, 0, k, k, k, 1.0, ln.rF, k, ln.rQ, k, 0.0, ln.rA, k, s));
+        count(h, 2); h->stats.gemm_flops += 2.0 * k * k * k;
       }
     } else if (left_side) {
       // (M M^T) U = M (M^T U)
-      BR_CUDA(h, f32_to_f64(Q, ln.rQ, k * k, s));          // the current basis, for the completion of a deficient product
-      count(h);
       BR_CUDA(h, sdgemm(1, 0, n, m, m, 1.0, Mo, n, Q, m, 0.0, ln.rZ, m, s));
       BR_CUDA(h, fdgemm(0, 0, m, m, n, 1.0, Mo, n, ln.rZ, m, 0.0, ln.rA, m, s));
       count(h, 2); h->stats.gemm_flops += 4.0 * m * m * n;
     } else {
       // (M^T M) V = M^T (M V)
-      BR_CUDA(h, f32_to_f64(Q, ln.rQ, k * k, s));
-      count(h);
       BR_CUDA(h, sdgemm(0, 0, m, n, n, 1.0, Mo, n, Q, n, 0.0, ln.rZ, n, s));
       BR_CUDA(h, fdgemm(1, 0, n, n, m, 1.0, Mo, n, ln.rZ, n, 0.0, ln.rA, n, s));
       count(h, 2); h->stats.gemm_flops += 4.0 * n * n * m;
@@ -463,7 +469,13 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
     // A product that is rank-deficient only numerically (gradients confined to a subspace) shows in the
     // factorisation itself: the orthonormalisation then repeats it, in the same call, on the completed
     // product, for which it needs the product once more (the factor's buffer is free by now) and the
-    // current basis (ln.rQ).
+    // current basis.
+    if (one) {
+      BR_CUDA(h, orth_whole(ln.rA, k, ln.rWork, fold ? F : nullptr, Q, ln.rF, Q, Q, left_side ? L.Uh : L.Vh,
+                            left_side ? L.Ul : L.Vl, h->d_status, h->d_cond + ci, s));
+      count(h); h->stats.gemm_flops += (fold ? 4.0 : 2.0) * k * k * k;
+      continue;
+    }
     BR_CUDA(h, cudaMemcpyAsync(ln.rF, ln.rA, sizeof(double) * (size_t)k * (size_t)k, cudaMemcpyDeviceToDevice, s));
     {
       br_status st = orthonormalise(h, ln, k, tcq, ci, s);
@@ -472,7 +484,7 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
     BR_CUDA(h, f64_to_f32(ln.rA, Q, k * k, s));
     count(h);
   }
-  if (L.use_tc) {
+  if (L.use_tc && !one) {
     BR_CUDA(h, split_bf16(Q, left_side ? L.Uh : L.Vh, left_side ? L.Ul : L.Vl, k * k, s));
     count(h);
   }
@@ -484,9 +496,11 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
 br_status refresh_layers(br_handle* h, const int* ids, int n_ids) {
   struct Job { int layer; bool left; double cost; int64_t k; bool needs_z; };
   std::vector<Job> jobs;
-  // time of one job when it runs alone (ms, measured: 11 at order 2560, 45 at order 6912): a cubic
-  // term for the products and a linear one for the chain of panel factorisations
-  auto cost = [](double k) { return 5.4e-11 * k * k * k + 3.9e-3 * k; };
+  // time of one job when it runs alone (ms, measured: 11 at order 2560, 45 at order 6912; 0.3 at 384 and 4 at
+  // 1536 on one cluster): a cubic term for the products and a linear one for the chain of panel factorisations
+  auto cost = [](double k) {
+    return qr_one_launch((int64_t)k) ? 1.0e-9 * k * k * k + 5e-4 * k : 5.4e-11 * k * k * k + 3.9e-3 * k;
+  };
   for (int j = 0; j < n_ids; ++j) {
     const Layer& L = h->layers[ids[j]];
     const bool z = L.d.src != BR_SRC_SECOND;
@@ -534,11 +548,14 @@ br_status refresh_layers(br_handle* h, const int* ids, int n_ids) {
   // the lanes forked from the handle's stream: join them again whatever happened above, so that
   // nothing of this call is still running on an internal stream once the handle's stream has passed it
   for (int i = 1; i < nl; ++i) {
-    cudaError_t je = cudaEventRecord(h->lanes[i].done, h->lanes[i].stream);
-    if (je == cudaSuccess) je = cudaStreamWaitEvent(h->stream, h->lanes[i].done, 0);
-    if (je != cudaSuccess && failed == BR_OK) {
-      h->err = format("joining a refresh lane failed: %s", cudaGetErrorString(je));
-      failed = BR_ERR_CUDA;
+    cudaError_t je = h->stats.inject() ? cudaErrorLaunchFailure : cudaEventRecord(h->lanes[i].done, h->lanes[i].stream);
+    if (je == cudaSuccess) je = h->stats.inject() ? cudaErrorLaunchFailure : cudaStreamWaitEvent(h->stream, h->lanes[i].done, 0);
+    if (je != cudaSuccess) {
+      cudaStreamSynchronize(h->lanes[i].stream);       // no event to wait for: wait here
+      if (failed == BR_OK) {
+        h->err = format("joining a refresh lane failed: %s", cudaGetErrorString(je));
+        failed = BR_ERR_CUDA;
+      }
     }
   }
   if (failed != BR_OK) return failed;

@@ -134,11 +134,43 @@ cudaError_t dgemm_ex(int ta, int tb, int64_t M, int64_t N, int64_t K, double alp
                      int nsplit, double* partial, const int* skip, cudaStream_t s);
 
 // ---------------------------------------------------------------------------------------------
+// Orthonormalisation by one thread-block cluster (orth.cu)
+// ---------------------------------------------------------------------------------------------
+constexpr int kOrthPanel = 64;             // panel width
+// A panel whose every column keeps at least this fraction of its squared norm against the columns
+// before it (at least 10 % of its length) needs no second Cholesky-QR pass: one pass loses orthogonality like
+// cond^2 * 1e-16, with cond^2 below about 64 / ratio for other than contrived panels.
+constexpr double kOrthPassRatio = 1e-2;
+// Squared-norm ratio below which the second sweep runs.  (With panels of 128 columns 1e-8 was enough; those of
+// 64 have one more level of projections: orders 1537 and 2047, a column at 1.2e-8, 1.4e-7 off the exact result
+// instead of 3.3e-8.)
+constexpr double kOrthIllRatio = 1e-7;
+constexpr double kOrthTcRatio = 1e-6;      // the same, when the projections ran on the tensor cores; also
+                                           // the ratio below which the next refresh must not use them
+constexpr double kOrthCompletion = 1e-6;   // a deficient column j is completed by this times its length times Q_j
+// Up to this order the product F Q is formed inside the factorisation's launch: the cluster's few SMs take
+// about as long for it (17 us at 128) as a launch of its own; above, the rest of the GPU is missed.
+constexpr int64_t kOrthFoldedProduct = 128;
+// The whole factorisation of a k x k product in one launch.  A: the product (overwritten), or, with F and Q0
+// (fp32), the buffer it is formed in.  Acopy / Qprev (both or none): as for qr_pos_inplace, the copy is made
+// here.  Results: Qout (fp32) and, optionally, its bf16 hi/lo pair; *cond_out as for qr_pos_inplace with
+// bit 1 set when the product was numerically rank-deficient.  work: orth_work_doubles(k).
+size_t orth_work_doubles(int64_t k);
+cudaError_t orth_whole(double* A, int64_t k, double* work, const float* F, const float* Q0, double* Acopy, const float* Qprev,
+                       float* Qout, __nv_bfloat16* Qh, __nv_bfloat16* Ql, int* status, int* cond_out, cudaStream_t s);
+// Columns [j0, j0 + w) only, as a part of one sweep of qr_pos_inplace (whose flag words `flags` are).
+// C: room for the largest coefficient block, (w / 2)^2 doubles.
+cudaError_t orth_part(double* A, int64_t k, int64_t j0, int64_t w, double* C, int first, double ill_ratio, const double* norm0,
+                      double* rdiag, int* status, int* flags, const int* skip, cudaStream_t s);
+
+// ---------------------------------------------------------------------------------------------
 // QR with positive diagonal in fp64 (qr.cu).  A (k x k, row-major, ld = k) is overwritten by
 // its Q factor.  work: at least qr_work_doubles(k) doubles.  status: device int, set to
 // BR_WARN_RANK_DEFICIENT when a pivot underflows.  Returns the number of launches in *launches.
 // ---------------------------------------------------------------------------------------------
 size_t qr_work_doubles(int64_t k);
+// Orders whose whole factorisation is one launch (orth_whole); the others go through qr_pos_inplace.
+bool qr_one_launch(int64_t k);
 // Optional tensor-core form of the block projections (see qr.cu): plans and scratch for one order
 // k, created once.  qr_tc_scratch_bytes is 0 when the order is not eligible.
 struct QrTc;

@@ -22,7 +22,7 @@
 namespace {
 
 constexpr int64_t kMaxOrder = 512;
-// k*k doubles for the product F*Q (rounded up to a 256-byte boundary), the QR work area (91,200
+// k*k doubles for the product F*Q (rounded up to a 256-byte boundary), the QR work area (82,432
 // doubles at order kMaxOrder, the largest over all orders up to it), and 64 doubles holding the
 // rank-deficiency flag.
 constexpr size_t kWorkDoubles = 98304;
@@ -71,8 +71,9 @@ extern "C" br_status br_power_static(void* cuda_stream, const float* F, float* Q
   // The array keeps whatever the previous call left.  Only the flag has to start at zero; every
   // other word is written by this call before it is read.
   if (cudaMemsetAsync(flag, 0, sizeof(int), s) != cudaSuccess) return BR_ERR_CUDA;
-  if (sdgemm(0, 0, k, k, k, 1.0, F, k, Q, k, 0.0, A, k, s) != cudaSuccess) return BR_ERR_CUDA;
-  if (qr_pos_inplace(A, k, work, flag, s, nullptr, nullptr) != cudaSuccess) return BR_ERR_CUDA;
-  if (f64_to_f32(A, Q, k * k, s) != cudaSuccess) return BR_ERR_CUDA;
+  const bool fold = k <= kOrthFoldedProduct;
+  if (!fold && sdgemm(0, 0, k, k, k, 1.0, F, k, Q, k, 0.0, A, k, s) != cudaSuccess) return BR_ERR_CUDA;
+  if (orth_whole(A, k, work, fold ? F : nullptr, Q, nullptr, nullptr, Q, nullptr, nullptr, flag, nullptr, s) != cudaSuccess)
+    return BR_ERR_CUDA;
   return BR_OK;
 }

@@ -1,0 +1,725 @@
+// Orthonormalisation Q <- qr(A).Q (positive diagonal of R, fp64) by one thread-block cluster.
+//
+// The factorisation of qr.cu (recursive block Gram-Schmidt over panels that are orthonormalised by
+// Cholesky-QR) is a chain of hundreds of short dependent steps: Gram matrix, Cholesky factor and its
+// inverse, panel update, projection coefficients, projection.  As launches of their own they cost more
+// in launch gaps than in work: at order 384, 248 launches of which 44 did something, 950 us a basis.
+// Here one cluster of up to 16 CTAs walks the whole chain of a range of columns in one launch, and the
+// steps are separated by the cluster's hardware barrier; the second sweep and the completion of a
+// rank-deficient product are branches instead of cancelled launches.  Measured, one basis alone: order 64
+// 37 us, 384 250 us, 1024 1.3 ms, 1536 3.9 ms; stand-alone Power() at order 384 1368 -> 314 us.
+//
+//  * Rows of A are dealt to the CTAs in contiguous chunks.  A CTA computes its rows' share of a panel's
+//    Gram matrix and applies R^-1 and the projections to its own rows only, so these steps need no
+//    barrier between them.  Only the Gram sums and the projection coefficients cross CTAs.
+//  * The Gram shares stay in shared memory: every CTA adds up one slice of rows over all shares (fixed
+//    order, through distributed shared memory), and after a second barrier every CTA reads all slices and
+//    computes the 64 x 64 Cholesky factor and its inverse for itself.  The redundant factorisation costs
+//    nothing (the other CTAs would wait for it) and saves the broadcast, and since all of them see the
+//    same bits, every decision (second pass, second sweep, completion) is taken alike without a word
+//    exchanged.
+//  * Projection coefficients Q_l^T A_r: one 64 x 64 tile per CTA, the contraction split over several CTAs
+//    when there are fewer tiles than CTAs (partial sums through distributed shared memory, fixed order).
+//
+// Products run on the fp64 matrix unit (mma.sync.m8n8k4.f64): 64 x 64 tiles, a warp 16 rows x 32 columns,
+// 16-deep stages, three of them in flight with cp.async.  111 KiB of shared memory and 128 registers, two CTAs
+// per SM, so that the clusters of several bases share SMs and one cluster's barriers are another's work.
+// Other CTAs write A and C while the kernel runs: plain loads are ordered by the acquire of the barrier
+// behind those writes, and none goes through the read-only path.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+#include <mutex>
+
+#include "br_internal.h"
+
+namespace cg = cooperative_groups;
+
+namespace br {
+namespace {
+
+constexpr int kT = 256;                       // threads per CTA
+constexpr int kW = kOrthPanel;                // panel width
+constexpr int kKs = 16;                       // contraction depth of a stage
+// Leading dimensions of staged tiles, 4 mod 16 doubles: the fragment loads of a half-warp (4 x 4 or
+// 4 contraction steps x 4 rows) then touch 16 different 8-byte banks.
+constexpr int kLdK = 68;                      // [contraction][64]
+constexpr int kLdI = 20;                      // [64][16 contraction steps]
+constexpr int kOper = 64 * kLdI;              // doubles of a staged first operand (either layout)
+constexpr int kOperB = kKs * kLdK;            // and of the second
+constexpr int kStages = 3;
+constexpr int kLdP = 72;                      // partial sums (16-byte stores of a quarter-warp: 8 different banks)
+constexpr int kMaxCluster = 16;
+constexpr int kStageD = kStages * (kOper + kOperB);   // operand stages; also one 64 x 64 tile of A (ld 68)
+constexpr int kPartD = 64 * kLdP;             // partial sums of this CTA, later R^-T (ld 68)
+constexpr int kSredD = 32 * 64;               // this CTA's slice of the summed Gram matrix (at most half of it)
+// One shared-memory array, carved at compile time (pointers kept in a structure would make every access a
+// generic one behind a reload of the pointer).
+extern __shared__ double sm[];
+constexpr int oStage = 0, oPart = oStage + kStageD, oSred = oPart + kPartD, oDiag0 = oSred + kSredD, oFloor = oDiag0 + 64,
+              oPiv = oFloor + 64, oN0 = oPiv + 64, kSmemD = oN0 + 64;
+constexpr int kSmemBytes = kSmemD * (int)sizeof(double);
+static_assert(kStageD >= 64 * kLdK && kOper >= kOperB, "staging area");
+
+__device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
+               : "+d"(c0), "+d"(c1) : "d"(a), "d"(b));
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// A 64 x 64 tile on 8 warps, 16 rows x 32 columns each: entry e of a thread's accumulator (mi = e / 8,
+// ni = e / 2 % 4) sits at row tile_row() + 8 mi, column tile_col() + 8 ni + e % 2 (8 x 64 per warp needs half
+// as much again from shared memory).  The warps of a scheduler take different rows, so that a short tile still
+// uses all four; with SYM only the 8 x 8 blocks on and above the diagonal are computed, and the warps are
+// paired so that the schedulers get 8 to 10 of the 36 blocks.
+template <bool SYM>
+__device__ __forceinline__ int warp_m() {
+  const int w = threadIdx.x >> 5;
+  return SYM ? (0x31322010 >> (4 * w)) & 3 : w >> 1;       // per warp, from warp 0 up: 0 1 0 2 2 3 1 3
+}
+template <bool SYM>
+__device__ __forceinline__ int warp_n() {
+  const int w = threadIdx.x >> 5;
+  return SYM ? (0x8B >> w) & 1 : w & 1;                    // 1 1 0 1 0 0 0 1
+}
+template <bool SYM> __device__ __forceinline__ int tile_row() { return 16 * warp_m<SYM>() + ((threadIdx.x & 31) >> 2); }
+template <bool SYM> __device__ __forceinline__ int tile_col() { return 32 * warp_n<SYM>() + 2 * (threadIdx.x & 3); }
+
+// One stage (16 contraction steps) of acc += (or -=, NEG) a b.  I: rows of the tile that exist.
+template <bool DIRECT, bool SYM, bool NEG>
+__device__ __forceinline__ void mma_stage(double (&acc)[16], const double* As, const double* Bs, int I) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, tig = lane & 3, wm = warp_m<SYM>(), wn = warp_n<SYM>();
+  As += DIRECT ? tig * kLdK + 16 * wm + g : (16 * wm + g) * kLdI + tig;
+  Bs += tig * kLdK + 32 * wn + g;
+  if (16 * wm >= I || (SYM && 4 * wn + 3 < 2 * wm)) return;
+  const bool two = 16 * wm + 8 < I;
+#pragma unroll
+  for (int k4 = 0; k4 < kKs; k4 += 4) {
+    double a0 = As[DIRECT ? k4 * kLdK : k4], a1 = As[DIRECT ? k4 * kLdK + 8 : 8 * kLdI + k4];
+    if (NEG) { a0 = -a0; a1 = -a1; }
+    double b[4];
+#pragma unroll
+    for (int ni = 0; ni < 4; ++ni) b[ni] = Bs[k4 * kLdK + 8 * ni];
+#pragma unroll
+    for (int ni = 0; ni < 4; ++ni)
+      if (!SYM || 4 * wn + ni >= 2 * wm) dmma(acc[2 * ni], acc[2 * ni + 1], a0, b[ni]);
+    if (two) {
+#pragma unroll
+      for (int ni = 0; ni < 4; ++ni)
+        if (!SYM || 4 * wn + ni >= 2 * wm + 1) dmma(acc[8 + 2 * ni], acc[9 + 2 * ni], a1, b[ni]);
+    }
+  }
+}
+// 16 or 8 bytes from global to shared memory, zero when !ok (the rows of an odd order are 8-byte aligned only)
+template <bool VEC>
+__device__ __forceinline__ void copy_async(double* dst, const double* src, bool ok) {
+  if (VEC)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 8 : 0) : "memory");
+}
+// acc += sum over kk < K of a(i, kk) b(kk, j), i < I <= 64, j < J <= 64 (NEG: -=).
+//   DIRECT: a(i, kk) = X[kk * lda + i]   otherwise a(i, kk) = X[i * lda + kk];   b(kk, j) = Y[kk * ldb + j].
+// VEC: all dimensions and leading dimensions that a copy runs along are even, and X and Y 16-byte aligned.
+template <bool VEC, bool DIRECT, bool SYM, bool NEG>
+__device__ __forceinline__ void mm64(double (&acc)[16], const double* X, int64_t lda, int I, const double* Y, int64_t ldb, int J, int K) {
+  constexpr int V = VEC ? 2 : 1, N = 4 / V;                // doubles per copy; copies per thread, operand and stage
+  const int t = threadIdx.x;
+  // thread -> first element of an operand tile, and the distance of its next one
+  constexpr int RK = kT / (64 / V), RI = kT / (kKs / V);   // rows of a [16][64] / [64][16] tile covered by one copy per thread
+  const int bk = t / (64 / V), bj = t % (64 / V) * V;
+  const int ak = DIRECT ? bk : t % (kKs / V) * V, ai = DIRECT ? bj : t / (kKs / V);
+  const double* px = X + (DIRECT ? (int64_t)ak * lda + ai : (int64_t)ai * lda + ak);
+  const double* py = Y + (int64_t)bk * ldb + bj;
+  const int64_t xq = (DIRECT ? RK : RI) * lda, xs = DIRECT ? kKs * lda : kKs, yq = RK * ldb, ys = kKs * ldb;
+  double* const dA = sm + oStage + (DIRECT ? ak * kLdK + ai : ai * kLdI + ak);
+  double* const dB = sm + oStage + kOper + bk * kLdK + bj;
+  const int nk = (K + kKs - 1) / kKs;
+  auto fetch = [&](int s) {
+    const int k0 = s * kKs, buf = (s % kStages) * (kOper + kOperB);
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const bool ok = DIRECT ? (ai < I && k0 + ak + q * RK < K) : (ai + q * RI < I && k0 + ak < K);
+      copy_async<VEC>(dA + buf + (DIRECT ? q * RK * kLdK : q * RI * kLdI), ok ? px + q * xq : X, ok);
+    }
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const bool ok = bj < J && k0 + bk + q * RK < K;
+      copy_async<VEC>(dB + buf + q * RK * kLdK, ok ? py + q * yq : Y, ok);
+    }
+    px += xs; py += ys;
+  };
+#pragma unroll
+  for (int s = 0; s < kStages - 1; ++s) {
+    if (s < nk) fetch(s);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  int buf = 0;
+  for (int s = 0; s < nk; ++s) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+    __syncthreads();                             // stage s is in place, and stage s - 1 has been read
+    if (s + kStages - 1 < nk) fetch(s + kStages - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const double* st = sm + oStage + buf * (kOper + kOperB);
+    mma_stage<DIRECT, SYM, NEG>(acc, st, st + kOper, I);
+    if (++buf == kStages) buf = 0;
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void clear(double (&acc)[16]) {
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = 0.0;
+}
+// the entries of a tile that exist: f(row, column, value)
+template <typename FN>
+__device__ __forceinline__ void each_entry(double (&acc)[16], int I, int J, FN f) {
+  const int r = tile_row<false>(), c = tile_col<false>();
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    const int row = r + 8 * (e >> 3), col = c + 8 * ((e >> 1) & 3) + (e & 1);
+    if (row < I && col < J) f(row, col, acc[e]);
+  }
+}
+
+// One tile of the product F Q of two fp32 matrices (row-major, widened while they are staged through
+// registers); only the smallest orders form it here.
+__device__ __noinline__ void product64(const float* X, int I, const float* Y, int J, int k, double* out) {
+  const int t = threadIdx.x;
+  double acc[16], ra[4], rb[4];
+  clear(acc);
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = (t >> 4) + 16 * q, ka = k0 + (t & 15), kb = k0 + (t >> 6) + 4 * q;
+      ra[q] = (i < I && ka < k) ? (double)X[(int64_t)i * k + ka] : 0.0;
+      rb[q] = ((t & 63) < J && kb < k) ? (double)Y[(int64_t)kb * k + (t & 63)] : 0.0;
+    }
+  };
+  auto store = [&](int buf) {
+    double* As = sm + oStage + buf * (kOper + kOperB);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      As[((t >> 4) + 16 * q) * kLdI + (t & 15)] = ra[q];
+      As[kOper + ((t >> 6) + 4 * q) * kLdK + (t & 63)] = rb[q];
+    }
+  };
+  const int nk = (k + kKs - 1) / kKs;
+  load(0);
+  store(0);
+  __syncthreads();
+  for (int s = 0; s < nk; ++s) {
+    if (s + 1 < nk) load((s + 1) * kKs);
+    const double* st = sm + oStage + (s & 1) * (kOper + kOperB);
+    mma_stage<false, false, false>(acc, st, st + kOper, I);
+    if (s + 1 < nk) store((s + 1) & 1);
+    __syncthreads();
+  }
+  each_entry(acc, I, J, [&](int i, int j, double v) { out[(int64_t)i * k + j] = v; });
+}
+
+struct OrthArgs {
+  double* A; int64_t k;          // k x k, row-major; columns [j0, j0 + w) are orthonormalised
+  int j0, w;
+  int whole;                     // 1: the complete factorisation (both sweeps, rank decision, completion, outputs)
+  int first;                     // part: this is the first sweep (watch the column norms)
+  double ill_ratio;              // part, first: squared-norm ratio below which the second sweep has to run
+  const double* norm0;           // part, first: squared norms of the columns before any projection
+  double *C, *normp, *rdiag;     // projection coefficients; 2 x cluster x k partial norms (whole); squared diagonal of R
+  const float *F, *Q0;           // whole: A <- F Q0 first (null: A holds the product)
+  double* Acopy; const float* Qprev;   // whole: buffer for a second copy of A, and the basis for its completion (both or none)
+  float* Qout; __nv_bfloat16 *Qh, *Ql; // whole: the result in fp32 and as a bf16 pair (optional)
+  int* status; int* flags; int* cond_out; const int* skip;
+};
+
+struct Ctx {
+  int64_t k;
+  double* A;
+  int rank, cs, r0, r1;
+};
+
+// Cholesky factor S = R^T R of the panel's Gram matrix (bw <= 64) and its inverse, as R^-T (ld 68), in the
+// area of the partial sums.
+//
+// Blocks of 8 x 8 in shared memory; block row c of [S | I] is solved with R_cc (forward substitution, a column
+// per thread) and subtracted, times R_ci^T, from the rows i below (matrix unit).  Column block j of S is dead
+// once block row j is done, and column block j of the identity's part is still a unit block until then, so
+// both share one 64 x 64 array.  The chain is bound by the 8 x 8 factorisations: warp 0 alone updates the
+// next diagonal block and factors it in registers (every lane the same: no shuffles, 8 dependent square
+// roots), while warp w updates block row c + w.  Two barriers a block instead of one a pivot: 64 pivots in
+// 12 us; 27 us with a barrier a pivot and the matrix in registers, 20 us with two pivots a barrier.
+// (Multiplying block row c by an explicit R_cc^-T instead loses the factorisation of a panel with a condition
+// number of 1e6, such as a completed rank-deficient product has: its error, 1e-16 times the condition number,
+// swamps pivots of 1e-12.  Substitution is backward stable like the unblocked elimination.)
+// The pivots end up at oPiv, the Gram diagonal at oDiag0.
+constexpr int oZ = oStage, oX = oZ + 64 * kLdK, oD = oX + 8 * kLdK;      // (in the operand stages)
+static_assert(64 * kLdK + 8 * kLdK + 8 * 8 + 8 <= kStageD, "the factorisation borrows the operand stages");
+
+// The diagonal block at Z (upper triangle) -> R_cc at oD (row-major 8 x 8), 1 / diagonal behind it, pivots at oPiv + 8 c
+__device__ __forceinline__ void factor8(const double* Z, int c) {
+  const int lane = threadIdx.x & 31;
+  double u[8][8], inv[8], piv[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = i; j < 8; ++j) u[i][j] = Z[i * kLdK + j];
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    const double fl = sm[oFloor + 8 * c + p];
+    piv[p] = u[p][p] > fl ? u[p][p] : fl;
+    inv[p] = rsqrt(piv[p]);
+#pragma unroll
+    for (int j = p + 1; j < 8; ++j) u[p][j] *= inv[p];
+#pragma unroll
+    for (int i = p + 1; i < 8; ++i)
+#pragma unroll
+      for (int j = i; j < 8; ++j) u[i][j] = fma(-u[p][i], u[p][j], u[i][j]);
+  }
+  if (lane == 0) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+#pragma unroll
+      for (int j = i + 1; j < 8; ++j) sm[oD + 8 * i + j] = u[i][j];
+      sm[oD + 64 + i] = inv[i];
+      sm[oPiv + 8 * c + i] = piv[i];
+    }
+  }
+}
+
+__device__ __noinline__ void chol64(const Ctx q, int bw) {
+  const int t = threadIdx.x, w = t >> 5, lane = t & 31, g = lane >> 2, tig = lane & 3;
+  const int rs = 64 / q.cs, nb = (bw + 7) / 8;
+  double* const Z = sm + oZ;
+  double* const RT = sm + oPart;
+  // upper block triangle of S (identity beyond the panel), zero below
+  double v[16];
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    const int i = (t >> 6) + 4 * u, j = t & 63;
+    v[u] = (i == j) ? 1.0 : 0.0;
+    if (j >= (i & ~7) && max(i, j) < bw) v[u] = q.cs == 1 ? sm[oPart + i * kLdP + j] : cg::this_cluster().map_shared_rank(sm + oSred, i / rs)[(i % rs) * 64 + j];
+  }
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    const int i = (t >> 6) + 4 * u, j = t & 63;
+    Z[i * kLdK + j] = v[u];
+    if (i == j) {
+      sm[oDiag0 + i] = v[u];
+      const double f = v[u] * 1e-24;
+      sm[oFloor + i] = f > 1e-300 ? f : 1e-300;      // a pivot at or below this is clamped
+    }
+  }
+  __syncthreads();
+  // block (i, j) of rows to come <- itself - R_ci^T X_j, with block row c of R | R^-T in oX
+  auto update = [&](int i, int j) {
+    double2* z = reinterpret_cast<double2*>(Z + (8 * i + g) * kLdK + 8 * j + 2 * tig);
+    double2 d = *z;
+#pragma unroll
+    for (int k4 = 0; k4 < 8; k4 += 4) {
+      const double* x = sm + oX + (k4 + tig) * kLdK + g;
+      dmma(d.x, d.y, -x[8 * i], x[8 * j]);
+    }
+    *z = d;
+  };
+#pragma unroll 1
+  for (int c = 0; c < nb; ++c) {
+    if (w == 0) {
+      if (c > 0) { update(c, c); __syncwarp(); }
+      factor8(Z + 8 * c * kLdK + 8 * c, c);
+    } else if (c > 0 && c - 1 + w < nb) {
+      const int i = c - 1 + w;
+      for (int j = 0; j < nb; ++j)
+        if (j < c || j > i || (j == i && i > c)) update(i, j);
+    }
+    __syncthreads();
+    // block row c: R right of the diagonal, R^-T up to it
+    if (t < 8 * nb) {
+      double x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = (t >> 3) == c ? ((t & 7) == i ? 1.0 : 0.0) : Z[(8 * c + i) * kLdK + t];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        x[i] *= sm[oD + 64 + i];
+#pragma unroll
+        for (int m = i + 1; m < 8; ++m) x[m] = fma(-sm[oD + 8 * i + m], x[i], x[m]);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) sm[oX + i * kLdK + t] = x[i];
+      if ((t >> 3) <= c) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) RT[(8 * c + i) * kLdK + t] = x[i];
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// own rows of columns [j0, j0 + bw) <- own rows * R^-1 (upper triangular)
+__device__ __noinline__ void apply_rinv(const Ctx q, int j0, int bw) {
+  const int t = threadIdx.x, lane = t & 31, g = lane >> 2, tig = lane & 3;
+  double pre[16];
+  auto load = [&](int r) {
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int i = (t >> 6) + 4 * u, kk = t & 63;
+      pre[u] = (r + i < q.r1 && kk < bw) ? __ldcg(q.A + (int64_t)(r + i) * q.k + j0 + kk) : 0.0;
+    }
+  };
+  if (q.r0 < q.r1) load(q.r0);
+  for (int r = q.r0; r < q.r1; r += 64) {
+#pragma unroll
+    for (int u = 0; u < 16; ++u) sm[oStage + ((t >> 6) + 4 * u) * kLdK + (t & 63)] = pre[u];
+    __syncthreads();
+    if (r + 64 < q.r1) load(r + 64);
+    const int wm = warp_m<false>(), wn = warp_n<false>();
+    if (r + 16 * wm < q.r1) {
+      double acc[16];
+      clear(acc);
+      const double* As = sm + oStage + (16 * wm + g) * kLdK + tig;
+      const double* Bs = sm + oPart + (32 * wn + g) * kLdK + tig;
+#pragma unroll
+      for (int k4 = 0; k4 < 64; k4 += 4) {
+        if (k4 >= 32 && wn == 0) break;                // R^-1 is upper triangular
+        const double a0 = As[k4], a1 = As[8 * kLdK + k4];
+#pragma unroll
+        for (int ni = 0; ni < 4; ++ni)
+          if (k4 < 32 ? (wn == 1 || k4 <= 8 * ni + 7) : k4 - 32 <= 8 * ni + 7) {
+            const double b = Bs[8 * ni * kLdK + k4];
+            dmma(acc[2 * ni], acc[2 * ni + 1], a0, b);
+            dmma(acc[8 + 2 * ni], acc[9 + 2 * ni], a1, b);
+          }
+      }
+      each_entry(acc, q.r1 - r, bw, [&](int i, int j, double v) { q.A[(int64_t)(r + i) * q.k + j0 + j] = v; });
+    }
+    __syncthreads();
+  }
+}
+
+// A[:, jt : jt + wt] -= Q (Q^T A[:, jt : jt + wt]), Q = A[:, jp : jp + wp] orthonormal, wp a multiple of 64.
+template <bool VEC>
+__device__ __noinline__ void project64(const Ctx q, double* C, int jp, int wp, int jt, int wt) {
+  const int t = threadIdx.x;
+  const int ntp = (wp + 63) / 64, ntt = (wt + 63) / 64, tiles = ntp * ntt;
+  const int sp = tiles < q.cs ? q.cs / tiles : 1;       // CTAs that share one tile's contraction
+  double acc[16];
+  cluster_sync();                                       // every CTA's rows of both blocks are written
+  auto tile_pos = [&](int tile, int* i0, int* c0, int* I, int* J) {
+    *i0 = (tile / ntt) * 64; *c0 = (tile % ntt) * 64; *I = min(64, wp - *i0); *J = min(64, wt - *c0);
+  };
+  if (sp == 1) {
+    for (int tile = q.rank; tile < tiles; tile += q.cs) {
+      int i0, c0, I, J;
+      tile_pos(tile, &i0, &c0, &I, &J);
+      clear(acc);
+      mm64<VEC, true, false, false>(acc, q.A + jp + i0, q.k, I, q.A + jt + c0, q.k, J, (int)q.k);
+      each_entry(acc, I, J, [&](int i, int j, double v) { C[(int64_t)(i0 + i) * wt + c0 + j] = v; });
+    }
+    cluster_sync();
+  } else {
+    const int tile = q.rank / sp, split = q.rank % sp;
+    int i0 = 0, c0 = 0, I = 0, J = 0;
+    if (tile < tiles) {
+      tile_pos(tile, &i0, &c0, &I, &J);
+      const int kc = ((int)((q.k + sp - 1) / sp) + kKs - 1) / kKs * kKs, k0 = min((int)q.k, split * kc);
+      const int kn = min(kc, (int)q.k - k0);
+      clear(acc);
+      mm64<VEC, true, false, false>(acc, q.A + (int64_t)k0 * q.k + jp + i0, q.k, I, q.A + (int64_t)k0 * q.k + jt + c0, q.k, J, kn);
+      each_entry(acc, 64, 64, [&](int i, int j, double v) { sm[oPart + i * kLdP + j] = v; });
+    }
+    cluster_sync();
+    if (tile < tiles) {
+      for (int e = split * kT + t; e < 64 * 64; e += sp * kT) {
+        const int i = e >> 6, j = e & 63;
+        double s = 0.0;
+        for (int z = 0; z < sp; ++z) s += cg::this_cluster().map_shared_rank(sm + oPart, tile * sp + z)[i * kLdP + j];
+        if (i < I && j < J) C[(int64_t)(i0 + i) * wt + c0 + j] = s;
+      }
+    }
+    cluster_sync();
+  }
+  for (int r = q.r0; r < q.r1; r += 64)
+    for (int c0 = 0; c0 < wt; c0 += 64) {
+      const int I = min(64, q.r1 - r), J = min(64, wt - c0);
+      // the accumulator starts from A itself: its loads overlap the first copies
+      double* p = q.A + (int64_t)r * q.k + jt + c0;
+      clear(acc);
+      each_entry(acc, I, J, [&](int i, int j, double& v) { v = __ldcg(p + (int64_t)i * q.k + j); });
+      mm64<VEC, false, false, true>(acc, q.A + (int64_t)r * q.k + jp, q.k, I, C + c0, wt, J, wp);
+      each_entry(acc, I, J, [&](int i, int j, double v) { p[(int64_t)i * q.k + j] = v; });
+    }
+  __syncthreads();
+}
+
+// What one sweep over the columns found (alike in every CTA).
+struct SweepNotes { bool ill = false, tc_bad = false, clamped = false; };
+
+// Cholesky-QR of the panel [j0, j0 + bw), repeated once unless every column kept kOrthPassRatio of its
+// squared norm against the panel's columns before it.
+template <bool VEC>
+__device__ __forceinline__ void panel64(const Ctx& q, int j0, int bw, bool first, double ill_ratio, double* rdiag, bool rdiag_init,
+                                        SweepNotes& notes) {
+  const int t = threadIdx.x;
+  for (int pass = 0; pass < 2; ++pass) {
+    double acc[16];
+    const double* P = q.A + (int64_t)q.r0 * q.k + j0;
+    clear(acc);
+    mm64<VEC, true, true, false>(acc, P, q.k, bw, P, q.k, bw, max(0, q.r1 - q.r0));
+    {
+      // (a warp whose blocks all lie below the diagonal writes zeros nobody reads)
+      const int row = tile_row<true>(), col = tile_col<true>();
+#pragma unroll
+      for (int e = 0; e < 16; e += 2)
+        *reinterpret_cast<double2*>(sm + oPart + (row + 8 * (e >> 3)) * kLdP + col + 8 * ((e >> 1) & 3)) = make_double2(acc[e], acc[e + 1]);
+    }
+    if (q.cs > 1) {
+      cluster_sync();
+      const int rs = 64 / q.cs;
+      for (int e = t; e < rs * 64; e += kT) {
+        const int i = q.rank * rs + (e >> 6), j = e & 63;
+        double s = 0.0;
+        if (j >= (i & ~7))
+          for (int z = 0; z < q.cs; ++z) s += cg::this_cluster().map_shared_rank(sm + oPart, z)[i * kLdP + j];
+        sm[oSred + e] = s;
+      }
+      cluster_sync();
+    } else {
+      __syncthreads();
+    }
+    chol64(q, bw);
+    // what the pivots say: pivot / Gram diagonal is the squared sine of the angle between a column and the
+    // span of the panel's columns before it
+    bool low = false, ill = false, bad = false, cl = false;
+    if (t < bw) {
+      const double piv = sm[oPiv + t], d0 = sm[oDiag0 + t];
+      low = !(d0 > 0.0 && piv >= kOrthPassRatio * d0);
+      cl = !(piv > sm[oFloor + t]);
+      if (first && pass == 0) { ill = d0 < ill_ratio * sm[oN0 + t]; bad = d0 < kOrthTcRatio * sm[oN0 + t]; }
+      if (q.rank == 0 && rdiag) rdiag[j0 + t] = (rdiag_init && pass == 0) ? piv : __ldcg(rdiag + j0 + t) * piv;
+    }
+    low = __syncthreads_or(low); notes.ill |= __syncthreads_or(ill) != 0;
+    notes.tc_bad |= __syncthreads_or(bad) != 0; notes.clamped |= __syncthreads_or(cl) != 0;
+    apply_rinv(q, j0, bw);
+    if (!low) break;
+  }
+}
+
+// One sweep over the columns [j0, j0 + w): the recursion "orthonormalise the left half, project it out of
+// the right half, orthonormalise the right half" in the order of its panels.  The node whose right part
+// starts at panel l is projected right before that panel.
+template <bool VEC>
+__device__ __forceinline__ SweepNotes sweep64(const Ctx& q, double* C, int j0, int w, bool first, double ill_ratio, const double* norm0,
+                                              int norm_parts, double* rdiag, bool rdiag_init) {
+  SweepNotes notes;
+  const int nl = (w + kW - 1) / kW;
+  for (int l = 0; l < nl; ++l) {
+    if (l > 0) {
+      int lo = 0, n = nl, h;
+      while (true) {
+        h = (n + 1) / 2;
+        if (l == lo + h) break;
+        if (l < lo + h) n = h; else { lo += h; n -= h; }
+      }
+      project64<VEC>(q, C, j0 + lo * kW, h * kW, j0 + l * kW, min(n * kW, w - lo * kW) - h * kW);
+    }
+    const int c0 = j0 + l * kW, bw = min(kW, j0 + w - c0);
+    if (first && (int)threadIdx.x < bw) {
+      double s = 0.0;
+      for (int z = 0; z < norm_parts; ++z) s += __ldcg(norm0 + (int64_t)z * q.k + c0 + threadIdx.x);
+      sm[oN0 + threadIdx.x] = s;
+    }
+    panel64<VEC>(q, c0, bw, first, ill_ratio, rdiag, rdiag_init, notes);
+  }
+  return notes;
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(kT, 2) k_orth_cluster(OrthArgs a) {
+  if (a.skip && *a.skip) return;               // uniform: a device-side flag cancels the whole launch
+  Ctx q;
+  q.k = a.k; q.A = a.A;
+  q.cs = (int)gridDim.x; q.rank = (int)blockIdx.x;
+  const int k = (int)a.k, rc = ((k + q.cs - 1) / q.cs + 7) / 8 * 8;
+  q.r0 = min(k, q.rank * rc); q.r1 = min(k, q.r0 + rc);
+  const int t = threadIdx.x;
+
+  if (!a.whole) {
+    const SweepNotes n = sweep64<VEC>(q, a.C, a.j0, a.w, a.first != 0, a.ill_ratio, a.norm0, 1, a.rdiag, false);
+    if (q.rank == 0 && t == 0) {
+      if (n.clamped) { atomicMax(a.status, (int)BR_WARN_RANK_DEFICIENT); a.flags[3] = 1; }
+      if (a.first && n.ill) a.flags[1] = 0;
+      if (a.first && n.tc_bad) a.flags[2] = 0;
+    }
+    cluster_sync();                              // no CTA leaves while another may still read its shared memory
+    return;
+  }
+
+  if (a.F) {
+    for (int r = q.r0; r < q.r1; r += 64)
+      for (int c0 = 0; c0 < k; c0 += 64)
+        product64(a.F + (int64_t)r * k, min(64, q.r1 - r), a.Q0 + c0, min(64, k - c0), k, q.A + (int64_t)r * k + c0);
+    __syncthreads();
+  }
+  bool clamped = false, tc_bad = false, deficient = false;
+  const bool fix = a.Acopy != nullptr && a.Qprev != nullptr;
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    double* normp = a.normp + (int64_t)attempt * q.cs * k;
+    for (int j = t; j < k; j += kT) {
+      double s = 0.0;
+      if (!attempt) {
+        // (rows come in eights: eight loads in flight)
+        for (int r = q.r0; r < q.r1; r += 8) {
+          double v[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) v[u] = r + u < q.r1 ? __ldcg(q.A + (int64_t)(r + u) * k + j) : 0.0;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            if (fix && r + u < q.r1) a.Acopy[(int64_t)(r + u) * k + j] = v[u];
+            s = fma(v[u], v[u], s);
+          }
+        }
+      } else {
+        // complete the product from the current basis: A_j + 1e-6 ||A_j|| Q_j (a zero column becomes Q_j)
+        double n2 = 0.0;
+        for (int z = 0; z < q.cs; ++z) n2 += __ldcg(a.normp + (int64_t)z * k + j);
+        const double d = n2 > 0.0 ? kOrthCompletion * sqrt(n2) : 1.0;
+        for (int r = q.r0; r < q.r1; ++r) {
+          const int64_t i = (int64_t)r * k + j;
+          const double v = fma(d, (double)a.Qprev[i], __ldcg(a.Acopy + i));
+          q.A[i] = v;
+          s = fma(v, v, s);
+        }
+      }
+      normp[(int64_t)q.rank * k + j] = s;
+    }
+    cluster_sync();
+    double* const rdiag = fix && !attempt ? a.rdiag : nullptr;
+    SweepNotes n = sweep64<VEC>(q, a.C, 0, k, true, kOrthIllRatio, normp, q.cs, rdiag, true);
+    clamped |= n.clamped;
+    if (!attempt) tc_bad = n.tc_bad;
+    if (n.ill) {
+      n = sweep64<VEC>(q, a.C, 0, k, false, 0.0, nullptr, 0, rdiag, false);
+      clamped |= n.clamped;
+    }
+    if (!fix || attempt) break;
+    // rank decision on the squared diagonal of R: deficient when some |R_jj| <= 1e-12 max |R_kk|
+    cluster_sync();
+    double lo = 1e300, hi = 0.0;
+    for (int j = t; j < k; j += kT) {
+      const double v = __ldcg(a.rdiag + j);
+      lo = v > 0.0 ? fmin(lo, v) : 0.0; hi = fmax(hi, v);
+    }
+    sm[oStage + t] = lo; sm[oStage + kT + t] = hi;
+    __syncthreads();
+    for (int s = kT / 2; s > 0; s >>= 1) {
+      if (t < s) {
+        sm[oStage + t] = fmin(sm[oStage + t], sm[oStage + t + s]);
+        sm[oStage + kT + t] = fmax(sm[oStage + kT + t], sm[oStage + kT + t + s]);
+      }
+      __syncthreads();
+    }
+    deficient = !(sm[oStage] > 1e-24 * sm[oStage + kT]);
+    __syncthreads();
+    if (!deficient) break;
+  }
+  // the result in fp32 and, for the tensor-core path, as a bf16 pair (own rows)
+  for (int64_t i0 = (int64_t)q.r0 * k; i0 < (int64_t)q.r1 * k; i0 += 8 * kT) {
+    float x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) { const int64_t i = i0 + u * kT + t; x[u] = i < (int64_t)q.r1 * k ? (float)__ldcg(q.A + i) : 0.f; }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int64_t i = i0 + u * kT + t;
+      if (i >= (int64_t)q.r1 * k) break;
+      a.Qout[i] = x[u];
+      if (a.Qh) {
+        const __nv_bfloat16 h = __float2bfloat16_rn(x[u]);
+        a.Qh[i] = h;
+        a.Ql[i] = __float2bfloat16_rn(x[u] - __bfloat162float(h));
+      }
+    }
+  }
+  if (q.rank == 0 && t == 0) {
+    if (clamped || deficient) atomicMax(a.status, (int)BR_WARN_RANK_DEFICIENT);
+    // bit 0: no column shrank below 1e-3 of its length; bit 1: numerically rank-deficient
+    if (a.cond_out) *a.cond_out = (tc_bad ? 0 : 1) | (clamped || deficient ? 2 : 0);
+  }
+  cluster_sync();
+}
+
+// Largest cluster the device schedules for this kernel (16 needs the non-portable size), per device.
+int max_cluster() {
+  static int cap[64] = {};
+  static std::mutex mu;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return 0; }
+  std::lock_guard<std::mutex> lock(mu);
+  if (cap[dev]) return cap[dev];
+  int best = kMaxCluster;
+  for (auto kernel : {k_orth_cluster<false>, k_orth_cluster<true>}) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) { cudaGetLastError(); return 0; }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kMaxCluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(kMaxCluster); cfg.blockDim = dim3(kT); cfg.dynamicSmemBytes = kSmemBytes; cfg.attrs = at; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1)
+      best = 8;
+  }
+  cudaGetLastError();
+  return cap[dev] = best;
+}
+
+// CTAs for order k: at least 32 rows each, a power of two.
+int cluster_for(int64_t k) {
+  int cs = 1;
+  while (cs < kMaxCluster && 32 * cs < k) cs *= 2;
+  return cs;
+}
+
+cudaError_t launch(const OrthArgs& a, cudaStream_t s) {
+  const int cap = max_cluster();
+  if (cap == 0) return cudaErrorInvalidConfiguration;
+  const int cs = std::min(cap, cluster_for(a.k));
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)cs); cfg.blockDim = dim3(kT); cfg.dynamicSmemBytes = kSmemBytes; cfg.stream = s;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  // 16-byte copies need even dimensions throughout (the buffers start on 256-byte boundaries)
+  return cudaLaunchKernelEx(&cfg, (a.k % 2 == 0) ? k_orth_cluster<true> : k_orth_cluster<false>, a);
+}
+
+inline int64_t pad32(int64_t doubles) { return (doubles + 31) / 32 * 32; }
+// The largest coefficient block: the root's is at most (k / 2)^2, a node of the left half (which may be
+// the larger one when the last panel is ragged) at most that or one panel squared.
+int64_t coef_doubles(int64_t k) { return pad32(std::max<int64_t>(((k + 1) / 2) * ((k + 1) / 2), kW * kW)); }
+
+}  // namespace
+
+size_t orth_work_doubles(int64_t k) {
+  return (size_t)(coef_doubles(k) + pad32(2 * cluster_for(k) * k) + pad32(k));
+}
+
+cudaError_t orth_whole(double* A, int64_t k, double* work, const float* F, const float* Q0, double* Acopy, const float* Qprev,
+                       float* Qout, __nv_bfloat16* Qh, __nv_bfloat16* Ql, int* status, int* cond_out, cudaStream_t s) {
+  OrthArgs a = {};
+  a.A = A; a.k = k; a.j0 = 0; a.w = (int)k; a.whole = 1;
+  a.C = work; a.normp = a.C + coef_doubles(k); a.rdiag = a.normp + pad32(2 * cluster_for(k) * k);
+  a.F = F; a.Q0 = Q0; a.Acopy = Acopy; a.Qprev = Qprev; a.Qout = Qout; a.Qh = Qh; a.Ql = Ql;
+  a.status = status; a.cond_out = cond_out;
+  return launch(a, s);
+}
+
+cudaError_t orth_part(double* A, int64_t k, int64_t j0, int64_t w, double* C, int first, double ill_ratio, const double* norm0,
+                      double* rdiag, int* status, int* flags, const int* skip, cudaStream_t s) {
+  OrthArgs a = {};
+  a.A = A; a.k = k; a.j0 = (int)j0; a.w = (int)w; a.first = first; a.ill_ratio = ill_ratio; a.norm0 = norm0;
+  a.C = C; a.rdiag = rdiag; a.status = status; a.flags = flags; a.skip = skip;
+  return launch(a, s);
+}
+
+}  // namespace br

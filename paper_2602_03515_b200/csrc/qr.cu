@@ -3,13 +3,11 @@
 // The factorisation wanted is the unique one with a positive diagonal of R.  It is computed by
 // a recursive block Gram-Schmidt whose floating-point work is almost entirely large fp64 matrix
 // products (dgemm.cu):
-//   orth(columns):  if the block is at most one panel (128 columns) wide, orthonormalise it by
-//                   Cholesky-QR; otherwise orth(left half), project the left half out of the right
-//                   half (C = Q_l^T A_r, A_r -= Q_l C), orth(right half).
-//   Cholesky-QR of a panel P: Gram matrix S = P^T P (split over the rows), Cholesky factor
-//   S = R^T R and its inverse in one CTA, P <- P R^-1.  The Cholesky factor has a positive
-//   diagonal, so the signs come out as required.  The step is repeated once unless the first
-//   factorisation showed the panel to be nearly orthogonal already (see k_chol_inverse).
+//   orth(columns):  a block of at most 256 columns is orthonormalised by one thread-block cluster
+//                   (orth.cu: the same recursion down to panels of 64 columns and Cholesky-QR of those);
+//                   otherwise orth(left half), project the left half out of the right half
+//                   (C = Q_l^T A_r, A_r -= Q_l C) with products over the whole GPU, orth(right half).
+// Orders below 2048 are one such block in all, second sweep and completion included.
 // Half of the floating-point work is in the two products of the top level and three quarters in
 // the top two, which is what lets the matrix unit run close to its peak.
 //
@@ -21,8 +19,8 @@
 // on its own output ("twice is enough"), which restores orthogonality to the rounding level.  The
 // second sweep is decided on the device: the first sweep compares the squared norm each column has
 // left when its panel is reached with the squared norm it started with, and clears a flag when the
-// ratio falls below 1e-8 (a column that kept less than 1e-4 of its length: one sweep then leaves an
-// orthogonality error of up to ~1e-16 * 1e4^2); every launch of the second sweep returns at once
+// ratio falls below 1e-7 (a column that kept less than 3e-4 of its length: one sweep then leaves an
+// orthogonality error of up to ~1e-16 / 1e-7); every launch of the second sweep returns at once
 // while the flag is set.
 // All reductions are done in a fixed order, so the result is bit-reproducible from run to run.
 //
@@ -36,7 +34,7 @@
 // fraction s of its length.  The caller therefore asks for this form only for a basis whose
 // previous refresh saw no column shrink below 1e-3 (cond_out), the sweep still measures the
 // shrinkage, and it runs the second (fp64) sweep already when a column keeps less than 1e-3 instead
-// of 1e-4.  The leaves (Cholesky-QR) and the power product stay in fp64.
+// of 3e-4.  The leaves (Cholesky-QR) and the power product stay in fp64.
 #include <algorithm>
 #include <cstdlib>
 #include <string>
@@ -47,150 +45,11 @@
 namespace br {
 namespace {
 
-constexpr int kB = 128;          // widest panel
-// A panel whose every column keeps at least this fraction of its squared norm against the columns
-// before it (at least 10 % of its length) needs no second Cholesky-QR pass.
-constexpr double kPassRatio = 1e-2;
-
 inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
-inline int panel_width(int64_t k) { return k >= 1024 ? 128 : 64; }
-inline int gram_splits(int64_t k) { return (int)std::min<int64_t>(64, std::max<int64_t>(1, cdiv(k, 128))); }
-inline int proj_splits_max(int64_t k) { return k >= 1024 ? 64 : 1; }
-constexpr double kIllRatio = 1e-8;   // squared-norm ratio below which the second sweep runs
-constexpr double kTcRatio = 1e-6;    // the same, when the projections ran on the tensor cores; also
-                                     // the ratio below which the next refresh must not use them
+constexpr int64_t kSplitUnit = 128;   // the recursion splits columns in multiples of this
+constexpr int kProjSplitsMax = 64;
 // sub-buffers of the work area start on 256-byte boundaries
 inline int64_t pad32(int64_t doubles) { return (doubles + 31) / 32 * 32; }
-
-// Cholesky factorisation S = R^T R of a bw x bw Gram matrix (bw <= 128) and R^-1, in one CTA.
-//
-// The matrix lives in registers: thread (ty, tx) of the 32 x 16 grid owns rows ty + 32 a (a < 4)
-// and columns tx + 16 b (b < 8), a cyclic distribution that keeps every thread busy while the
-// elimination shrinks the active part.  Row c reaches the other threads through shared memory,
-// posted by its owners at the end of step c - 1; in step c every thread derives 1 / R_cc from it
-// (redundantly, so no thread waits for another inside a step), scales the row and subtracts R_ci
-// times it from each of its rows i > c.  The same row operations applied to the identity give
-// R^-T; because column j of the Gram matrix is dead once step j is done and column j of R^-T is
-// still a unit vector until then, both share one register array: entry (i, j) holds the Gram
-// entry while j > c and the entry of R^-T afterwards.  Row c of R^-T is final after step c and is
-// written out (as column c of R^-1) straight from the scaled row.
-//
-// A pivot that underflows 1e-24 of the column's squared norm is clamped and reported as a
-// numerically rank-deficient factor.  pivot_c / S_cc is the squared sine of the angle between
-// column c and the span of the panel's columns before it.  One Cholesky-QR pass loses orthogonality
-// like cond^2 * 1e-16 with cond the condition number of the column-scaled panel; while every column
-// keeps at least kPassRatio of its squared norm, cond^2 stays (for other than contrived matrices)
-// below ~128 / kPassRatio ~ 1e4 and one pass is accurate far beyond the fp32 result, so *skip_next
-// is set and the kernels of the second pass return at once.  norm0 (optional):
-// squared norms the panel's columns had before any projection; a column that has lost more than
-// 1 - kIllRatio of it marks the input as ill-conditioned by clearing *ill_clear.
-__global__ void __launch_bounds__(512)
-k_chol_inverse(const double* __restrict__ S, int bw, double* __restrict__ Rinv, int* __restrict__ status,
-               int* __restrict__ skip_next, const int* __restrict__ skip_self,
-               const double* __restrict__ norm0, int* __restrict__ ill_clear, double ill_ratio,
-               int* __restrict__ tc_ok_clear, double* __restrict__ rdiag) {
-  if (skip_self && *skip_self) {
-    if (skip_next && threadIdx.x == 0) *skip_next = 1;
-    return;
-  }
-  __shared__ double rowS[2][kB];
-  __shared__ double diag0[kB], diag0_inv[kB], nrm_floor[kB], tc_floor[kB];
-  const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
-  if (t < kB) {
-    const double n0 = (norm0 && t < bw) ? norm0[t] : 0.0;
-    nrm_floor[t] = ill_ratio * n0;
-    tc_floor[t] = kTcRatio * n0;
-  }
-  double Z[4][8];
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int i = ty + 32 * a;
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-      const int j = tx + 16 * b;
-      const double v = (i < bw && j < bw) ? S[(int64_t)i * bw + j] : (i == j ? 1.0 : 0.0);
-      Z[a][b] = v;
-      if (i == j) { diag0[i] = v; diag0_inv[i] = v > 0.0 ? 1.0 / v : 0.0; }
-    }
-  }
-  if (ty == 0) {
-#pragma unroll
-    for (int b = 0; b < 8; ++b) rowS[0][tx + 16 * b] = Z[0][b];
-  }
-  __syncthreads();
-  double min_ratio = 1.0;    // tracked by thread 0 (every thread sees every pivot)
-  bool ill = false, tc_bad = false, any_clamped = false;
-
-  for (int c = 0; c < bw; ++c) {
-    const int buf = c & 1;
-    const double orig = diag0[c];
-    double piv = rowS[buf][c];
-    double floor_ = orig * 1e-24;
-    if (!(floor_ > 1e-300)) floor_ = 1e-300;
-    const bool clamped = !(piv > floor_);
-    if (clamped) piv = floor_;
-    if (t == 0) {
-      if (clamped) { atomicMax(status, (int)BR_WARN_RANK_DEFICIENT); any_clamped = true; }
-      min_ratio = fmin(min_ratio, piv * diag0_inv[c]);
-      // R_cc^2 of the whole factorisation is the product of this column's pivots over every pass and sweep
-      if (rdiag) rdiag[c] *= piv;
-      if (orig < nrm_floor[c]) ill = true;
-      if (orig < tc_floor[c]) tc_bad = true;
-    }
-    const double inv_d = rsqrt(piv);
-    double rj[8];
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-      const int j = tx + 16 * b;
-      rj[b] = (j == c) ? inv_d : rowS[buf][j] * inv_d;
-    }
-    // row c of R^-T is final: column c of R^-1 (zero below the diagonal)
-    if (ty == 0) {
-#pragma unroll
-      for (int b = 0; b < 8; ++b) {
-        const int j = tx + 16 * b;
-        if (j < bw) Rinv[(int64_t)j * bw + c] = (j <= c) ? rj[b] : 0.0;
-      }
-    }
-    double f[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int i = ty + 32 * a;
-      f[a] = (i > c) ? rowS[buf][i] * inv_d : 0.0;   // R_ci (row c of R, by symmetry); 0 leaves dead rows alone
-#pragma unroll
-      for (int b = 0; b < 8; ++b) Z[a][b] = fma(-f[a], rj[b], Z[a][b]);
-    }
-    // column c turns from a Gram column into a column of R^-T: entry (i, c) = -R_ci / R_cc
-    if (tx == (c & 15)) {
-      switch (c >> 4) {
-#define BR_FIX(B)                                                          \
-  case B:                                                                  \
-    _Pragma("unroll") for (int a = 0; a < 4; ++a) Z[a][B] = -f[a] * inv_d; \
-    break;
-        BR_FIX(0) BR_FIX(1) BR_FIX(2) BR_FIX(3) BR_FIX(4) BR_FIX(5) BR_FIX(6) BR_FIX(7)
-#undef BR_FIX
-      }
-    }
-    // post row c + 1 for the next step
-    if (ty == ((c + 1) & 31)) {
-      switch ((c + 1) >> 5) {
-#define BR_POST(A)                                                                          \
-  case A:                                                                                   \
-    _Pragma("unroll") for (int b = 0; b < 8; ++b) rowS[buf ^ 1][tx + 16 * b] = Z[A][b];     \
-    break;
-        BR_POST(0) BR_POST(1) BR_POST(2) BR_POST(3)
-#undef BR_POST
-      }
-    }
-    __syncthreads();
-  }
-  if (t == 0) {
-    if (skip_next) *skip_next = (min_ratio >= kPassRatio) ? 1 : 0;
-    if (ill && ill_clear) *ill_clear = 0;
-    if (tc_bad && tc_ok_clear) *tc_ok_clear = 0;
-    if (any_clamped && tc_ok_clear) tc_ok_clear[1] = 1;      // numerically rank-deficient: noted for the next refresh
-  }
-}
 
 // flags at the start of a QR: second sweep cancelled, basis well enough conditioned for the
 // tensor-core projections next time; and the copy of the latter to its long-lived home at the end
@@ -290,6 +149,8 @@ inline int64_t env_or(const char* name, int64_t dflt, int64_t lo, int64_t hi) {
 // tuning aids: BR_QR_TC_MIN_NODE (entries of the coefficient block), BR_QR_TC_MIN_ORDER
 inline int64_t tc_min_node() { static const int64_t v = env_or("BR_QR_TC_MIN_NODE", (int64_t)1 << 18, 1 << 14, (int64_t)1 << 40); return v; }
 inline int64_t tc_min_order() { static const int64_t v = env_or("BR_QR_TC_MIN_ORDER", 2048, 1024, (int64_t)1 << 30); return v; }
+// widest range of columns one cluster orthonormalises by itself
+constexpr int64_t kPartWidth = 256;
 inline bool tc_node(int64_t wp, int64_t wt) { return wp * wt >= tc_min_node(); }
 
 void enumerate_nodes(int64_t j0, int64_t w, int64_t b, std::vector<ProjNode>* out) {
@@ -448,13 +309,13 @@ cudaError_t qr_tc_power(QrTc* t, const double* Frest, const double* U, int* stat
 namespace {
 
 struct Sweep {
-  double* A; int64_t k; int b, sg, sp_max;
-  double *gram_part, *S, *Rinv, *norm0, *C, *proj_part;
+  double* A; int64_t k;
+  double *norm0, *C, *proj_part;
   double* rdiag = nullptr;    // squared diagonal of R, accumulated over passes and sweeps
-  int *skip2, *sweep2_skip;   // sweep2_skip[1] is the "tensor cores allowed next time" flag
+  int* flags;                 // [1] second sweep cancelled, [2] tensor cores allowed next time, [3] a pivot was clamped
   QrTc* tc = nullptr;         // non-null: block projections of the first sweep on the tensor cores
   int node = 0;               // running index of the projection in recursion order
-  double ill_ratio = kIllRatio;
+  double ill_ratio = kOrthIllRatio;
   int* status;
   cudaStream_t s;
   const int* skip;        // non-null: every launch of this sweep returns while *skip != 0
@@ -463,25 +324,6 @@ struct Sweep {
   double flops = 0.0;
   cudaError_t err = cudaSuccess;
 };
-
-// Cholesky-QR (at most twice) of the panel of columns [j0, j0 + bw).
-void leaf(Sweep& q, int64_t j0, int bw) {
-  double* P = q.A + j0;
-  const int64_t k = q.k;
-  for (int pass = 0; pass < 2 && q.err == cudaSuccess; ++pass) {
-    const int* skip = pass ? q.skip2 : q.skip;
-    cudaError_t e = dgemm_ex(1, 0, bw, bw, k, 1.0, P, k, P, k, 0.0, q.S, bw, q.sg, q.gram_part, skip, q.s);
-    if (e != cudaSuccess) { q.err = e; return; }
-    k_chol_inverse<<<1, 512, 0, q.s>>>(q.S, bw, q.Rinv, q.status, pass ? nullptr : q.skip2, skip,
-                                       (q.first && !pass) ? q.norm0 + j0 : nullptr, q.sweep2_skip, q.ill_ratio,
-                                       q.sweep2_skip + 1, q.rdiag ? q.rdiag + j0 : nullptr);
-    // P <- P R^-1 (in place: a CTA reads only the rows it writes, and writes after its last read)
-    e = dgemm_ex(0, 0, k, bw, bw, 1.0, P, k, q.Rinv, bw, 0.0, P, k, 1, nullptr, skip, q.s);
-    if (e != cudaSuccess) { q.err = e; return; }
-    q.launches += 3 + (q.sg > 1 ? 1 : 0);
-    if (q.first && !pass) q.flops += 4.0 * (double)k * bw * bw;
-  }
-}
 
 // A[:, jt : jt + wt] -= Q (Q^T A[:, jt : jt + wt]) with Q = A[:, jp : jp + wp] orthonormal.
 void project(Sweep& q, int64_t jp, int64_t wp, int64_t jt, int64_t wt) {
@@ -494,7 +336,7 @@ void project(Sweep& q, int64_t jp, int64_t wp, int64_t jt, int64_t wt) {
   }
   const int64_t tiles = cdiv(wp, 128) * cdiv(wt, 128);
   int sp = 1;
-  if (tiles < 148) sp = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(cdiv(296, tiles), q.sp_max), k / 128));
+  if (tiles < 148) sp = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(cdiv(296, tiles), kProjSplitsMax), k / 128));
   cudaError_t e = dgemm_ex(1, 0, wp, wt, k, 1.0, q.A + jp, k, q.A + jt, k, 0.0, q.C, wt, sp, q.proj_part, q.skip, q.s);
   if (e == cudaSuccess)
     e = dgemm_ex(0, 0, k, wt, wp, -1.0, q.A + jp, k, q.C, wt, 1.0, q.A + jt, k, 1, nullptr, q.skip, q.s);
@@ -505,24 +347,26 @@ void project(Sweep& q, int64_t jp, int64_t wp, int64_t jt, int64_t wt) {
 
 void orth(Sweep& q, int64_t j0, int64_t w) {
   if (q.err != cudaSuccess) return;
-  if (w <= q.b) { leaf(q, j0, (int)w); return; }
-  const int64_t h = cdiv(w, 2 * q.b) * q.b;     // left part: a whole number of panels
+  if (w <= kPartWidth) {
+    q.err = orth_part(q.A, q.k, j0, w, q.C, q.first ? 1 : 0, q.ill_ratio, q.norm0, q.rdiag, q.status, q.flags, q.skip, q.s);
+    q.launches += 1;
+    if (q.first) q.flops += 2.0 * (double)q.k * w * w;
+    return;
+  }
+  const int64_t h = cdiv(w, 2 * kSplitUnit) * kSplitUnit;
   orth(q, j0, h);
   project(q, j0, h, j0 + h, w - h);
   orth(q, j0 + h, w - h);
 }
 
+// a projection is split only while it has fewer than 148 tiles of 128 x 128
 inline int64_t proj_part_doubles(int64_t k) {
-  const int sp = proj_splits_max(k);
-  if (sp <= 1) return 0;
-  // a projection is split only while it has fewer than 148 tiles of 128 x 128
-  return std::min<int64_t>((int64_t)sp * ((k + 1) / 2) * ((k + 1) / 2), (int64_t)(296 + 148) * 128 * 128);
+  return std::min<int64_t>((int64_t)kProjSplitsMax * ((k + 1) / 2) * ((k + 1) / 2), (int64_t)(296 + 148) * 128 * 128);
 }
 
 }  // namespace
 
 namespace {
-constexpr double kCompletion = 1e-6;
 template <typename TQ>
 __global__ void __launch_bounds__(256)
 k_complete_columns(double* __restrict__ A, const TQ* __restrict__ Q, int64_t k, const double* __restrict__ norm2,
@@ -533,7 +377,7 @@ k_complete_columns(double* __restrict__ A, const TQ* __restrict__ Q, int64_t k, 
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t c = i % k;
     const double n2 = norm2[c];
-    const double d = n2 > 0.0 ? kCompletion * sqrt(n2) : 1.0;
+    const double d = n2 > 0.0 ? kOrthCompletion * sqrt(n2) : 1.0;
     A[i] = fma(d, (double)Q[i], A[i]);
   }
 }
@@ -562,10 +406,12 @@ cudaError_t qr_complete_columns(double* A, const float* Q, int64_t k, double* wo
   return complete_columns<float>(A, Q, k, work, status, nullptr, s);
 }
 
+bool qr_one_launch(int64_t k) { return k < tc_min_order(); }
+
 size_t qr_work_doubles(int64_t k) {
-  const int64_t b = std::min<int64_t>(panel_width(k), k);
-  return (size_t)(pad32((int64_t)gram_splits(k) * b * b) + 2 * pad32(b * b) + 64 + pad32(k) +
-                  pad32(((k + 1) / 2) * ((k + 1) / 2)) + pad32(proj_part_doubles(k)) + pad32(k));
+  const int64_t norms = (kNormChunks + 1) * k + 64;        // complete_columns
+  if (qr_one_launch(k)) return (size_t)std::max<int64_t>((int64_t)orth_work_doubles(k), norms);
+  return (size_t)(64 + pad32(k) + pad32(((k + 1) / 2) * ((k + 1) / 2)) + pad32(proj_part_doubles(k)) + pad32(k));
 }
 
 namespace {
@@ -575,19 +421,10 @@ namespace {
 cudaError_t run_qr(double* A, int64_t k, double* work, int flag_base, int* status, cudaStream_t s, const int* skip_all,
                    QrTc* tc, bool track_rdiag, int64_t* launches, double* flops) {
   Sweep q;
-  if (tc && tc->k == k) { q.tc = tc; q.ill_ratio = kTcRatio; }
+  if (tc && tc->k == k) { q.tc = tc; q.ill_ratio = kOrthTcRatio; }
   q.A = A; q.k = k; q.s = s; q.status = status;
-  q.b = (int)std::min<int64_t>(panel_width(k), k);
-  q.sg = gram_splits(k);
-  q.sp_max = proj_splits_max(k);
-  const int64_t b = q.b;
-  q.gram_part = work;
-  q.S = q.gram_part + pad32((int64_t)q.sg * b * b);
-  q.Rinv = q.S + pad32(b * b);
-  int* flags = reinterpret_cast<int*>(q.Rinv + pad32(b * b)) + flag_base;      // 64 doubles reserved for flags
-  q.skip2 = flags;
-  q.sweep2_skip = flags + 1;
-  q.norm0 = q.Rinv + pad32(b * b) + 64;
+  q.flags = reinterpret_cast<int*>(work) + flag_base;                          // 64 doubles reserved for flags
+  q.norm0 = work + 64;
   q.C = q.norm0 + pad32(k);
   q.proj_part = q.C + pad32(((k + 1) / 2) * ((k + 1) / 2));
   q.rdiag = track_rdiag ? q.proj_part + pad32(proj_part_doubles(k)) : nullptr;
@@ -599,13 +436,13 @@ cudaError_t run_qr(double* A, int64_t k, double* work, int flag_base, int* statu
     const int used = (int)cdiv(k, rows_per_chunk);
     dim3 grid((unsigned)cdiv(k, 256), (unsigned)used);
     k_column_norms_partial<<<grid, 256, 0, s>>>(A, k, rows_per_chunk, q.C, skip_all);
-    k_column_norms_sum<<<(unsigned)cdiv(k, 256), 256, 0, s>>>(q.C, k, used, q.norm0, q.sweep2_skip, q.rdiag, skip_all);
+    k_column_norms_sum<<<(unsigned)cdiv(k, 256), 256, 0, s>>>(q.C, k, used, q.norm0, q.flags + 1, q.rdiag, skip_all);
   }
   q.skip = skip_all; q.first = true;
   orth(q, 0, k);
   if (q.err != cudaSuccess) return q.err;
   // second sweep, cancelled on the device unless the first one met an ill-conditioned input
-  q.skip = q.sweep2_skip; q.first = false;
+  q.skip = q.flags + 1; q.first = false;
   orth(q, 0, k);
   if (q.err != cudaSuccess) return q.err;
   if (launches) *launches += q.launches + 2;
@@ -620,8 +457,7 @@ cudaError_t qr_pos_inplace(double* A, int64_t k, double* work, int* status, cuda
   const bool fix = Acopy != nullptr && Qprev != nullptr;
   cudaError_t e = run_qr(A, k, work, 0, status, s, nullptr, tc, fix, launches, flops);
   if (e != cudaSuccess) return e;
-  const int64_t b = std::min<int64_t>(panel_width(k), k);
-  int* flags = reinterpret_cast<int*>(work + pad32((int64_t)gram_splits(k) * b * b) + 2 * pad32(b * b));
+  int* flags = reinterpret_cast<int*>(work);
   if (fix) {
     // The oracle's rule for a rank-deficient product (decided on the diagonal of R, as the oracle decides
     // it): factorise A with 1e-6 ||A_j|| Qprev_j added to every column instead.  Everything is enqueued
@@ -631,7 +467,7 @@ cudaError_t qr_pos_inplace(double* A, int64_t k, double* work, int* status, cuda
     k_rank_decide<<<1, 256, 0, s>>>(rdiag, k, skip_fix, status, flags + 1);
     const int64_t n = k * k, blocks = cdiv(n, 256);
     k_copy_unless<<<(unsigned)(blocks < 1184 ? blocks : 1184), 256, 0, s>>>(A, Acopy, n, skip_fix);
-    if ((e = complete_columns<double>(A, Qprev, k, work, status, skip_fix, s)) != cudaSuccess) return e;
+    if ((e = complete_columns<double>(A, Qprev, k, work + 64 + pad32(k), status, skip_fix, s)) != cudaSuccess) return e;
     if ((e = run_qr(A, k, work, 8, status, s, skip_fix, nullptr, false, launches, nullptr)) != cudaSuccess) return e;
     if (launches) *launches += 5;
   }

@@ -385,6 +385,7 @@ int reexpress_chunk(Chunk& c, std::vector<Layer>& layers, const std::vector<int>
                     Launcher& lz) {
   for (int j : slots) {
     const Layer& L = layers[c.ids[j]];
+    if (lz.stats->inject()) return lz.fail("split_bf16", cudaErrorLaunchFailure);
     cudaError_t e = split_bf16(L.M, c.scr[j].B[0], c.scr[j].B[1], L.d.m * L.d.n, lz.s);
     if (e != cudaSuccess) return lz.fail("split_bf16", e);
     lz.stats->launches += 1;

@@ -1,0 +1,51 @@
+"""The one-launch factorisation Q <- qr(F Q).Q of orders below 2048, through the C-ABI (set_state, refresh_basis,
+get_state), at the orders where its tiling can go wrong: less than one panel, whole and ragged panels, one CTA
+more or less in the cluster, odd orders (8-byte instead of 16-byte copies), the product formed inside or outside
+the launch, the largest order, and the first orders that go through the chain of launches.
+
+Reference: LAPACK QR of the float64 product with a positive diagonal of R.  Both sides then round to (library) or
+start from (reference) the same fp32 inputs, so what remains is the rounding of Q to fp32 -- at most 2^-24 relative
+per entry, 6e-8 of a column's length -- and what one sweep of block Gram-Schmidt leaves when no second one runs, up
+to 1e-16 / 1e-7 = 1e-9 per column in each of up to k directions (4.5e-8 at order 2047; the factors with a strong
+signal come close to that threshold).  The asserted 1.2e-7 is their sum, rounded up."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+TOL = 1.2e-7
+
+
+def _refresh(k, F, Q0):
+    import torch
+    import paper_2602_03515_b200 as br
+    from workloads import LayerSpec
+    w = torch.zeros(k, 8, device="cuda")
+    opt = br.BasisRotation([LayerSpec("W", k, 8, br.BR_GEOM_BILATERAL, br.BR_SRC_SECOND, 0)], [w], grad_dtype="f32",
+                           gemm_prec=br.BR_GEMM_FP32, freq=10 ** 6)
+    try:
+        opt.step([torch.randn(k, 8, device="cuda") * 0.01], 0)
+        opt.set_state(0, br.BR_BUF_L, torch.from_numpy(F))
+        opt.set_state(0, br.BR_BUF_U, torch.from_numpy(Q0))
+        opt.refresh_basis(0)
+        opt.sync_status()
+        return opt.get_state(0, br.BR_BUF_U).numpy().astype(np.float64)
+    finally:
+        opt.close()
+
+
+@pytest.mark.parametrize("signal", [0.0, 300.0])      # well-conditioned: one sweep; a strong low-rank part: two
+@pytest.mark.parametrize("k", [1, 7, 8, 63, 64, 65, 127, 128, 129, 130, 255, 384, 511, 513, 1000, 1537, 2047, 2049])
+def test_order(k, signal):
+    rng = np.random.default_rng(k)
+    N = rng.standard_normal((k, k)) / np.sqrt(k)
+    F = np.eye(k) + 0.1 * (N + N.T)
+    if signal and k > 4:
+        A = signal * rng.standard_normal((k, 4)) / np.sqrt(k)
+        F += A @ A.T
+    F = F.astype(np.float32)
+    Q0 = np.linalg.qr(rng.standard_normal((k, k)))[0].astype(np.float32)
+    want, R = np.linalg.qr(F.astype(np.float64) @ Q0.astype(np.float64))
+    want *= np.sign(np.diag(R))
+    got = _refresh(k, F, Q0)
+    err = np.linalg.norm(got - want) / np.linalg.norm(want)
+    assert err <= TOL, (k, signal, err)

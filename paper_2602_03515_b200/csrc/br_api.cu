@@ -93,8 +93,9 @@ struct br_handle {
   char* slab = nullptr;
   size_t slab_bytes = 0;
   int* d_status = nullptr;
-  // scratch of the SIMT path (one layer at a time)
-  float *sG = nullptr, *sT = nullptr, *sGt = nullptr, *sMt = nullptr;
+  // scratch of the SIMT path, shared by the layers of one chunk (simt_need() floats each)
+  float* simt_scratch = nullptr;
+  size_t simt_floats = 0;
   // The refresh runs independent Power() applications (one per layer and side) on a few lanes at
   // once: lane 0 is the handle's own stream, the others are internal streams that wait for the
   // handle's stream before they start and that the handle's stream waits for when they are done.
@@ -172,12 +173,16 @@ struct Bump {
   }
 };
 
+// Scratch of one layer on the fp32 path: the gradient in fp32, the two first-side products, X.  Layers share
+// grouped launches as far as 64 MiB of it go (one layer alone takes what it needs).
+inline size_t simt_need(const Layer& L) { return 4 * (((size_t)L.d.m * L.d.n + 63) / 64 * 64); }
+constexpr size_t kSimtScratch = 16u << 20;
+
 // Lays out every buffer of the handle in one slab.  With base == nullptr only sizes are computed.
 void layout(br_handle* h, Bump& b, Sizes* sz) {
   const br_hparams& hp = h->hp;
   if (hp.flags & BR_FLAG_DEBUG_CANARY) { b.guard = kAlign; b.guards = &h->guard_offsets; h->guard_offsets.clear(); }
-  size_t max_numel = 0, max_k = 0, max_z = 0, n_sides = 0;
-  bool any_simt = false;
+  size_t simt_max = 0, simt_total = 0, max_k = 0, max_z = 0, n_sides = 0;
   for (Layer& L : h->layers) {
     const size_t mn = (size_t)L.d.m * L.d.n;
     L.M = b.take<float>(mn);
@@ -200,17 +205,15 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
       L.ring = b.take<char>(L.slot_stride * (size_t)L.ring_slots);
     }
     if (L.d.geom != BR_GEOM_NONE) {
-      if (!L.use_tc) { any_simt = true; max_numel = std::max(max_numel, mn); }
+      if (!L.use_tc) { simt_max = std::max(simt_max, simt_need(L)); simt_total += simt_need(L); }
       if (L.left) { max_k = std::max(max_k, (size_t)L.d.m); ++n_sides; }
       if (L.right) { max_k = std::max(max_k, (size_t)L.d.n); ++n_sides; }
       if (!second) max_z = std::max(max_z, mn);
     }
   }
-  if (any_simt) {
-    h->sG = b.take<float>(max_numel);
-    h->sT = b.take<float>(max_numel);
-    h->sGt = b.take<float>(max_numel);
-    h->sMt = b.take<float>(max_numel);
+  if (simt_total) {
+    h->simt_floats = std::max(simt_max, std::min(simt_total, kSimtScratch));
+    h->simt_scratch = b.take<float>(h->simt_floats);
   }
   h->tcq_bytes = 0;
   for (const Layer& L : h->layers) {
@@ -423,15 +426,11 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
   QrTc* tcq = nullptr;
   if (L.use_tc && (h->cond_known[ci] & 1) && !complete)
     for (QrTc* t : ln.tcq) if (qr_tc_order(t) == k) tcq = t;
-  // a small order is factorised in one launch of one cluster; with the smallest the product goes along
-  const bool one = qr_one_launch(k);
-  const bool fold = one && k <= kOrthFoldedProduct && L.d.src == BR_SRC_SECOND && !complete;
+  const bool one = qr_one_launch(k);      // a small order is factorised in one launch of one cluster
   const float* F = left_side ? L.L : L.R;
   for (int it = 0; it < h->hp.power_iters; ++it) {
     if (!one) { BR_CUDA(h, f32_to_f64(Q, ln.rQ, k * k, s)); count(h); }       // the current basis, for the product and its completion
-    if (fold) {
-      // inside the launch below
-    } else if (L.d.src == BR_SRC_SECOND) {
+    if (L.d.src == BR_SRC_SECOND) {
       if (tcq) {
         // widen once, then fp64 products (the products of fp32 values are exact either way)
         BR_CUDA(h, f32_to_f64(F, ln.rF, k * k, s));
@@ -471,9 +470,9 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
     // product, for which it needs the product once more (the factor's buffer is free by now) and the
     // current basis.
     if (one) {
-      BR_CUDA(h, orth_whole(ln.rA, k, ln.rWork, fold ? F : nullptr, Q, ln.rF, Q, Q, left_side ? L.Uh : L.Vh,
-                            left_side ? L.Ul : L.Vl, h->d_status, h->d_cond + ci, s));
-      count(h); h->stats.gemm_flops += (fold ? 4.0 : 2.0) * k * k * k;
+      BR_CUDA(h, orth_whole(ln.rA, k, ln.rWork, ln.rF, Q, Q, left_side ? L.Uh : L.Vh, left_side ? L.Ul : L.Vl,
+                            h->d_status, h->d_cond + ci, s));
+      count(h); h->stats.gemm_flops += 2.0 * k * k * k;
       continue;
     }
     BR_CUDA(h, cudaMemcpyAsync(ln.rF, ln.rA, sizeof(double) * (size_t)k * (size_t)k, cudaMemcpyDeviceToDevice, s));
@@ -561,33 +560,13 @@ br_status refresh_layers(br_handle* h, const int* ids, int n_ids) {
   if (failed != BR_OK) return failed;
   h->stats.prof.end(span, h->stream, h->stats.gemm_flops - f0);
   BR_CUDA(h, cudaMemcpyAsync(h->h_cond, h->d_cond, sizeof(int) * h->cond_known.size(), cudaMemcpyDeviceToHost, h->stream));
+  count(h);
   BR_CUDA(h, cudaEventRecord(h->ev_cond, h->stream));
   h->cond_pending = true;
   for (int j = 0; j < n_ids; ++j) {
     Layer& L = h->layers[ids[j]];
     if (L.left || L.right) L.refresh_count += 1;
   }
-  return BR_OK;
-}
-
-br_status refresh_layer(br_handle* h, Layer& L) {
-  const int id = (int)(&L - h->layers.data());
-  return refresh_layers(h, &id, 1);
-}
-
-// L <- beta L + (1-beta) G G^T ; R <- beta R + (1-beta) G^T G   (Alg. 2), fp32 FFMA
-br_status accumulate_factors_simt(br_handle* h, Layer& L, const float* G) {
-  const float beta = h->hp.beta_factor < 0.f ? h->hp.beta2 : h->hp.beta_factor;
-  const int64_t m = L.d.m, n = L.d.n;
-  if (L.L) {
-    BR_CUDA(h, sgemm(0, 1, m, m, n, 1.0f - beta, G, n, G, n, beta, L.L, m, h->stream));
-    count(h); h->stats.gemm_flops += 2.0 * m * m * n;
-  }
-  if (L.R) {
-    BR_CUDA(h, sgemm(1, 0, n, n, m, 1.0f - beta, G, n, G, n, beta, L.R, n, h->stream));
-    count(h); h->stats.gemm_flops += 2.0 * n * n * m;
-  }
-  L.n_accum += 1;
   return BR_OK;
 }
 
@@ -639,47 +618,97 @@ void tmp_free(br_handle* h, void* p) {
   if (h->alloc.alloc) h->alloc.free(p, h->alloc.ctx); else cudaFree(p);
 }
 
-// One update of one layer on the accurate (fp32 FFMA) path.  G: the gradient to apply.
-br_status update_layer_simt(br_handle* h, Layer& L, const void* G, const float* gscale) {
+// One update of the given layers on the accurate (fp32 FFMA) path, phase by phase, each phase one grouped
+// launch: a layer of this path alone neither fills the GPU nor outlasts a launch.  G[i] / GS[i]: the gradient
+// layer i applies and its clipping factor.
+br_status update_layers_simt(br_handle* h, const std::vector<int>& ids, const std::vector<const void*>& G,
+                             const std::vector<const float*>& GS) {
   const br_hparams& hp = h->hp;
   cudaStream_t s = h->stream;
-  const int64_t m = L.d.m, n = L.d.n, mn = m * n;
-  const int bf = L.d.grad_dtype == BR_BF16;
-  br_status st;
-  // Alg. 1 (momentum update) (and widen a bf16 gradient once)
-  // (a clipped gradient is materialised in fp32 too: everything below works on the scaled values)
-  const bool copy = bf || gscale != nullptr;
-  BR_CUDA(h, ema_momentum(L.M, G, bf, mn, hp.beta1, copy ? h->sG : nullptr, nullptr, nullptr, gscale, s));
-  count(h);
-  const float* G32 = copy ? h->sG : reinterpret_cast<const float*>(G);
-  const bool second = L.d.src == BR_SRC_SECOND;
-  if (second && hp.accum == BR_ACCUM_EVERY_STEP && (st = accumulate_factors_simt(h, L, G32)) != BR_OK) return st;
-  // Alg. 1 (periodic refresh)
-  if (L.t % L.freq == 0) {
-    if (second && hp.accum == BR_ACCUM_ON_REFRESH && (st = accumulate_factors_simt(h, L, G32)) != BR_OK) return st;
-    if ((st = refresh_layer(h, L)) != BR_OK) return st;
+  const float beta_f = hp.beta_factor < 0.f ? hp.beta2 : hp.beta_factor, decay = 1.0f - hp.lr * hp.weight_decay;
+  struct Work { Layer* L; const float* G; float *T, *Tm, *X; };
+  std::vector<Work> work;
+  std::vector<EmaJob> ema;
+  std::vector<int> due;
+  std::vector<SimtProblem> factors, first, dual, back, write;
+  auto group = [&](std::vector<SimtProblem>& v, bool is_dual) -> br_status {
+    if (v.empty()) return BR_OK;
+    BR_CUDA(h, simt_group(v.data(), (int)v.size(), is_dual, s));
+    count(h, ((int)v.size() + 31) / 32);
+    for (const SimtProblem& p : v) h->stats.gemm_flops += (is_dual ? 4.0 : 2.0) * p.M * p.N * p.K;
+    return BR_OK;
+  };
+  auto flush = [&]() -> br_status {
+    if (work.empty()) return BR_OK;
+    br_status st;
+    BR_CUDA(h, ema_momentum(ema.data(), (int)ema.size(), hp.beta1, s));      // Alg. 1 (momentum update)
+    count(h, ((int)ema.size() + 31) / 32);
+    for (const Work& w : work) {
+      Layer& L = *w.L;
+      const int64_t m = L.d.m, n = L.d.n;
+      // L <- beta L + (1-beta) G G^T ; R <- beta R + (1-beta) G^T G   (Alg. 2)
+      const bool is_due = L.t % L.freq == 0;
+      if (L.d.src == BR_SRC_SECOND && (hp.accum == BR_ACCUM_EVERY_STEP || is_due)) {
+        if (L.L) factors.push_back(simt_problem(0, 1, m, m, n, 1.0f - beta_f, w.G, n, w.G, n, beta_f, L.L, m));
+        if (L.R) factors.push_back(simt_problem(1, 0, n, n, m, 1.0f - beta_f, w.G, n, w.G, n, beta_f, L.R, n));
+        L.n_accum += 1;
+      }
+      if (is_due) due.push_back((int)(w.L - h->layers.data()));
+    }
+    if (!due.empty()) {                                                      // Alg. 1 (periodic refresh)
+      if ((st = group(factors, false)) != BR_OK) return st;
+      factors.clear();
+      if ((st = refresh_layers(h, due.data(), (int)due.size())) != BR_OK) return st;
+    }
+    for (const Work& w : work) {
+      Layer& L = *w.L;
+      const int64_t m = L.d.m, n = L.d.n;
+      // Alg. 1 (rotation of G and M): the first side, beside the factors; then the second with the second-moment
+      // update and the scaling in its epilogue, X = M~ / sqrt(V~ + eps)
+      SimtProblem q;
+      if (L.left && L.right) {
+        first.push_back(simt_problem(1, 0, m, n, m, 1.f, L.U, m, w.G, n, 0.f, w.T, n));
+        first.push_back(simt_problem(1, 0, m, n, m, 1.f, L.U, m, L.M, n, 0.f, w.Tm, n));
+        q = simt_problem(0, 0, m, n, n, 1.0f - hp.beta2, w.T, n, L.V, n, hp.beta2, w.X, n);
+        q.A[1] = w.Tm;
+        back.push_back(simt_problem(0, 0, m, n, m, 1.f, L.U, m, w.X, n, 0.f, w.T, n));
+        write.push_back(simt_problem(0, 1, m, n, n, -hp.lr, w.T, n, L.V, n, decay, L.d.weight, n));
+      } else if (L.left) {
+        q = simt_problem(1, 0, m, n, m, 1.0f - hp.beta2, L.U, m, w.G, n, hp.beta2, w.X, n);
+        q.B[1] = L.M;
+        write.push_back(simt_problem(0, 0, m, n, m, -hp.lr, L.U, m, w.X, n, decay, L.d.weight, n));
+      } else {
+        q = simt_problem(0, 0, m, n, n, 1.0f - hp.beta2, w.G, n, L.V, n, hp.beta2, w.X, n);
+        q.A[1] = L.M;
+        write.push_back(simt_problem(0, 1, m, n, n, -hp.lr, w.X, n, L.V, n, decay, L.d.weight, n));
+      }
+      q.V2 = L.V2; q.eps = hp.eps;
+      dual.push_back(q);
+    }
+    factors.insert(factors.end(), first.begin(), first.end());
+    if ((st = group(factors, false)) != BR_OK || (st = group(dual, true)) != BR_OK || (st = group(back, false)) != BR_OK ||
+        (st = group(write, false)) != BR_OK)                                 // W <- (1 - eta lambda) W - eta U X V^T
+      return st;
+    work.clear(); ema.clear(); due.clear(); factors.clear(); first.clear(); dual.clear(); back.clear(); write.clear();
+    return BR_OK;
+  };
+  size_t used = 0;
+  for (int i : ids) {
+    Layer& L = h->layers[i];
+    if (used + simt_need(L) > h->simt_floats) {
+      const br_status st = flush();
+      if (st != BR_OK) return st;
+      used = 0;
+    }
+    const size_t part = simt_need(L) / 4;
+    float* base = h->simt_scratch + used;
+    used += 4 * part;
+    // a bf16 gradient is widened once, and a clipped one is materialised too: everything works on the scaled values
+    const bool bf = L.d.grad_dtype == BR_BF16, copy = bf || GS[i] != nullptr;
+    work.push_back({&L, copy ? base : reinterpret_cast<const float*>(G[i]), base + part, base + 2 * part, base + 3 * part});
+    ema.push_back({L.M, G[i], copy ? base : nullptr, GS[i], L.d.m * L.d.n, bf ? 1 : 0});
   }
-  // Alg. 1 (rotation of G and M)
-  if ((st = rotate_simt(h, L, G32, h->sT, h->sGt)) != BR_OK) return st;
-  if ((st = rotate_simt(h, L, L.M, h->sT, h->sMt)) != BR_OK) return st;
-  // second-moment update and scaling, element-wise part: X overwrites sMt
-  BR_CUDA(h, second_moment_scale(L.V2, h->sGt, h->sMt, mn, hp.beta2, hp.eps, s));
-  count(h);
-  // weight update: W <- (1 - eta lambda) W - eta U X V^T
-  const float decay = 1.0f - hp.lr * hp.weight_decay;
-  float* W = L.d.weight;
-  if (L.left && L.right) {
-    BR_CUDA(h, sgemm(0, 0, m, n, m, 1.f, L.U, m, h->sMt, n, 0.f, h->sT, n, s));
-    BR_CUDA(h, sgemm(0, 1, m, n, n, -hp.lr, h->sT, n, L.V, n, decay, W, n, s));
-    count(h, 2); h->stats.gemm_flops += 2.0 * m * n * (m + n);
-  } else if (L.left) {
-    BR_CUDA(h, sgemm(0, 0, m, n, m, -hp.lr, L.U, m, h->sMt, n, decay, W, n, s));
-    count(h); h->stats.gemm_flops += 2.0 * m * n * m;
-  } else {
-    BR_CUDA(h, sgemm(0, 1, m, n, n, -hp.lr, h->sMt, n, L.V, n, decay, W, n, s));
-    count(h); h->stats.gemm_flops += 2.0 * m * n * n;
-  }
-  return BR_OK;
+  return flush();
 }
 
 br_status check_handle(br_handle* h) {
@@ -957,6 +986,7 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
   }
   // ---- enqueue the updates ----------------------------------------------------------------
   const br_hparams& hp = h->hp;
+  std::vector<int> simt_ids;
   for (int i = 0; i < nl; ++i) {
     Layer& L = h->layers[i];
     if (!G[i]) continue;
@@ -977,11 +1007,12 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
         h->stats.gemm_flops += (acc ? 2.0 : 0.0) * ((L.L ? m * m * n : 0) + (L.R ? n * n * m : 0)) +
                                6.0 * m * n * ((L.left ? m : 0) + (L.right ? n : 0));
         if (acc) L.n_accum += 1;
-      } else if ((st = update_layer_simt(h, L, G[i], GS[i])) != BR_OK) {
-        return st;
+      } else {
+        simt_ids.push_back(i);
       }
     }
   }
+  if (!simt_ids.empty() && (st = update_layers_simt(h, simt_ids, G, GS)) != BR_OK) return st;
   if (h->tc) {
     struct StepCtx { br_handle* h; const void* const* grads; std::vector<char>* stored; bool copied; };
     StepCtx sc{h, grads, &stored, false};

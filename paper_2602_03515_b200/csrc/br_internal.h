@@ -64,11 +64,14 @@ struct LaunchStats {
 // ---------------------------------------------------------------------------------------------
 cudaError_t set_identity(float* Q, int64_t k, cudaStream_t s);
 
-// Alg. 1 (momentum update): M <- beta1 M + (1-beta1) G.  G is fp32 or bf16 (g_is_bf16).  Optional outputs:
-// Gf32 (G widened to fp32), Mh/Ml (bf16 hi/lo split of the new M).
-// gscale (optional, DEVICE): clipping factor the gradient is multiplied by
-cudaError_t ema_momentum(float* M, const void* G, int g_is_bf16, int64_t numel, float beta1,
-                         float* Gf32, __nv_bfloat16* Mh, __nv_bfloat16* Ml, const float* gscale, cudaStream_t s);
+// Alg. 1 (momentum update): M <- beta1 M + (1-beta1) G for a group of matrices in one launch per 32 of them.
+// G is fp32 or bf16; gscale (optional, DEVICE): clipping factor the gradient is multiplied by; Gf32
+// (optional): the gradient as it was applied, in fp32.
+struct EmaJob {
+  float* M; const void* G; float* Gf32; const float* gscale;
+  int64_t numel; int g_is_bf16;
+};
+cudaError_t ema_momentum(const EmaJob* jobs, int n, float beta1, cudaStream_t s);
 // Global-norm clipping factor of one call: *out = min(1, clip / ||all gradients||_2).  part: scratch of
 // 296 * ceil(n / 64) doubles.  Fixed summation order.
 cudaError_t clip_factor(const void* const* grads, const int64_t* numel, const int* is_bf16, int n, float clip,
@@ -77,11 +80,6 @@ cudaError_t clip_factor(const void* const* grads, const int64_t* numel, const in
 // Eq. (adam): plain Adam, eps inside the sqrt, no bias correction, decoupled weight decay.
 cudaError_t plain_adam(float* W, float* M, float* V, const void* G, int g_is_bf16, int64_t numel,
                        float lr, float beta1, float beta2, float eps, float wd, const float* gscale, cudaStream_t s);
-
-// Alg. 1 (second-moment update and scaling) (element-wise part): V~ <- beta2 V~ + (1-beta2) G~^2 ; X = M~/sqrt(V~+eps).
-// X overwrites Mt.
-cudaError_t second_moment_scale(float* V2, const float* Gt, float* Mt, int64_t numel, float beta2,
-                                float eps, cudaStream_t s);
 
 // fp32 -> bf16 hi (+ optional lo = bf16(x - hi)).
 cudaError_t split_bf16(const float* X, __nv_bfloat16* hi, __nv_bfloat16* lo, int64_t numel,
@@ -116,6 +114,19 @@ cudaError_t guard_check(const char* slab, const unsigned long long* offs, int n,
 // SIMT contractions (gemm_simt.cu):  C = alpha * op(A) op(B) + beta * C, row-major.
 // op(X) = X or X^T (ta / tb).  M, N, K are the dimensions of the product.
 // ---------------------------------------------------------------------------------------------
+// One product of a grouped launch.  A launch is either of plain products (A[0], B[0]) or of dual ones: with
+// g = op(A[0]) op(B[0]) and m = op(A[1]) op(B[1]), V2 <- beta V2 + alpha g^2 and C <- m / sqrt(V2 + eps)
+// (Alg. 1 (second-moment update and scaling), without either product in memory).
+struct SimtProblem {
+  const float *A[2], *B[2];
+  float *C, *V2;
+  int32_t M, N, K, lda, ldb, ldc, ta, tb;
+  float alpha, beta, eps;
+};
+SimtProblem simt_problem(int ta, int tb, int64_t M, int64_t N, int64_t K, float alpha, const float* A, int64_t lda, const float* B,
+                         int64_t ldb, float beta, float* C, int64_t ldc);
+// All problems in one launch per 32 of them; they must be independent of one another.
+cudaError_t simt_group(const SimtProblem* problems, int n, bool dual, cudaStream_t s);
 cudaError_t sgemm(int ta, int tb, int64_t M, int64_t N, int64_t K, float alpha, const float* A,
                   int64_t lda, const float* B, int64_t ldb, float beta, float* C, int64_t ldc,
                   cudaStream_t s);
@@ -148,20 +159,21 @@ constexpr double kOrthIllRatio = 1e-7;
 constexpr double kOrthTcRatio = 1e-6;      // the same, when the projections ran on the tensor cores; also
                                            // the ratio below which the next refresh must not use them
 constexpr double kOrthCompletion = 1e-6;   // a deficient column j is completed by this times its length times Q_j
-// Up to this order the product F Q is formed inside the factorisation's launch: the cluster's few SMs take
-// about as long for it (17 us at 128) as a launch of its own; above, the rest of the GPU is missed.
-constexpr int64_t kOrthFoldedProduct = 128;
-// The whole factorisation of a k x k product in one launch.  A: the product (overwritten), or, with F and Q0
-// (fp32), the buffer it is formed in.  Acopy / Qprev (both or none): as for qr_pos_inplace, the copy is made
-// here.  Results: Qout (fp32) and, optionally, its bf16 hi/lo pair; *cond_out as for qr_pos_inplace with
+// The whole factorisation of a k x k product A (overwritten) in one launch.  Acopy / Qprev (both or none): as
+// for qr_pos_inplace, the copy is made here.  Results: Qout (fp32) and, optionally, its bf16 hi/lo pair; *cond_out as for qr_pos_inplace with
 // bit 1 set when the product was numerically rank-deficient.  work: orth_work_doubles(k).
 size_t orth_work_doubles(int64_t k);
-cudaError_t orth_whole(double* A, int64_t k, double* work, const float* F, const float* Q0, double* Acopy, const float* Qprev,
+cudaError_t orth_whole(double* A, int64_t k, double* work, double* Acopy, const float* Qprev,
                        float* Qout, __nv_bfloat16* Qh, __nv_bfloat16* Ql, int* status, int* cond_out, cudaStream_t s);
 // Columns [j0, j0 + w) only, as a part of one sweep of qr_pos_inplace (whose flag words `flags` are).
 // C: room for the largest coefficient block, (w / 2)^2 doubles.
 cudaError_t orth_part(double* A, int64_t k, int64_t j0, int64_t w, double* C, int first, double ill_ratio, const double* norm0,
                       double* rdiag, int* status, int* flags, const int* skip, cudaStream_t s);
+// C = alpha op(A) B + beta C with fp64 accumulation and output, in tiles of 64 x 64.
+cudaError_t product64(int ta, int64_t M, int64_t N, int64_t K, double alpha, const float* A, int64_t lda, const float* B,
+                      int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t s);
+cudaError_t product64(int ta, int64_t M, int64_t N, int64_t K, double alpha, const float* A, int64_t lda, const double* B,
+                      int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t s);
 
 // ---------------------------------------------------------------------------------------------
 // QR with positive diagonal in fp64 (qr.cu).  A (k x k, row-major, ld = k) is overwritten by

@@ -72,45 +72,44 @@ __global__ void k_set_identity(float* Q, int64_t k) {
   }
 }
 
+constexpr int kMaxEmaJobs = 32;
+struct EmaArgs {                  // passed by value
+  EmaJob j[kMaxEmaJobs];
+  int block_begin[kMaxEmaJobs + 1];
+  int n;
+};
+
 template <bool G_BF16>
-__global__ void __launch_bounds__(kThreads)
-k_ema_momentum(float* __restrict__ M, const void* __restrict__ G, int64_t numel, float beta1,
-               float* __restrict__ Gf32, __nv_bfloat16* __restrict__ Mh,
-               __nv_bfloat16* __restrict__ Ml, const float* __restrict__ gscale) {
-  const float gs = gscale ? *gscale : 1.0f;     // clipping factor of the call this gradient came with
+__device__ __forceinline__ void ema_one(const EmaJob& j, int block, int blocks, float beta1) {
+  const float gs = j.gscale ? *j.gscale : 1.0f;     // clipping factor of the call this gradient came with
   const float omb = 1.0f - beta1;
-  const int64_t nvec = numel >> 2;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nvec; v += stride) {
+  const int64_t nvec = j.numel >> 2, stride = (int64_t)blocks * kThreads;
+  for (int64_t v = block * (int64_t)kThreads + threadIdx.x; v < nvec; v += stride) {
     const int64_t i = v << 2;
-    float4 g = load_grad4<G_BF16>(G, i);
+    float4 g = load_grad4<G_BF16>(j.G, i);
     g.x *= gs; g.y *= gs; g.z *= gs; g.w *= gs;
-    float4 m = ld4(M + i);
+    float4 m = ld4(j.M + i);
     m.x = beta1 * m.x + omb * g.x;
     m.y = beta1 * m.y + omb * g.y;
     m.z = beta1 * m.z + omb * g.z;
     m.w = beta1 * m.w + omb * g.w;
-    st4(M + i, m);
-    if (Gf32) st4(Gf32 + i, g);
-    if (Mh) {
-      float4 h = make_float4(bf16_round(m.x), bf16_round(m.y), bf16_round(m.z), bf16_round(m.w));
-      st4_bf16(Mh + i, h);
-      if (Ml) st4_bf16(Ml + i, make_float4(m.x - h.x, m.y - h.y, m.z - h.z, m.w - h.w));
-    }
+    st4(j.M + i, m);
+    if (j.Gf32) st4(j.Gf32 + i, g);
   }
   // ragged tail (numel not a multiple of 4)
-  for (int64_t i = (nvec << 2) + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < numel;
-       i += stride) {
-    float g = gs * load_grad1<G_BF16>(G, i);
-    float m = beta1 * M[i] + omb * g;
-    M[i] = m;
-    if (Gf32) Gf32[i] = g;
-    if (Mh) {
-      float h = bf16_round(m);
-      Mh[i] = __float2bfloat16_rn(m);
-      if (Ml) Ml[i] = __float2bfloat16_rn(m - h);
-    }
+  for (int64_t i = (nvec << 2) + block * (int64_t)kThreads + threadIdx.x; i < j.numel; i += stride) {
+    const float g = gs * load_grad1<G_BF16>(j.G, i);
+    j.M[i] = beta1 * j.M[i] + omb * g;
+    if (j.Gf32) j.Gf32[i] = g;
   }
+}
+
+// The momentum EMA of every layer of the fp32 path: blocks are dealt to the layers in proportion to their size.
+__global__ void __launch_bounds__(kThreads) k_ema_momentum(const __grid_constant__ EmaArgs a, float beta1) {
+  int i = 0;
+  while (i + 1 < a.n && (int)blockIdx.x >= a.block_begin[i + 1]) ++i;
+  const int block = (int)blockIdx.x - a.block_begin[i], blocks = a.block_begin[i + 1] - a.block_begin[i];
+  if (a.j[i].g_is_bf16) ema_one<true>(a.j[i], block, blocks, beta1); else ema_one<false>(a.j[i], block, blocks, beta1);
 }
 
 template <bool G_BF16>
@@ -145,31 +144,6 @@ k_plain_adam(float* __restrict__ W, float* __restrict__ M, float* __restrict__ V
     M[i] = m;
     V[i] = s;
     W[i] = decay * W[i] - lr * (m / sqrtf(s + eps));
-  }
-}
-
-__global__ void __launch_bounds__(kThreads)
-k_second_moment_scale(float* __restrict__ V2, const float* __restrict__ Gt, float* __restrict__ Mt,
-                      int64_t numel, float beta2, float eps) {
-  const float omb2 = 1.0f - beta2;
-  const int64_t nvec = numel >> 2;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nvec; v += stride) {
-    const int64_t i = v << 2;
-    float4 g = ld4(Gt + i), s = ld4(V2 + i), m = ld4(Mt + i);
-    s.x = beta2 * s.x + omb2 * g.x * g.x;  m.x = m.x / sqrtf(s.x + eps);
-    s.y = beta2 * s.y + omb2 * g.y * g.y;  m.y = m.y / sqrtf(s.y + eps);
-    s.z = beta2 * s.z + omb2 * g.z * g.z;  m.z = m.z / sqrtf(s.z + eps);
-    s.w = beta2 * s.w + omb2 * g.w * g.w;  m.w = m.w / sqrtf(s.w + eps);
-    st4(V2 + i, s);
-    st4(Mt + i, m);
-  }
-  for (int64_t i = (nvec << 2) + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < numel;
-       i += stride) {
-    float g = Gt[i];
-    float s = beta2 * V2[i] + omb2 * g * g;
-    V2[i] = s;
-    Mt[i] = Mt[i] / sqrtf(s + eps);
   }
 }
 
@@ -325,14 +299,22 @@ cudaError_t set_identity(float* Q, int64_t k, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t ema_momentum(float* M, const void* G, int g_is_bf16, int64_t numel, float beta1,
-                         float* Gf32, __nv_bfloat16* Mh, __nv_bfloat16* Ml, const float* gscale, cudaStream_t s) {
-  int grid = grid_for((numel + 3) / 4);
-  if (g_is_bf16)
-    k_ema_momentum<true><<<grid, kThreads, 0, s>>>(M, G, numel, beta1, Gf32, Mh, Ml, gscale);
-  else
-    k_ema_momentum<false><<<grid, kThreads, 0, s>>>(M, G, numel, beta1, Gf32, Mh, Ml, gscale);
-  return cudaGetLastError();
+cudaError_t ema_momentum(const EmaJob* jobs, int n, float beta1, cudaStream_t s) {
+  EmaArgs a;
+  for (int at = 0; at < n; at += kMaxEmaJobs) {
+    a.n = n - at < kMaxEmaJobs ? n - at : kMaxEmaJobs;
+    int blocks = 0;
+    for (int i = 0; i < a.n; ++i) {
+      a.j[i] = jobs[at + i];
+      a.block_begin[i] = blocks;
+      blocks += grid_for((a.j[i].numel + 3) / 4);
+    }
+    a.block_begin[a.n] = blocks;
+    k_ema_momentum<<<blocks, kThreads, 0, s>>>(a, beta1);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t plain_adam(float* W, float* M, float* V, const void* G, int g_is_bf16, int64_t numel,
@@ -343,12 +325,6 @@ cudaError_t plain_adam(float* W, float* M, float* V, const void* G, int g_is_bf1
     k_plain_adam<true><<<grid, kThreads, 0, s>>>(W, M, V, G, numel, lr, beta1, beta2, eps, decay, gscale);
   else
     k_plain_adam<false><<<grid, kThreads, 0, s>>>(W, M, V, G, numel, lr, beta1, beta2, eps, decay, gscale);
-  return cudaGetLastError();
-}
-
-cudaError_t second_moment_scale(float* V2, const float* Gt, float* Mt, int64_t numel, float beta2,
-                                float eps, cudaStream_t s) {
-  k_second_moment_scale<<<grid_for((numel + 3) / 4), kThreads, 0, s>>>(V2, Gt, Mt, numel, beta2, eps);
   return cudaGetLastError();
 }
 

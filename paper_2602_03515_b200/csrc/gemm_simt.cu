@@ -1,111 +1,187 @@
-// SIMT (FFMA) contractions: the accurate fp32 path.  Used for BR_GEMM_FP32 and for layers whose
+// Grouped fp32 (FFMA) contractions: the accurate path.  Used for BR_GEMM_FP32 and for layers whose
 // shapes the tensor-core tiles do not take.  (The fp64 contractions of the basis refresh live in
-// dgemm.cu.)
+// dgemm.cu and orth.cu.)
 //
-// C = alpha * op(A) op(B) + beta * C, all row-major.  op(A) is M x K, op(B) is K x N.
+//   C = alpha * op(A) op(B) + beta * C, all row-major, op(A) M x K, op(B) K x N
+//
+// or, DUAL, two products with the same shapes whose tiles meet in one epilogue (the rotated gradient and
+// the rotated momentum, see SimtProblem).  One launch covers the same phase of every layer of a handle: the
+// matrices of this path are small, and a launch of their own for each product left most SMs idle and cost
+// 40 us for what a CTA computes in 10 (four ragged layers of 37 x 53 to 333 x 257: 1.1 ms an update as 40
+// launches, of which 1.0 ms in the products).
+//
+// A CTA computes one tile; the next 16 steps of the contraction are fetched into registers while the
+// current ones are multiplied out of shared memory, and every entry is one chain of fused multiply-adds in
+// the order of the contraction.  The tile follows from the work of the launch: 32 x 32 on 64 threads while
+// those tiles fit on the GPU at once (the time is then that of one tile's chain, and a small tile's step is
+// the shortest), 64 x 64 up to a few waves, 128 x 128 (8 x 8 per thread, half the shared-memory reads per
+// multiply-add) above.
 #include "br_internal.h"
 #include "step_tc.h"
 
 namespace br {
 namespace {
 
-template <typename TA, typename TB, typename TC, int BM, int BN, int BK, int TM, int TN>
+constexpr int BK = 16;
+constexpr int kMaxProblems = 32;      // by value: 3.2 KB of launch parameters
+
+struct GroupArgs {
+  SimtProblem p[kMaxProblems];
+  int tile_begin[kMaxProblems + 1];
+  int n;
+};
+
+template <int BM, int BN, int TM, int TN, bool DUAL>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
-k_gemm(int ta, int tb, int64_t M, int64_t N, int64_t K, TC alpha, const TA* __restrict__ A,
-       int64_t lda, const TB* __restrict__ B, int64_t ldb, TC beta, TC* __restrict__ C,
-       int64_t ldc) {
-  constexpr int NT = (BM / TM) * (BN / TN);
-  constexpr int PAD = 4;
-  __shared__ TC As[BK][BM + PAD];
-  __shared__ TC Bs[BK][BN + PAD];
+k_simt_group(const __grid_constant__ GroupArgs ga) {
+  constexpr int NT = (BM / TM) * (BN / TN), NP = DUAL ? 2 : 1;
+  constexpr int LA = BM * BK / NT, LB = BN * BK / NT;
+  __shared__ __align__(16) float As[NP][BK][BM + 4];
+  __shared__ __align__(16) float Bs[NP][BK][BN + 4];
+  int pi = 0;
+  while (pi + 1 < ga.n && (int)blockIdx.x >= ga.tile_begin[pi + 1]) ++pi;
+  const SimtProblem& p = ga.p[pi];
+  const int tiles_n = (p.N + BN - 1) / BN, tile = (int)blockIdx.x - ga.tile_begin[pi];
+  const int m0 = tile / tiles_n * BM, n0 = tile % tiles_n * BN;
+  const int M = p.M, N = p.N, K = p.K;
+  const int t = threadIdx.x, tx = t % (BN / TN), ty = t / (BN / TN);
 
-  const int t = threadIdx.x;
-  const int tx = t % (BN / TN), ty = t / (BN / TN);
-  const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
-
-  TC acc[TM][TN];
+  float ra[NP][LA], rb[NP][LB];
+  auto fetch = [&](int k0) {
 #pragma unroll
-  for (int i = 0; i < TM; ++i)
+    for (int u = 0; u < LA; ++u) {
+      const int idx = t + u * NT;
+      const int i = p.ta ? idx % BM : idx / BK, kk = p.ta ? idx / BM : idx % BK;
+      const bool ok = m0 + i < M && k0 + kk < K;
+      const int64_t at = p.ta ? (int64_t)(k0 + kk) * p.lda + m0 + i : (int64_t)(m0 + i) * p.lda + k0 + kk;
 #pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = TC(0);
-
-  for (int64_t k0 = 0; k0 < K; k0 += BK) {
-    // ---- stage op(A)[m0:m0+BM, k0:k0+BK] as As[kk][i] --------------------------------------
-#pragma unroll 1
-    for (int idx = t; idx < BM * BK; idx += NT) {
-      int i, kk;
-      if (ta) { i = idx % BM; kk = idx / BM; } else { kk = idx % BK; i = idx / BK; }
-      const int64_t gm = m0 + i, gk = k0 + kk;
-      TC v = TC(0);
-      if (gm < M && gk < K) v = (TC)(ta ? A[gk * lda + gm] : A[gm * lda + gk]);
-      As[kk][i] = v;
+      for (int z = 0; z < NP; ++z) ra[z][u] = ok ? p.A[z][at] : 0.f;
     }
-    // ---- stage op(B)[k0:k0+BK, n0:n0+BN] as Bs[kk][j] --------------------------------------
-#pragma unroll 1
-    for (int idx = t; idx < BN * BK; idx += NT) {
-      int j, kk;
-      if (tb) { kk = idx % BK; j = idx / BK; } else { j = idx % BN; kk = idx / BN; }
-      const int64_t gn = n0 + j, gk = k0 + kk;
-      TC v = TC(0);
-      if (gn < N && gk < K) v = (TC)(tb ? B[gn * ldb + gk] : B[gk * ldb + gn]);
-      Bs[kk][j] = v;
+#pragma unroll
+    for (int u = 0; u < LB; ++u) {
+      const int idx = t + u * NT;
+      const int j = p.tb ? idx / BK : idx % BN, kk = p.tb ? idx % BK : idx / BN;
+      const bool ok = n0 + j < N && k0 + kk < K;
+      const int64_t at = p.tb ? (int64_t)(n0 + j) * p.ldb + k0 + kk : (int64_t)(k0 + kk) * p.ldb + n0 + j;
+#pragma unroll
+      for (int z = 0; z < NP; ++z) rb[z][u] = ok ? p.B[z][at] : 0.f;
+    }
+  };
+  float acc[NP][TM][TN];
+#pragma unroll
+  for (int z = 0; z < NP; ++z)
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) acc[z][i][j] = 0.f;
+  // thread rows ty * 4 + i % 4 (+ BM / 2 for i >= 4), columns likewise: 16-byte reads, neighbours adjacent
+  auto sub = [](int base, int i, int half) { return (i < 4 ? 0 : half) + base * 4 + (i & 3); };
+  fetch(0);
+  for (int k0 = 0; k0 < K; k0 += BK) {
+#pragma unroll
+    for (int u = 0; u < LA; ++u) {
+      const int idx = t + u * NT;
+      const int i = p.ta ? idx % BM : idx / BK, kk = p.ta ? idx / BM : idx % BK;
+#pragma unroll
+      for (int z = 0; z < NP; ++z) As[z][kk][i] = ra[z][u];
+    }
+#pragma unroll
+    for (int u = 0; u < LB; ++u) {
+      const int idx = t + u * NT;
+      const int j = p.tb ? idx / BK : idx % BN, kk = p.tb ? idx % BK : idx / BN;
+#pragma unroll
+      for (int z = 0; z < NP; ++z) Bs[z][kk][j] = rb[z][u];
     }
     __syncthreads();
+    if (k0 + BK < K) fetch(k0 + BK);
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      TC a[TM], b[TN];
+    for (int kk = 0; kk < BK; ++kk)
 #pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = As[kk][ty * TM + i];
+      for (int z = 0; z < NP; ++z) {
+        float a[TM], b[TN];
 #pragma unroll
-      for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx * TN + j];
+        for (int i = 0; i < TM; i += 4) *reinterpret_cast<float4*>(a + i) = *reinterpret_cast<const float4*>(&As[z][kk][sub(ty, i, BM / 2)]);
 #pragma unroll
-      for (int i = 0; i < TM; ++i)
+        for (int j = 0; j < TN; j += 4) *reinterpret_cast<float4*>(b + j) = *reinterpret_cast<const float4*>(&Bs[z][kk][sub(tx, j, BN / 2)]);
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[z][i][j] = fmaf(a[i], b[j], acc[z][i][j]);
+      }
     __syncthreads();
   }
-
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
-    const int64_t gm = m0 + ty * TM + i;
+    const int gm = m0 + sub(ty, i, BM / 2);
     if (gm >= M) continue;
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
-      const int64_t gn = n0 + tx * TN + j;
+      const int gn = n0 + sub(tx, j, BN / 2);
       if (gn >= N) continue;
-      TC* p = C + gm * ldc + gn;
-      TC v = alpha * acc[i][j];
-      if (beta != TC(0)) v = fma(beta, *p, v);
-      *p = v;
+      const int64_t at = (int64_t)gm * p.ldc + gn;
+      if (DUAL) {
+        const float g = acc[0][i][j], v2 = p.beta * p.V2[at] + p.alpha * g * g;
+        p.V2[at] = v2;
+        p.C[at] = acc[NP - 1][i][j] / sqrtf(v2 + p.eps);
+      } else {
+        float v = p.alpha * acc[0][i][j];
+        if (p.beta != 0.f) v = fmaf(p.beta, p.C[at], v);
+        p.C[at] = v;
+      }
     }
   }
 }
 
-template <typename TA, typename TB, typename TC>
-cudaError_t launch(int ta, int tb, int64_t M, int64_t N, int64_t K, TC alpha, const TA* A,
-                   int64_t lda, const TB* B, int64_t ldb, TC beta, TC* C, int64_t ldc,
-                   cudaStream_t s) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
-  const int64_t tiles_big = ((M + 127) / 128) * ((N + 127) / 128);
-  if (tiles_big >= 148) {
-    dim3 grid((unsigned)((N + 127) / 128), (unsigned)((M + 127) / 128));
-    k_gemm<TA, TB, TC, 128, 128, 8, 8, 8><<<grid, 256, 0, s>>>(ta, tb, M, N, K, alpha, A, lda, B, ldb,
-                                                              beta, C, ldc);
-  } else {
-    dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64));
-    k_gemm<TA, TB, TC, 64, 64, 16, 4, 4><<<grid, 256, 0, s>>>(ta, tb, M, N, K, alpha, A, lda, B, ldb,
-                                                             beta, C, ldc);
+template <int BM, int BN, int TM, int TN, bool DUAL>
+cudaError_t launch(GroupArgs& ga, cudaStream_t s) {
+  int64_t tiles = 0;
+  for (int i = 0; i < ga.n; ++i) {
+    ga.tile_begin[i] = (int)tiles;
+    tiles += (int64_t)((ga.p[i].M + BM - 1) / BM) * ((ga.p[i].N + BN - 1) / BN);
   }
+  ga.tile_begin[ga.n] = (int)tiles;
+  if (tiles > 0x7fffffff) return cudaErrorInvalidConfiguration;
+  k_simt_group<BM, BN, TM, TN, DUAL><<<(unsigned)tiles, (BM / TM) * (BN / TN), 0, s>>>(ga);
   return cudaGetLastError();
+}
+
+template <bool DUAL>
+cudaError_t launch_sized(GroupArgs& ga, cudaStream_t s) {
+  double area = 0.0;                                       // in tiles of 32 x 32
+  for (int i = 0; i < ga.n; ++i) area += (double)((ga.p[i].M + 31) / 32) * ((ga.p[i].N + 31) / 32);
+  if (area <= 148 * 12) return launch<32, 32, 4, 4, DUAL>(ga, s);
+  if (DUAL || area <= 148 * 64) return launch<64, 64, 4, 4, DUAL>(ga, s);
+  return launch<128, 128, 8, 8, false>(ga, s);
 }
 
 }  // namespace
 
-cudaError_t sgemm(int ta, int tb, int64_t M, int64_t N, int64_t K, float alpha, const float* A,
-                  int64_t lda, const float* B, int64_t ldb, float beta, float* C, int64_t ldc,
-                  cudaStream_t s) {
-  return launch<float, float, float>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s);
+cudaError_t simt_group(const SimtProblem* problems, int n, bool dual, cudaStream_t s) {
+  GroupArgs ga;
+  for (int at = 0; at < n; at += kMaxProblems) {
+    ga.n = 0;
+    for (int i = at; i < n && i < at + kMaxProblems; ++i)
+      if (problems[i].M > 0 && problems[i].N > 0) ga.p[ga.n++] = problems[i];
+    if (ga.n == 0) continue;
+    const cudaError_t e = dual ? launch_sized<true>(ga, s) : launch_sized<false>(ga, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+SimtProblem simt_problem(int ta, int tb, int64_t M, int64_t N, int64_t K, float alpha, const float* A, int64_t lda, const float* B,
+                         int64_t ldb, float beta, float* C, int64_t ldc) {
+  SimtProblem p = {};
+  p.A[0] = p.A[1] = A; p.B[0] = p.B[1] = B; p.C = C;
+  p.M = (int)M; p.N = (int)N; p.K = (int)K; p.lda = (int)lda; p.ldb = (int)ldb; p.ldc = (int)ldc;
+  p.ta = ta; p.tb = tb; p.alpha = alpha; p.beta = beta;
+  return p;
+}
+
+cudaError_t sgemm(int ta, int tb, int64_t M, int64_t N, int64_t K, float alpha, const float* A, int64_t lda, const float* B,
+                  int64_t ldb, float beta, float* C, int64_t ldc, cudaStream_t s) {
+  const SimtProblem p = simt_problem(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
+  return simt_group(&p, 1, false, s);
 }
 
 }  // namespace br

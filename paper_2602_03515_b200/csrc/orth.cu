@@ -7,7 +7,7 @@
 // Here one cluster of up to 16 CTAs walks the whole chain of a range of columns in one launch, and the
 // steps are separated by the cluster's hardware barrier; the second sweep and the completion of a
 // rank-deficient product are branches instead of cancelled launches.  Measured, one basis alone: order 64
-// 37 us, 384 250 us, 1024 1.3 ms, 1536 3.9 ms; stand-alone Power() at order 384 1368 -> 314 us.
+// 32 us, 384 240 us, 1024 1.3 ms, 1536 3.9 ms; stand-alone Power() at order 384 1368 -> 267 us.
 //
 //  * Rows of A are dealt to the CTAs in contiguous chunks.  A CTA computes its rows' share of a panel's
 //    Gram matrix and applies R^-1 and the projections to its own rows only, so these steps need no
@@ -183,40 +183,62 @@ __device__ __forceinline__ void each_entry(double (&acc)[16], int I, int J, FN f
   }
 }
 
-// One tile of the product F Q of two fp32 matrices (row-major, widened while they are staged through
-// registers); only the smallest orders form it here.
-__device__ __noinline__ void product64(const float* X, int I, const float* Y, int J, int k, double* out) {
-  const int t = threadIdx.x;
-  double acc[16], ra[4], rb[4];
+// C = alpha op(X) Y + beta C, X fp32, Y fp32 or fp64, widened while they are staged through registers: one
+// 64 x 64 tile per CTA, for the products of a refresh that have too few tiles of 128 x 128 to fill the GPU.
+template <bool TRANS, typename TB>
+__global__ void __launch_bounds__(kT, 2)
+k_product64(int M, int N, int K, double alpha, const float* __restrict__ X, int64_t lda, const TB* __restrict__ Y, int64_t ldb,
+            double beta, double* __restrict__ C, int64_t ldc) {
+  const int t = threadIdx.x, m0 = (int)blockIdx.y * 64, n0 = (int)blockIdx.x * 64;
+  double acc[16];
+  float ra[4];
+  TB rb[4];
   clear(acc);
   auto load = [&](int k0) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int i = (t >> 4) + 16 * q, ka = k0 + (t & 15), kb = k0 + (t >> 6) + 4 * q;
-      ra[q] = (i < I && ka < k) ? (double)X[(int64_t)i * k + ka] : 0.0;
-      rb[q] = ((t & 63) < J && kb < k) ? (double)Y[(int64_t)kb * k + (t & 63)] : 0.0;
+      const int i = m0 + (TRANS ? (t & 63) : (t >> 4) + 16 * q), ka = k0 + (TRANS ? (t >> 6) + 4 * q : (t & 15));
+      const int j = n0 + (t & 63), kb = k0 + (t >> 6) + 4 * q;
+      ra[q] = (i < M && ka < K) ? X[TRANS ? (int64_t)ka * lda + i : (int64_t)i * lda + ka] : 0.f;
+      rb[q] = (j < N && kb < K) ? Y[(int64_t)kb * ldb + j] : (TB)0;
     }
   };
   auto store = [&](int buf) {
     double* As = sm + oStage + buf * (kOper + kOperB);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      As[((t >> 4) + 16 * q) * kLdI + (t & 15)] = ra[q];
-      As[kOper + ((t >> 6) + 4 * q) * kLdK + (t & 63)] = rb[q];
+      As[TRANS ? ((t >> 6) + 4 * q) * kLdK + (t & 63) : ((t >> 4) + 16 * q) * kLdI + (t & 15)] = (double)ra[q];
+      As[kOper + ((t >> 6) + 4 * q) * kLdK + (t & 63)] = (double)rb[q];
     }
   };
-  const int nk = (k + kKs - 1) / kKs;
+  const int nk = (K + kKs - 1) / kKs;
   load(0);
   store(0);
   __syncthreads();
   for (int s = 0; s < nk; ++s) {
     if (s + 1 < nk) load((s + 1) * kKs);
     const double* st = sm + oStage + (s & 1) * (kOper + kOperB);
-    mma_stage<false, false, false>(acc, st, st + kOper, I);
+    mma_stage<TRANS, false, false>(acc, st, st + kOper, M - m0);
     if (s + 1 < nk) store((s + 1) & 1);
     __syncthreads();
   }
-  each_entry(acc, I, J, [&](int i, int j, double v) { out[(int64_t)i * k + j] = v; });
+  each_entry(acc, M - m0, N - n0, [&](int i, int j, double v) {
+    double* c = C + (int64_t)(m0 + i) * ldc + n0 + j;
+    v *= alpha;
+    *c = beta != 0.0 ? fma(beta, *c, v) : v;
+  });
+}
+
+template <typename TB>
+cudaError_t launch_product(int ta, int64_t M, int64_t N, int64_t K, double alpha, const float* A, int64_t lda, const TB* B,
+                           int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t s) {
+  const dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64));
+  const size_t bytes = 2 * (kOper + kOperB) * sizeof(double);
+  if (ta)
+    k_product64<true, TB><<<grid, kT, bytes, s>>>((int)M, (int)N, (int)K, alpha, A, lda, B, ldb, beta, C, ldc);
+  else
+    k_product64<false, TB><<<grid, kT, bytes, s>>>((int)M, (int)N, (int)K, alpha, A, lda, B, ldb, beta, C, ldc);
+  return cudaGetLastError();
 }
 
 struct OrthArgs {
@@ -227,7 +249,6 @@ struct OrthArgs {
   double ill_ratio;              // part, first: squared-norm ratio below which the second sweep has to run
   const double* norm0;           // part, first: squared norms of the columns before any projection
   double *C, *normp, *rdiag;     // projection coefficients; 2 x cluster x k partial norms (whole); squared diagonal of R
-  const float *F, *Q0;           // whole: A <- F Q0 first (null: A holds the product)
   double* Acopy; const float* Qprev;   // whole: buffer for a second copy of A, and the basis for its completion (both or none)
   float* Qout; __nv_bfloat16 *Qh, *Ql; // whole: the result in fp32 and as a bf16 pair (optional)
   int* status; int* flags; int* cond_out; const int* skip;
@@ -554,12 +575,6 @@ __global__ void __launch_bounds__(kT, 2) k_orth_cluster(OrthArgs a) {
     return;
   }
 
-  if (a.F) {
-    for (int r = q.r0; r < q.r1; r += 64)
-      for (int c0 = 0; c0 < k; c0 += 64)
-        product64(a.F + (int64_t)r * k, min(64, q.r1 - r), a.Q0 + c0, min(64, k - c0), k, q.A + (int64_t)r * k + c0);
-    __syncthreads();
-  }
   bool clamped = false, tc_bad = false, deficient = false;
   const bool fix = a.Acopy != nullptr && a.Qprev != nullptr;
   for (int attempt = 0; attempt < 2; ++attempt) {
@@ -704,12 +719,12 @@ size_t orth_work_doubles(int64_t k) {
   return (size_t)(coef_doubles(k) + pad32(2 * cluster_for(k) * k) + pad32(k));
 }
 
-cudaError_t orth_whole(double* A, int64_t k, double* work, const float* F, const float* Q0, double* Acopy, const float* Qprev,
+cudaError_t orth_whole(double* A, int64_t k, double* work, double* Acopy, const float* Qprev,
                        float* Qout, __nv_bfloat16* Qh, __nv_bfloat16* Ql, int* status, int* cond_out, cudaStream_t s) {
   OrthArgs a = {};
   a.A = A; a.k = k; a.j0 = 0; a.w = (int)k; a.whole = 1;
   a.C = work; a.normp = a.C + coef_doubles(k); a.rdiag = a.normp + pad32(2 * cluster_for(k) * k);
-  a.F = F; a.Q0 = Q0; a.Acopy = Acopy; a.Qprev = Qprev; a.Qout = Qout; a.Qh = Qh; a.Ql = Ql;
+  a.Acopy = Acopy; a.Qprev = Qprev; a.Qout = Qout; a.Qh = Qh; a.Ql = Ql;
   a.status = status; a.cond_out = cond_out;
   return launch(a, s);
 }
@@ -720,6 +735,15 @@ cudaError_t orth_part(double* A, int64_t k, int64_t j0, int64_t w, double* C, in
   a.A = A; a.k = k; a.j0 = (int)j0; a.w = (int)w; a.first = first; a.ill_ratio = ill_ratio; a.norm0 = norm0;
   a.C = C; a.rdiag = rdiag; a.status = status; a.flags = flags; a.skip = skip;
   return launch(a, s);
+}
+
+cudaError_t product64(int ta, int64_t M, int64_t N, int64_t K, double alpha, const float* A, int64_t lda, const float* B,
+                      int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t s) {
+  return launch_product(ta, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s);
+}
+cudaError_t product64(int ta, int64_t M, int64_t N, int64_t K, double alpha, const float* A, int64_t lda, const double* B,
+                      int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t s) {
+  return launch_product(ta, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s);
 }
 
 }  // namespace br

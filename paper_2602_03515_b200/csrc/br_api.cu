@@ -987,6 +987,7 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
   // ---- enqueue the updates ----------------------------------------------------------------
   const br_hparams& hp = h->hp;
   std::vector<int> simt_ids;
+  std::vector<SmallJob> small;
   for (int i = 0; i < nl; ++i) {
     Layer& L = h->layers[i];
     if (!G[i]) continue;
@@ -1000,10 +1001,8 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
       if (small_on && L.t % L.freq != 0 && small_step_eligible(L.d.m, L.d.n, L.left, L.right)) {
         const bool acc = L.d.src == BR_SRC_SECOND && hp.accum == BR_ACCUM_EVERY_STEP;
         const int64_t m = L.d.m, n = L.d.n;
-        BR_CUDA(h, small_step(m, n, L.left, L.right, G[i], L.d.grad_dtype == BR_BF16, GS[i], L.M, L.V2, L.U, L.V, L.L, L.R,
-                              L.d.weight, acc ? 1 : 0, hp.lr, hp.beta1, hp.beta2, hp.eps, hp.weight_decay,
-                              hp.beta_factor < 0.f ? hp.beta2 : hp.beta_factor, h->stream));
-        count(h);
+        small.push_back({(int)m, (int)n, L.left, L.right, L.d.grad_dtype == BR_BF16, acc ? 1 : 0, G[i], GS[i], L.M, L.V2, L.U, L.V,
+                         L.L, L.R, L.d.weight});
         h->stats.gemm_flops += (acc ? 2.0 : 0.0) * ((L.L ? m * m * n : 0) + (L.R ? n * n * m : 0)) +
                                6.0 * m * n * ((L.left ? m : 0) + (L.right ? n : 0));
         if (acc) L.n_accum += 1;
@@ -1011,6 +1010,11 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
         simt_ids.push_back(i);
       }
     }
+  }
+  if (!small.empty()) {
+    BR_CUDA(h, small_step(small.data(), (int)small.size(), hp.lr, hp.beta1, hp.beta2, hp.eps, hp.weight_decay,
+                          hp.beta_factor < 0.f ? hp.beta2 : hp.beta_factor, h->stream));
+    count(h, ((int)small.size() + 23) / 24);
   }
   if (!simt_ids.empty() && (st = update_layers_simt(h, simt_ids, G, GS)) != BR_OK) return st;
   if (h->tc) {

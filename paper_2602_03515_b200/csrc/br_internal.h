@@ -99,12 +99,18 @@ cudaError_t sub_f32_from_f64(double* A, int64_t ld, int64_t rows, int64_t cols, 
 cudaError_t ema_out(float* out, const float* M, const void* G, int g_is_bf16, int64_t numel, float beta1,
                     const float* gscale, cudaStream_t s);
 
-// One whole update (Alg. 1 (momentum, rotation, second moment, weight update) and the factor EMAs of Alg. 2, no refresh) of a matrix with both
-// dimensions <= 128 in a single one-CTA launch (small_step.cu).  accumulate: update L and R as well.
+// One whole update (Alg. 1 (momentum, rotation, second moment, weight update) and the factor EMAs of Alg. 2, no refresh) of
+// matrices with both dimensions <= 128, a CTA each, in one launch per 24 of them (small_step.cu).  accumulate:
+// update L and R as well.
 bool small_step_eligible(int64_t m, int64_t n, bool left, bool right);
-cudaError_t small_step(int64_t m, int64_t n, bool left, bool right, const void* G, int g_is_bf16, const float* gscale,
-                       float* M, float* V2, float* U, float* V, float* L, float* R, float* W, int accumulate, float lr,
-                       float beta1, float beta2, float eps, float weight_decay, float beta_factor, cudaStream_t s);
+struct SmallJob {
+  int m, n, left, right;    // shape, and which sides are rotated
+  int g_is_bf16, accumulate;
+  const void* G; const float* gscale;      // gradient, and its call's clipping factor or null
+  float *M, *V2, *U, *V, *L, *R, *W;
+};
+cudaError_t small_step(const SmallJob* jobs, int n, float lr, float beta1, float beta2, float eps, float weight_decay,
+                       float beta_factor, cudaStream_t s);
 
 // Debug canaries (BR_FLAG_DEBUG_CANARY): n guards of 256 bytes at byte offsets offs[] (DEVICE array) of the slab.
 cudaError_t guard_fill(char* slab, const unsigned long long* offs, int n, cudaStream_t s);

@@ -11,11 +11,12 @@
 // launches, of which 1.0 ms in the products).
 //
 // A CTA computes one tile; the next 16 steps of the contraction are fetched into registers while the
-// current ones are multiplied out of shared memory, and every entry is one chain of fused multiply-adds in
-// the order of the contraction.  The tile follows from the work of the launch: 32 x 32 on 64 threads while
-// those tiles fit on the GPU at once (the time is then that of one tile's chain, and a small tile's step is
-// the shortest), 64 x 64 up to a few waves, 128 x 128 (8 x 8 per thread, half the shared-memory reads per
-// multiply-add) above.
+// current ones are multiplied out of shared memory.  The tile follows from the work of the launch: 32 x 32 on
+// 64 threads while those tiles fit on the GPU at once (the time is then that of one tile's chain, and a small
+// tile's step is the shortest), 64 x 64 up to a few waves, 128 x 128 (8 x 8 per thread, half the shared-memory
+// reads per multiply-add) above.  With at most four tiles of 32 x 32 per SM a step is bound by the latency of
+// its loads, and four groups of 64 threads take a quarter of the contraction each: the dual launch of the four
+// ragged layers 54 -> 30 us, the others 30 -> 16 us.
 #include "br_internal.h"
 #include "step_tc.h"
 
@@ -31,20 +32,28 @@ struct GroupArgs {
   int n;
 };
 
-template <int BM, int BN, int TM, int TN, bool DUAL>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
+// KS groups of NT threads share one tile's contraction (a range of it each) and add up their sums at the end.
+template <int BM, int BN, int TM, int TN, bool DUAL, int KS>
+__global__ void __launch_bounds__(KS * (BM / TM) * (BN / TN))
 k_simt_group(const __grid_constant__ GroupArgs ga) {
   constexpr int NT = (BM / TM) * (BN / TN), NP = DUAL ? 2 : 1;
-  constexpr int LA = BM * BK / NT, LB = BN * BK / NT;
-  __shared__ __align__(16) float As[NP][BK][BM + 4];
-  __shared__ __align__(16) float Bs[NP][BK][BN + 4];
+  constexpr int LA = BM * BK / NT, LB = BN * BK / NT, FA = BK * (BM + 4), FB = BK * (BN + 4);
+  static_assert(KS == 1 || (TM == 4 && TN == 4 && KS == TM && NP * TM * NT * 4 <= NP * (FA + FB)), "partial sums fit the operand area");
+  __shared__ __align__(16) float area[KS][NP * (FA + FB)];
+  const int group = KS == 1 ? 0 : (int)threadIdx.x / NT;
+  float(*As)[BK][BM + 4] = reinterpret_cast<float(*)[BK][BM + 4]>(area[group]);
+  float(*Bs)[BK][BN + 4] = reinterpret_cast<float(*)[BK][BN + 4]>(area[group] + NP * FA);
+  auto sync = [&] {      // the groups run at their own pace
+    if (KS == 1) __syncthreads(); else asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(NT) : "memory");
+  };
   int pi = 0;
   while (pi + 1 < ga.n && (int)blockIdx.x >= ga.tile_begin[pi + 1]) ++pi;
   const SimtProblem& p = ga.p[pi];
   const int tiles_n = (p.N + BN - 1) / BN, tile = (int)blockIdx.x - ga.tile_begin[pi];
   const int m0 = tile / tiles_n * BM, n0 = tile % tiles_n * BN;
-  const int M = p.M, N = p.N, K = p.K;
-  const int t = threadIdx.x, tx = t % (BN / TN), ty = t / (BN / TN);
+  const int M = p.M, N = p.N;
+  const int kc = KS == 1 ? p.K : (p.K + KS * BK - 1) / (KS * BK) * BK, kbeg = min(p.K, group * kc), K = min(p.K, kbeg + kc);
+  const int t = threadIdx.x % NT, tx = t % (BN / TN), ty = t / (BN / TN);
 
   float ra[NP][LA], rb[NP][LB];
   auto fetch = [&](int k0) {
@@ -76,8 +85,8 @@ k_simt_group(const __grid_constant__ GroupArgs ga) {
       for (int j = 0; j < TN; ++j) acc[z][i][j] = 0.f;
   // thread rows ty * 4 + i % 4 (+ BM / 2 for i >= 4), columns likewise: 16-byte reads, neighbours adjacent
   auto sub = [](int base, int i, int half) { return (i < 4 ? 0 : half) + base * 4 + (i & 3); };
-  fetch(0);
-  for (int k0 = 0; k0 < K; k0 += BK) {
+  if (kbeg < K) fetch(kbeg);
+  for (int k0 = kbeg; k0 < K; k0 += BK) {
 #pragma unroll
     for (int u = 0; u < LA; ++u) {
       const int idx = t + u * NT;
@@ -92,7 +101,7 @@ k_simt_group(const __grid_constant__ GroupArgs ga) {
 #pragma unroll
       for (int z = 0; z < NP; ++z) Bs[z][kk][j] = rb[z][u];
     }
-    __syncthreads();
+    sync();
     if (k0 + BK < K) fetch(k0 + BK);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk)
@@ -108,11 +117,31 @@ k_simt_group(const __grid_constant__ GroupArgs ga) {
 #pragma unroll
           for (int j = 0; j < TN; ++j) acc[z][i][j] = fmaf(a[i], b[j], acc[z][i][j]);
       }
-    __syncthreads();
+    sync();
   }
+  if (KS > 1) {
+    // [product][row of the thread's tile][thread], four columns each; group g then finishes row g of every tile
+    float4* mine = reinterpret_cast<float4*>(area[group]);
 #pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    const int gm = m0 + sub(ty, i, BM / 2);
+    for (int z = 0; z < NP; ++z)
+#pragma unroll
+      for (int i = 0; i < TM; ++i) mine[(z * TM + i) * NT + t] = make_float4(acc[z][i][0], acc[z][i][1], acc[z][i][2], acc[z][i][3]);
+    __syncthreads();
+#pragma unroll
+    for (int z = 0; z < NP; ++z) {
+      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int g = 0; g < KS; ++g) {
+        const float4 o = reinterpret_cast<const float4*>(area[g])[(z * TM + group) * NT + t];
+        s.x += o.x; s.y += o.y; s.z += o.z; s.w += o.w;
+      }
+      acc[z][0][0] = s.x; acc[z][0][1] = s.y; acc[z][0][2] = s.z; acc[z][0][3] = s.w;
+    }
+  }
+  constexpr int ROWS = KS > 1 ? 1 : TM;
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i) {
+    const int gm = m0 + sub(ty, KS > 1 ? group : i, BM / 2);
     if (gm >= M) continue;
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
@@ -132,7 +161,7 @@ k_simt_group(const __grid_constant__ GroupArgs ga) {
   }
 }
 
-template <int BM, int BN, int TM, int TN, bool DUAL>
+template <int BM, int BN, int TM, int TN, bool DUAL, int KS = 1>
 cudaError_t launch(GroupArgs& ga, cudaStream_t s) {
   int64_t tiles = 0;
   for (int i = 0; i < ga.n; ++i) {
@@ -141,7 +170,7 @@ cudaError_t launch(GroupArgs& ga, cudaStream_t s) {
   }
   ga.tile_begin[ga.n] = (int)tiles;
   if (tiles > 0x7fffffff) return cudaErrorInvalidConfiguration;
-  k_simt_group<BM, BN, TM, TN, DUAL><<<(unsigned)tiles, (BM / TM) * (BN / TN), 0, s>>>(ga);
+  k_simt_group<BM, BN, TM, TN, DUAL, KS><<<(unsigned)tiles, KS * (BM / TM) * (BN / TN), 0, s>>>(ga);
   return cudaGetLastError();
 }
 
@@ -149,6 +178,7 @@ template <bool DUAL>
 cudaError_t launch_sized(GroupArgs& ga, cudaStream_t s) {
   double area = 0.0;                                       // in tiles of 32 x 32
   for (int i = 0; i < ga.n; ++i) area += (double)((ga.p[i].M + 31) / 32) * ((ga.p[i].N + 31) / 32);
+  if (area <= 148 * 4) return launch<32, 32, 4, 4, DUAL, 4>(ga, s);
   if (area <= 148 * 12) return launch<32, 32, 4, 4, DUAL>(ga, s);
   if (DUAL || area <= 148 * 64) return launch<64, 64, 4, 4, DUAL>(ga, s);
   return launch<128, 128, 8, 8, false>(ga, s);

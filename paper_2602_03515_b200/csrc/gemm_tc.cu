@@ -13,7 +13,8 @@
 // operand tile is fetched from L2 once per k-block instead of once per pair.
 //
 // One persistent CTA per SM walks a static tile list that spans every problem of a launch
-// (all layers of one phase of the step), so small and large matrices share one launch.
+// (all layers of one phase of the step), so small and large matrices share one launch; the lists are made on
+// the host, longest tiles first (make_schedule).
 // Two 256-column accumulators in tensor memory let the epilogue of a tile overlap the main
 // loop of the next one.
 //
@@ -53,8 +54,11 @@
 #include <cuda.h>
 
 #include <cstdlib>
+#include <algorithm>
 #include <cstring>
+#include <functional>
 #include <mutex>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -96,6 +100,7 @@ constexpr int MAX_PAIRS = 3;
 // Tile rasterisation: a group of row-blocks (or, transposed, of column-blocks) is swept across the
 // other dimension, so that the group's operand panel stays in L2 while the other operand streams
 // through once per group.  The host picks orientation and group size per problem (see plan creation).
+constexpr int kTileCost = 6, kFoldTileCost = 24;  // see make_schedule
 constexpr double kL2PanelBytes = 40e6;           // what one resident operand panel may take of the 126 MB L2
 
 struct alignas(128) DevProblem {
@@ -397,8 +402,8 @@ __device__ __forceinline__ TileInfo locate_tile(const DevProblem* probs, int n_p
 // ---------------------------------------------------------------------------------------------
 template <bool SHARED, bool PAIR, bool FOLD = false>
 __global__ void __launch_bounds__(FOLD ? FOLD_THREADS : NUM_THREADS, 1)
-k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int total_tiles, long long calls,
-          int tau, float dyn_alpha, float dyn_beta, int* status) {
+k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int total_tiles, const int* __restrict__ schedule,
+          long long calls, int tau, float dyn_alpha, float dyn_beta, int* status) {
   using F = Form<SHARED, PAIR>;
   constexpr int NST = F::NST;
   constexpr int TM = F::TM;
@@ -461,7 +466,11 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
   }
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
-  if (dead) first_tile = total_tiles;          // every role finds an empty tile list
+  // this unit's tiles: entries [walk_begin, walk_end) of the schedule's list behind its n_units + 1 offsets, or,
+  // without a schedule, every n_units-th tile of the range.  A dead pair finds an empty list in every role.
+  const int walk_begin = schedule ? schedule[unit] : first_tile + unit, walk_step = schedule ? 1 : n_units;
+  const int walk_end = dead ? walk_begin : schedule ? schedule[unit + 1] : total_tiles;
+  auto tile_at = [&](int i) { return schedule ? schedule[n_units + 1 + i] : i; };
 
   if (warp == 0) {
     // ======================= TMA producer =======================
@@ -473,8 +482,8 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
       auto load = [&](uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z) {
         if (PAIR) tma_load_3d_pair(dst, map, bar, x, y, z); else tma_load_3d(dst, map, bar, x, y, z);
       };
-      for (int tile = first_tile + unit; tile < total_tiles && !*abort_flag; tile += n_units) {
-        const TileInfo ti = locate_tile<TM>(probs, n_probs, tile, calls, tau);
+      for (int wi = walk_begin; wi < walk_end && !*abort_flag; wi += walk_step) {
+        const TileInfo ti = locate_tile<TM>(probs, n_probs, tile_at(wi), calls, tau);
         if (!ti.active) continue;
         const DevProblem* p = ti.p;
         const int nkb = (p->K + BK - 1) / BK;
@@ -535,8 +544,8 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
       auto commit = [&](uint32_t bar) {
         if (PAIR) { umma_commit_pair(bar); umma_commit_pair(map_to_cta(bar, 1)); } else { umma_commit(bar); }
       };
-      for (int tile = first_tile + unit; tile < total_tiles && !*abort_flag; tile += n_units) {
-        const TileInfo ti = locate_tile<TM>(probs, n_probs, tile, calls, tau);
+      for (int wi = walk_begin; wi < walk_end && !*abort_flag; wi += walk_step) {
+        const TileInfo ti = locate_tile<TM>(probs, n_probs, tile_at(wi), calls, tau);
         if (!ti.active) continue;
         const DevProblem* p = ti.p;
         const int nkb = (p->K + BK - 1) / BK;
@@ -630,8 +639,8 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
     const int sub_r = lane >> 3, sub_c = (lane & 7) * 4;
     int acc = 0; uint32_t acc_phase = 0;
     uint32_t fold_seq = 0;
-    for (int tile_i = first_tile + unit; tile_i < total_tiles && !*abort_flag; tile_i += n_units) {
-      const TileInfo ti = locate_tile<TM>(probs, n_probs, tile_i, calls, tau);
+    for (int wi = walk_begin; wi < walk_end && !*abort_flag; wi += walk_step) {
+      const TileInfo ti = locate_tile<TM>(probs, n_probs, tile_at(wi), calls, tau);
       if (!ti.active) continue;
       const DevProblem* p = ti.p;
       float alpha = p->dyn_scalars ? dyn_alpha : p->alpha;
@@ -1003,7 +1012,7 @@ bool encode_operand(CUtensorMap* map, const TcOperand& op, int64_t rows, int64_t
   return true;
 }
 
-typedef void (*TcKernel)(const DevProblem*, int, int, int, long long, int, float, float, int*);
+typedef void (*TcKernel)(const DevProblem*, int, int, int, const int*, long long, int, float, float, int*);
 TcKernel kernel_of(bool shared, bool pair, bool fold = false) {
   if (fold) return pair ? k_tc_gemm<false, true, true> : k_tc_gemm<false, false, true>;
   if (pair) return shared ? k_tc_gemm<true, true> : k_tc_gemm<false, true>;
@@ -1043,6 +1052,39 @@ int pair_capacity(bool shared) {
   return c;
 }
 
+// Longest tiles first, each to the unit with the least work so far.  The round-robin walk of the plan's order
+// leaves units idle at the end when a launch mixes contraction lengths (the factor products of a decoder layer with
+// its embedding: 55 tiles of 500 k-blocks behind 1739 of 40 to 108) or has few tiles per unit.  Tiles of equal
+// length keep their order, so that neighbours in the walk still run at the same time and share operands in L2.
+// A tile costs its k-blocks plus `fixed` (the part of its epilogue that the next tile's main loop does not
+// cover, in k-blocks).  Layout: units + 1 offsets, then the tiles.
+std::vector<int> make_schedule(const std::vector<DevProblem>& probs, int total, int units, int fixed) {
+  struct Tile { int cost, index; };
+  std::vector<Tile> tiles;
+  tiles.reserve((size_t)total);
+  for (const DevProblem& d : probs)
+    for (int i = 0; i < d.tile_count; ++i) tiles.push_back({d.n_pairs * ((d.K + BK - 1) / BK) + fixed, d.tile_begin + i});
+  std::stable_sort(tiles.begin(), tiles.end(), [](const Tile& a, const Tile& b) { return a.cost > b.cost; });
+  typedef std::pair<long long, int> Load;                     // (work so far, unit)
+  std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
+  for (int u = 0; u < units; ++u) heap.push({0, u});
+  std::vector<std::vector<int>> list((size_t)units);
+  for (const Tile& t : tiles) {
+    Load l = heap.top();
+    heap.pop();
+    list[(size_t)l.second].push_back(t.index);
+    l.first += t.cost;
+    heap.push(l);
+  }
+  std::vector<int> out;
+  out.reserve((size_t)(units + 1 + total));
+  int at = 0;
+  for (int u = 0; u < units; ++u) { out.push_back(at); at += (int)list[(size_t)u].size(); }
+  out.push_back(at);
+  for (const auto& l : list) out.insert(out.end(), l.begin(), l.end());
+  return out;
+}
+
 }  // namespace
 
 struct TcPlan {
@@ -1053,6 +1095,8 @@ struct TcPlan {
   std::vector<int> tile_begin;  // per problem, plus the total at the end
   std::vector<double> prob_flops;
   DevProblem* d_probs = nullptr;
+  int* d_schedule = nullptr;    // tile lists of the whole plan's units (see make_schedule), or null
+  int units = 0;                // CTA pairs (or CTAs) of a launch of the whole plan
   int n = 0;
   int total_tiles = 0;
   double flops = 0.0;
@@ -1231,10 +1275,17 @@ TcPlan* tc_plan_create(const TcProblem* problems, int n, int device, cudaStream_
   plan->flops = flops;
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, device) == cudaSuccess) plan->sm_count = prop.multiProcessorCount;
-  cudaError_t ce = cudaMalloc(&plan->d_probs, sizeof(DevProblem) * n);
-  if (ce == cudaSuccess)
+  const int cap = pair ? pairs : plan->sm_count;
+  plan->units = tile_begin < cap ? tile_begin : cap;
+  const std::vector<int> schedule = make_schedule(host, tile_begin, plan->units, fold ? kFoldTileCost : kTileCost);
+  cudaError_t ce = cudaMalloc(&plan->d_probs, sizeof(DevProblem) * n + sizeof(int) * schedule.size());
+  if (ce == cudaSuccess) {
+    plan->d_schedule = reinterpret_cast<int*>(plan->d_probs + n);
     ce = cudaMemcpyAsync(plan->d_probs, host.data(), sizeof(DevProblem) * n, cudaMemcpyHostToDevice, s);
-  if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);   // `host` goes out of scope
+  }
+  if (ce == cudaSuccess)
+    ce = cudaMemcpyAsync(plan->d_schedule, schedule.data(), sizeof(int) * schedule.size(), cudaMemcpyHostToDevice, s);
+  if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);   // `host` and `schedule` go out of scope
   if (ce != cudaSuccess) {
     if (plan->d_probs) cudaFree(plan->d_probs);
     delete plan;
@@ -1262,19 +1313,21 @@ cudaError_t tc_plan_launch_range(TcPlan* p, int first, int count, long long call
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
+  const bool whole = first == 0 && count == p->n;
   if (p->pair) {
-    const int units = tiles < p->max_pairs ? tiles : p->max_pairs;
+    const int units = whole ? p->units : tiles < p->max_pairs ? tiles : p->max_pairs;
     cfg.gridDim = dim3(2u * (unsigned)units);
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
   } else {
-    cfg.gridDim = dim3((unsigned)(tiles < p->sm_count ? tiles : p->sm_count));
+    cfg.gridDim = dim3((unsigned)(whole ? p->units : tiles < p->sm_count ? tiles : p->sm_count));
   }
   cfg.blockDim = dim3(p->fold ? FOLD_THREADS : NUM_THREADS);
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = s;
-  return cudaLaunchKernelEx(&cfg, kernel, (const DevProblem*)p->d_probs, p->n, t0, t1, calls, tau, dyn_alpha,
+  return cudaLaunchKernelEx(&cfg, kernel, (const DevProblem*)p->d_probs, p->n, t0, t1,
+                            (const int*)(whole ? p->d_schedule : nullptr), calls, tau, dyn_alpha,
                             dyn_beta, status_word);
 }
 

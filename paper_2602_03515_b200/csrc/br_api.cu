@@ -507,6 +507,14 @@ br_status refresh_layers(br_handle* h, const int* ids, int n_ids) {
     if (L.right) jobs.push_back({ids[j], false, cost((double)L.d.n), L.d.n, z});
   }
   if (jobs.empty()) return BR_OK;
+  for (int j = 0; j < n_ids; ++j) {
+    Layer& L = h->layers[ids[j]];
+    if (!L.lower_stale) continue;
+    cudaError_t e;
+    const int n = h->stats.inject() ? (e = cudaErrorLaunchFailure, -1) : complete_factors(L, h->stream, &e);
+    if (n < 0) { h->err = format("completing the factors failed: %s", cudaGetErrorString(e)); return BR_ERR_CUDA; }
+    count(h, n);
+  }
   if (h->cond_pending) {
     // the notes of the previous batch: long since on the host unless the two refreshes are back to back
     BR_CUDA(h, cudaEventSynchronize(h->ev_cond));
@@ -1231,6 +1239,12 @@ br_status br_get_state(br_handle* h, int layer, int which, void* host_dst, size_
   const size_t want = buf_bytes(L, which, &p);
   if (!p || want == 0) { h->err = "this layer has no such buffer"; return BR_ERR_STATE; }
   if (bytes != want) { h->err = format("buffer is %zu bytes, caller passed %zu", want, bytes); return BR_ERR_SHAPE; }
+  if (which == BR_BUF_L || which == BR_BUF_R) {
+    cudaError_t e;
+    const int n = complete_factors(h->layers[layer], h->stream, &e);
+    if (n < 0) { h->err = format("completing the factors failed: %s", cudaGetErrorString(e)); return BR_ERR_CUDA; }
+    count(h, n);
+  }
   BR_CUDA(h, cudaStreamSynchronize(h->stream));
   if (which == BR_BUF_M && L.use_tc) {
     // the state is M~: hand out M = U M~ V^T, computed with fp32 FFMA products into temporaries
@@ -1269,6 +1283,12 @@ br_status br_set_state(br_handle* h, int layer, int which, const void* host_src,
   const size_t want = buf_bytes(L, which, &p);
   if (!p || want == 0) { h->err = "this layer has no such buffer"; return BR_ERR_STATE; }
   if (bytes != want) { h->err = format("buffer is %zu bytes, caller passed %zu", want, bytes); return BR_ERR_SHAPE; }
+  if (which == BR_BUF_L || which == BR_BUF_R) {        // (the other factor of the layer is completed; this one is replaced whole)
+    cudaError_t e;
+    const int n = complete_factors(L, h->stream, &e);
+    if (n < 0) { h->err = format("completing the factors failed: %s", cudaGetErrorString(e)); return BR_ERR_CUDA; }
+    count(h, n);
+  }
   BR_CUDA(h, cudaStreamSynchronize(h->stream));
   const size_t mn_bytes = 4 * (size_t)L.d.m * L.d.n;
   if (L.use_tc && (which == BR_BUF_M || which == BR_BUF_U || which == BR_BUF_V)) {

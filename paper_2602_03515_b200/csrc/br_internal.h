@@ -81,6 +81,8 @@ cudaError_t clip_factor(const void* const* grads, const int64_t* numel, const in
 cudaError_t plain_adam(float* W, float* M, float* V, const void* G, int g_is_bf16, int64_t numel,
                        float lr, float beta1, float beta2, float eps, float wd, const float* gscale, cudaStream_t s);
 
+// F[j][i] <- F[i][j] for the 32 x 32 blocks (j, i) strictly below the diagonal of the k x k matrix F.
+cudaError_t mirror_lower(float* F, int64_t k, cudaStream_t s);
 // fp32 -> bf16 hi (+ optional lo = bf16(x - hi)).
 cudaError_t split_bf16(const float* X, __nv_bfloat16* hi, __nv_bfloat16* lo, int64_t numel,
                        cudaStream_t s);
@@ -252,8 +254,9 @@ struct TcProblem {
   const float* clip = nullptr; int32_t clip_slots = 0; int32_t clip_mode = 0;
   int32_t fold_kb = 0;            // > 0: accumulate in chunks of this many 64-deep k-blocks, summed outside the tensor
                                   // core (a plan whose problems all ask for it runs the folded form of the kernel)
-  int32_t symmetric = 0;          // 1: A_p = B_p and D is square: only tiles touching the upper triangle are
-                                  // computed, the rest of D is written as their mirror image (EPI_AXPBY_F32 only)
+  int32_t symmetric = 0;          // 1: A_p = B_p and D is square (EPI_AXPBY_F32 only): only the 32 x 32 blocks on and above
+                                  // the diagonal are computed, read and written; D below them keeps what it holds
+                                  // until mirror_lower() copies it over
   float alpha = 1.f, beta = 0.f, eps = 0.f, beta1 = 0.f;
   float* D = nullptr; int64_t ldd = 0;                                   // fp32 in/out
   float* D2 = nullptr;                                                   // second fp32 in/out (same ld)

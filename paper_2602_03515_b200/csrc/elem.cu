@@ -147,6 +147,26 @@ k_plain_adam(float* __restrict__ W, float* __restrict__ M, float* __restrict__ V
   }
 }
 
+// One 32 x 32 block pair per CTA of 32 x 8 threads, through a padded shared-memory tile.  Blocks are numbered along
+// the columns of the strict upper block triangle (block b of column c, b < c, is number c (c - 1) / 2 + b).  Bound by memory, 8 bytes per pair of entries.
+__global__ void __launch_bounds__(256) k_mirror_lower(float* __restrict__ F, int64_t k) {
+  __shared__ float tile[32][33];
+  const int id = (int)blockIdx.x;
+  int c = (int)((sqrtf(8.0f * (float)id + 1.0f) + 1.0f) * 0.5f);
+  while (c * (c - 1) / 2 > id) --c;
+  while (c * (c + 1) / 2 <= id) ++c;
+  const int b = id - c * (c - 1) / 2;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t r0 = 32 * (int64_t)b, c0 = 32 * (int64_t)c;
+#pragma unroll
+  for (int i = ty; i < 32; i += 8)
+    if (c0 + tx < k) tile[i][tx] = F[(r0 + i) * k + c0 + tx];
+  __syncthreads();
+#pragma unroll
+  for (int i = ty; i < 32; i += 8)
+    if (c0 + i < k) F[(c0 + i) * k + r0 + tx] = tile[tx][i];
+}
+
 __global__ void __launch_bounds__(kThreads)
 k_split_bf16(const float* __restrict__ X, __nv_bfloat16* __restrict__ hi,
              __nv_bfloat16* __restrict__ lo, int64_t numel) {
@@ -296,6 +316,13 @@ k_f64_to_f32(const double* __restrict__ X, float* __restrict__ out, int64_t nume
 
 cudaError_t set_identity(float* Q, int64_t k, cudaStream_t s) {
   k_set_identity<<<grid_for(k * k), kThreads, 0, s>>>(Q, k);
+  return cudaGetLastError();
+}
+
+cudaError_t mirror_lower(float* F, int64_t k, cudaStream_t s) {
+  const int nb = (int)((k + 31) / 32);
+  if (nb < 2) return cudaSuccess;
+  k_mirror_lower<<<(unsigned)((int64_t)nb * (nb - 1) / 2), 256, 0, s>>>(F, k);
   return cudaGetLastError();
 }
 

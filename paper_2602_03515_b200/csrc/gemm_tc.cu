@@ -45,8 +45,10 @@
 // 128 result columns each) add every finished chunk, round to nearest on the CUDA cores, to a running
 // sum they keep in registers, while the tensor core is already working on the next chunk.  Chains
 // are 8 to 16 instructions on partial sums a tenth the size: the error drops by the number of chunks.
-// The final epilogue (factor EMA and its mirror image) runs from the registers while the first two
-// chunks of the next tile accumulate.
+// The final epilogue (factor EMA) runs from the registers while the first two chunks of the next tile
+// accumulate.  It is bound by the traffic between L2 and the SMs, which all of them cause at the same time:
+// 19 to 25 thousand cycles a tile when it wrote the mirror image of every block as well, against 26 thousand
+// for the chunks of a tile of K = 2560.
 //
 // Every wait on an mbarrier is bounded: when a wait gives up the CTA raises an abort flag,
 // records BR_ERR_TIMEOUT in the status word, leaves its loops, frees its tensor memory and
@@ -95,7 +97,9 @@ struct Form {
 constexpr int TMEM_COLS = 512;
 constexpr int NUM_THREADS = 192;                 // warp 0: TMA, warp 1: MMA, warps 2..5: epilogue
 constexpr int FOLD_THREADS = 320;                // folded form: warps 2..9 fold and write (two per lane quadrant)
-constexpr int SMEM_BYTES_FOLD = OPERAND_BYTES + 2 * EPI_BYTES + 1024;
+// folded form: 160 KiB of operand stages, and two blocks of 32 x 32 floats for each of its eight epilogue warps
+constexpr int FOLD_OPERAND_BYTES = 160 * 1024, FOLD_BLOCK = 32 * 32;
+constexpr int SMEM_BYTES_FOLD = FOLD_OPERAND_BYTES + 8 * 2 * FOLD_BLOCK * 4 + 1024;
 constexpr int MAX_PAIRS = 3;
 // Tile rasterisation: a group of row-blocks (or, transposed, of column-blocks) is swept across the
 // other dimension, so that the group's operand panel stays in L2 while the other operand streams
@@ -405,7 +409,7 @@ __global__ void __launch_bounds__(FOLD ? FOLD_THREADS : NUM_THREADS, 1)
 k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int total_tiles, const int* __restrict__ schedule,
           long long calls, int tau, float dyn_alpha, float dyn_beta, int* status) {
   using F = Form<SHARED, PAIR>;
-  constexpr int NST = F::NST;
+  constexpr int NST = FOLD ? FOLD_OPERAND_BYTES / F::STAGE : F::NST;      // folded: 5 paired, 3 unpaired
   constexpr int TM = F::TM;
   extern __shared__ uint8_t smem_raw[];
   __shared__ alignas(8) uint64_t bars[2 * MAX_STAGES + 4];
@@ -431,7 +435,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
     return SHARED ? tiles_base + (uint32_t)s * F::STAGE + 2u * A_BYTES + (uint32_t)i * F::BB
                   : tiles_base + (uint32_t)NST * A_BYTES + (uint32_t)s * F::BB;
   };
-  float* epi_tiles = reinterpret_cast<float*>(smem_raw + ((tiles_base - smem_u32(smem_raw)) + (uint32_t)OPERAND_BYTES));
+  float* epi_tiles = reinterpret_cast<float*>(smem_raw + ((tiles_base - smem_u32(smem_raw)) + (uint32_t)(FOLD ? FOLD_OPERAND_BYTES : OPERAND_BYTES)));
   const uint32_t bar0 = smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
@@ -632,8 +636,8 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
     // tile so that global memory is accessed along rows: 8 lanes cover 128 contiguous bytes of one
     // row, a warp instruction four whole rows.  The values a read-modify-write epilogue needs are
     // prefetched into L2 while the main loop of the tile is still running and then loaded eight
-    // rows deep before the first one is used.  A symmetric product (the factor EMAs) writes its
-    // strictly-upper blocks a second time, transposed, instead of computing the lower triangle.
+    // rows deep before the first one is used.  A symmetric product (the factor EMAs) computes and writes only
+    // the 32 x 32 blocks on and above the diagonal (see TcProblem::symmetric).
     const int quad = warp & 3;                    // tensor-memory lane quadrant this warp may read
     float* tile = epi_tiles + quad * (32 * EPI_LD);
     const int sub_r = lane >> 3, sub_c = (lane & 7) * 4;
@@ -658,7 +662,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
       const bool quad_ok = row_base < p->Md;      // uniform across the warp
       const bool reads_d = (epi == EPI_AXPBY_F32 && beta != 0.0f) || epi == EPI_ROTATED_ADAM ||
                            epi == EPI_SECOND_MOMENT || epi == EPI_SCALE_BF16;
-      if (reads_d && row_base + lane < p->Md) {
+      if (!FOLD && reads_d && row_base + lane < p->Md) {
         const float* d = p->D + (long long)(row_base + lane) * p->ldd + ti.n0;
 #pragma unroll
         for (int q = 0; q < BN / 32; ++q)
@@ -671,7 +675,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
       if (FOLD) {
         // ---- folded form: this warp owns 32 rows (its lane quadrant) x 128 columns (its half) ----
         const int half = (warp - 2) >> 2;
-        float* ftile = epi_tiles + (warp - 2) * (32 * EPI_LD);
+        float* const fbuf = epi_tiles + (warp - 2) * (2 * FOLD_BLOCK);
         const int nkb = (p->K + BK - 1) / BK;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * 128);
         // which of the four 32-column blocks are written at all (uniform across the warp)
@@ -681,6 +685,31 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
           const int col0 = ti.n0 + half * 128 + 32 * b;
           if (col0 < p->Nd && quad_ok && !(p->symmetric && row_base >= col0 + 32)) need |= 1u << b;
         }
+        // The old values of D are copied to shared memory asynchronously, two of the four blocks while the chunks
+        // of the tile accumulate and the others as soon as a buffer is free: 16-byte pieces, piece c of row r at
+        // c ^ (r % 8), so that both the copies (a row's 128 bytes by eight lanes) and a thread's walk along its own
+        // row are free of bank conflicts.  (Loaded into registers beside the 128 running sums they were spilled, or
+        // exposed the latency of memory once per half block.)
+        auto piece = [&](int buf, int r, int c) { return fbuf + buf * FOLD_BLOCK + r * 32 + ((c ^ (r & 7)) * 4); };
+        const int cp_r = lane >> 3, cp_c = lane & 7;
+        float* const d0 = p->D + (long long)(row_base + cp_r) * p->ldd + ti.n0 + half * 128 + cp_c * 4;
+        const long long step = 4 * p->ldd;
+        auto rows_of = [&](int b) {                // groups of four rows of block b that exist in this lane's columns
+          if (!((need >> b) & 1u) || ti.n0 + half * 128 + 32 * b + cp_c * 4 >= p->Nd) return 0;
+          const int n_it = (p->Md - row_base - cp_r + 3) >> 2;
+          return n_it > 8 ? 8 : n_it;
+        };
+        auto fetch_old = [&](int b) {
+          const int n_it = beta != 0.0f ? rows_of(b) : 0;
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (i < n_it)
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(piece(b & 1, 4 * i + cp_r, cp_c))),
+                           "l"(d0 + 32 * b + i * step) : "memory");
+          asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        fetch_old(0);
+        fetch_old(1);
         // The running sum of this thread: its row, its warp's 128 columns.  The first chunk is loaded
         // straight into these registers; every later one is added with packed fp32 adds, one 32-column
         // block at a time (the other warp of the quadrant covers the load latency).
@@ -722,56 +751,31 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
           ++fold_seq;
         }
         if (!ok) break;
-        // ---- factor EMA D <- alpha sum + beta D on the blocks that touch the upper triangle, and their mirror image ----
+        // ---- factor EMA D <- alpha sum + beta D on the blocks that touch the upper triangle ----
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-          if (!((need >> b) & 1u)) continue;
-          const int col0 = ti.n0 + half * 128 + 32 * b;
+          asm volatile("cp.async.wait_group 1;" ::: "memory");
           __syncwarp();
+          if ((need >> b) & 1u) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) ftile[lane * EPI_LD + j] = __uint_as_float(sum[b][j]);
-          __syncwarp();
-          const int col = col0 + sub_c;
-          int n_it = 0;
-          if (col < p->Nd) { n_it = (p->Md - row_base - sub_r + 3) >> 2; n_it = n_it > 8 ? 8 : n_it; }
-          float* d = p->D + (long long)(row_base + sub_r) * p->ldd + col;
-          const long long step = 4 * p->ldd;
-          const bool mirror = p->symmetric && col0 >= row_base + 32;
-          // four row groups at a time (registers): read the old values, combine, write, and put the
-          // result back into the tile for the mirror image
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            float4 o[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              if (beta != 0.0f && 4 * h + i < n_it) o[i] = *reinterpret_cast<const float4*>(d + (4 * h + i) * step);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int it = 4 * h + i;
-              float* t4 = ftile + (it * 4 + sub_r) * EPI_LD + sub_c;
-              float4 r = make_float4(alpha * t4[0], alpha * t4[1], alpha * t4[2], alpha * t4[3]);
-              if (beta != 0.0f && it < n_it) {
-                r.x = fmaf(beta, o[i].x, r.x); r.y = fmaf(beta, o[i].y, r.y);
-                r.z = fmaf(beta, o[i].z, r.z); r.w = fmaf(beta, o[i].w, r.w);
+            for (int c = 0; c < 8; ++c) {
+              float4* q = reinterpret_cast<float4*>(piece(b & 1, lane, c));
+              float4 r = make_float4(alpha * __uint_as_float(sum[b][4 * c]), alpha * __uint_as_float(sum[b][4 * c + 1]),
+                                     alpha * __uint_as_float(sum[b][4 * c + 2]), alpha * __uint_as_float(sum[b][4 * c + 3]));
+              if (beta != 0.0f) {
+                const float4 o = *q;
+                r.x = fmaf(beta, o.x, r.x); r.y = fmaf(beta, o.y, r.y); r.z = fmaf(beta, o.z, r.z); r.w = fmaf(beta, o.w, r.w);
               }
-              if (it < n_it) *reinterpret_cast<float4*>(d + it * step) = r;
-              if (mirror) { t4[0] = r.x; t4[1] = r.y; t4[2] = r.z; t4[3] = r.w; }     // (each thread rewrites only what it read)
+              *q = r;
             }
           }
-          if (mirror) {
-            __syncwarp();
-            const int mrow0 = col0 + sub_r, mcol = row_base + sub_c;
-            if (mcol < p->Nd) {
+          __syncwarp();
+          const int n_it = rows_of(b);
 #pragma unroll
-              for (int it = 0; it < 8; ++it) {
-                const int mrow = mrow0 + it * 4;
-                if (mrow >= p->Md) break;
-                const float* t1 = ftile + sub_c * EPI_LD + (it * 4 + sub_r);
-                *reinterpret_cast<float4*>(p->D + (long long)mrow * p->ldd + mcol) =
-                    make_float4(t1[0], t1[EPI_LD], t1[2 * EPI_LD], t1[3 * EPI_LD]);
-              }
-            }
-          }
+          for (int i = 0; i < 8; ++i)
+            if (i < n_it) *reinterpret_cast<float4*>(d0 + 32 * b + i * step) = *reinterpret_cast<const float4*>(piece(b & 1, 4 * i + cp_r, cp_c));
+          __syncwarp();
+          if (b < 2) fetch_old(b + 2); else asm volatile("cp.async.commit_group;" ::: "memory");
         }
         continue;
       }
@@ -784,7 +788,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
         float v[32];
         tmem_ld32(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + c0), v);
         // nothing to write: rows beyond the matrix, or a block strictly below the diagonal of a
-        // symmetric product (its mirror image is written by the block above the diagonal)
+        // symmetric product
         if (!quad_ok || (p->symmetric && row_base >= col0 + 32)) continue;
         __syncwarp();
 #pragma unroll
@@ -818,27 +822,6 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
             }
             if (it < n_it) *reinterpret_cast<float4*>(d + it * step) = o;
             a[it] = o;
-          }
-          if (p->symmetric && col0 >= row_base + 32) {
-            // mirror image: element (r, c) of this block also is element (c, r) of the result
-            __syncwarp();
-#pragma unroll
-            for (int it = 0; it < 8; ++it) {
-              float* t4 = tile + (it * 4 + sub_r) * EPI_LD + sub_c;
-              t4[0] = a[it].x; t4[1] = a[it].y; t4[2] = a[it].z; t4[3] = a[it].w;
-            }
-            __syncwarp();
-            const int mrow0 = col0 + sub_r, mcol = row_base + sub_c;   // transposed block: rows col0.., columns row_base..
-            if (mcol < p->Nd) {
-#pragma unroll
-              for (int it = 0; it < 8; ++it) {
-                const int mrow = mrow0 + it * 4;
-                if (mrow >= p->Md) break;
-                const float* t1 = tile + sub_c * EPI_LD + (it * 4 + sub_r);
-                *reinterpret_cast<float4*>(p->D + (long long)mrow * p->ldd + mcol) =
-                    make_float4(t1[0], t1[EPI_LD], t1[2 * EPI_LD], t1[3 * EPI_LD]);
-              }
-            }
           }
         } else if (epi == EPI_ROTATED_ADAM) {
           float* d = p->D + (long long)(row_base + sub_r) * p->ldd + col;      // V~

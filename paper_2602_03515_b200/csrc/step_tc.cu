@@ -247,6 +247,16 @@ void destroy(RxPlans& r) {
 
 }  // namespace
 
+int complete_factors(Layer& L, cudaStream_t s, cudaError_t* e) {
+  *e = cudaSuccess;
+  if (!L.lower_stale) return 0;
+  int n = 0;
+  if (L.L) { if ((*e = mirror_lower(L.L, L.d.m, s)) != cudaSuccess) return -1; ++n; }
+  if (L.R) { if ((*e = mirror_lower(L.R, L.d.n, s)) != cudaSuccess) return -1; ++n; }
+  L.lower_stale = false;
+  return n;
+}
+
 struct TcStep {
   std::vector<Chunk> chunks;
   std::vector<TcPlan*> factor_plan;   // per layer, BR_ACCUM_ON_REFRESH only
@@ -434,7 +444,7 @@ int tc_step_run(TcStep* t, std::vector<Layer>& layers, const std::vector<const v
     int rc;
     if ((rc = lz.run(c.factors, "factor launch", calls, tau, dyn_alpha, dyn_beta))) return rc;
     if (c.factors)
-      for (int i : c.ids) if (G[i]) layers[i].n_accum += 1;
+      for (int i : c.ids) if (G[i]) { layers[i].n_accum += 1; layers[i].lower_stale = layers[i].L || layers[i].R; }
     std::vector<int> due, due_slots;
     for (size_t j = 0; j < c.ids.size(); ++j) {
       const int i = c.ids[j];
@@ -443,6 +453,7 @@ int tc_step_run(TcStep* t, std::vector<Layer>& layers, const std::vector<const v
       if (t->factor_plan[i]) {
         if ((rc = lz.run(t->factor_plan[i], "factor launch", calls, tau, dyn_alpha, dyn_beta))) return rc;
         L.n_accum += 1;
+        L.lower_stale = true;
       }
       due.push_back(i);
       due_slots.push_back((int)j);

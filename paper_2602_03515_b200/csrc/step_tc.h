@@ -17,6 +17,8 @@ struct Layer {
   float *M = nullptr, *V2 = nullptr, *U = nullptr, *V = nullptr, *L = nullptr, *R = nullptr;
   float* Morig = nullptr;             // tensor-core layers with S = 1st: M_t in the original space for a refresh
   __nv_bfloat16 *Uh = nullptr, *Ul = nullptr, *Vh = nullptr, *Vl = nullptr;  // bf16 hi/lo of U, V
+  // tensor-core layers accumulate the upper block triangles of L and R only; set while their lower ones lag behind
+  bool lower_stale = false;
   char* ring = nullptr;
   int ring_slots = 0;                 // physical slots: tau_max, or 1 for a tensor-core layer without delay
   size_t slot_stride = 0;             // bytes between ring slots
@@ -31,6 +33,10 @@ void rotated_sides(int64_t m, int64_t n, int geom, bool* left, bool* right);
 cudaError_t fdgemm(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha, const float* A,
                    int64_t lda, const double* B, int64_t ldb, double beta, double* C, int64_t ldc,
                    cudaStream_t s);
+
+// Brings the lower block triangles of L and R up to date if they lag behind.  Returns the number of launches, or -1
+// with the error in *e.
+int complete_factors(Layer& L, cudaStream_t s, cudaError_t* e);
 
 struct TcStep;
 struct TcStepCallbacks {

@@ -343,7 +343,7 @@ br_status deflated_power(br_handle* h, br_handle::Lane& ln, QrTc* tcq, int64_t k
   double* T1 = W1 + r;                                // leading dimension 2r
   const size_t rb = sizeof(double) * r, pk = sizeof(double) * k, p2 = sizeof(double) * r2;
   // B = F U_s ; Lam = U_s^T B ; C1 = U_s^T Q ; C2 = B^T Q
-  BR_CUDA(h, dgemm(0, 0, k, r, k, 1.0, F, k, Us, k, 0.0, B, r2, s));
+  BR_CUDA(h, dgemm_ex(0, 0, k, r, k, 1.0, F, k, Us, k, 0.0, B, r2, 4, part, nullptr, s));
   BR_CUDA(h, dgemm_ex(1, 0, r, r, k, 1.0, Us, k, B, r2, 0.0, Lam, r, sp_small, part, nullptr, s));
   BR_CUDA(h, dgemm_ex(1, 0, r, k, k, 1.0, Us, k, Q, k, 0.0, C1, k, 4, part, nullptr, s));
   BR_CUDA(h, dgemm_ex(1, 0, r, k, k, 1.0, B, r2, Q, k, 0.0, C2, k, 4, part, nullptr, s));
@@ -361,7 +361,7 @@ br_status deflated_power(br_handle* h, br_handle::Lane& ln, QrTc* tcq, int64_t k
   BR_CUDA(h, dgemm(0, 0, r, k, r, -1.0, Lam, r, C1, k, 1.0, C2, k, s));
   BR_CUDA(h, f32_to_f64(Af, ln.rA, k * k, s));
   BR_CUDA(h, dgemm(0, 0, k, k, r2, 1.0, W2, r2, C1, k, 1.0, ln.rA, k, s));
-  count(h, 20);
+  count(h, 21);
   h->stats.gemm_flops += 14.0 * k * k * r;
   return BR_OK;
 }
@@ -438,7 +438,7 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
         br_status st = deflated_power(h, ln, tcq, k, s);
         if (st != BR_OK) return st;
       } else if (one) {
-        BR_CUDA(h, sdgemm(0, 0, k, k, k, 1.0, F, k, Q, k, 0.0, ln.rA, k, s));
+        BR_CUDA(h, sdgemm(0, k, k, k, 1.0, F, k, Q, k, 0.0, ln.rA, k, s));
         count(h); h->stats.gemm_flops += 2.0 * k * k * k;
       } else {
         BR_CUDA(h, f32_to_f64(F, ln.rF, k * k, s));
@@ -447,13 +447,13 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
       }
     } else if (left_side) {
       // (M M^T) U = M (M^T U)
-      BR_CUDA(h, sdgemm(1, 0, n, m, m, 1.0, Mo, n, Q, m, 0.0, ln.rZ, m, s));
-      BR_CUDA(h, fdgemm(0, 0, m, m, n, 1.0, Mo, n, ln.rZ, m, 0.0, ln.rA, m, s));
+      BR_CUDA(h, sdgemm(1, n, m, m, 1.0, Mo, n, Q, m, 0.0, ln.rZ, m, s));
+      BR_CUDA(h, fdgemm(0, m, m, n, 1.0, Mo, n, ln.rZ, m, 0.0, ln.rA, m, s));
       count(h, 2); h->stats.gemm_flops += 4.0 * m * m * n;
     } else {
       // (M^T M) V = M^T (M V)
-      BR_CUDA(h, sdgemm(0, 0, m, n, n, 1.0, Mo, n, Q, n, 0.0, ln.rZ, n, s));
-      BR_CUDA(h, fdgemm(1, 0, n, n, m, 1.0, Mo, n, ln.rZ, n, 0.0, ln.rA, n, s));
+      BR_CUDA(h, sdgemm(0, m, n, n, 1.0, Mo, n, Q, n, 0.0, ln.rZ, n, s));
+      BR_CUDA(h, fdgemm(1, n, n, m, 1.0, Mo, n, ln.rZ, n, 0.0, ln.rA, n, s));
       count(h, 2); h->stats.gemm_flops += 4.0 * n * n * m;
     }
     // A rank-deficient product has no unique Q factor.  Which products are is known on the host: with

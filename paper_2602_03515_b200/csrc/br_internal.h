@@ -139,9 +139,11 @@ cudaError_t sgemm(int ta, int tb, int64_t M, int64_t N, int64_t K, float alpha, 
                   int64_t lda, const float* B, int64_t ldb, float beta, float* C, int64_t ldc,
                   cudaStream_t s);
 // fp32 inputs, fp64 accumulation and output (power step F Q of a refresh)
-cudaError_t sdgemm(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha, const float* A,
-                   int64_t lda, const float* B, int64_t ldb, double beta, double* C, int64_t ldc,
-                   cudaStream_t s);
+cudaError_t sdgemm(int ta, int64_t M, int64_t N, int64_t K, double alpha, const float* A, int64_t lda, const float* B,
+                   int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t s);
+// the same with an fp64 second operand
+cudaError_t fdgemm(int ta, int64_t M, int64_t N, int64_t K, double alpha, const float* A, int64_t lda, const double* B,
+                   int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t s);
 cudaError_t dgemm(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha, const double* A,
                   int64_t lda, const double* B, int64_t ldb, double beta, double* C, int64_t ldc,
                   cudaStream_t s);
@@ -177,6 +179,10 @@ cudaError_t orth_whole(double* A, int64_t k, double* work, double* Acopy, const 
 // C: room for the largest coefficient block, (w / 2)^2 doubles.
 cudaError_t orth_part(double* A, int64_t k, int64_t j0, int64_t w, double* C, int first, double ill_ratio, const double* norm0,
                       double* rdiag, int* status, int* flags, const int* skip, cudaStream_t s);
+// fp64 products in tiles of 64 x 64; with nsplit > 1 the partial sums only, nsplit x M x N at `partial`.
+cudaError_t dgemm64(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha, const double* A, int64_t lda, const double* B,
+                    int64_t ldb, double beta, double* C, int64_t ldc, int nsplit, int64_t k_per_split, double* partial, const int* skip,
+                    cudaStream_t s);
 // C = alpha op(A) B + beta C with fp64 accumulation and output, in tiles of 64 x 64.
 cudaError_t product64(int ta, int64_t M, int64_t N, int64_t K, double alpha, const float* A, int64_t lda, const float* B,
                       int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t s);

@@ -71,7 +71,7 @@ extern "C" br_status br_power_static(void* cuda_stream, const float* F, float* Q
   // The array keeps whatever the previous call left.  Only the flag has to start at zero; every
   // other word is written by this call before it is read.
   if (cudaMemsetAsync(flag, 0, sizeof(int), s) != cudaSuccess) return BR_ERR_CUDA;
-  if (sdgemm(0, 0, k, k, k, 1.0, F, k, Q, k, 0.0, A, k, s) != cudaSuccess) return BR_ERR_CUDA;
+  if (sdgemm(0, k, k, k, 1.0, F, k, Q, k, 0.0, A, k, s) != cudaSuccess) return BR_ERR_CUDA;
   if (orth_whole(A, k, work, nullptr, nullptr, Q, nullptr, nullptr, flag, nullptr, s) != cudaSuccess) return BR_ERR_CUDA;
   return BR_OK;
 }

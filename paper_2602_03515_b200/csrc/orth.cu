@@ -88,11 +88,12 @@ template <bool SYM> __device__ __forceinline__ int tile_row() { return 16 * warp
 template <bool SYM> __device__ __forceinline__ int tile_col() { return 32 * warp_n<SYM>() + 2 * (threadIdx.x & 3); }
 
 // One stage (16 contraction steps) of acc += (or -=, NEG) a b.  I: rows of the tile that exist.
-template <bool DIRECT, bool SYM, bool NEG>
+// BT: the second operand is staged [64][contraction] like a first operand that is not DIRECT.
+template <bool DIRECT, bool SYM, bool NEG, bool BT = false>
 __device__ __forceinline__ void mma_stage(double (&acc)[16], const double* As, const double* Bs, int I) {
   const int lane = threadIdx.x & 31, g = lane >> 2, tig = lane & 3, wm = warp_m<SYM>(), wn = warp_n<SYM>();
   As += DIRECT ? tig * kLdK + 16 * wm + g : (16 * wm + g) * kLdI + tig;
-  Bs += tig * kLdK + 32 * wn + g;
+  Bs += BT ? (32 * wn + g) * kLdI + tig : tig * kLdK + 32 * wn + g;
   if (16 * wm >= I || (SYM && 4 * wn + 3 < 2 * wm)) return;
   const bool two = 16 * wm + 8 < I;
 #pragma unroll
@@ -101,7 +102,7 @@ __device__ __forceinline__ void mma_stage(double (&acc)[16], const double* As, c
     if (NEG) { a0 = -a0; a1 = -a1; }
     double b[4];
 #pragma unroll
-    for (int ni = 0; ni < 4; ++ni) b[ni] = Bs[k4 * kLdK + 8 * ni];
+    for (int ni = 0; ni < 4; ++ni) b[ni] = Bs[BT ? 8 * ni * kLdI + k4 : k4 * kLdK + 8 * ni];
 #pragma unroll
     for (int ni = 0; ni < 4; ++ni)
       if (!SYM || 4 * wn + ni >= 2 * wm) dmma(acc[2 * ni], acc[2 * ni + 1], a0, b[ni]);
@@ -122,23 +123,25 @@ __device__ __forceinline__ void copy_async(double* dst, const double* src, bool 
 }
 // acc += sum over kk < K of a(i, kk) b(kk, j), i < I <= 64, j < J <= 64 (NEG: -=).
 //   DIRECT: a(i, kk) = X[kk * lda + i]   otherwise a(i, kk) = X[i * lda + kk];   b(kk, j) = Y[kk * ldb + j].
+//   BT: b(kk, j) = Y[j * ldb + kk].
 // VEC: all dimensions and leading dimensions that a copy runs along are even, and X and Y 16-byte aligned.
-template <bool VEC, bool DIRECT, bool SYM, bool NEG>
+template <bool VEC, bool DIRECT, bool SYM, bool NEG, bool BT = false>
 __device__ __forceinline__ void mm64(double (&acc)[16], const double* X, int64_t lda, int I, const double* Y, int64_t ldb, int J, int K) {
   constexpr int V = VEC ? 2 : 1, N = 4 / V;                // doubles per copy; copies per thread, operand and stage
   const int t = threadIdx.x;
   // thread -> first element of an operand tile, and the distance of its next one
   constexpr int RK = kT / (64 / V), RI = kT / (kKs / V);   // rows of a [16][64] / [64][16] tile covered by one copy per thread
-  const int bk = t / (64 / V), bj = t % (64 / V) * V;
-  const int ak = DIRECT ? bk : t % (kKs / V) * V, ai = DIRECT ? bj : t / (kKs / V);
+  constexpr int STAGE = kOper + (BT ? kOper : kOperB);
+  const int dk = t / (64 / V), di = t % (64 / V) * V, sk = t % (kKs / V) * V, si = t / (kKs / V);   // [16][64] and [64][16] tiles
+  const int ak = DIRECT ? dk : sk, ai = DIRECT ? di : si, bk = BT ? sk : dk, bj = BT ? si : di;
   const double* px = X + (DIRECT ? (int64_t)ak * lda + ai : (int64_t)ai * lda + ak);
-  const double* py = Y + (int64_t)bk * ldb + bj;
-  const int64_t xq = (DIRECT ? RK : RI) * lda, xs = DIRECT ? kKs * lda : kKs, yq = RK * ldb, ys = kKs * ldb;
+  const double* py = Y + (BT ? (int64_t)bj * ldb + bk : (int64_t)bk * ldb + bj);
+  const int64_t xq = (DIRECT ? RK : RI) * lda, xs = DIRECT ? kKs * lda : kKs, yq = (BT ? RI : RK) * ldb, ys = BT ? kKs : kKs * ldb;
   double* const dA = sm + oStage + (DIRECT ? ak * kLdK + ai : ai * kLdI + ak);
-  double* const dB = sm + oStage + kOper + bk * kLdK + bj;
+  double* const dB = sm + oStage + kOper + (BT ? bj * kLdI + bk : bk * kLdK + bj);
   const int nk = (K + kKs - 1) / kKs;
   auto fetch = [&](int s) {
-    const int k0 = s * kKs, buf = (s % kStages) * (kOper + kOperB);
+    const int k0 = s * kKs, buf = (s % kStages) * STAGE;
 #pragma unroll
     for (int q = 0; q < N; ++q) {
       const bool ok = DIRECT ? (ai < I && k0 + ak + q * RK < K) : (ai + q * RI < I && k0 + ak < K);
@@ -146,8 +149,8 @@ __device__ __forceinline__ void mm64(double (&acc)[16], const double* X, int64_t
     }
 #pragma unroll
     for (int q = 0; q < N; ++q) {
-      const bool ok = bj < J && k0 + bk + q * RK < K;
-      copy_async<VEC>(dB + buf + q * RK * kLdK, ok ? py + q * yq : Y, ok);
+      const bool ok = BT ? (bj + q * RI < J && k0 + bk < K) : (bj < J && k0 + bk + q * RK < K);
+      copy_async<VEC>(dB + buf + (BT ? q * RI * kLdI : q * RK * kLdK), ok ? py + q * yq : Y, ok);
     }
     px += xs; py += ys;
   };
@@ -162,8 +165,8 @@ __device__ __forceinline__ void mm64(double (&acc)[16], const double* X, int64_t
     __syncthreads();                             // stage s is in place, and stage s - 1 has been read
     if (s + kStages - 1 < nk) fetch(s + kStages - 1);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    const double* st = sm + oStage + buf * (kOper + kOperB);
-    mma_stage<DIRECT, SYM, NEG>(acc, st, st + kOper, I);
+    const double* st = sm + oStage + buf * STAGE;
+    mma_stage<DIRECT, SYM, NEG, BT>(acc, st, st + kOper, I);
     if (++buf == kStages) buf = 0;
   }
   __syncthreads();
@@ -227,6 +230,45 @@ k_product64(int M, int N, int K, double alpha, const float* __restrict__ X, int6
     v *= alpha;
     *c = beta != 0.0 ? fma(beta, *c, v) : v;
   });
+}
+
+// C = alpha op(X) op(Y) + beta C in fp64, one 64 x 64 tile and a range of the contraction per CTA (split over
+// blockIdx.z: partial sums, added by a second kernel).
+template <bool VEC, bool TRANS, bool BT>
+__global__ void __launch_bounds__(kT, 2)
+k_dgemm64(int M, int N, int K, double alpha, const double* X, int64_t lda, const double* Y, int64_t ldb, double beta, double* C,
+          int64_t ldc, int k_per_split, double* partial, const int* skip) {
+  if (skip && *skip) return;            // uniform: a device-side flag cancels the whole launch
+  const int m0 = (int)blockIdx.y * 64, n0 = (int)blockIdx.x * 64, k0 = (int)blockIdx.z * k_per_split;
+  double acc[16];
+  clear(acc);
+  mm64<VEC, TRANS, false, false, BT>(acc, X + (TRANS ? (int64_t)k0 * lda + m0 : (int64_t)m0 * lda + k0), lda, min(64, M - m0),
+                                     Y + (BT ? (int64_t)n0 * ldb + k0 : (int64_t)k0 * ldb + n0), ldb, min(64, N - n0), min(k_per_split, K - k0));
+  const bool split = gridDim.z > 1;
+  each_entry(acc, M - m0, N - n0, [&](int i, int j, double v) {
+    if (split) { partial[((int64_t)blockIdx.z * M + m0 + i) * N + n0 + j] = v; return; }
+    double* c = C + (int64_t)(m0 + i) * ldc + n0 + j;
+    v *= alpha;
+    *c = beta != 0.0 ? fma(beta, *c, v) : v;
+  });
+}
+constexpr int kDgemmSmem = kStages * 2 * kOper * (int)sizeof(double);
+
+template <bool VEC, bool TRANS, bool BT>
+cudaError_t launch_dgemm(dim3 grid, int64_t M, int64_t N, int64_t K, double alpha, const double* A, int64_t lda, const double* B,
+                         int64_t ldb, double beta, double* C, int64_t ldc, int64_t k_per_split, double* partial, const int* skip,
+                         cudaStream_t s) {
+  static bool attr_set[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < 64 && !attr_set[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(k_dgemm64<VEC, TRANS, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDgemmSmem);
+    if (e != cudaSuccess) return e;
+    attr_set[dev] = true;
+  }
+  k_dgemm64<VEC, TRANS, BT><<<grid, kT, kDgemmSmem, s>>>((int)M, (int)N, (int)K, alpha, A, lda, B, ldb, beta, C, ldc, (int)k_per_split,
+                                                        partial, skip);
+  return cudaGetLastError();
 }
 
 template <typename TB>
@@ -744,6 +786,20 @@ cudaError_t product64(int ta, int64_t M, int64_t N, int64_t K, double alpha, con
 cudaError_t product64(int ta, int64_t M, int64_t N, int64_t K, double alpha, const float* A, int64_t lda, const double* B,
                       int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t s) {
   return launch_product(ta, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s);
+}
+
+cudaError_t dgemm64(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha, const double* A, int64_t lda, const double* B,
+                    int64_t ldb, double beta, double* C, int64_t ldc, int nsplit, int64_t k_per_split, double* partial, const int* skip,
+                    cudaStream_t s) {
+  const dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64), (unsigned)nsplit);
+  const bool vec = ((M | N | K | lda | ldb) & 1) == 0 && ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0;
+#define BR_DGEMM64(T, B_) \
+  return vec ? launch_dgemm<true, T, B_>(grid, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, k_per_split, partial, skip, s) \
+             : launch_dgemm<false, T, B_>(grid, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, k_per_split, partial, skip, s)
+  if (ta) { if (tb) BR_DGEMM64(true, true); BR_DGEMM64(true, false); }
+  if (tb) BR_DGEMM64(false, true);
+  BR_DGEMM64(false, false);
+#undef BR_DGEMM64
 }
 
 }  // namespace br

@@ -334,9 +334,10 @@ void project(Sweep& q, int64_t jp, int64_t wp, int64_t jt, int64_t wt) {
     q.launches += 13;
     return;
   }
-  const int64_t tiles = cdiv(wp, 128) * cdiv(wt, 128);
+  // fewer tiles of 64 x 64 than two per SM: split the contraction until there are four
+  const int64_t tiles = cdiv(wp, 64) * cdiv(wt, 64);
   int sp = 1;
-  if (tiles < 148) sp = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(cdiv(296, tiles), kProjSplitsMax), k / 128));
+  if (tiles < 296) sp = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(cdiv(592, tiles), kProjSplitsMax), k / 128));
   cudaError_t e = dgemm_ex(1, 0, wp, wt, k, 1.0, q.A + jp, k, q.A + jt, k, 0.0, q.C, wt, sp, q.proj_part, q.skip, q.s);
   if (e == cudaSuccess)
     e = dgemm_ex(0, 0, k, wt, wp, -1.0, q.A + jp, k, q.C, wt, 1.0, q.A + jt, k, 1, nullptr, q.skip, q.s);
@@ -359,9 +360,9 @@ void orth(Sweep& q, int64_t j0, int64_t w) {
   orth(q, j0 + h, w - h);
 }
 
-// a projection is split only while it has fewer than 148 tiles of 128 x 128
+// a projection is split only while it has fewer than 296 tiles of 64 x 64
 inline int64_t proj_part_doubles(int64_t k) {
-  return std::min<int64_t>((int64_t)kProjSplitsMax * ((k + 1) / 2) * ((k + 1) / 2), (int64_t)(296 + 148) * 128 * 128);
+  return std::min<int64_t>((int64_t)kProjSplitsMax * ((k + 1) / 2) * ((k + 1) / 2), (int64_t)(592 + 296) * 64 * 64);
 }
 
 }  // namespace

@@ -30,10 +30,6 @@ std::string format(const char* fmt, ...);
 size_t dtype_size(int dt);
 void rotated_sides(int64_t m, int64_t n, int geom, bool* left, bool* right);
 
-cudaError_t fdgemm(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha, const float* A,
-                   int64_t lda, const double* B, int64_t ldb, double beta, double* C, int64_t ldc,
-                   cudaStream_t s);
-
 // Brings the lower block triangles of L and R up to date if they lag behind.  Returns the number of launches, or -1
 // with the error in *e.
 int complete_factors(Layer& L, cudaStream_t s, cudaError_t* e);

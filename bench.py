@@ -573,7 +573,7 @@ def main():
         ref_flops = sum((2.0 + 8.0 / 3.0) * float(k) ** 3 for k in orders)
         ref_tflops = ref_flops / (refresh_ms / 1e3) / 1e12
         fp64_peak = 148 * 64 * 2 * 1.965e9 / 1e12       # 148 SMs x 64 fp64 FMA per clock (mma.sync.m8n8k4.f64) x 2 x 1.965 GHz
-        roofline_refresh = {"bound": "fp64 matrix unit / tensor", "kernel": "k_dgemm + k_chol_inverse + k_tc_gemm (three-term bf16 splits)",
+        roofline_refresh = {"bound": "fp64 matrix unit / tensor", "kernel": "k_orth_cluster + k_dgemm64 + k_tc_gemm (three-term bf16 splits)",
                             "bases": len(orders), "algorithmic_flops": ref_flops, "achieved": ref_tflops, "unit": "TFLOP/s",
                             "peak_fp64_unit": fp64_peak, "frac_of_fp64_unit": ref_tflops / fp64_peak,
                             "peak_bf16_split6": peaks["tf_sustained"] / 6.0, "frac_of_bf16_split6": ref_tflops / (peaks["tf_sustained"] / 6.0),

@@ -108,17 +108,18 @@ struct br_handle {
     char* tcq_scratch = nullptr;          // scratch of the tensor-core projections (largest eligible order)
     std::vector<QrTc*> tcq;               // their plans, one per distinct eligible order
     int64_t cap_k = 0;                    // largest order this lane's buffers hold
-    // The orthonormalisation of one basis is several hundred dependent launches whose arguments
-    // depend only on the lane (its buffers) and on the order: it is captured into a CUDA graph the
-    // first time and replayed afterwards, one launch per basis.  Key: 2 * order + (tensor-core form).
+    // The orthonormalisation of one basis of an order from 2048 on is a chain of launches whose arguments depend
+    // only on the lane (its buffers) and on the order: it is captured into a CUDA graph the first time and
+    // replayed afterwards, one launch per basis.  Key: 2 * order + (tensor-core form).
     struct QrGraph { cudaGraphExec_t exec = nullptr; int64_t launches = 0; double flops = 0.0; };
     std::map<int64_t, QrGraph> qr_graphs;
     int* cond = nullptr;                  // conditioning note of the lane's current job (device)
   };
   bool use_graphs = true;                 // cleared when a capture fails (BR_REFRESH_GRAPHS=0 switches it off)
-  // Up to three lanes hold the largest order; up to five more hold only the small orders (at most
-  // 1/sqrt(2) of the largest, S = 2nd), whose refresh is a chain of short launches that leaves most of
-  // the GPU idle: eight streams in all, the default number of hardware queues.
+  // Eight streams in all, the default number of hardware queues.  When the largest order is one that a single
+  // cluster factorises, every lane holds it: a cluster leaves 132 SMs to the others (ten steps and the 32 bases of a d = 384 decoder:
+  // 27.2 -> 16.2 ms against three full-size lanes).  Otherwise three lanes do, whose products fill the GPU, and up to
+  // five more hold only the small orders (at most 1/sqrt(2) of the largest, S = 2nd).
   static constexpr int kBigLanes = 3;       // default number of full-size lanes (BR_REFRESH_LANES: 1..6)
   static constexpr int kMaxBigLanes = 6;
   static constexpr int kMaxLanes = 8;       // lanes of both kinds

@@ -6,11 +6,28 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <atomic>
 #include <vector>
 
 #include "br.h"
 
 namespace br {
+
+// Something that has to be done once per device before a kernel's first launch there (its shared-memory
+// attribute).  Host threads that drive different handles may come here at the same time: each that finds it undone
+// does it, which is harmless, and what it noted is seen only after it is done.
+struct OncePerDevice {
+  std::atomic<bool> done[64] = {};
+  template <typename FN> cudaError_t run(FN set) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool tracked = dev >= 0 && dev < 64;
+    if (tracked && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    if ((e = set()) == cudaSuccess && tracked) done[dev].store(true, std::memory_order_release);
+    return e;
+  }
+};
 
 // ---------------------------------------------------------------------------------------------
 // Launch accounting (reported through br_get_launch_stats)

@@ -258,14 +258,9 @@ template <bool VEC, bool TRANS, bool BT>
 cudaError_t launch_dgemm(dim3 grid, int64_t M, int64_t N, int64_t K, double alpha, const double* A, int64_t lda, const double* B,
                          int64_t ldb, double beta, double* C, int64_t ldc, int64_t k_per_split, double* partial, const int* skip,
                          cudaStream_t s) {
-  static bool attr_set[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(k_dgemm64<VEC, TRANS, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDgemmSmem);
-    if (e != cudaSuccess) return e;
-    attr_set[dev] = true;
-  }
+  static OncePerDevice once;
+  const cudaError_t e = once.run([] { return cudaFuncSetAttribute(k_dgemm64<VEC, TRANS, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDgemmSmem); });
+  if (e != cudaSuccess) return e;
   k_dgemm64<VEC, TRANS, BT><<<grid, kT, kDgemmSmem, s>>>((int)M, (int)N, (int)K, alpha, A, lda, B, ldb, beta, C, ldc, (int)k_per_split,
                                                         partial, skip);
   return cudaGetLastError();

@@ -256,14 +256,9 @@ namespace {
 template <int NJ>
 cudaError_t launch(const SmallJob* jobs, int n, float lr, float beta1, float beta2, float eps, float weight_decay, float beta_factor,
                    cudaStream_t s) {
-  static bool attr_set[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(k_small_step<NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-    if (e != cudaSuccess) return e;
-    attr_set[dev] = true;
-  }
+  static OncePerDevice once;
+  const cudaError_t e = once.run([] { return cudaFuncSetAttribute(k_small_step<NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem); });
+  if (e != cudaSuccess) return e;
   SmallGroup<NJ> g;
   g.lr = lr; g.beta1 = beta1; g.beta2 = beta2; g.eps = eps; g.decay = 1.0f - lr * weight_decay; g.beta_factor = beta_factor;
   size_t bytes = 0;

@@ -176,11 +176,12 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-// Hands an accumulator back.  What it orders are tcgen05.ld of this warp (tcgen05.fence::before_thread_sync stands in
-// front of it); no data in memory passes with it, so the default scope is enough.  A release at cluster scope
-// would make the warp wait for its global stores of the tile before (a quarter of all stalls of the folded form).
+// Hands an accumulator back to the CTA that issues the MMAs, which may be the other one of the pair: cluster scope.
+// What it orders are tcgen05.ld of this warp, and those are ordered by the tcgen05.fence::before_thread_sync in front
+// of it; no data in memory passes with it, so it need not be a release.  (A release at cluster scope would make the
+// warp wait for its global stores of the tile before, a quarter of all stalls of the folded form.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 __device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t cluster_addr) {
   uint32_t v;

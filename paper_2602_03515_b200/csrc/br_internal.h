@@ -119,8 +119,8 @@ cudaError_t ema_out(float* out, const float* M, const void* G, int g_is_bf16, in
                     const float* gscale, cudaStream_t s);
 
 // One whole update (Alg. 1 (momentum, rotation, second moment, weight update) and the factor EMAs of Alg. 2, no refresh) of
-// matrices with both dimensions <= 128, a CTA each, in one launch per 24 of them (small_step.cu).  accumulate:
-// update L and R as well.
+// matrices with both dimensions <= 128, a cluster of up to four CTAs each, in one launch per 24 of them
+// (small_step.cu).  accumulate: update L and R as well.
 bool small_step_eligible(int64_t m, int64_t n, bool left, bool right);
 struct SmallJob {
   int m, n, left, right;    // shape, and which sides are rotated

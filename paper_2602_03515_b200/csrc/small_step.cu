@@ -10,8 +10,11 @@
 // operands whose contraction index is the slow one (an 8- and a 16-byte read per step for 8 multiply-adds; the
 // rotation of G and of M shares the basis' read).  That takes G, U and V in both orientations; T, X and Y are
 // written in the one the next product reads.  Bound by the shared-memory reads of one SM, hence the cluster:
-// a 64 x 32 matrix took 33 us with a dot product per thread, 18 us with 4 x 4 tiles on one CTA, 13 us now.
+// a 64 x 32 matrix took 33 us with a dot product per thread, 18 us with 4 x 4 tiles on one CTA, 13 us now.  Matrices
+// of a few hundred entries keep the dot product per thread (k_tiny_step).
 #include <cooperative_groups.h>
+
+#include <algorithm>
 
 #include "br_internal.h"
 
@@ -236,6 +239,110 @@ __global__ void __launch_bounds__(kThreads) k_small_step(const __grid_constant__
   }
 }
 
+// The same update for launches of tiny matrices only (tiny_eligible), a CTA each and a dot product per thread.  Such a
+// matrix is bound by the latency of its loads and barriers: the form above stages more copies, zero-padded, behind
+// index arithmetic and a second set of barriers.  Kernel time on one matrix, here and above, us: 8 x 8 4.8 and 7.4,
+// 16 x 16 5.7 and 7.2, 32 x 4 6.3 and 9.0, 40 x 8 rotated on the right only 4.4 and 6.0.
+constexpr int kTinyThreads = 512, kTinySmem = 80 * 1024;
+template <int NJ>
+__global__ void __launch_bounds__(kTinyThreads) k_tiny_step(const __grid_constant__ SmallGroup<NJ> grp) {
+  extern __shared__ __align__(16) float sm[];
+  const SmallJob& a = grp.j[blockIdx.x];
+  const int m = a.m, n = a.n, mn = m * n, t = threadIdx.x;
+  const int ln = n | 1, lm = m | 1;           // odd: a walk along a column touches different banks
+  float* sG = sm;                             // G, later X
+  float* sM = sG + m * ln;                    // M, later Y
+  float* sT1 = sM + m * ln;                   // first-side products of G and of M
+  float* sT2 = sT1 + m * ln;
+  float* sU = sT2 + m * ln;                   // m x m (left side rotated)
+  float* sV = sU + (a.left ? m * lm : 0);     // n x n (right side rotated)
+  const float gs = a.gscale ? *a.gscale : 1.0f;
+  for (int e = t; e < mn; e += kTinyThreads) {
+    const float g = gs * (a.g_is_bf16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(a.G)[e]) : reinterpret_cast<const float*>(a.G)[e]);
+    const float mo = grp.beta1 * a.M[e] + (1.0f - grp.beta1) * g;
+    const int at = e / n * ln + e % n;
+    sG[at] = g; sM[at] = mo; a.M[e] = mo;
+  }
+  if (a.left) for (int e = t; e < m * m; e += kTinyThreads) sU[e / m * lm + e % m] = a.U[e];
+  if (a.right) for (int e = t; e < n * n; e += kTinyThreads) sV[e / n * ln + e % n] = a.V[e];
+  __syncthreads();
+  if (a.accumulate) {                         // L <- b L + (1 - b) G G^T ; R <- b R + (1 - b) G^T G
+    const float b = grp.beta_factor, ob = 1.0f - grp.beta_factor;
+    if (a.L)
+      for (int e = t; e < m * m; e += kTinyThreads) {
+        const int i = e / m, j = e % m;
+        float s = 0.f;
+        for (int k = 0; k < n; ++k) s = fmaf(sG[i * ln + k], sG[j * ln + k], s);
+        a.L[e] = b * a.L[e] + ob * s;
+      }
+    if (a.R)
+      for (int e = t; e < n * n; e += kTinyThreads) {
+        const int i = e / n, j = e % n;
+        float s = 0.f;
+        for (int k = 0; k < m; ++k) s = fmaf(sG[k * ln + i], sG[k * ln + j], s);
+        a.R[e] = b * a.R[e] + ob * s;
+      }
+  }
+  for (int e = t; e < mn; e += kTinyThreads) {           // T1 = U^T G, T2 = U^T M
+    const int i = e / n, j = e % n;
+    float s1 = sG[i * ln + j], s2 = sM[i * ln + j];
+    if (a.left) {
+      s1 = 0.f; s2 = 0.f;
+      for (int k = 0; k < m; ++k) { const float u = sU[k * lm + i]; s1 = fmaf(u, sG[k * ln + j], s1); s2 = fmaf(u, sM[k * ln + j], s2); }
+    }
+    sT1[i * ln + j] = s1; sT2[i * ln + j] = s2;
+  }
+  __syncthreads();
+  for (int e = t; e < mn; e += kTinyThreads) {           // G~ = T1 V, M~ = T2 V, second moment, X
+    const int i = e / n, j = e % n;
+    float gt = sT1[i * ln + j], mt = sT2[i * ln + j];
+    if (a.right) {
+      gt = 0.f; mt = 0.f;
+      for (int k = 0; k < n; ++k) { const float v = sV[k * ln + j]; gt = fmaf(sT1[i * ln + k], v, gt); mt = fmaf(sT2[i * ln + k], v, mt); }
+    }
+    const float v2 = grp.beta2 * a.V2[e] + (1.0f - grp.beta2) * gt * gt;
+    a.V2[e] = v2;
+    sG[i * ln + j] = mt / sqrtf(v2 + grp.eps);
+  }
+  __syncthreads();
+  for (int e = t; e < mn; e += kTinyThreads) {           // Y = U X
+    const int i = e / n, j = e % n;
+    float y = sG[i * ln + j];
+    if (a.left) {
+      y = 0.f;
+      for (int k = 0; k < m; ++k) y = fmaf(sU[i * lm + k], sG[k * ln + j], y);
+    }
+    sM[i * ln + j] = y;
+  }
+  __syncthreads();
+  for (int e = t; e < mn; e += kTinyThreads) {           // W <- decay W - eta Y V^T
+    const int i = e / n, j = e % n;
+    float d = sM[i * ln + j];
+    if (a.right) {
+      d = 0.f;
+      for (int k = 0; k < n; ++k) d = fmaf(sM[i * ln + k], sV[j * ln + k], d);
+    }
+    a.W[e] = grp.decay * a.W[e] - grp.lr * d;
+  }
+}
+
+size_t tiny_bytes(int64_t m, int64_t n, bool left, bool right) {
+  return sizeof(float) * (size_t)(4 * m * (n | 1) + (left ? m * (m | 1) : 0) + (right ? n * (n | 1) : 0));
+}
+// In this range the form above takes about as long for every size, and this one as many steps as its phases have
+// passes over their entries times terms of a dot product: 264 steps are 9 to 11 us either way while a pass covers the
+// matrix, and beyond that the lines are where a sweep of 259 shapes, each with one and with two rotated sides, with
+// and without factors, has the two level (the worst of the 1036 is 14 % above what the one form alone took before the
+// other existed, 24 are more than 3 %).
+bool tiny_eligible(const SmallJob& j) {
+  const int m = j.m, n = j.n;
+  auto passes = [](int entries) { return (entries + kTinyThreads - 1) / kTinyThreads; };
+  int steps = 2 * passes(m * n) * ((j.left ? m : 0) + (j.right ? n : 0));
+  if (j.accumulate) steps += (j.L ? passes(m * m) * n : 0) + (j.R ? passes(n * n) * m : 0);
+  return m * n < 1024 && steps <= (m * n <= kTinyThreads ? 264 : j.left && j.right ? 240 : 136) &&
+         tiny_bytes(m, n, j.left != 0, j.right != 0) <= (size_t)kTinySmem;
+}
+
 size_t small_bytes(int64_t m64, int64_t n64, bool left, bool right) {
   const int m = (int)m64, n = (int)n64, mp = up4(m), np = up4(n), lm = ldp(m), ln = ldp(n);
   size_t f = (size_t)mp * ln + (size_t)np * lm + 2 * (left ? (size_t)mp * ln : (size_t)np * lm);
@@ -254,17 +361,32 @@ bool small_step_eligible(int64_t m, int64_t n, bool left, bool right) {
 
 namespace {
 template <int NJ>
+SmallGroup<NJ> group(const SmallJob* jobs, int n, float lr, float beta1, float beta2, float eps, float weight_decay, float beta_factor) {
+  SmallGroup<NJ> g;
+  g.lr = lr; g.beta1 = beta1; g.beta2 = beta2; g.eps = eps; g.decay = 1.0f - lr * weight_decay; g.beta_factor = beta_factor;
+  for (int i = 0; i < n; ++i) g.j[i] = jobs[i];
+  return g;
+}
+template <int NJ>
+cudaError_t launch_tiny(const SmallJob* jobs, int n, float lr, float beta1, float beta2, float eps, float weight_decay, float beta_factor,
+                        cudaStream_t s) {
+  static OncePerDevice once;
+  const cudaError_t e = once.run([] { return cudaFuncSetAttribute(k_tiny_step<NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTinySmem); });
+  if (e != cudaSuccess) return e;
+  size_t bytes = 0;
+  for (int i = 0; i < n; ++i) bytes = std::max(bytes, tiny_bytes(jobs[i].m, jobs[i].n, jobs[i].left != 0, jobs[i].right != 0));
+  k_tiny_step<NJ><<<n, kTinyThreads, bytes, s>>>(group<NJ>(jobs, n, lr, beta1, beta2, eps, weight_decay, beta_factor));
+  return cudaGetLastError();
+}
+template <int NJ>
 cudaError_t launch(const SmallJob* jobs, int n, float lr, float beta1, float beta2, float eps, float weight_decay, float beta_factor,
                    cudaStream_t s) {
   static OncePerDevice once;
   const cudaError_t e = once.run([] { return cudaFuncSetAttribute(k_small_step<NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem); });
   if (e != cudaSuccess) return e;
-  SmallGroup<NJ> g;
-  g.lr = lr; g.beta1 = beta1; g.beta2 = beta2; g.eps = eps; g.decay = 1.0f - lr * weight_decay; g.beta_factor = beta_factor;
   size_t bytes = 0;
   int rows = 0;
   for (int i = 0; i < n; ++i) {
-    g.j[i] = jobs[i];
     const size_t need = small_bytes(jobs[i].m, jobs[i].n, jobs[i].left != 0, jobs[i].right != 0);
     if (need > bytes) bytes = need;
     if (jobs[i].m > rows) rows = jobs[i].m;
@@ -277,17 +399,22 @@ cudaError_t launch(const SmallJob* jobs, int n, float lr, float beta1, float bet
   at[0].val.clusterDim.x = (unsigned)cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3((unsigned)(n * cs)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = bytes; cfg.stream = s;
   cfg.attrs = at; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_small_step<NJ>, g);
+  return cudaLaunchKernelEx(&cfg, k_small_step<NJ>, group<NJ>(jobs, n, lr, beta1, beta2, eps, weight_decay, beta_factor));
 }
 }  // namespace
 
 cudaError_t small_step(const SmallJob* jobs, int n, float lr, float beta1, float beta2, float eps, float weight_decay,
                        float beta_factor, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
+  const bool tiny = std::all_of(jobs, jobs + n, tiny_eligible);      // (among larger ones they go along in the launch of those)
   for (int at = 0; at < n && e == cudaSuccess; at += kMaxJobs) {
     const int cnt = n - at < kMaxJobs ? n - at : kMaxJobs;
-    e = cnt == 1 ? launch<1>(jobs + at, 1, lr, beta1, beta2, eps, weight_decay, beta_factor, s)
-                 : launch<kMaxJobs>(jobs + at, cnt, lr, beta1, beta2, eps, weight_decay, beta_factor, s);
+    if (tiny)
+      e = cnt == 1 ? launch_tiny<1>(jobs + at, 1, lr, beta1, beta2, eps, weight_decay, beta_factor, s)
+                   : launch_tiny<kMaxJobs>(jobs + at, cnt, lr, beta1, beta2, eps, weight_decay, beta_factor, s);
+    else
+      e = cnt == 1 ? launch<1>(jobs + at, 1, lr, beta1, beta2, eps, weight_decay, beta_factor, s)
+                   : launch<kMaxJobs>(jobs + at, cnt, lr, beta1, beta2, eps, weight_decay, beta_factor, s);
   }
   return e;
 }

@@ -182,8 +182,8 @@ BR_API br_status br_set_lr(br_handle* h, float lr);
  * Bases are refreshed several at a time on internal streams that fork from and join the
  * handle's stream inside the call (the same happens for the periodic refresh inside br_step, which
  * also stores the call's gradients through an internal stream that joins before it returns).  The
- * launch chain of a basis of order 2048 or more is captured into a CUDA graph the first time its (order, form) occurs and
- * replayed afterwards (plain launches if that capture fails).  Neither this call nor br_step may be
+ * launch chain of a basis of order 1600 or more is captured into a CUDA graph the first time its
+ * (order, form) occurs and replayed afterwards (plain launches if that capture fails).  Neither this call nor br_step may be
  * issued while the handle's stream is being captured by the caller: both read conditioning notes of
  * the previous refresh back from the device. */
 BR_API br_status br_refresh_basis(br_handle* h, int layer);

@@ -108,7 +108,7 @@ struct br_handle {
     char* tcq_scratch = nullptr;          // scratch of the tensor-core projections (largest eligible order)
     std::vector<QrTc*> tcq;               // their plans, one per distinct eligible order
     int64_t cap_k = 0;                    // largest order this lane's buffers hold
-    // The orthonormalisation of one basis of an order from 2048 on is a chain of launches whose arguments depend
+    // The orthonormalisation of one basis of an order from 1600 on is a chain of launches whose arguments depend
     // only on the lane (its buffers) and on the order: it is captured into a CUDA graph the first time and
     // replayed afterwards, one launch per basis.  Key: 2 * order + (tensor-core form).
     struct QrGraph { cudaGraphExec_t exec = nullptr; int64_t launches = 0; double flops = 0.0; };
@@ -118,10 +118,12 @@ struct br_handle {
   bool use_graphs = true;                 // cleared when a capture fails (BR_REFRESH_GRAPHS=0 switches it off)
   // Eight streams in all, the default number of hardware queues.  When the largest order is one that a single
   // cluster factorises, every lane holds it: a cluster leaves 132 SMs to the others (ten steps and the 32 bases of a d = 384 decoder:
-  // 27.2 -> 16.2 ms against three full-size lanes).  Otherwise three lanes do, whose products fill the GPU, and up to
-  // five more hold only the small orders (at most 1/sqrt(2) of the largest, S = 2nd).
-  static constexpr int kBigLanes = 3;       // default number of full-size lanes (BR_REFRESH_LANES: 1..6)
+  // 27.2 -> 16.2 ms against three full-size lanes).  From order 2048 on three lanes do, whose products fill the GPU, and
+  // between the two six (sixteen bases of order 1792: 24.0 ms on three lanes, 19.6 on four, 17.6 on six); the others hold
+  // only the small orders (at most 1/sqrt(2) of the largest, S = 2nd).
+  static constexpr int kBigLanes = 3;       // default number of full-size lanes from order 2048 on (BR_REFRESH_LANES: 1..6)
   static constexpr int kMaxBigLanes = 6;
+  static constexpr int64_t kBigOrder = 2048;
   static constexpr int kMaxLanes = 8;       // lanes of both kinds
   Lane lanes[kMaxLanes];
   int n_lanes = 1;
@@ -224,7 +226,8 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
   }
   if (max_k) {
     // an order that one cluster factorises leaves most of the GPU to others: every lane holds the largest
-    int want_big = qr_one_launch((int64_t)max_k) ? br_handle::kMaxLanes : br_handle::kBigLanes;
+    int want_big = qr_one_launch((int64_t)max_k) ? br_handle::kMaxLanes
+                   : (int64_t)max_k < br_handle::kBigOrder ? br_handle::kMaxBigLanes : br_handle::kBigLanes;
     // tuning aid: BR_REFRESH_LANES=1..6 sets the number of concurrent full-size refresh lanes
     if (const char* env = std::getenv("BR_REFRESH_LANES")) {
       const int v = std::atoi(env);
@@ -496,10 +499,11 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
 br_status refresh_layers(br_handle* h, const int* ids, int n_ids) {
   struct Job { int layer; bool left; double cost; int64_t k; bool needs_z; };
   std::vector<Job> jobs;
-  // time of one job when it runs alone (ms, measured: 11 at order 2560, 45 at order 6912; 0.3 at 384 and 4 at
-  // 1536 on one cluster): a cubic term for the products and a linear one for the chain of panel factorisations
+  // time of one job when it runs alone (ms, measured: on one cluster 0.29 at order 384, 1.4 at 1024, 4.2 at 1536; the
+  // chain 2.8 at 1792, 3.9 at 2048, 5.8 at 2560, 13 at 4096, 36 at 6912 with the products of a tracking basis on the tensor
+  // cores): a cubic term for the products and a linear one for the chain of panel factorisations
   auto cost = [](double k) {
-    return qr_one_launch((int64_t)k) ? 1.0e-9 * k * k * k + 5e-4 * k : 5.4e-11 * k * k * k + 3.9e-3 * k;
+    return qr_one_launch((int64_t)k) ? 1.0e-9 * k * k * k + 5e-4 * k : 9.0e-11 * k * k * k + 1.6e-3 * k;
   };
   for (int j = 0; j < n_ids; ++j) {
     const Layer& L = h->layers[ids[j]];

@@ -7,7 +7,7 @@
 //                   (orth.cu: the same recursion down to panels of 64 columns and Cholesky-QR of those);
 //                   otherwise orth(left half), project the left half out of the right half
 //                   (C = Q_l^T A_r, A_r -= Q_l C) with products over the whole GPU, orth(right half).
-// Orders below 2048 are one such block in all, second sweep and completion included.
+// Orders below 1600 are one such block in all, second sweep and completion included (see qr_one_launch).
 // Half of the floating-point work is in the two products of the top level and three quarters in
 // the top two, which is what lets the matrix unit run close to its peak.
 //
@@ -407,7 +407,14 @@ cudaError_t qr_complete_columns(double* A, const float* Q, int64_t k, double* wo
   return complete_columns<float>(A, Q, k, work, status, nullptr, s);
 }
 
-bool qr_one_launch(int64_t k) { return k < tc_min_order(); }
+// Up to here one cluster's launch is at least as fast as the launches of 128-column panels were that it replaced (one
+// basis of 1536 4.5 -> 4.2 ms, of 1664 5.1 -> 5.2, of 2040 6.8 -> 8.2), and from here on the chain of 256-column
+// launches is faster than the cluster for any number of bases, on the lanes that a handle has in either case (ms, cluster
+// and chain): 1600 alone 4.9 and 2.4, eight 9.8 and 7.7, sixteen 16.2 and 13.3; 2040 alone 8.2 and 3.5, eight 17.5 and
+// 13.3, sixteen 30.4 and 24.5.  (It is the faster one alone from 1024 on, and with eight from about 1152; the cluster
+// needs a third of its memory there.)
+constexpr int64_t kOneLaunchEnd = 1600;
+bool qr_one_launch(int64_t k) { return k < std::min(kOneLaunchEnd, tc_min_order()); }
 
 size_t qr_work_doubles(int64_t k) {
   const int64_t norms = (kNormChunks + 1) * k + 64;        // complete_columns

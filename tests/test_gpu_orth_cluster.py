@@ -1,7 +1,7 @@
-"""The one-launch factorisation Q <- qr(F Q).Q of orders below 2048, through the C-ABI (set_state, refresh_basis,
+"""The one-launch factorisation Q <- qr(F Q).Q of orders below 1600, through the C-ABI (set_state, refresh_basis,
 get_state), at the orders where its tiling can go wrong: less than one panel, whole and ragged panels, one CTA
-more or less in the cluster, odd orders (8-byte instead of 16-byte copies), the product formed inside or outside
-the launch, the largest order, and the first orders that go through the chain of launches.
+more or less in the cluster, odd orders (8-byte instead of 16-byte copies), the largest order, and orders that go
+through the chain of launches.
 
 Reference: LAPACK QR of the float64 product with a positive diagonal of R.  Both sides then round to (library) or
 start from (reference) the same fp32 inputs, so what remains is the rounding of Q to fp32 -- at most 2^-24 relative
@@ -33,8 +33,27 @@ def _refresh(k, F, Q0):
         opt.close()
 
 
+@pytest.mark.parametrize("k,one", [(1599, True), (1600, False), (2040, False)])
+def test_form_by_order(k, one):
+    """Which form a refresh takes, told by its launches: the product and the factorisation, or the chain."""
+    import torch
+    import paper_2602_03515_b200 as br
+    from workloads import LayerSpec
+    opt = br.BasisRotation([LayerSpec("W", k, k, br.BR_GEOM_UNILATERAL, br.BR_SRC_SECOND, 0)], [torch.zeros(k, k, device="cuda")],
+                           grad_dtype="f32", gemm_prec=br.BR_GEMM_FP32, freq=10 ** 6)
+    try:
+        opt.step([torch.randn(k, k, device="cuda") * 0.01], 0)
+        before, _ = opt.launch_stats()
+        opt.refresh_basis(0)
+        launches = opt.launch_stats()[0] - before
+        assert opt.sync_status() == br.BR_OK
+        assert launches <= 4 if one else launches > 20, launches
+    finally:
+        opt.close()
+
+
 @pytest.mark.parametrize("signal", [0.0, 300.0])      # well-conditioned: one sweep; a strong low-rank part: two
-@pytest.mark.parametrize("k", [1, 7, 8, 63, 64, 65, 127, 128, 129, 130, 255, 384, 511, 513, 1000, 1537, 2047, 2049])
+@pytest.mark.parametrize("k", [1, 7, 8, 63, 64, 65, 127, 128, 129, 130, 255, 384, 511, 513, 1000, 1537, 1599, 1600, 1601, 2047, 2049])
 def test_order(k, signal):
     rng = np.random.default_rng(k)
     N = rng.standard_normal((k, k)) / np.sqrt(k)

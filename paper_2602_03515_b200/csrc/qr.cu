@@ -146,7 +146,8 @@ inline int64_t env_or(const char* name, int64_t dflt, int64_t lo, int64_t hi) {
   }
   return dflt;
 }
-// tuning aids: BR_QR_TC_MIN_NODE (entries of the coefficient block), BR_QR_TC_MIN_ORDER
+// tuning aids: BR_QR_TC_MIN_NODE (entries of the coefficient block), BR_QR_TC_MIN_ORDER (smallest order with tensor-core
+// forms; those are part of the launch chain, so a lower value brings its orders there too)
 inline int64_t tc_min_node() { static const int64_t v = env_or("BR_QR_TC_MIN_NODE", (int64_t)1 << 18, 1 << 14, (int64_t)1 << 40); return v; }
 inline int64_t tc_min_order() { static const int64_t v = env_or("BR_QR_TC_MIN_ORDER", 2048, 1024, (int64_t)1 << 30); return v; }
 // widest range of columns one cluster orthonormalises by itself

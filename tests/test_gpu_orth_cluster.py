@@ -33,7 +33,7 @@ def _refresh(k, F, Q0):
         opt.close()
 
 
-@pytest.mark.parametrize("k,one", [(1599, True), (1600, False), (2040, False)])
+@pytest.mark.parametrize("k,one", [(1599, True), (1600, False), (2040, False), (2304, False)])
 def test_form_by_order(k, one):
     """Which form a refresh takes, told by its launches: the product and the factorisation, or the chain."""
     import torch

@@ -1,7 +1,8 @@
 """The library's alternative forms are selected by environment variables that are read once per
 process (tuning aids: the unpaired tensor-core kernel, stream launches instead of graph replay for the
-refresh, no small-order lanes).  Each is exercised here in a child process that runs a few of the
-ordinary parity tests under that setting, so that the forms a user can fall back to stay correct."""
+refresh, no small-order lanes, the smallest order whose refresh uses the tensor cores).  Each is
+exercised here in a child process that runs a few of the ordinary parity tests under that setting, so that
+the forms a user can fall back to stay correct."""
 import os
 import subprocess
 import sys
@@ -32,3 +33,12 @@ def test_refresh_without_graphs_and_small_lanes():
           "tests/test_gpu_full_size.py::test_refresh_tensor_core_projections",
           "tests/test_gpu_parity_fp32.py::test_numerically_rank_deficient_refresh_is_completed_in_the_same_call",
           "tests/test_gpu_parity_bf16.py", "-k", "not checkpoint"])
+
+
+def test_refresh_without_tensor_cores():
+    """A raised line keeps the tensor cores out of the refresh and leaves the form of the factorisation alone."""
+    _run({"BR_QR_TC_MIN_ORDER": str(1 << 30)}, ["tests/test_gpu_orth_cluster.py", "-k", "form_by_order or 1599 or 2049"])
+
+
+def test_refresh_with_tensor_cores_from_order_1024():
+    _run({"BR_QR_TC_MIN_ORDER": "1024"}, ["tests/test_gpu_full_size.py::test_refresh_order_1024_against_oracle_power"])

@@ -260,7 +260,7 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
       ln.cap_k = (int64_t)cap;
       ln.rA = b.take<double>(cap * cap);
       ln.rF = b.take<double>(cap * cap);
-      ln.rQ = b.take<double>(cap * cap);
+      if (!qr_one_launch((int64_t)cap)) ln.rQ = b.take<double>(cap * cap);      // (one launch reads the fp32 basis itself)
       size_t work = 1056;                                  // (also 1025 doubles of norm scratch)
       for (size_t k : orders) if (k <= cap) work = std::max(work, qr_work_doubles((int64_t)k));
       ln.rWork = b.take<double>(work);

@@ -181,6 +181,15 @@ struct Bump {
 inline size_t simt_need(const Layer& L) { return 4 * (((size_t)L.d.m * L.d.n + 63) / 64 * 64); }
 constexpr size_t kSimtScratch = 16u << 20;
 
+// S = 1st: the half product of a refresh (M^T U, or M V) is formed in equal slices of the unrotated dimension, each
+// at most 128 MiB of fp64 in every lane.  (Whole, it was 393 MB a lane for an embedding of 32000 x 1536.  Slices of half
+// the size cost 1 to 2 % of such a refresh.)
+constexpr int64_t kZSlice = 16 << 20;
+inline int64_t z_slice(int64_t k, int64_t other) {
+  const int64_t rows = std::max<int64_t>(1, kZSlice / k), slices = (other + rows - 1) / rows;
+  return std::min(std::min(rows, other), ((other + slices - 1) / slices + 63) / 64 * 64);      // (whole tiles)
+}
+
 // Lays out every buffer of the handle in one slab.  With base == nullptr only sizes are computed.
 void layout(br_handle* h, Bump& b, Sizes* sz) {
   const br_hparams& hp = h->hp;
@@ -211,7 +220,9 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
       if (!L.use_tc) { simt_max = std::max(simt_max, simt_need(L)); simt_total += simt_need(L); }
       if (L.left) { max_k = std::max(max_k, (size_t)L.d.m); ++n_sides; }
       if (L.right) { max_k = std::max(max_k, (size_t)L.d.n); ++n_sides; }
-      if (!second) max_z = std::max(max_z, mn);
+      if (!second)
+        for (int64_t k : {L.left ? L.d.m : (int64_t)0, L.right ? L.d.n : (int64_t)0})
+          if (k) max_z = std::max(max_z, (size_t)(k * z_slice(k, L.d.m * L.d.n / k)));
     }
   }
   if (simt_total) {
@@ -449,16 +460,17 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
         BR_CUDA(h, dgemm(0, 0, k, k, k, 1.0, ln.rF, k, ln.rQ, k, 0.0, ln.rA, k, s));
         count(h, 2); h->stats.gemm_flops += 2.0 * k * k * k;
       }
-    } else if (left_side) {
-      // (M M^T) U = M (M^T U)
-      BR_CUDA(h, sdgemm(1, n, m, m, 1.0, Mo, n, Q, m, 0.0, ln.rZ, m, s));
-      BR_CUDA(h, fdgemm(0, m, m, n, 1.0, Mo, n, ln.rZ, m, 0.0, ln.rA, m, s));
-      count(h, 2); h->stats.gemm_flops += 4.0 * m * m * n;
     } else {
-      // (M^T M) V = M^T (M V)
-      BR_CUDA(h, sdgemm(0, m, n, n, 1.0, Mo, n, Q, n, 0.0, ln.rZ, n, s));
-      BR_CUDA(h, fdgemm(1, n, n, m, 1.0, Mo, n, ln.rZ, n, 0.0, ln.rA, n, s));
-      count(h, 2); h->stats.gemm_flops += 4.0 * n * n * m;
+      // (M M^T) U = M (M^T U), or (M^T M) V = M^T (M V), a slice of M's columns (rows) after the other
+      const int64_t slice = z_slice(k, other);
+      for (int64_t o = 0; o < other; o += slice) {
+        const int64_t w = std::min(slice, other - o);
+        const float* Ms = left_side ? Mo + o : Mo + o * n;
+        BR_CUDA(h, sdgemm(left_side ? 1 : 0, w, k, k, 1.0, Ms, n, Q, k, 0.0, ln.rZ, k, s));
+        BR_CUDA(h, fdgemm(left_side ? 0 : 1, k, k, w, 1.0, Ms, n, ln.rZ, k, o ? 1.0 : 0.0, ln.rA, k, s));
+        count(h, 2);
+      }
+      h->stats.gemm_flops += 4.0 * k * k * other;
     }
     // A rank-deficient product has no unique Q factor.  Which products are is known on the host: with
     // S = 1st, M M^T (M^T M) has rank <= min(m, n), short of the larger side; with S = 2nd, a factor that

@@ -52,6 +52,38 @@ def test_form_by_order(k, one):
         opt.close()
 
 
+@pytest.mark.parametrize("m,n", [(66000, 260), (260, 66000), (66001, 257), (4200, 4100)])
+def test_first_source_product_in_slices(m, n):
+    """S = 1st with a momentum of more than 2^24 entries: M^T (M V), or M (M^T U), in slices of the unrotated dimension.
+    The error is that of the orders above: the products are exact up to fp64 rounding whatever the slices."""
+    import torch
+    import paper_2602_03515_b200 as br
+    from workloads import LayerSpec
+    rng = np.random.default_rng(m)
+    k = min(m, n)
+    M = rng.standard_normal((m, n)).astype(np.float32)
+    if (m, n) == (4200, 4100):
+        M += 60 * np.eye(m, n, dtype=np.float32)           # (a square random matrix alone is nearly singular)
+    Q0 = np.linalg.qr(rng.standard_normal((k, k)))[0].astype(np.float32)
+    M64, Q64 = M.astype(np.float64), Q0.astype(np.float64)
+    want, R = np.linalg.qr(M64 @ (M64.T @ Q64) if m <= n else M64.T @ (M64 @ Q64))
+    want *= np.sign(np.diag(R))
+    which = br.BR_BUF_U if m <= n else br.BR_BUF_V
+    opt = br.BasisRotation([LayerSpec("W", m, n, br.BR_GEOM_UNILATERAL, br.BR_SRC_FIRST, 0)], [torch.zeros(m, n, device="cuda")],
+                           grad_dtype="f32", gemm_prec=br.BR_GEMM_FP32, freq=10 ** 6)
+    try:
+        opt.step([torch.randn(m, n, device="cuda") * 0.01], 0)
+        opt.set_state(0, br.BR_BUF_M, torch.from_numpy(M))
+        opt.set_state(0, which, torch.from_numpy(Q0))
+        opt.refresh_basis(0)
+        assert opt.sync_status() == br.BR_OK
+        got = opt.get_state(0, which).numpy().astype(np.float64)
+    finally:
+        opt.close()
+    err = np.linalg.norm(got - want) / np.linalg.norm(want)
+    assert err <= TOL, (m, n, err)
+
+
 @pytest.mark.parametrize("signal", [0.0, 300.0])      # well-conditioned: one sweep; a strong low-rank part: two
 @pytest.mark.parametrize("k", [1, 7, 8, 63, 64, 65, 127, 128, 129, 130, 255, 384, 511, 513, 1000, 1537, 1599, 1600, 1601, 2047, 2049])
 def test_order(k, signal):

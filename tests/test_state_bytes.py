@@ -29,3 +29,16 @@ def test_a_lane_of_one_launch_orders(k):
     copy (k^2 doubles each) and the factorisation's work (coefficients k^2 / 4, column norms 2 x 16 k, diagonal k)."""
     want = 4 * 4 * k * k + 4 * 4 * k * k + 8 * (2 * k * k + k * k / 4 + 33 * k)
     assert total_bytes([(k, k)], GEOM_UNI, SRC_SECOND, br.BR_GEMM_FP32, tau=0) <= want + 16 * 1024 + 8 * k
+
+
+@pytest.mark.parametrize("emb,d,ffn", [(32000, 1536, 6144), (50257, 768, 3072)])
+def test_first_source_buffers_do_not_grow_with_the_largest_matrix(emb, d, ffn):
+    """The half product of an S = 1st refresh has at most 128 MiB in each of at most eight lanes."""
+    blk = total_bytes(block(d, ffn), GEOM_UNI, SRC_FIRST, br.BR_GEMM_BF16)
+    both = total_bytes([(emb, d)] + block(d, ffn), GEOM_UNI, SRC_FIRST, br.BR_GEMM_BF16)
+    tc = emb % 8 == 0
+    # the layer itself: M, V~ (and the momentum of the original space), ring of four bf16 slots, basis and its bf16 pair; on
+    # the fp32 path its step's scratch of 4 m n floats, on the tensor-core path the operands of its chunk, 11 bytes an entry
+    layer = emb * d * (8 + (4 + 11 if tc else 16) + 4 * 2) + d * d * 8
+    lane = 8 * (2 * d * d + d * d / 4 + 33 * d)
+    assert both - blk <= layer + 8 * (128 << 20) + 2 * lane

@@ -153,9 +153,12 @@ typedef enum {
   BR_BUF_CLIP = 9
 } br_buf;
 
-/* Bytes of device memory br_create would request for these layers (state, ring, operand
- * shadows and scratch).  Host only.  App. H's table is overhead_bytes: rotation matrices
- * plus factor buffers in fp32, summed over layers (either out pointer may be NULL). */
+/* Bytes of device memory br_create requests for these layers (state, ring, operand shadows and
+ * scratch).  If that request is refused and a layout with fewer concurrent refresh lanes is smaller,
+ * br_create asks once more, for that one (a refresh takes longer; fp32 layers are grouped into other
+ * launches, which may round differently).  Host only.  App. H's
+ * table is overhead_bytes: rotation matrices plus factor buffers in fp32, summed over layers (either
+ * out pointer may be NULL). */
 BR_API br_status br_state_bytes(const br_layer_desc* layers, int n_layers, const br_hparams* hp,
                          size_t* total_bytes, size_t* overhead_bytes);
 

@@ -124,6 +124,8 @@ struct br_handle {
   static constexpr int kBigLanes = 3;       // default number of full-size lanes from order 2048 on (BR_REFRESH_LANES: 1..6)
   static constexpr int kMaxBigLanes = 6;
   static constexpr int64_t kBigOrder = 2048;
+  // The layout of a handle whose allocator refused the usual one: three full-size lanes, fp32 scratch for one layer.
+  bool compact = false;
   static constexpr int kMaxLanes = 8;       // lanes of both kinds
   Lane lanes[kMaxLanes];
   int n_lanes = 1;
@@ -226,7 +228,7 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
     }
   }
   if (simt_total) {
-    h->simt_floats = std::max(simt_max, std::min(simt_total, kSimtScratch));
+    h->simt_floats = h->compact ? simt_max : std::max(simt_max, std::min(simt_total, kSimtScratch));
     h->simt_scratch = b.take<float>(h->simt_floats);
   }
   h->tcq_bytes = 0;
@@ -237,7 +239,8 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
   }
   if (max_k) {
     // an order that one cluster factorises leaves most of the GPU to others: every lane holds the largest
-    int want_big = qr_one_launch((int64_t)max_k) ? br_handle::kMaxLanes
+    int want_big = h->compact ? br_handle::kBigLanes
+                   : qr_one_launch((int64_t)max_k) ? br_handle::kMaxLanes
                    : (int64_t)max_k < br_handle::kBigOrder ? br_handle::kMaxBigLanes : br_handle::kBigLanes;
     // tuning aid: BR_REFRESH_LANES=1..6 sets the number of concurrent full-size refresh lanes
     if (const char* env = std::getenv("BR_REFRESH_LANES")) {
@@ -842,17 +845,23 @@ br_status br_create(br_handle** out, const br_layer_desc* layers, int n_layers, 
   if (a && a->alloc && a->free) h->alloc = *a;
   init_layers(h, layers, n_layers);
 
-  Bump sizing;
   Sizes sz;
-  layout(h, sizing, &sz);
   const size_t tc_bytes = align_up(tc_step_scratch_bytes(h->layers, h->hp));
-  h->slab_bytes = sz.total + tc_bytes;
   void* p = nullptr;
-  if (h->alloc.alloc) {
-    p = h->alloc.alloc(h->slab_bytes, h->alloc.ctx);
-  } else if (cudaMalloc(&p, h->slab_bytes) != cudaSuccess) {
-    (void)cudaGetLastError();
-    p = nullptr;
+  for (int attempt = 0; attempt < 2 && !p; ++attempt) {      // the usual layout, then the compact one if that is smaller
+    h->compact = attempt == 1;
+    Bump sizing;
+    Sizes s;
+    layout(h, sizing, &s);
+    if (attempt == 1 && s.total >= sz.total) break;
+    sz = s;
+    h->slab_bytes = sz.total + tc_bytes;
+    if (h->alloc.alloc) {
+      p = h->alloc.alloc(h->slab_bytes, h->alloc.ctx);
+    } else if (cudaMalloc(&p, h->slab_bytes) != cudaSuccess) {
+      (void)cudaGetLastError();
+      p = nullptr;
+    }
   }
   if (!p) {
     g_create_error = format("allocation of %zu bytes failed", h->slab_bytes);

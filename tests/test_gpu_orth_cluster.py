@@ -52,6 +52,54 @@ def test_form_by_order(k, one):
         opt.close()
 
 
+@pytest.mark.parametrize("k", [130, 1599, 1601, 2304])
+def test_rank_deficient_product(k):
+    """A factor with an exactly empty block, whose rank the host does not know: the factorisation finds the product
+    F Q short of rank (some |R_jj| <= 1e-12 of the largest) and, in the same refresh, factorises it with
+    1e-6 ||(F Q)_j|| Q_j added to every column -- as branches of the one launch, and from order 1600 on as launches of the
+    chain that a device flag turns on.  The completed product has full rank and the completed directions come out of
+    it at 1e-6 of its columns: fp64 rounding is 1e-10 of them, far below the fp32 result."""
+    import torch
+    import paper_2602_03515_b200 as br
+    from workloads import LayerSpec
+    rng = np.random.default_rng(k)
+    r = k - k // 5
+    N = rng.standard_normal((r, r)) / np.sqrt(r)
+    F = np.zeros((k, k), dtype=np.float32)
+    F[:r, :r] = np.eye(r) + 0.1 * (N + N.T)
+    Q0 = np.linalg.qr(rng.standard_normal((k, k)))[0].astype(np.float32)
+    A = F.astype(np.float64) @ Q0.astype(np.float64)
+    A += 1e-6 * np.linalg.norm(A, axis=0) * Q0.astype(np.float64)
+    want, R = np.linalg.qr(A)
+    want *= np.sign(np.diag(R))
+    opt = br.BasisRotation([LayerSpec("W", k, k, br.BR_GEOM_UNILATERAL, br.BR_SRC_SECOND, 0)], [torch.zeros(k, k, device="cuda")],
+                           grad_dtype="f32", gemm_prec=br.BR_GEMM_FP32, freq=10 ** 6)
+    try:
+        opt.step([torch.randn(k, k, device="cuda") * 0.01], 0)
+        opt.set_state(0, br.BR_BUF_L, torch.from_numpy(F))
+        opt.set_state(0, br.BR_BUF_U, torch.from_numpy(Q0))
+        for again in range(2):                 # (the second time the chain comes out of its graph)
+            opt.refresh_basis(0)
+            assert opt.sync_status() == br.BR_WARN_RANK_DEFICIENT
+            got = opt.get_state(0, br.BR_BUF_U).numpy().astype(np.float64)
+            assert br.br_get_basis_flags(opt.handle, 0) & 4
+            err = np.linalg.norm(got - want) / np.linalg.norm(want)
+            assert err <= TOL, (k, again, err)
+            opt.set_state(0, br.BR_BUF_U, torch.from_numpy(Q0))
+        # a full-rank factor on the same handle: nothing of the completion runs
+        F[r:, r:] = np.eye(k - r)
+        want, R = np.linalg.qr(F.astype(np.float64) @ Q0.astype(np.float64))
+        want *= np.sign(np.diag(R))
+        opt.set_state(0, br.BR_BUF_L, torch.from_numpy(F))
+        opt.refresh_basis(0)
+        assert opt.sync_status() == br.BR_OK
+        got = opt.get_state(0, br.BR_BUF_U).numpy().astype(np.float64)
+        err = np.linalg.norm(got - want) / np.linalg.norm(want)
+        assert err <= TOL, (k, err)
+    finally:
+        opt.close()
+
+
 @pytest.mark.parametrize("m,n", [(66000, 260), (260, 66000), (66001, 257), (4200, 4100)])
 def test_first_source_product_in_slices(m, n):
     """S = 1st with a momentum of more than 2^24 entries: M^T (M V), or M (M^T U), in slices of the unrotated dimension.

@@ -15,7 +15,6 @@
 #include <algorithm>
 
 #include "br_internal.h"
-#include "step_tc.h"
 
 namespace br {
 namespace {

@@ -11,14 +11,13 @@
 // launches, of which 1.0 ms in the products).
 //
 // A CTA computes one tile; the next 16 steps of the contraction are fetched into registers while the
-// current ones are multiplied out of shared memory.  The tile follows from the work of the launch: 32 x 32 on
-// 64 threads while those tiles fit on the GPU at once (the time is then that of one tile's chain, and a small
+// current ones are multiplied out of shared memory.  The tile follows from the size of the launch's results (launch_sized):
+// 32 x 32 on 64 threads while those tiles fit on the GPU at once (the time is then that of one tile's chain, and a small
 // tile's step is the shortest), 64 x 64 up to a few waves, 128 x 128 (8 x 8 per thread, half the shared-memory
 // reads per multiply-add) above.  With at most four tiles of 32 x 32 per SM a step is bound by the latency of
 // its loads, and four groups of 64 threads take a quarter of the contraction each: the dual launch of the four
 // ragged layers 54 -> 30 us, the others 30 -> 16 us.
 #include "br_internal.h"
-#include "step_tc.h"
 
 namespace br {
 namespace {
@@ -174,6 +173,11 @@ cudaError_t launch(GroupArgs& ga, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// The lines, in result tiles of 32 x 32, measured on updates of one k x k matrix rotated on one side (us, the form below
+// the line and the one above): 592: k = 640 (400 tiles) 110 and 134, 900 (841) 281 and 249.  1776: 1400 (1936) 789 and
+// 711; 64 x 64 is the faster one already at 1000 (1024) with 343 and 282 and at 1300 (1681) with 639 and 524.  9472: level
+// within 2 % from 2800 to 4200.  How long the contraction is does not enter: a result of few tiles with a contraction of
+// tens of thousands is one chain per tile.
 template <bool DUAL>
 cudaError_t launch_sized(GroupArgs& ga, cudaStream_t s) {
   double area = 0.0;                                       // in tiles of 32 x 32

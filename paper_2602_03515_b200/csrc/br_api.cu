@@ -1035,8 +1035,10 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
       if (small_on && L.t % L.freq != 0 && small_step_eligible(L.d.m, L.d.n, L.left, L.right)) {
         const bool acc = L.d.src == BR_SRC_SECOND && hp.accum == BR_ACCUM_EVERY_STEP;
         const int64_t m = L.d.m, n = L.d.n;
+        void* ring = L.ring_slots > 0 ? const_cast<void*>(ring_slot_ptr(L, (h->calls - 1) % L.ring_slots)) : nullptr;
         small.push_back({(int)m, (int)n, L.left, L.right, L.d.grad_dtype == BR_BF16, acc ? 1 : 0, G[i], GS[i], L.M, L.V2, L.U, L.V,
-                         L.L, L.R, L.d.weight});
+                         L.L, L.R, L.d.weight, grads[i], ring});
+        if (ring) stored[i] = 1;
         h->stats.gemm_flops += (acc ? 2.0 : 0.0) * ((L.L ? m * m * n : 0) + (L.R ? n * n * m : 0)) +
                                6.0 * m * n * ((L.left ? m : 0) + (L.right ? n : 0));
         if (acc) L.n_accum += 1;

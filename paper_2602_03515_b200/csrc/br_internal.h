@@ -127,6 +127,7 @@ struct SmallJob {
   int g_is_bf16, accumulate;
   const void* G; const float* gscale;      // gradient, and its call's clipping factor or null
   float *M, *V2, *U, *V, *L, *R, *W;
+  const void* grad; void* ring;            // this call's gradient, and the slot it is stored in (or null), which may be G
 };
 cudaError_t small_step(const SmallJob* jobs, int n, float lr, float beta1, float beta2, float eps, float weight_decay,
                        float beta_factor, cudaStream_t s);

@@ -1047,12 +1047,26 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
       }
     }
   }
+  // the small matrices beside the grouped launches of the others, where there are any (the update of four ragged layers,
+  // one of them small: 146 -> 133 us)
+  const bool beside = !small.empty() && !simt_ids.empty();
   if (!small.empty()) {
+    cudaStream_t ss = beside ? h->copy_stream : h->stream;
+    if (beside) {
+      BR_CUDA(h, cudaEventRecord(h->ev_consumed, h->stream));
+      BR_CUDA(h, cudaStreamWaitEvent(ss, h->ev_consumed, 0));
+    }
     BR_CUDA(h, small_step(small.data(), (int)small.size(), hp.lr, hp.beta1, hp.beta2, hp.eps, hp.weight_decay,
-                          hp.beta_factor < 0.f ? hp.beta2 : hp.beta_factor, h->stream));
+                          hp.beta_factor < 0.f ? hp.beta2 : hp.beta_factor, ss));
     count(h, ((int)small.size() + 23) / 24);
   }
-  if (!simt_ids.empty() && (st = update_layers_simt(h, simt_ids, G, GS)) != BR_OK) return st;
+  if (!simt_ids.empty()) st = update_layers_simt(h, simt_ids, G, GS);
+  if (beside) {
+    // (also on a failed step: the side stream must not outlive the caller's view of this call)
+    cudaEventRecord(h->ev_copied, h->copy_stream);
+    cudaStreamWaitEvent(h->stream, h->ev_copied, 0);
+  }
+  if (st != BR_OK) return st;
   if (h->tc) {
     struct StepCtx { br_handle* h; const void* const* grads; std::vector<char>* stored; bool copied; };
     StepCtx sc{h, grads, &stored, false};

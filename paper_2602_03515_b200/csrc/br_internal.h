@@ -250,11 +250,9 @@ cudaError_t qr_pos_inplace(double* A, int64_t k, double* work, int* status, cuda
 enum Epilogue : int32_t {
   EPI_AXPBY_F32 = 0,    // D <- alpha*acc + beta*D                 (factor EMA, weight write, plain)
   EPI_SPLIT_BF16 = 1,   // Dh <- bf16(acc), Dl <- bf16(acc - Dh)   (Dl optional)
-  EPI_SECOND_MOMENT = 2,// D(V~) <- beta*D + alpha*acc^2
-  EPI_SCALE_BF16 = 3,   // Dh(X) <- bf16(acc / sqrt(D(V~) + eps))
   // Alg. 1 (momentum and second-moment updates, scaling) in rotated coordinates, acc = G~:
   //   D2(M~) <- beta1 D2 + (1-beta1) acc ; D(V~) <- beta D + alpha acc^2 ; Dh(X) <- bf16(D2 / sqrt(D + eps))
-  EPI_ROTATED_ADAM = 4
+  EPI_ROTATED_ADAM = 2
 };
 
 struct TcOperand {

@@ -2,7 +2,7 @@
 //   D_tile = sum over operand pairs p and k-blocks of A_p[128 x 64] * B_p[256 x 64]^T
 // TMA (cp.async.bulk.tensor, 128-byte swizzle) stages operand tiles in shared memory, one elected
 // thread issues tcgen05.mma (kind::f16, bf16 operands, fp32 accumulation) into tensor memory,
-// four epilogue warps read the accumulator back with tcgen05.ld, turn it through shared memory so
+// eight epilogue warps read the accumulator back with tcgen05.ld, turn it through shared memory so
 // that global memory is accessed along rows, and apply a fused epilogue
 // (factor EMA, bf16 hi/lo split, second-moment update, Adam scaling, weight write).
 //
@@ -79,8 +79,8 @@ constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int SH_STAGES = 2;                     // shared-operand form: two stages of 2 A tiles + 2 B tiles
 constexpr int SH_STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
 static_assert(SH_STAGES * SH_STAGE_BYTES == STAGES * STAGE_BYTES, "both forms use the same operand area");
-constexpr int EPI_LD = 33;                       // padded row of an epilogue tile (floats): rows and columns both conflict-free
-constexpr int EPI_BYTES = 4 * 32 * EPI_LD * 4;   // one 32 x 32 fp32 tile per epilogue warp
+constexpr int EPI_WARPS = 8;
+constexpr int EPI_BYTES = EPI_WARPS * 32 * 32 * 4;   // one 32 x 32 fp32 block per epilogue warp
 constexpr int OPERAND_BYTES = STAGES * STAGE_BYTES;                   // 192 KiB of operand stages in every form
 constexpr int SMEM_BYTES = OPERAND_BYTES + EPI_BYTES + 1024;          // + slack to align the tiles to 1 KiB
 constexpr int MAX_STAGES = 6;
@@ -95,8 +95,7 @@ struct Form {
   static_assert(NST <= MAX_STAGES && NST * STAGE == OPERAND_BYTES, "stages fill the operand area");
 };
 constexpr int TMEM_COLS = 512;
-constexpr int NUM_THREADS = 192;                 // warp 0: TMA, warp 1: MMA, warps 2..5: epilogue
-constexpr int FOLD_THREADS = 320;                // folded form: warps 2..9 fold and write (two per lane quadrant)
+constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS; // warp 0: TMA, warp 1: MMA, warps 2..9: epilogue (two per lane quadrant)
 // folded form: 160 KiB of operand stages, and two blocks of 32 x 32 floats for each of its eight epilogue warps
 constexpr int FOLD_OPERAND_BYTES = 160 * 1024, FOLD_BLOCK = 32 * 32;
 constexpr int SMEM_BYTES_FOLD = FOLD_OPERAND_BYTES + 8 * 2 * FOLD_BLOCK * 4 + 1024;
@@ -207,20 +206,21 @@ template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                           int* status, uint64_t limit_ns = kWaitLimitNs) {
   auto try_wait = [&] { return CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
-  if (try_wait()) return true;
-  const uint64_t t0 = global_timer_ns();
+  // (the timer is read only when a wait has become a long one)
+  uint64_t t0 = 0;
   uint32_t spins = 0;
-  while (true) {
-    if (try_wait()) return true;
-    if ((++spins & 0xFF) == 0) {
-      if (*abort_flag) return false;
-      if (global_timer_ns() - t0 > limit_ns) {
-        *abort_flag = 1;
-        atomicMin(status, (int)BR_ERR_TIMEOUT);
-        return false;
-      }
+  while (!try_wait()) {
+    if ((++spins & 0xFF) != 0) continue;
+    if (*abort_flag) return false;
+    const uint64_t now = global_timer_ns();
+    if (t0 == 0) t0 = now;
+    if (now - t0 > limit_ns) {
+      *abort_flag = 1;
+      atomicMin(status, (int)BR_ERR_TIMEOUT);
+      return false;
     }
   }
+  return true;
 }
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
@@ -346,6 +346,13 @@ __device__ __forceinline__ uint32_t make_idesc(int a_mn, int b_mn, int rows = BM
   return d;
 }
 
+// 1 / sqrt(x): the hardware's approximation and one Newton step, without the branches that sqrtf and a division take
+// for their special cases (an approximation of 0 or infinity stands as it is).
+__device__ __forceinline__ float inv_sqrt(float x) {
+  const float r = rsqrtf(x), n = fmaf(0.5f * r, fmaf(-(x * r), r, 1.0f), r);
+  return x > 0.0f && x < __int_as_float(0x7f800000) ? n : r;
+}
+
 __device__ __forceinline__ uint32_t pack2_bf16(float a, float b) {
   __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t*>(&v);
@@ -409,7 +416,7 @@ __device__ __forceinline__ TileInfo locate_tile(const DevProblem* probs, int n_p
 // The kernel
 // ---------------------------------------------------------------------------------------------
 template <bool SHARED, bool PAIR, bool FOLD = false>
-__global__ void __launch_bounds__(FOLD ? FOLD_THREADS : NUM_THREADS, 1)
+__global__ void __launch_bounds__(NUM_THREADS, 1)
 k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int total_tiles, const int* __restrict__ schedule,
           long long calls, int tau, float dyn_alpha, float dyn_beta, int* status) {
   using F = Form<SHARED, PAIR>;
@@ -448,8 +455,8 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    // accumulator hand-back: four epilogue warps, of both CTAs in the paired form
-    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), (FOLD ? 2 : 1) * (PAIR ? 8 : 4)); }
+    // accumulator hand-back: every epilogue warp, of both CTAs in the paired form
+    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), (PAIR ? 2 : 1) * EPI_WARPS); }
     abort_word = 0;
     dead_word = (*reinterpret_cast<volatile int*>(status) < 0) ? 1u : 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -636,14 +643,19 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
   } else {
     // ======================= epilogue warps =======================
     // A warp may read only its own quadrant of tensor memory, where lane = accumulator row: a
-    // 32 x 32 block arrives with one row per lane.  It is turned through a padded shared-memory
-    // tile so that global memory is accessed along rows: 8 lanes cover 128 contiguous bytes of one
+    // 32 x 32 block arrives with one row per lane.  It is turned through a swizzled shared-memory
+    // block so that global memory is accessed along rows: 8 lanes cover 128 contiguous bytes of one
     // row, a warp instruction four whole rows.  The values a read-modify-write epilogue needs are
-    // prefetched into L2 while the main loop of the tile is still running and then loaded eight
-    // rows deep before the first one is used.  A symmetric product (the factor EMAs) computes and writes only
+    // prefetched into L2 while the main loop of the tile is still running; those of a warp's first block are loaded
+    // before it waits for the accumulator, those of the next one in place of the ones just used.  (Four warps, one
+    // block's loads behind the other's stores and IEEE division and square root: 34 us for a tile of the rotated Adam
+    // at d = 1024, three times its main loop.)  A symmetric product (the factor EMAs) computes and writes only
     // the 32 x 32 blocks on and above the diagonal (see TcProblem::symmetric).
     const int quad = warp & 3;                    // tensor-memory lane quadrant this warp may read
-    float* tile = epi_tiles + quad * (32 * EPI_LD);
+    const int half = (warp - 2) >> 2;             // and its half of the result columns
+    float* const block = epi_tiles + (warp - 2) * (32 * 32);
+    // 16-byte piece c of row r of the warp's block: a thread's own row and a row by eight lanes are both conflict-free
+    auto piece = [&](int r, int c) { return block + r * 32 + ((c ^ (r & 7)) * 4); };
     const int sub_r = lane >> 3, sub_c = (lane & 7) * 4;
     int acc = 0; uint32_t acc_phase = 0;
     uint32_t fold_seq = 0;
@@ -663,22 +675,20 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
         if (p->clip_mode == 2) alpha *= gclip * gclip;
       }
       const int row_base = ti.m0 + (int)rank * BM + quad * 32;
+      const int col_base = ti.n0 + half * (BN / 2);
       const bool quad_ok = row_base < p->Md;      // uniform across the warp
-      const bool reads_d = (epi == EPI_AXPBY_F32 && beta != 0.0f) || epi == EPI_ROTATED_ADAM ||
-                           epi == EPI_SECOND_MOMENT || epi == EPI_SCALE_BF16;
+      const bool reads_d = (epi == EPI_AXPBY_F32 && beta != 0.0f) || epi == EPI_ROTATED_ADAM;
       if (!FOLD && reads_d && row_base + lane < p->Md) {
-        const float* d = p->D + (long long)(row_base + lane) * p->ldd + ti.n0;
+        const long long at = (long long)(row_base + lane) * p->ldd + col_base;
 #pragma unroll
-        for (int q = 0; q < BN / 32; ++q)
-          if (ti.n0 + 32 * q < p->Nd) {
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(d + 32 * q));
-            if (epi == EPI_ROTATED_ADAM)
-              asm volatile("prefetch.global.L2 [%0];" ::"l"(p->D2 + (long long)(row_base + lane) * p->ldd + ti.n0 + 32 * q));
+        for (int q = 0; q < BN / 64; ++q)
+          if (col_base + 32 * q < p->Nd) {
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p->D + at + 32 * q));
+            if (epi == EPI_ROTATED_ADAM) asm volatile("prefetch.global.L2 [%0];" ::"l"(p->D2 + at + 32 * q));
           }
       }
-      if (FOLD) {
+      if constexpr (FOLD) {
         // ---- folded form: this warp owns 32 rows (its lane quadrant) x 128 columns (its half) ----
-        const int half = (warp - 2) >> 2;
         float* const fbuf = epi_tiles + (warp - 2) * (2 * FOLD_BLOCK);
         const int nkb = (p->K + BK - 1) / BK;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * 128);
@@ -686,7 +696,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
         uint32_t need = 0;
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-          const int col0 = ti.n0 + half * 128 + 32 * b;
+          const int col0 = col_base + 32 * b;
           if (col0 < p->Nd && quad_ok && !(p->symmetric && row_base >= col0 + 32)) need |= 1u << b;
         }
         // The old values of D are copied to shared memory asynchronously, two of the four blocks while the chunks
@@ -694,12 +704,12 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
         // c ^ (r % 8), so that both the copies (a row's 128 bytes by eight lanes) and a thread's walk along its own
         // row are free of bank conflicts.  (Loaded into registers beside the 128 running sums they were spilled, or
         // exposed the latency of memory once per half block.)
-        auto piece = [&](int buf, int r, int c) { return fbuf + buf * FOLD_BLOCK + r * 32 + ((c ^ (r & 7)) * 4); };
-        const int cp_r = lane >> 3, cp_c = lane & 7;
-        float* const d0 = p->D + (long long)(row_base + cp_r) * p->ldd + ti.n0 + half * 128 + cp_c * 4;
+        auto piece2 = [&](int buf, int r, int c) { return fbuf + buf * FOLD_BLOCK + r * 32 + ((c ^ (r & 7)) * 4); };
+        const int cp_r = sub_r, cp_c = lane & 7;
+        float* const d0 = p->D + (long long)(row_base + cp_r) * p->ldd + col_base + cp_c * 4;
         const long long step = 4 * p->ldd;
         auto rows_of = [&](int b) {                // groups of four rows of block b that exist in this lane's columns
-          if (!((need >> b) & 1u) || ti.n0 + half * 128 + 32 * b + cp_c * 4 >= p->Nd) return 0;
+          if (!((need >> b) & 1u) || col_base + 32 * b + cp_c * 4 >= p->Nd) return 0;
           const int n_it = (p->Md - row_base - cp_r + 3) >> 2;
           return n_it > 8 ? 8 : n_it;
         };
@@ -708,7 +718,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             if (i < n_it)
-              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(piece(b & 1, 4 * i + cp_r, cp_c))),
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(piece2(b & 1, 4 * i + cp_r, cp_c))),
                            "l"(d0 + 32 * b + i * step) : "memory");
           asm volatile("cp.async.commit_group;" ::: "memory");
         };
@@ -763,7 +773,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
           if ((need >> b) & 1u) {
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-              float4* q = reinterpret_cast<float4*>(piece(b & 1, lane, c));
+              float4* q = reinterpret_cast<float4*>(piece2(b & 1, lane, c));
               float4 r = make_float4(alpha * __uint_as_float(sum[b][4 * c]), alpha * __uint_as_float(sum[b][4 * c + 1]),
                                      alpha * __uint_as_float(sum[b][4 * c + 2]), alpha * __uint_as_float(sum[b][4 * c + 3]));
               if (beta != 0.0f) {
@@ -777,138 +787,138 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
           const int n_it = rows_of(b);
 #pragma unroll
           for (int i = 0; i < 8; ++i)
-            if (i < n_it) *reinterpret_cast<float4*>(d0 + 32 * b + i * step) = *reinterpret_cast<const float4*>(piece(b & 1, 4 * i + cp_r, cp_c));
+            if (i < n_it) *reinterpret_cast<float4*>(d0 + 32 * b + i * step) = *reinterpret_cast<const float4*>(piece2(b & 1, 4 * i + cp_r, cp_c));
           __syncwarp();
           if (b < 2) fetch_old(b + 2); else asm volatile("cp.async.commit_group;" ::: "memory");
         }
         continue;
       }
-      if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag, status)) break;
-      tc_fence_after();
-#pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
-        const int col0 = ti.n0 + c0;
-        if (col0 >= p->Nd) break;                 // uniform across the warp
+      // The blocks of 32 columns that this warp writes (uniform across it), and the groups of four rows of block b that
+      // exist in this lane's columns (columns come in multiples of 8: a group of four is all in or all out).
+      auto writes = [&](int b) {
+        const int col0 = col_base + 32 * b;
+        return quad_ok && b < BN / 64 && col0 < p->Nd && !(p->symmetric && row_base >= col0 + 32);
+      };
+      auto rows_of = [&](int b) {
+        if (!writes(b) || col_base + 32 * b + sub_c >= p->Nd) return 0;
+        const int n_it = (p->Md - row_base - sub_r + 3) >> 2;
+        return n_it > 8 ? 8 : n_it;
+      };
+      const long long at_d = (long long)(row_base + sub_r) * p->ldd + col_base + sub_c, step_d = 4 * p->ldd;
+      const long long at_h = (long long)(row_base + sub_r) * p->ldh + col_base + sub_c, step_h = 4 * p->ldh;
+      // block b of the accumulator, turned: entry `it` of this lane is row 4 it + sub_r, columns sub_c .. sub_c + 3
+      auto turn = [&](int b) {
         float v[32];
-        tmem_ld32(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + c0), v);
-        // nothing to write: rows beyond the matrix, or a block strictly below the diagonal of a
-        // symmetric product
-        if (!quad_ok || (p->symmetric && row_base >= col0 + 32)) continue;
+        tmem_ld32(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + half * (BN / 2) + 32 * b), v);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) *reinterpret_cast<float4*>(piece(lane, c)) = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
         __syncwarp();
+      };
+      auto turned = [&](int it) { return *reinterpret_cast<const float4*>(piece(4 * it + sub_r, lane & 7)); };
+      if (epi == EPI_ROTATED_ADAM) {
+        const float b1 = p->beta1, ob1 = 1.0f - p->beta1;
+        float* const pv = p->D + at_d;                 // V~
+        float* const pm = p->D2 + at_d;                // M~
+        float4 mm[8], ss[8];
+        int n_it = rows_of(0);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) tile[lane * EPI_LD + j] = v[j];
-        __syncwarp();
-        const int col = col0 + sub_c;
-        // columns come in multiples of 8: a group of four is all in or all out
-        int n_it = 0;
-        if (col < p->Nd) { n_it = (p->Md - row_base - sub_r + 3) >> 2; n_it = n_it > 8 ? 8 : n_it; }
-        float4 a[8];
-#pragma unroll
-        for (int it = 0; it < 8; ++it) {
-          const float* t4 = tile + (it * 4 + sub_r) * EPI_LD + sub_c;
-          a[it] = make_float4(t4[0], t4[1], t4[2], t4[3]);
-        }
-        if (epi == EPI_AXPBY_F32) {
-          float* d = p->D + (long long)(row_base + sub_r) * p->ldd + col;
-          const long long step = 4 * p->ldd;
-          float4 old[8];
-          if (beta != 0.0f) {
-#pragma unroll
-            for (int it = 0; it < 8; ++it)
-              if (it < n_it) old[it] = *reinterpret_cast<const float4*>(d + it * step);
+        for (int it = 0; it < 8; ++it)
+          if (it < n_it) {
+            mm[it] = *reinterpret_cast<const float4*>(pm + it * step_d);
+            ss[it] = *reinterpret_cast<const float4*>(pv + it * step_d);
           }
+        if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag, status)) break;
+        tc_fence_after();
+#pragma unroll 1
+        for (int b = 0; b < BN / 64; ++b) {
+          if (!writes(b)) break;
+          turn(b);
+          const int n_next = rows_of(b + 1);
+          float *const dv = pv + 32 * b, *const dm = pm + 32 * b;
+          __nv_bfloat16* const xh = p->Dh + at_h + 32 * b;
 #pragma unroll
           for (int it = 0; it < 8; ++it) {
-            float4 o = make_float4(alpha * a[it].x, alpha * a[it].y, alpha * a[it].z, alpha * a[it].w);
-            if (beta != 0.0f && it < n_it) {
-              o.x = fmaf(beta, old[it].x, o.x); o.y = fmaf(beta, old[it].y, o.y);
-              o.z = fmaf(beta, old[it].z, o.z); o.w = fmaf(beta, old[it].w, o.w);
-            }
-            if (it < n_it) *reinterpret_cast<float4*>(d + it * step) = o;
-          }
-        } else if (epi == EPI_ROTATED_ADAM) {
-          float* d = p->D + (long long)(row_base + sub_r) * p->ldd + col;      // V~
-          float* m2 = p->D2 + (long long)(row_base + sub_r) * p->ldd + col;    // M~
-          __nv_bfloat16* xh = p->Dh + (long long)(row_base + sub_r) * p->ldh + col;
-          const long long step = 4 * p->ldd, steph = 4 * p->ldh;
-          const float b1 = p->beta1, ob1 = 1.0f - p->beta1;
-          float4 mm[8], ss[8];
-#pragma unroll
-          for (int it = 0; it < 8; ++it)
             if (it < n_it) {
-              mm[it] = *reinterpret_cast<const float4*>(m2 + it * step);
-              ss[it] = *reinterpret_cast<const float4*>(d + it * step);
-            }
-#pragma unroll
-          for (int it = 0; it < 8; ++it)
-            if (it < n_it) {
-              const float4 g = make_float4(gclip * a[it].x, gclip * a[it].y, gclip * a[it].z, gclip * a[it].w);
+              const float4 x = turned(it);
+              const float4 g = make_float4(gclip * x.x, gclip * x.y, gclip * x.z, gclip * x.w);
               float4 m = mm[it], q = ss[it];
               m.x = b1 * m.x + ob1 * g.x; m.y = b1 * m.y + ob1 * g.y;
               m.z = b1 * m.z + ob1 * g.z; m.w = b1 * m.w + ob1 * g.w;
               q.x = fmaf(beta, q.x, alpha * g.x * g.x); q.y = fmaf(beta, q.y, alpha * g.y * g.y);
               q.z = fmaf(beta, q.z, alpha * g.z * g.z); q.w = fmaf(beta, q.w, alpha * g.w * g.w);
-              *reinterpret_cast<float4*>(m2 + it * step) = m;
-              *reinterpret_cast<float4*>(d + it * step) = q;
+              *reinterpret_cast<float4*>(dm + it * step_d) = m;
+              *reinterpret_cast<float4*>(dv + it * step_d) = q;
               uint2 o;
-              o.x = pack2_bf16(m.x / sqrtf(q.x + eps), m.y / sqrtf(q.y + eps));
-              o.y = pack2_bf16(m.z / sqrtf(q.z + eps), m.w / sqrtf(q.w + eps));
-              *reinterpret_cast<uint2*>(xh + it * steph) = o;
+              o.x = pack2_bf16(m.x * inv_sqrt(q.x + eps), m.y * inv_sqrt(q.y + eps));
+              o.y = pack2_bf16(m.z * inv_sqrt(q.z + eps), m.w * inv_sqrt(q.w + eps));
+              *reinterpret_cast<uint2*>(xh + it * step_h) = o;
             }
-        } else if (epi == EPI_SECOND_MOMENT) {
-          float* d = p->D + (long long)(row_base + sub_r) * p->ldd + col;
-          const long long step = 4 * p->ldd;
-          float4 ss[8];
+            if (it < n_next) {
+              mm[it] = *reinterpret_cast<const float4*>(dm + 32 + it * step_d);
+              ss[it] = *reinterpret_cast<const float4*>(dv + 32 + it * step_d);
+            }
+          }
+          n_it = n_next;
+          __syncwarp();                           // the block's buffer is rewritten by the next one
+        }
+      } else if (epi == EPI_AXPBY_F32) {
+        float* const pd = p->D + at_d;
+        float4 old[8];
+        const bool rd = beta != 0.0f;
+        int n_it = rows_of(0);
 #pragma unroll
-          for (int it = 0; it < 8; ++it)
-            if (it < n_it) ss[it] = *reinterpret_cast<const float4*>(d + it * step);
+        for (int it = 0; it < 8; ++it)
+          if (rd && it < n_it) old[it] = *reinterpret_cast<const float4*>(pd + it * step_d);
+        if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag, status)) break;
+        tc_fence_after();
+#pragma unroll 1
+        for (int b = 0; b < BN / 64; ++b) {
+          const int n_next = rows_of(b + 1);
+          float* const d = pd + 32 * b;
+          if (writes(b)) turn(b);
+#pragma unroll
+          for (int it = 0; it < 8; ++it) {
+            if (it < n_it) {
+              const float4 x = turned(it);
+              float4 o = make_float4(alpha * x.x, alpha * x.y, alpha * x.z, alpha * x.w);
+              if (rd) {
+                o.x = fmaf(beta, old[it].x, o.x); o.y = fmaf(beta, old[it].y, o.y);
+                o.z = fmaf(beta, old[it].z, o.z); o.w = fmaf(beta, old[it].w, o.w);
+              }
+              *reinterpret_cast<float4*>(d + it * step_d) = o;
+            }
+            if (rd && it < n_next) old[it] = *reinterpret_cast<const float4*>(d + 32 + it * step_d);
+          }
+          n_it = n_next;
+          __syncwarp();
+        }
+      } else {  // EPI_SPLIT_BF16
+        if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag, status)) break;
+        tc_fence_after();
+#pragma unroll 1
+        for (int b = 0; b < BN / 64; ++b) {
+          if (!writes(b)) break;
+          turn(b);
+          const int n_it = rows_of(b);
+          __nv_bfloat16* const dh = p->Dh + at_h + 32 * b;
+          __nv_bfloat16* const dl = p->Dl ? p->Dl + at_h + 32 * b : nullptr;
 #pragma unroll
           for (int it = 0; it < 8; ++it)
             if (it < n_it) {
-              const float4 g = a[it];
-              float4 q = ss[it];
-              q.x = fmaf(beta, q.x, alpha * g.x * g.x); q.y = fmaf(beta, q.y, alpha * g.y * g.y);
-              q.z = fmaf(beta, q.z, alpha * g.z * g.z); q.w = fmaf(beta, q.w, alpha * g.w * g.w);
-              *reinterpret_cast<float4*>(d + it * step) = q;
-            }
-        } else if (epi == EPI_SCALE_BF16) {
-          const float* d = p->D + (long long)(row_base + sub_r) * p->ldd + col;
-          __nv_bfloat16* xh = p->Dh + (long long)(row_base + sub_r) * p->ldh + col;
-          const long long step = 4 * p->ldd, steph = 4 * p->ldh;
-          float4 ss[8];
-#pragma unroll
-          for (int it = 0; it < 8; ++it)
-            if (it < n_it) ss[it] = *reinterpret_cast<const float4*>(d + it * step);
-#pragma unroll
-          for (int it = 0; it < 8; ++it)
-            if (it < n_it) {
-              const float4 g = a[it], q = ss[it];
-              uint2 o;
-              o.x = pack2_bf16(g.x / sqrtf(q.x + eps), g.y / sqrtf(q.y + eps));
-              o.y = pack2_bf16(g.z / sqrtf(q.z + eps), g.w / sqrtf(q.w + eps));
-              *reinterpret_cast<uint2*>(xh + it * steph) = o;
-            }
-        } else {  // EPI_SPLIT_BF16
-          __nv_bfloat16* dh = p->Dh + (long long)(row_base + sub_r) * p->ldh + col;
-          __nv_bfloat16* dl = p->Dl ? p->Dl + (long long)(row_base + sub_r) * p->ldh + col : nullptr;
-          const long long steph = 4 * p->ldh;
-#pragma unroll
-          for (int it = 0; it < 8; ++it)
-            if (it < n_it) {
-              const float4 g = a[it];
+              const float4 g = turned(it);
               const float h0 = __bfloat162float(__float2bfloat16_rn(g.x)), h1 = __bfloat162float(__float2bfloat16_rn(g.y));
               const float h2 = __bfloat162float(__float2bfloat16_rn(g.z)), h3 = __bfloat162float(__float2bfloat16_rn(g.w));
               uint2 o;
               o.x = pack2_bf16(h0, h1); o.y = pack2_bf16(h2, h3);
-              *reinterpret_cast<uint2*>(dh + it * steph) = o;
+              *reinterpret_cast<uint2*>(dh + it * step_h) = o;
               if (dl) {
                 uint2 l;
                 l.x = pack2_bf16(g.x - h0, g.y - h1); l.y = pack2_bf16(g.z - h2, g.w - h3);
-                *reinterpret_cast<uint2*>(dl + it * steph) = l;
+                *reinterpret_cast<uint2*>(dl + it * step_h) = l;
               }
             }
+          __syncwarp();
         }
-        __syncwarp();                             // the tile is rewritten by the next block
       }
       // all tcgen05.ld of this warp have completed (wait::ld): hand the accumulator back
       tc_fence_before();
@@ -1228,7 +1238,7 @@ TcPlan* tc_plan_create(const TcProblem* problems, int n, int device, cudaStream_
       return fail("tensor-core problem: a symmetric product needs a square fp32 result");
     d.D = q.D; d.ldd = q.ldd; d.Dh = q.Dh; d.Dl = q.Dl; d.ldh = q.ldh; d.D2 = q.D2;
     const bool need_D = q.epilogue != EPI_SPLIT_BF16;
-    const bool need_H = q.epilogue == EPI_SPLIT_BF16 || q.epilogue == EPI_SCALE_BF16 || q.epilogue == EPI_ROTATED_ADAM;
+    const bool need_H = q.epilogue == EPI_SPLIT_BF16 || q.epilogue == EPI_ROTATED_ADAM;
     if (q.epilogue == EPI_ROTATED_ADAM && (!q.D2 || (reinterpret_cast<uintptr_t>(q.D2) & 15)))
       return fail("tensor-core problem: second in/out pointer missing or misaligned");
     if ((need_D && (!q.D || (q.ldd % 4) || (reinterpret_cast<uintptr_t>(q.D) & 15))) ||
@@ -1309,7 +1319,7 @@ cudaError_t tc_plan_launch_range(TcPlan* p, int first, int count, long long call
   } else {
     cfg.gridDim = dim3((unsigned)(whole ? p->units : tiles < p->sm_count ? tiles : p->sm_count));
   }
-  cfg.blockDim = dim3(p->fold ? FOLD_THREADS : NUM_THREADS);
+  cfg.blockDim = dim3(NUM_THREADS);
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = s;
   return cudaLaunchKernelEx(&cfg, kernel, (const DevProblem*)p->d_probs, p->n, t0, t1,

@@ -183,6 +183,9 @@ struct Bump {
 inline size_t simt_need(const Layer& L) { return 4 * (((size_t)L.d.m * L.d.n + 63) / 64 * 64); }
 constexpr size_t kSimtScratch = 16u << 20;
 
+// A gradient of this size is copied by itself (164 MB: 52 us, 64 in the grouped kernel).
+constexpr size_t kCopyAlone = 4u << 20;
+
 // S = 1st: the half product of a refresh (M^T U, or M V) is formed in equal slices of the unrotated dimension, each
 // at most 128 MiB of fp64 in every lane.  (Whole, it was 393 MB a lane for an embedding of 32000 x 1536.  Slices of half
 // the size cost 1 to 2 % of such a refresh.)
@@ -903,7 +906,11 @@ br_status br_create(br_handle** out, const br_layer_desc* layers, int n_layers, 
     if ((e = cudaEventCreateWithFlags(&h->lanes[i].done, cudaEventDisableTiming)) != cudaSuccess) return fail("cudaEventCreate", e);
   }
   if ((e = cudaEventCreateWithFlags(&h->ev_begin, cudaEventDisableTiming)) != cudaSuccess) return fail("cudaEventCreate", e);
-  if ((e = cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking)) != cudaSuccess) return fail("cudaStreamCreate", e);
+  // The side stream of a step has the highest priority: the CTAs of a launch that waits for SMs behind a running one (the
+  // next phase of the step) would otherwise keep back those of the copies, which fit beside the running ones.
+  int least = 0, greatest = 0;
+  if ((e = cudaDeviceGetStreamPriorityRange(&least, &greatest)) != cudaSuccess) return fail("cudaDeviceGetStreamPriorityRange", e);
+  if ((e = cudaStreamCreateWithPriority(&h->copy_stream, cudaStreamNonBlocking, greatest)) != cudaSuccess) return fail("cudaStreamCreate", e);
   if ((e = cudaEventCreateWithFlags(&h->ev_consumed, cudaEventDisableTiming)) != cudaSuccess) return fail("cudaEventCreate", e);
   if ((e = cudaEventCreateWithFlags(&h->ev_copied, cudaEventDisableTiming)) != cudaSuccess) return fail("cudaEventCreate", e);
   if ((e = cudaEventCreateWithFlags(&h->ev_cond, cudaEventDisableTiming)) != cudaSuccess) return fail("cudaEventCreate", e);
@@ -1081,15 +1088,17 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
       br_handle* h = c->h;
       BR_CUDA(h, cudaEventRecord(h->ev_consumed, h->stream));
       BR_CUDA(h, cudaStreamWaitEvent(h->copy_stream, h->ev_consumed, 0));
+      std::vector<CopyJob> copies;
       for (int j = 0; j < n; ++j) {
         Layer& L = h->layers[ids[j]];
         if (L.ring_slots <= 0 || (*c->stored)[ids[j]]) continue;
-        const size_t bytes = (size_t)L.d.m * L.d.n * dtype_size(L.d.grad_dtype);
-        void* dst = const_cast<void*>(ring_slot_ptr(L, (h->calls - 1) % L.ring_slots));
-        BR_CUDA(h, cudaMemcpyAsync(dst, c->grads[ids[j]], bytes, cudaMemcpyDeviceToDevice, h->copy_stream));
+        copies.push_back({c->grads[ids[j]], const_cast<void*>(ring_slot_ptr(L, (h->calls - 1) % L.ring_slots)),
+                          (size_t)L.d.m * L.d.n * dtype_size(L.d.grad_dtype)});
         (*c->stored)[ids[j]] = 1;
-        c->copied = true;
       }
+      if (copies.empty()) return (int)BR_OK;
+      c->copied = true;
+      BR_CUDA(h, ring_copy(copies.data(), (int)copies.size(), true, h->copy_stream));
       return (int)BR_OK;
     };
     const char* terr = nullptr;
@@ -1105,13 +1114,16 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
     }
   }
   // ---- store g_c in the ring (after every reader of the slot it may overwrite) --------------
+  std::vector<CopyJob> copies;
   for (int i = 0; i < nl; ++i) {
     Layer& L = h->layers[i];
     if (L.ring_slots <= 0 || stored[i]) continue;
+    void* const slot = const_cast<void*>(ring_slot_ptr(L, (h->calls - 1) % L.ring_slots));
     const size_t bytes = (size_t)L.d.m * L.d.n * dtype_size(L.d.grad_dtype);
-    void* dst = const_cast<void*>(ring_slot_ptr(L, (h->calls - 1) % L.ring_slots));
-    BR_CUDA(h, cudaMemcpyAsync(dst, grads[i], bytes, cudaMemcpyDeviceToDevice, h->stream));
+    if (bytes >= kCopyAlone) BR_CUDA(h, cudaMemcpyAsync(slot, grads[i], bytes, cudaMemcpyDeviceToDevice, h->stream));
+    else copies.push_back({grads[i], slot, bytes});
   }
+  if (!copies.empty()) BR_CUDA(h, ring_copy(copies.data(), (int)copies.size(), false, h->stream));
   return any ? BR_OK : BR_WARMUP;
 }
 

@@ -98,6 +98,11 @@ cudaError_t clip_factor(const void* const* grads, const int64_t* numel, const in
 cudaError_t plain_adam(float* W, float* M, float* V, const void* G, int g_is_bf16, int64_t numel,
                        float lr, float beta1, float beta2, float eps, float wd, const float* gscale, cudaStream_t s);
 
+// Matrices of one launch at most (by value).
+constexpr int kElemGroup = 64;
+// dst <- src (an even number of bytes; dst on a 16-byte boundary); beside: one CTA per SM, next to contraction launches
+struct CopyJob { const void* src; void* dst; size_t bytes; };
+cudaError_t ring_copy(const CopyJob* jobs, int n, bool beside, cudaStream_t s);
 // F[j][i] <- F[i][j] for the 32 x 32 blocks (j, i) strictly below the diagonal of the k x k matrix F.
 cudaError_t mirror_lower(float* F, int64_t k, cudaStream_t s);
 // fp32 -> bf16 hi (+ optional lo = bf16(x - hi)).

@@ -1,6 +1,8 @@
 // Fused element-wise kernels of the rotated Adam step.  All are HBM-bound: one pass over the
 // data, 128-bit accesses on the aligned body, grid-stride loops on a grid sized as a multiple of
 // the SM count.
+#include <algorithm>
+
 #include "br_internal.h"
 
 namespace br {
@@ -295,6 +297,40 @@ __global__ void __launch_bounds__(kThreads) k_clip_final(const double* __restric
   *out = (nrm > (double)clip) ? (float)((double)clip / nrm) : 1.0f;
 }
 
+// Copies (a call's gradients into the ring) that run beside the contraction launches: one CTA of 256 threads and 40
+// registers per SM is what an SM has room for next to one of those (it leaves 11.7 of 64 thousand registers and 1.9 KB of shared
+// memory, of which every CTA takes one; two copy CTAs on an SM would keep the next contraction launch off it until they are
+// done).  One cudaMemcpyAsync per gradient takes 2.7 us each at the sizes of a d = 384 layer, 43 us a step, and finds no room there.
+constexpr int kCopyThreads = 256, kCopyLoads = 4;
+struct CopyArgs { CopyJob j[kElemGroup]; long long begin[kElemGroup + 1]; int n; };     // begin: in 16-byte pieces
+__global__ void __launch_bounds__(kCopyThreads, 6) k_ring_copy(const __grid_constant__ CopyArgs a) {
+  const long long total = a.begin[a.n], stride = (long long)gridDim.x * kCopyThreads;
+  int job = 0;
+  for (long long i = (long long)blockIdx.x * kCopyThreads + threadIdx.x; i < total; i += kCopyLoads * stride) {
+    uint4 v[kCopyLoads];
+    uint4* d[kCopyLoads];
+#pragma unroll
+    for (int u = 0; u < kCopyLoads; ++u) {
+      const long long at = i + u * stride;
+      d[u] = nullptr;
+      if (at >= total) continue;
+      while (a.begin[job + 1] <= at) ++job;
+      const CopyJob& j = a.j[job];
+      const size_t off = (size_t)(at - a.begin[job]) * 16;
+      const char* s = static_cast<const char*>(j.src) + off;
+      if (reinterpret_cast<uintptr_t>(s) % 16 == 0 && off + 16 <= j.bytes) {
+        v[u] = __ldg(reinterpret_cast<const uint4*>(s));
+        d[u] = reinterpret_cast<uint4*>(static_cast<char*>(j.dst) + off);
+      } else {                                 // (gradients are 2-byte aligned at least; the slots are 256-byte aligned)
+        for (size_t b = off; b < off + 16 && b < j.bytes; b += 2)
+          *reinterpret_cast<uint16_t*>(static_cast<char*>(j.dst) + b) = *reinterpret_cast<const uint16_t*>(static_cast<const char*>(j.src) + b);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kCopyLoads; ++u) if (d[u]) *d[u] = v[u];
+  }
+}
+
 // x (rounded to fp32) = p1 + p2 + p3 with three bf16 terms: all 24 significant bits survive.
 __device__ __forceinline__ void split3(float f, __nv_bfloat16& p1, __nv_bfloat16& p2, __nv_bfloat16& p3) {
   const float h1 = bf16_round(f);
@@ -351,6 +387,21 @@ k_f64_to_f32(const double* __restrict__ X, float* __restrict__ out, int64_t nume
 
 cudaError_t set_identity(float* Q, int64_t k, cudaStream_t s) {
   k_set_identity<<<grid_for(k * k), kThreads, 0, s>>>(Q, k);
+  return cudaGetLastError();
+}
+
+cudaError_t ring_copy(const CopyJob* jobs, int n, bool beside, cudaStream_t s) {
+  for (int first = 0; first < n; first += kElemGroup) {
+    CopyArgs a;
+    a.n = std::min(kElemGroup, n - first);
+    a.begin[0] = 0;
+    for (int i = 0; i < a.n; ++i) {
+      a.j[i] = jobs[first + i];
+      a.begin[i + 1] = a.begin[i] + (long long)((a.j[i].bytes + 15) / 16);
+    }
+    const long long want = (a.begin[a.n] + kCopyThreads - 1) / kCopyThreads;
+    k_ring_copy<<<(unsigned)std::min<long long>(want, 148 * (beside ? 1 : 6)), kCopyThreads, 0, s>>>(a);
+  }
   return cudaGetLastError();
 }
 

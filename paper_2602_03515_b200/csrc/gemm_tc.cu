@@ -429,9 +429,6 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
   __shared__ uint32_t dead_word;
   volatile int* abort_flag = &abort_word;
 
-  // an earlier launch failed: nothing to do (a pair takes the decision from its leader, below)
-  if (!PAIR && *reinterpret_cast<volatile int*>(status) < 0) return;
-
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;        // 0: leader of the pair
   const int unit = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;      // index of this CTA (pair) in the tile walk
@@ -458,7 +455,6 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
     // accumulator hand-back: every epilogue warp, of both CTAs in the paired form
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), (PAIR ? 2 : 1) * EPI_WARPS); }
     abort_word = 0;
-    dead_word = (*reinterpret_cast<volatile int*>(status) < 0) ? 1u : 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -470,9 +466,15 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
       asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
   }
+  // Up to here nothing of the launches before was touched: a launch may begin while the last CTAs of the one before it
+  // are still working (programmatic dependent launch), and its CTAs find their set-up done when those have finished.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // an earlier launch failed: nothing to do
+  if (threadIdx.x == 0) dead_word = (*reinterpret_cast<volatile int*>(status) < 0) ? 1u : 0u;
   tc_fence_before();
   __syncthreads();
-  bool dead = false;
+  bool dead = dead_word != 0u;
   if (PAIR) {
     // both CTAs have initialised their barriers before either signals the other; the pair skips its
     // work together when the leader saw a failed status word
@@ -1298,8 +1300,9 @@ void tc_plan_destroy(TcPlan* p) {
 
 double tc_plan_flops(const TcPlan* p) { return p ? p->flops : 0.0; }
 
-cudaError_t tc_plan_launch_range(TcPlan* p, int first, int count, long long calls, int tau, float dyn_alpha,
-                                 float dyn_beta, int* status_word, cudaStream_t s) {
+namespace {
+cudaError_t launch_range(TcPlan* p, int first, int count, long long calls, int tau, float dyn_alpha, float dyn_beta, int* status_word,
+                         cudaStream_t s, bool overlap) {
   if (first < 0 || count < 1 || first + count > p->n) return cudaErrorInvalidValue;
   const int t0 = p->tile_begin[first], t1 = p->tile_begin[first + count];
   const int tiles = t1 - t0;
@@ -1308,14 +1311,20 @@ cudaError_t tc_plan_launch_range(TcPlan* p, int first, int count, long long call
   const int smem_bytes = p->fold ? SMEM_BYTES_FOLD : SMEM_BYTES;
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   const bool whole = first == 0 && count == p->n;
+  cfg.attrs = attr;
+  if (overlap) {
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 1;
+  }
   if (p->pair) {
     const int units = whole ? p->units : tiles < p->max_pairs ? tiles : p->max_pairs;
     cfg.gridDim = dim3(2u * (unsigned)units);
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    cudaLaunchAttribute& a = attr[cfg.numAttrs++];
+    a.id = cudaLaunchAttributeClusterDimension;
+    a.val.clusterDim.x = 2; a.val.clusterDim.y = 1; a.val.clusterDim.z = 1;
   } else {
     cfg.gridDim = dim3((unsigned)(whole ? p->units : tiles < p->sm_count ? tiles : p->sm_count));
   }
@@ -1327,9 +1336,17 @@ cudaError_t tc_plan_launch_range(TcPlan* p, int first, int count, long long call
                             dyn_beta, status_word);
 }
 
+}  // namespace
+
+cudaError_t tc_plan_launch_range(TcPlan* p, int first, int count, long long calls, int tau, float dyn_alpha,
+                                 float dyn_beta, int* status_word, cudaStream_t s) {
+  return launch_range(p, first, count, calls, tau, dyn_alpha, dyn_beta, status_word, s, false);
+}
+
+// The phases of a step follow one another on the stream: each launch's set-up overlaps the tail of the one before.
 cudaError_t tc_plan_launch(TcPlan* p, long long calls, int tau, float dyn_alpha, float dyn_beta,
                            int* status_word, cudaStream_t s) {
-  return tc_plan_launch_range(p, 0, p->n, calls, tau, dyn_alpha, dyn_beta, status_word, s);
+  return launch_range(p, 0, p->n, calls, tau, dyn_alpha, dyn_beta, status_word, s, true);
 }
 
 cudaError_t tc_wait_probe(uint64_t limit_ns, int* status_word, cudaStream_t s) {

@@ -13,7 +13,7 @@
 //    Gram matrix and applies R^-1 and the projections to its own rows only, so these steps need no
 //    barrier between them.  Only the Gram sums and the projection coefficients cross CTAs.
 //  * The Gram shares stay in shared memory: every CTA adds up one slice of rows over all shares (fixed
-//    order, through distributed shared memory), and after a second barrier every CTA reads all slices and
+//    order, through distributed shared memory) and writes it into every CTA, and after a second barrier each
 //    computes the 64 x 64 Cholesky factor and its inverse for itself.  The redundant factorisation costs
 //    nothing (the other CTAs would wait for it) and saves the broadcast, and since all of them see the
 //    same bits, every decision (second pass, second sweep, completion) is taken alike without a word
@@ -22,7 +22,7 @@
 //    when there are fewer tiles than CTAs (partial sums through distributed shared memory, fixed order).
 //
 // Products run on the fp64 matrix unit (mma.sync.m8n8k4.f64): 64 x 64 tiles, a warp 16 rows x 32 columns,
-// 16-deep stages, three of them in flight with cp.async.  111 KiB of shared memory and 128 registers, two CTAs
+// 16-deep stages, three of them in flight with cp.async.  95 KiB of shared memory and 128 registers, two CTAs
 // per SM, so that the clusters of several bases share SMs and one cluster's barriers are another's work.
 // Other CTAs write A and C while the kernel runs: plain loads are ordered by the acquire of the barrier
 // behind those writes, and none goes through the read-only path.
@@ -52,11 +52,10 @@ constexpr int kLdP = 72;                      // partial sums (16-byte stores of
 constexpr int kMaxCluster = 16;
 constexpr int kStageD = kStages * (kOper + kOperB);   // operand stages; also one 64 x 64 tile of A (ld 68)
 constexpr int kPartD = 64 * kLdP;             // partial sums of this CTA, later R^-T (ld 68)
-constexpr int kSredD = 32 * 64;               // this CTA's slice of the summed Gram matrix (at most half of it)
 // One shared-memory array, carved at compile time (pointers kept in a structure would make every access a
 // generic one behind a reload of the pointer).
 extern __shared__ double sm[];
-constexpr int oStage = 0, oPart = oStage + kStageD, oSred = oPart + kPartD, oDiag0 = oSred + kSredD, oFloor = oDiag0 + 64,
+constexpr int oStage = 0, oPart = oStage + kStageD, oDiag0 = oPart + kPartD, oFloor = oDiag0 + 64,
               oPiv = oFloor + 64, oN0 = oPiv + 64, kSmemD = oN0 + 64;
 constexpr int kSmemBytes = kSmemD * (int)sizeof(double);
 static_assert(kStageD >= 64 * kLdK && kOper >= kOperB, "staging area");
@@ -307,8 +306,9 @@ struct Ctx {
 // once block row j is done, and column block j of the identity's part is still a unit block until then, so
 // both share one 64 x 64 array.  The chain is bound by the 8 x 8 factorisations: warp 0 alone updates the
 // next diagonal block and factors it in registers (every lane the same: no shuffles, 8 dependent square
-// roots), while warp w updates block row c + w.  Two barriers a block instead of one a pivot: 64 pivots in
-// 12 us; 27 us with a barrier a pivot and the matrix in registers, 20 us with two pivots a barrier.
+// roots), while the other warps update the rest, all of a warp's blocks at once (a block row to a warp took as long as two
+// factorisations).  Two barriers a block instead of one a pivot: 27 us with a barrier a pivot and the matrix in registers,
+// 20 us with two pivots a barrier, 13.3 us with a block row to a warp and CUDA's rsqrt().
 // (Multiplying block row c by an explicit R_cc^-T instead loses the factorisation of a panel with a condition
 // number of 1e6, such as a completed rank-deficient product has: its error, 1e-16 times the condition number,
 // swamps pivots of 1e-12.  Substitution is backward stable like the unblocked elimination.)
@@ -316,19 +316,43 @@ struct Ctx {
 constexpr int oZ = oStage, oX = oZ + 64 * kLdK, oD = oX + 8 * kLdK;      // (in the operand stages)
 static_assert(64 * kLdK + 8 * kLdK + 8 * 8 + 8 <= kStageD, "the factorisation borrows the operand stages");
 
+// 1 / sqrt(x) of a positive normal number: the hardware's approximation y (relative error 1e-6) and the third-order
+// iteration y (1 + e / 2 + 3 e^2 / 8), e = 1 - x y^2, four dependent operations: 49 cycles, rsqrt() 61 (the square roots are the
+// chain's critical path).  Largest relative error over 1e-260 .. 1e260: 2.2e-16.
+__device__ __forceinline__ double inv_sqrt(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
+// The blocks that step c updates with block row c - 1, its own diagonal block excepted: rows i >= c, columns j > i, j = i
+// and (the identity's part) j < c.  Entries beyond the count are valid blocks whose result is dropped.
+struct Updates { unsigned char ij[8][35]; unsigned char n[8]; };
+constexpr Updates make_updates() {
+  Updates u = {};
+  for (int c = 1; c < 8; ++c)
+    for (int i = c; i < 8; ++i)
+      for (int j = 0; j < 8; ++j)
+        if (j < c || j > i || (j == i && i > c)) u.ij[c][u.n[c]++] = (unsigned char)(8 * i + j);
+  return u;
+}
+__constant__ const Updates kUpdates = make_updates();
+
 // The diagonal block at Z (upper triangle) -> R_cc at oD (row-major 8 x 8), 1 / diagonal behind it, pivots at oPiv + 8 c
 __device__ __forceinline__ void factor8(const double* Z, int c) {
   const int lane = threadIdx.x & 31;
-  double u[8][8], inv[8], piv[8];
+  double u[8][8], inv[8], piv[8], fl[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) fl[i] = sm[oFloor + 8 * c + i];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
     for (int j = i; j < 8; ++j) u[i][j] = Z[i * kLdK + j];
 #pragma unroll
   for (int p = 0; p < 8; ++p) {
-    const double fl = sm[oFloor + 8 * c + p];
-    piv[p] = u[p][p] > fl ? u[p][p] : fl;
-    inv[p] = rsqrt(piv[p]);
+    piv[p] = u[p][p] > fl[p] ? u[p][p] : fl[p];
+    inv[p] = inv_sqrt(piv[p]);
 #pragma unroll
     for (int j = p + 1; j < 8; ++j) u[p][j] *= inv[p];
 #pragma unroll
@@ -347,50 +371,57 @@ __device__ __forceinline__ void factor8(const double* Z, int c) {
   }
 }
 
-__device__ __noinline__ void chol64(const Ctx q, int bw) {
+__device__ __noinline__ void chol64(int bw) {
   const int t = threadIdx.x, w = t >> 5, lane = t & 31, g = lane >> 2, tig = lane & 3;
-  const int rs = 64 / q.cs, nb = (bw + 7) / 8;
+  const int nb = (bw + 7) / 8;
   double* const Z = sm + oZ;
   double* const RT = sm + oPart;
-  // upper block triangle of S (identity beyond the panel), zero below
-  double v[16];
-#pragma unroll
-  for (int u = 0; u < 16; ++u) {
-    const int i = (t >> 6) + 4 * u, j = t & 63;
-    v[u] = (i == j) ? 1.0 : 0.0;
-    if (j >= (i & ~7) && max(i, j) < bw) v[u] = q.cs == 1 ? sm[oPart + i * kLdP + j] : cg::this_cluster().map_shared_rank(sm + oSred, i / rs)[(i % rs) * 64 + j];
-  }
-#pragma unroll
-  for (int u = 0; u < 16; ++u) {
-    const int i = (t >> 6) + 4 * u, j = t & 63;
-    Z[i * kLdK + j] = v[u];
-    if (i == j) {
-      sm[oDiag0 + i] = v[u];
-      const double f = v[u] * 1e-24;
-      sm[oFloor + i] = f > 1e-300 ? f : 1e-300;      // a pivot at or below this is clamped
-    }
+  if (t < 64) {
+    const double d = Z[t * kLdK + t], f = d * 1e-24;
+    sm[oDiag0 + t] = d;
+    sm[oFloor + t] = f > 1e-300 ? f : 1e-300;        // a pivot at or below this is clamped
   }
   __syncthreads();
-  // block (i, j) of rows to come <- itself - R_ci^T X_j, with block row c of R | R^-T in oX
-  auto update = [&](int i, int j) {
-    double2* z = reinterpret_cast<double2*>(Z + (8 * i + g) * kLdK + 8 * j + 2 * tig);
-    double2 d = *z;
-#pragma unroll
-    for (int k4 = 0; k4 < 8; k4 += 4) {
-      const double* x = sm + oX + (k4 + tig) * kLdK + g;
-      dmma(d.x, d.y, -x[8 * i], x[8 * j]);
-    }
-    *z = d;
-  };
 #pragma unroll 1
   for (int c = 0; c < nb; ++c) {
     if (w == 0) {
-      if (c > 0) { update(c, c); __syncwarp(); }
+      if (c > 0) {
+        // block (c, c) <- itself - R_{c-1,c}^T R_{c-1,c}, and its factorisation
+        double2* z = reinterpret_cast<double2*>(Z + (8 * c + g) * kLdK + 8 * c + 2 * tig);
+        double2 d = *z;
+#pragma unroll
+        for (int k4 = 0; k4 < 8; k4 += 4) {
+          const double x = sm[oX + (k4 + tig) * kLdK + g + 8 * c];
+          dmma(d.x, d.y, -x, x);
+        }
+        *z = d;
+        __syncwarp();
+      }
       factor8(Z + 8 * c * kLdK + 8 * c, c);
-    } else if (c > 0 && c - 1 + w < nb) {
-      const int i = c - 1 + w;
-      for (int j = 0; j < nb; ++j)
-        if (j < c || j > i || (j == i && i > c)) update(i, j);
+    } else if (c > 0) {
+      // the other blocks (i, j) of rows to come <- themselves - R_{c-1,i}^T X_j, with block row c - 1 of R | R^-T in oX:
+      // at most 34, dealt to seven warps, all of a warp's in flight at once
+      constexpr int U = 5;
+      double2 d[U];
+      int bi[U], bj[U];
+      bool ok[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int e = w - 1 + 7 * u, ij = kUpdates.ij[c][e];
+        bi[u] = ij >> 3; bj[u] = ij & 7;
+        ok[u] = e < kUpdates.n[c] && max(bi[u], bj[u]) < nb;
+        d[u] = *reinterpret_cast<const double2*>(Z + (8 * bi[u] + g) * kLdK + 8 * bj[u] + 2 * tig);
+      }
+#pragma unroll
+      for (int k4 = 0; k4 < 8; k4 += 4)
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const double* x = sm + oX + (k4 + tig) * kLdK + g;
+          dmma(d[u].x, d[u].y, -x[8 * bi[u]], x[8 * bj[u]]);
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (ok[u]) *reinterpret_cast<double2*>(Z + (8 * bi[u] + g) * kLdK + 8 * bj[u] + 2 * tig) = d[u];
     }
     __syncthreads();
     // block row c: R right of the diagonal, R^-T up to it
@@ -461,43 +492,34 @@ template <bool VEC>
 __device__ __noinline__ void project64(const Ctx q, double* C, int jp, int wp, int jt, int wt) {
   const int t = threadIdx.x;
   const int ntp = (wp + 63) / 64, ntt = (wt + 63) / 64, tiles = ntp * ntt;
-  const int sp = tiles < q.cs ? q.cs / tiles : 1;       // CTAs that share one tile's contraction
   double acc[16];
   cluster_sync();                                       // every CTA's rows of both blocks are written
-  auto tile_pos = [&](int tile, int* i0, int* c0, int* I, int* J) {
-    *i0 = (tile / ntt) * 64; *c0 = (tile % ntt) * 64; *I = min(64, wp - *i0); *J = min(64, wt - *c0);
-  };
-  if (sp == 1) {
-    for (int tile = q.rank; tile < tiles; tile += q.cs) {
-      int i0, c0, I, J;
-      tile_pos(tile, &i0, &c0, &I, &J);
-      clear(acc);
-      mm64<VEC, true, false, false>(acc, q.A + jp + i0, q.k, I, q.A + jt + c0, q.k, J, (int)q.k);
+  // A tile per CTA while there are as many left; of fewer, as many as are a power of two at a time, their contractions
+  // shared (nine tiles on 16 CTAs: eight on two CTAs each, then one on all, 9 / 16 of the time of one tile instead of all of it)
+  for (int done = 0; done < tiles;) {
+    const int left = tiles - done, n = left >= q.cs ? q.cs : 1 << (31 - __clz(left)), sp = q.cs / n;
+    const int tile = done + q.rank / sp, split = q.rank % sp;
+    const int i0 = (tile / ntt) * 64, c0 = (tile % ntt) * 64, I = min(64, wp - i0), J = min(64, wt - c0);
+    const int kc = ((int)((q.k + sp - 1) / sp) + kKs - 1) / kKs * kKs, k0 = min((int)q.k, split * kc), kn = min(kc, (int)q.k - k0);
+    clear(acc);
+    mm64<VEC, true, false, false>(acc, q.A + (int64_t)k0 * q.k + jp + i0, q.k, I, q.A + (int64_t)k0 * q.k + jt + c0, q.k, J, kn);
+    if (sp == 1) {
       each_entry(acc, I, J, [&](int i, int j, double v) { C[(int64_t)(i0 + i) * wt + c0 + j] = v; });
-    }
-    cluster_sync();
-  } else {
-    const int tile = q.rank / sp, split = q.rank % sp;
-    int i0 = 0, c0 = 0, I = 0, J = 0;
-    if (tile < tiles) {
-      tile_pos(tile, &i0, &c0, &I, &J);
-      const int kc = ((int)((q.k + sp - 1) / sp) + kKs - 1) / kKs * kKs, k0 = min((int)q.k, split * kc);
-      const int kn = min(kc, (int)q.k - k0);
-      clear(acc);
-      mm64<VEC, true, false, false>(acc, q.A + (int64_t)k0 * q.k + jp + i0, q.k, I, q.A + (int64_t)k0 * q.k + jt + c0, q.k, J, kn);
+    } else {
       each_entry(acc, 64, 64, [&](int i, int j, double v) { sm[oPart + i * kLdP + j] = v; });
-    }
-    cluster_sync();
-    if (tile < tiles) {
+      cluster_sync();
       for (int e = split * kT + t; e < 64 * 64; e += sp * kT) {
         const int i = e >> 6, j = e & 63;
         double s = 0.0;
-        for (int z = 0; z < sp; ++z) s += cg::this_cluster().map_shared_rank(sm + oPart, tile * sp + z)[i * kLdP + j];
+#pragma unroll 4
+        for (int z = 0; z < sp; ++z) s += cg::this_cluster().map_shared_rank(sm + oPart, q.rank - split + z)[i * kLdP + j];
         if (i < I && j < J) C[(int64_t)(i0 + i) * wt + c0 + j] = s;
       }
+      if (done + n < tiles) cluster_sync();             // before the partial sums are overwritten
     }
-    cluster_sync();
+    done += n;
   }
+  cluster_sync();
   for (int r = q.r0; r < q.r1; r += 64)
     for (int c0 = 0; c0 < wt; c0 += 64) {
       const int I = min(64, q.r1 - r), J = min(64, wt - c0);
@@ -532,21 +554,27 @@ __device__ __forceinline__ void panel64(const Ctx& q, int j0, int bw, bool first
       for (int e = 0; e < 16; e += 2)
         *reinterpret_cast<double2*>(sm + oPart + (row + 8 * (e >> 3)) * kLdP + col + 8 * ((e >> 1) & 3)) = make_double2(acc[e], acc[e + 1]);
     }
+    // the summed matrix at oZ of every CTA: its upper block triangle, the identity beyond the panel, zero elsewhere
+    auto entry = [&](int i, int j, double v) { return max(i, j) >= bw ? (i == j ? 1.0 : 0.0) : j >= (i & ~7) ? v : 0.0; };
     if (q.cs > 1) {
       cluster_sync();
       const int rs = 64 / q.cs;
       for (int e = t; e < rs * 64; e += kT) {
         const int i = q.rank * rs + (e >> 6), j = e & 63;
         double s = 0.0;
-        if (j >= (i & ~7))
-          for (int z = 0; z < q.cs; ++z) s += cg::this_cluster().map_shared_rank(sm + oPart, z)[i * kLdP + j];
-        sm[oSred + e] = s;
+#pragma unroll 8
+        for (int z = 0; z < q.cs; ++z) s += cg::this_cluster().map_shared_rank(sm + oPart, z)[i * kLdP + j];
+        s = entry(i, j, s);
+#pragma unroll 8
+        for (int z = 0; z < q.cs; ++z) cg::this_cluster().map_shared_rank(sm + oZ, z)[i * kLdK + j] = s;
       }
       cluster_sync();
     } else {
       __syncthreads();
+      for (int e = t; e < 64 * 64; e += kT) sm[oZ + (e >> 6) * kLdK + (e & 63)] = entry(e >> 6, e & 63, sm[oPart + (e >> 6) * kLdP + (e & 63)]);
+      __syncthreads();
     }
-    chol64(q, bw);
+    chol64(bw);
     // what the pivots say: pivot / Gram diagonal is the squared sine of the angle between a column and the
     // span of the panel's columns before it
     bool low = false, ill = false, bad = false, cl = false;

@@ -115,6 +115,14 @@ struct br_handle {
     std::map<int64_t, QrGraph> qr_graphs;
     int* cond = nullptr;                  // conditioning note of the lane's current job (device)
   };
+  // S = 2nd bases of one-launch orders need no lane: all of them are refreshed by one grouped product and one grouped
+  // factorisation (as many at a time as the pool has room for), so that a cluster that is done makes room for the next
+  // basis.  (Dealt to eight lanes ahead of time, the 32 bases of four d = 384 blocks took 10.0 ms, 9.1 now: clusters that
+  // share their SMs with another run half as long again, so no estimate of the lanes' loads was right.)
+  char* pool = nullptr;
+  size_t pool_bytes = 0;
+  struct Side { cudaStream_t stream = nullptr; cudaEvent_t done = nullptr; };
+  Side group_side[2];                     // beside the handle's stream (created when there is a pool)
   bool use_graphs = true;                 // cleared when a capture fails (BR_REFRESH_GRAPHS=0 switches it off)
   // Eight streams in all, the default number of hardware queues.  When the largest order is one that a single
   // cluster factorises, every lane holds it: a cluster leaves 132 SMs to the others (ten steps and the 32 bases of a d = 384 decoder:
@@ -195,11 +203,19 @@ inline int64_t z_slice(int64_t k, int64_t other) {
   return std::min(std::min(rows, other), ((other + slices - 1) / slices + 63) / 64 * 64);      // (whole tiles)
 }
 
+constexpr size_t kPoolOfLargest = 12, kPoolCompact = 3;
+constexpr int64_t kSmallGroup = 128;
+// A side whose refresh is part of the grouped launches, and what it needs of the pool.
+inline bool grouped_side(const Layer& L, int64_t k) { return L.d.src == BR_SRC_SECOND && qr_one_launch(k); }
+inline size_t pool_need(int64_t k) {
+  return align_up(sizeof(double) * (size_t)k * (size_t)k) + align_up(sizeof(double) * orth_work_doubles(k));
+}
+
 // Lays out every buffer of the handle in one slab.  With base == nullptr only sizes are computed.
 void layout(br_handle* h, Bump& b, Sizes* sz) {
   const br_hparams& hp = h->hp;
   if (hp.flags & BR_FLAG_DEBUG_CANARY) { b.guard = kAlign; b.guards = &h->guard_offsets; h->guard_offsets.clear(); }
-  size_t simt_max = 0, simt_total = 0, max_k = 0, max_z = 0, n_sides = 0;
+  size_t simt_max = 0, simt_total = 0, max_k = 0, max_z = 0, n_sides = 0, pool_sum = 0, pool_max = 0;
   for (Layer& L : h->layers) {
     const size_t mn = (size_t)L.d.m * L.d.n;
     L.M = b.take<float>(mn);
@@ -223,8 +239,11 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
     }
     if (L.d.geom != BR_GEOM_NONE) {
       if (!L.use_tc) { simt_max = std::max(simt_max, simt_need(L)); simt_total += simt_need(L); }
-      if (L.left) { max_k = std::max(max_k, (size_t)L.d.m); ++n_sides; }
-      if (L.right) { max_k = std::max(max_k, (size_t)L.d.n); ++n_sides; }
+      for (int64_t k : {L.left ? L.d.m : (int64_t)0, L.right ? L.d.n : (int64_t)0}) {
+        if (!k) continue;
+        if (grouped_side(L, k)) { pool_sum += pool_need(k); pool_max = std::max(pool_max, pool_need(k)); }
+        else { max_k = std::max(max_k, (size_t)k); ++n_sides; }
+      }
       if (!second)
         for (int64_t k : {L.left ? L.d.m : (int64_t)0, L.right ? L.d.n : (int64_t)0})
           if (k) max_z = std::max(max_z, (size_t)(k * z_slice(k, L.d.m * L.d.n / k)));
@@ -234,6 +253,10 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
     h->simt_floats = h->compact ? simt_max : std::max(simt_max, std::min(simt_total, kSimtScratch));
     h->simt_scratch = b.take<float>(h->simt_floats);
   }
+  // the pool: every grouped basis at once, up to twelve of the largest (three in the compact layout)
+  h->pool_bytes = std::min(pool_sum, (h->compact ? kPoolCompact : kPoolOfLargest) * pool_max);
+  if (h->pool_bytes) h->pool = b.take<char>(h->pool_bytes);
+  h->n_lanes = 1;
   h->tcq_bytes = 0;
   for (const Layer& L : h->layers) {
     if (!L.use_tc) continue;
@@ -257,7 +280,7 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
     for (const Layer& L : h->layers) {
       if (L.d.geom == BR_GEOM_NONE) continue;
       for (size_t k : {L.left ? (size_t)L.d.m : (size_t)0, L.right ? (size_t)L.d.n : (size_t)0}) {
-        if (!k) continue;
+        if (!k || grouped_side(L, (int64_t)k)) continue;
         orders.push_back(k);
         if (L.d.src == BR_SRC_SECOND && 2 * k * k <= max_k * max_k) { small_k = std::max(small_k, k); ++n_small_sides; }
       }
@@ -447,7 +470,7 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
   QrTc* tcq = nullptr;
   if (L.use_tc && (h->cond_known[ci] & 1) && !complete)
     for (QrTc* t : ln.tcq) if (qr_tc_order(t) == k) tcq = t;
-  const bool one = qr_one_launch(k);      // a small order is factorised in one launch of one cluster
+  const bool one = qr_one_launch(k);      // a small order (S = 1st here) is factorised in one launch of one cluster
   const float* F = left_side ? L.L : L.R;
   for (int it = 0; it < h->hp.power_iters; ++it) {
     if (!one) { BR_CUDA(h, f32_to_f64(Q, ln.rQ, k * k, s)); count(h); }       // the current basis, for the product and its completion
@@ -458,9 +481,6 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
         count(h);
         br_status st = deflated_power(h, ln, tcq, k, s);
         if (st != BR_OK) return st;
-      } else if (one) {
-        BR_CUDA(h, sdgemm(0, k, k, k, 1.0, F, k, Q, k, 0.0, ln.rA, k, s));
-        count(h); h->stats.gemm_flops += 2.0 * k * k * k;
       } else {
         BR_CUDA(h, f32_to_f64(F, ln.rF, k * k, s));
         BR_CUDA(h, dgemm(0, 0, k, k, k, 1.0, ln.rF, k, ln.rQ, k, 0.0, ln.rA, k, s));
@@ -483,7 +503,7 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
     // has accumulated a gradients has rank <= a * (the other dimension).  The directions outside the
     // range of F Q are then completed from the current basis: what is orthonormalised is F Q with
     // 1e-6 ||(F Q)_j|| Q_j added to every column j (full rank whenever Q is).
-    if (complete) {
+    if (complete && !one) {
       BR_CUDA(h, qr_complete_columns(ln.rA, Q, k, ln.rWork, h->d_status, s));
       count(h, 3);
     }
@@ -492,8 +512,11 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
     // product, for which it needs the product once more (the factor's buffer is free by now) and the
     // current basis.
     if (one) {
-      BR_CUDA(h, orth_whole(ln.rA, k, ln.rWork, ln.rF, Q, Q, left_side ? L.Uh : L.Vh, left_side ? L.Ul : L.Vl,
-                            h->d_status, h->d_cond + ci, s));
+      OrthJob job = {};
+      job.A = ln.rA; job.k = k; job.Acopy = ln.rF; job.Qprev = Q; job.complete = complete ? 1 : 0;
+      job.Qout = Q; job.Qh = left_side ? L.Uh : L.Vh; job.Ql = left_side ? L.Ul : L.Vl; job.cond_out = h->d_cond + ci;
+      orth_job_work(&job, ln.rWork);
+      BR_CUDA(h, orth_group(&job, 1, h->d_status, s));
       count(h); h->stats.gemm_flops += 2.0 * k * k * k;
       continue;
     }
@@ -512,11 +535,49 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
   return BR_OK;
 }
 
-// Refresh the bases of the given layers: every (layer, side) is an independent job; jobs are
-// dealt to the lanes largest first, each to the lane with the least work so far.
+struct GroupSide { int layer; bool left; int64_t k; };
+
+// The grouped refreshes `v` (longest first) on one stream, as many at a time as `bytes` of the pool hold.
+br_status refresh_group(br_handle* h, const GroupSide* v, int n, char* pool, size_t bytes, cudaStream_t s) {
+  std::vector<OrthJob> jobs;
+  for (int first = 0; first < n; first += (int)jobs.size()) {
+    jobs.clear();
+    size_t need = 0, used = 0;
+    int end = first;
+    for (; end < n && need + pool_need(v[end].k) <= bytes; ++end) need += pool_need(v[end].k);
+    for (int i = first; i < end; ++i) {
+      Layer& L = h->layers[v[i].layer];
+      const bool left = v[i].left;
+      const int64_t k = v[i].k, other = left ? L.d.n : L.d.m;
+      OrthJob j = {};
+      j.A = reinterpret_cast<double*>(pool + used); j.k = k;
+      used += align_up(sizeof(double) * (size_t)k * (size_t)k);
+      j.F = left ? L.L : L.R; j.Qprev = j.Qout = left ? L.U : L.V;
+      j.Qh = left ? L.Uh : L.Vh; j.Ql = left ? L.Ul : L.Vl;
+      j.cond_out = h->d_cond + 2 * v[i].layer + (left ? 0 : 1);
+      j.complete = L.n_accum < (k + other - 1) / other;        // (see refresh_side)
+      jobs.push_back(j);
+    }
+    for (OrthJob& j : jobs) {
+      orth_job_work(&j, reinterpret_cast<double*>(pool + used));
+      used += align_up(sizeof(double) * orth_work_doubles(j.k));
+    }
+    for (int it = 0; it < h->hp.power_iters; ++it) {
+      BR_CUDA(h, product_group(jobs.data(), (int)jobs.size(), s));
+      BR_CUDA(h, orth_group(jobs.data(), (int)jobs.size(), h->d_status, s));
+      count(h, 2 * (((int)jobs.size() + kOrthGroup - 1) / kOrthGroup));
+      for (const OrthJob& j : jobs) h->stats.gemm_flops += 4.0 * j.k * j.k * j.k;
+    }
+  }
+  return BR_OK;
+}
+
+// Refresh the bases of the given layers: every (layer, side) is an independent job.  Those that grouped_side() names are
+// refreshed together; the others are dealt to the lanes largest first, each to the lane with the least work so far.
 br_status refresh_layers(br_handle* h, const int* ids, int n_ids) {
   struct Job { int layer; bool left; double cost; int64_t k; bool needs_z; };
   std::vector<Job> jobs;
+  std::vector<GroupSide> grouped;
   // time of one job when it runs alone (ms, measured: on one cluster 0.29 at order 384, 1.4 at 1024, 4.2 at 1536; the
   // chain 2.8 at 1792, 3.9 at 2048, 5.8 at 2560, 13 at 4096, 36 at 6912 with the products of a tracking basis on the tensor
   // cores): a cubic term for the products and a linear one for the chain of panel factorisations
@@ -526,15 +587,20 @@ br_status refresh_layers(br_handle* h, const int* ids, int n_ids) {
   for (int j = 0; j < n_ids; ++j) {
     const Layer& L = h->layers[ids[j]];
     const bool z = L.d.src != BR_SRC_SECOND;
-    if (L.left) jobs.push_back({ids[j], true, cost((double)L.d.m), L.d.m, z});
-    if (L.right) jobs.push_back({ids[j], false, cost((double)L.d.n), L.d.n, z});
+    for (const bool left : {true, false}) {
+      const int64_t k = left ? L.d.m : L.d.n;
+      if (!(left ? L.left : L.right)) continue;
+      if (grouped_side(L, k)) grouped.push_back({ids[j], left, k});
+      else jobs.push_back({ids[j], left, cost((double)k), k, z});
+    }
   }
-  if (jobs.empty()) return BR_OK;
-  for (int j = 0; j < n_ids; ++j) {
-    Layer& L = h->layers[ids[j]];
-    if (!L.lower_stale) continue;
+  if (jobs.empty() && grouped.empty()) return BR_OK;
+  std::vector<Layer*> stale;
+  for (int j = 0; j < n_ids; ++j)
+    if (h->layers[ids[j]].lower_stale) stale.push_back(&h->layers[ids[j]]);
+  if (!stale.empty()) {
     cudaError_t e;
-    const int n = h->stats.inject() ? (e = cudaErrorLaunchFailure, -1) : complete_factors(L, h->stream, &e);
+    const int n = h->stats.inject() ? (e = cudaErrorLaunchFailure, -1) : complete_factors(stale.data(), (int)stale.size(), h->stream, &e);
     if (n < 0) { h->err = format("completing the factors failed: %s", cudaGetErrorString(e)); return BR_ERR_CUDA; }
     count(h, n);
   }
@@ -559,16 +625,38 @@ br_status refresh_layers(br_handle* h, const int* ids, int n_ids) {
     per_lane[best].push_back(jb);
     load[best] += jb.cost;
   }
+  // The grouped launches: orders that need fewer CTAs (one, up to order 32; up to four, beside orders above kSmallGroup) by
+  // themselves when the pool holds all of them; on the handle's own stream where that is free.
+  std::stable_sort(grouped.begin(), grouped.end(), [](const GroupSide& a, const GroupSide& b) { return a.k > b.k; });
+  size_t need = 0, need_large = 0;
+  int n_large = 0;
+  const int64_t line = !grouped.empty() && grouped.front().k > kSmallGroup ? kSmallGroup : 32;
+  for (const GroupSide& g : grouped) {
+    need += pool_need(g.k);
+    if (g.k > line) { need_large += pool_need(g.k); ++n_large; }
+  }
+  const int n_grouped = (int)grouped.size();
+  const bool apart = n_large > 0 && n_large < n_grouped && need <= h->pool_bytes;
+  struct Batch { int first, n; char* pool; size_t bytes; br_handle::Side* side; };
+  std::vector<Batch> batches;
+  if (n_grouped) {
+    const size_t small = apart ? need - need_large : 0;
+    batches.push_back({0, apart ? n_large : n_grouped, h->pool + small, h->pool_bytes - small, jobs.empty() ? nullptr : &h->group_side[0]});
+    if (apart) batches.push_back({n_large, n_grouped - n_large, h->pool, small, &h->group_side[1]});
+  }
   const double f0 = h->stats.gemm_flops;
   const int span = h->stats.prof.begin(PROF_REFRESH, h->stream);
-  if (nl > 1) {
-    BR_CUDA(h, cudaEventRecord(h->ev_begin, h->stream));
+  if (!jobs.empty() || apart) BR_CUDA(h, cudaEventRecord(h->ev_begin, h->stream));
+  if (!jobs.empty())
     for (int i = 1; i < nl; ++i) BR_CUDA(h, cudaStreamWaitEvent(h->lanes[i].stream, h->ev_begin, 0));
-  }
+  for (const Batch& bt : batches)
+    if (bt.side) BR_CUDA(h, cudaStreamWaitEvent(bt.side->stream, h->ev_begin, 0));
   // interleave the enqueueing so that every lane has work early
   size_t longest = 0;
   for (auto& v : per_lane) longest = std::max(longest, v.size());
   br_status failed = BR_OK;
+  for (const Batch& bt : batches)
+    if (failed == BR_OK) failed = refresh_group(h, grouped.data() + bt.first, bt.n, bt.pool, bt.bytes, bt.side ? bt.side->stream : h->stream);
   for (size_t r = 0; r < longest && failed == BR_OK; ++r)
     for (int i = 0; i < nl && failed == BR_OK; ++i) {
       if (r >= per_lane[i].size()) continue;
@@ -577,17 +665,20 @@ br_status refresh_layers(br_handle* h, const int* ids, int n_ids) {
     }
   // the lanes forked from the handle's stream: join them again whatever happened above, so that
   // nothing of this call is still running on an internal stream once the handle's stream has passed it
-  for (int i = 1; i < nl; ++i) {
-    cudaError_t je = h->stats.inject() ? cudaErrorLaunchFailure : cudaEventRecord(h->lanes[i].done, h->lanes[i].stream);
-    if (je == cudaSuccess) je = h->stats.inject() ? cudaErrorLaunchFailure : cudaStreamWaitEvent(h->stream, h->lanes[i].done, 0);
-    if (je != cudaSuccess) {
-      cudaStreamSynchronize(h->lanes[i].stream);       // no event to wait for: wait here
-      if (failed == BR_OK) {
-        h->err = format("joining a refresh lane failed: %s", cudaGetErrorString(je));
-        failed = BR_ERR_CUDA;
-      }
+  auto join = [&](cudaStream_t side, cudaEvent_t done) {
+    cudaError_t je = h->stats.inject() ? cudaErrorLaunchFailure : cudaEventRecord(done, side);
+    if (je == cudaSuccess) je = h->stats.inject() ? cudaErrorLaunchFailure : cudaStreamWaitEvent(h->stream, done, 0);
+    if (je == cudaSuccess) return;
+    cudaStreamSynchronize(side);                       // no event to wait for: wait here
+    if (failed == BR_OK) {
+      h->err = format("joining a refresh lane failed: %s", cudaGetErrorString(je));
+      failed = BR_ERR_CUDA;
     }
-  }
+  };
+  if (!jobs.empty())
+    for (int i = 1; i < nl; ++i) join(h->lanes[i].stream, h->lanes[i].done);
+  for (const Batch& bt : batches)
+    if (bt.side) join(bt.side->stream, bt.side->done);
   if (failed != BR_OK) return failed;
   h->stats.prof.end(span, h->stream, h->stats.gemm_flops - f0);
   BR_CUDA(h, cudaMemcpyAsync(h->h_cond, h->d_cond, sizeof(int) * h->cond_known.size(), cudaMemcpyDeviceToHost, h->stream));
@@ -775,6 +866,10 @@ void release(br_handle* h) {
     if (h->lanes[i].stream) { cudaStreamSynchronize(h->lanes[i].stream); cudaStreamDestroy(h->lanes[i].stream); }
     if (h->lanes[i].done) cudaEventDestroy(h->lanes[i].done);
   }
+  for (br_handle::Side& g : h->group_side) {
+    if (g.stream) { cudaStreamSynchronize(g.stream); cudaStreamDestroy(g.stream); }
+    if (g.done) cudaEventDestroy(g.done);
+  }
   if (h->ev_begin) cudaEventDestroy(h->ev_begin);
   if (h->ev_cond) cudaEventDestroy(h->ev_cond);
   if (h->copy_stream) { cudaStreamSynchronize(h->copy_stream); cudaStreamDestroy(h->copy_stream); }
@@ -904,6 +999,11 @@ br_status br_create(br_handle** out, const br_layer_desc* layers, int n_layers, 
   for (int i = 1; i < h->n_lanes; ++i) {
     if ((e = cudaStreamCreateWithFlags(&h->lanes[i].stream, cudaStreamNonBlocking)) != cudaSuccess) return fail("cudaStreamCreate", e);
     if ((e = cudaEventCreateWithFlags(&h->lanes[i].done, cudaEventDisableTiming)) != cudaSuccess) return fail("cudaEventCreate", e);
+  }
+  for (br_handle::Side& g : h->group_side) {
+    if (!h->pool) break;
+    if ((e = cudaStreamCreateWithFlags(&g.stream, cudaStreamNonBlocking)) != cudaSuccess) return fail("cudaStreamCreate", e);
+    if ((e = cudaEventCreateWithFlags(&g.done, cudaEventDisableTiming)) != cudaSuccess) return fail("cudaEventCreate", e);
   }
   if ((e = cudaEventCreateWithFlags(&h->ev_begin, cudaEventDisableTiming)) != cudaSuccess) return fail("cudaEventCreate", e);
   // The side stream of a step has the highest priority: the CTAs of a launch that waits for SMs behind a running one (the
@@ -1295,7 +1395,8 @@ br_status br_get_state(br_handle* h, int layer, int which, void* host_dst, size_
   if (bytes != want) { h->err = format("buffer is %zu bytes, caller passed %zu", want, bytes); return BR_ERR_SHAPE; }
   if (which == BR_BUF_L || which == BR_BUF_R) {
     cudaError_t e;
-    const int n = complete_factors(h->layers[layer], h->stream, &e);
+    Layer* one = &h->layers[layer];
+    const int n = complete_factors(&one, 1, h->stream, &e);
     if (n < 0) { h->err = format("completing the factors failed: %s", cudaGetErrorString(e)); return BR_ERR_CUDA; }
     count(h, n);
   }
@@ -1339,7 +1440,8 @@ br_status br_set_state(br_handle* h, int layer, int which, const void* host_src,
   if (bytes != want) { h->err = format("buffer is %zu bytes, caller passed %zu", want, bytes); return BR_ERR_SHAPE; }
   if (which == BR_BUF_L || which == BR_BUF_R) {        // (the other factor of the layer is completed; this one is replaced whole)
     cudaError_t e;
-    const int n = complete_factors(L, h->stream, &e);
+    Layer* one = &L;
+    const int n = complete_factors(&one, 1, h->stream, &e);
     if (n < 0) { h->err = format("completing the factors failed: %s", cudaGetErrorString(e)); return BR_ERR_CUDA; }
     count(h, n);
   }

@@ -104,10 +104,15 @@ constexpr int kElemGroup = 64;
 struct CopyJob { const void* src; void* dst; size_t bytes; };
 cudaError_t ring_copy(const CopyJob* jobs, int n, bool beside, cudaStream_t s);
 // F[j][i] <- F[i][j] for the 32 x 32 blocks (j, i) strictly below the diagonal of the k x k matrix F.
-cudaError_t mirror_lower(float* F, int64_t k, cudaStream_t s);
+struct MirrorJob { float* F; int64_t k; };
+cudaError_t mirror_lower(const MirrorJob* jobs, int n, cudaStream_t s);
 // fp32 -> bf16 hi (+ optional lo = bf16(x - hi)).
-cudaError_t split_bf16(const float* X, __nv_bfloat16* hi, __nv_bfloat16* lo, int64_t numel,
-                       cudaStream_t s);
+struct SplitJob { const float* X; __nv_bfloat16 *hi, *lo; int64_t numel; };
+cudaError_t split_bf16(const SplitJob* jobs, int n, cudaStream_t s);
+inline cudaError_t split_bf16(const float* X, __nv_bfloat16* hi, __nv_bfloat16* lo, int64_t numel, cudaStream_t s) {
+  const SplitJob j = {X, hi, lo, numel};
+  return split_bf16(&j, 1, s);
+}
 cudaError_t widen_bf16(const __nv_bfloat16* X, float* out, int64_t numel, cudaStream_t s);
 // out(double) <- in(float) ; out(float) <- in(double)
 cudaError_t f64_to_f32(const double* X, float* out, int64_t numel, cudaStream_t s);
@@ -192,12 +197,25 @@ constexpr double kOrthIllRatio = 1e-7;
 constexpr double kOrthTcRatio = 1e-6;      // the same, when the projections ran on the tensor cores; also
                                            // the ratio below which the next refresh must not use them
 constexpr double kOrthCompletion = 1e-6;   // a deficient column j is completed by this times its length times Q_j
-// The whole factorisation of a k x k product A (overwritten) in one launch.  Acopy / Qprev (both or none): as
-// for qr_pos_inplace, the copy is made here.  Results: Qout (fp32) and, optionally, its bf16 hi/lo pair; *cond_out as for qr_pos_inplace with
-// bit 1 set when the product was numerically rank-deficient.  work: orth_work_doubles(k).
+// Whole factorisations of k x k products (overwritten), one cluster each.  Results: Qout (fp32) and, optionally, its bf16
+// hi/lo pair; *cond_out (or null): bit 0 as for qr_pos_inplace, bit 1 set when the product was numerically
+// rank-deficient.  Such a product is factorised again, completed from Qprev, if Qprev is given and either Acopy (room for
+// a copy of A) or F (the product is formed again as F Qprev); complete: the product is known to be short of rank and is
+// completed before it is factorised.  Qprev may be Qout.
+struct OrthJob {
+  double* A; int64_t k;
+  double *C, *normp, *rdiag;          // work area, laid out by orth_job_work
+  double* Acopy; const float *F, *Qprev;
+  float* Qout; __nv_bfloat16 *Qh, *Ql;
+  int* cond_out;
+  int complete;
+};
+constexpr int kOrthGroup = 32;        // jobs of one launch at most (by value: 3.4 KB of launch parameters)
 size_t orth_work_doubles(int64_t k);
-cudaError_t orth_whole(double* A, int64_t k, double* work, double* Acopy, const float* Qprev,
-                       float* Qout, __nv_bfloat16* Qh, __nv_bfloat16* Ql, int* status, int* cond_out, cudaStream_t s);
+void orth_job_work(OrthJob* j, double* work);
+cudaError_t orth_group(const OrthJob* jobs, int n, int* status, cudaStream_t s);
+// A <- F Qprev of every job (fp32 operands, fp64 sums)
+cudaError_t product_group(const OrthJob* jobs, int n, cudaStream_t s);
 // Columns [j0, j0 + w) only, as a part of one sweep of qr_pos_inplace (whose flag words `flags` are).
 // C: room for the largest coefficient block, (w / 2)^2 doubles.
 cudaError_t orth_part(double* A, int64_t k, int64_t j0, int64_t w, double* C, int first, double ill_ratio, const double* norm0,
@@ -218,7 +236,7 @@ cudaError_t product64(int ta, int64_t M, int64_t N, int64_t K, double alpha, con
 // BR_WARN_RANK_DEFICIENT when a pivot underflows.  Returns the number of launches in *launches.
 // ---------------------------------------------------------------------------------------------
 size_t qr_work_doubles(int64_t k);
-// Orders whose whole factorisation is one launch (orth_whole); the others go through qr_pos_inplace.
+// Orders whose whole factorisation is one launch (orth_group); the others go through qr_pos_inplace.
 bool qr_one_launch(int64_t k);
 // Optional tensor-core form of the block projections (see qr.cu): plans and scratch for one order
 // k, created once.  qr_tc_scratch_bytes is 0 when the order is not eligible.

@@ -151,9 +151,14 @@ k_plain_adam(float* __restrict__ W, float* __restrict__ M, float* __restrict__ V
 
 // One 32 x 32 block pair per CTA of 32 x 8 threads, through a padded shared-memory tile.  Blocks are numbered along
 // the columns of the strict upper block triangle (block b of column c, b < c, is number c (c - 1) / 2 + b).  Bound by memory, 8 bytes per pair of entries.
-__global__ void __launch_bounds__(256) k_mirror_lower(float* __restrict__ F, int64_t k) {
+struct MirrorArgs { float* F[kElemGroup]; int k[kElemGroup], begin[kElemGroup + 1], n; };
+__global__ void __launch_bounds__(256) k_mirror_lower(const __grid_constant__ MirrorArgs a) {
   __shared__ float tile[32][33];
-  const int id = (int)blockIdx.x;
+  int job = 0;
+  while (job + 1 < a.n && a.begin[job + 1] <= (int)blockIdx.x) ++job;
+  float* const F = a.F[job];
+  const int64_t k = a.k[job];
+  const int id = (int)blockIdx.x - a.begin[job];
   int c = (int)((sqrtf(8.0f * (float)id + 1.0f) + 1.0f) * 0.5f);
   while (c * (c - 1) / 2 > id) --c;
   while (c * (c + 1) / 2 <= id) ++c;
@@ -169,20 +174,24 @@ __global__ void __launch_bounds__(256) k_mirror_lower(float* __restrict__ F, int
     if (c0 + i < k) F[(c0 + i) * k + r0 + tx] = tile[tx][i];
 }
 
+struct SplitArgs { SplitJob j[kElemGroup]; int begin[kElemGroup + 1], n; };
 __global__ void __launch_bounds__(kThreads)
-k_split_bf16(const float* __restrict__ X, __nv_bfloat16* __restrict__ hi,
-             __nv_bfloat16* __restrict__ lo, int64_t numel) {
+k_split_bf16(const __grid_constant__ SplitArgs a) {
+  int job = 0;
+  while (job + 1 < a.n && a.begin[job + 1] <= (int)blockIdx.x) ++job;
+  const float* const X = a.j[job].X;
+  __nv_bfloat16 *const hi = a.j[job].hi, *const lo = a.j[job].lo;
+  const int64_t numel = a.j[job].numel, block = (int)blockIdx.x - a.begin[job];
   const int64_t nvec = numel >> 2;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nvec; v += stride) {
+  const int64_t stride = (int64_t)(a.begin[job + 1] - a.begin[job]) * blockDim.x;
+  for (int64_t v = block * blockDim.x + threadIdx.x; v < nvec; v += stride) {
     const int64_t i = v << 2;
     float4 x = ld4(X + i);
     float4 h = make_float4(bf16_round(x.x), bf16_round(x.y), bf16_round(x.z), bf16_round(x.w));
     st4_bf16(hi + i, h);
     if (lo) st4_bf16(lo + i, make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w));
   }
-  for (int64_t i = (nvec << 2) + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < numel;
-       i += stride) {
+  for (int64_t i = (nvec << 2) + block * blockDim.x + threadIdx.x; i < numel; i += stride) {
     float x = X[i], h = bf16_round(x);
     hi[i] = __float2bfloat16_rn(x);
     if (lo) lo[i] = __float2bfloat16_rn(x - h);
@@ -405,10 +414,18 @@ cudaError_t ring_copy(const CopyJob* jobs, int n, bool beside, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t mirror_lower(float* F, int64_t k, cudaStream_t s) {
-  const int nb = (int)((k + 31) / 32);
-  if (nb < 2) return cudaSuccess;
-  k_mirror_lower<<<(unsigned)((int64_t)nb * (nb - 1) / 2), 256, 0, s>>>(F, k);
+cudaError_t mirror_lower(const MirrorJob* jobs, int n, cudaStream_t s) {
+  for (int first = 0; first < n; first += kElemGroup) {
+    MirrorArgs a;
+    a.n = std::min(kElemGroup, n - first);
+    a.begin[0] = 0;
+    for (int i = 0; i < a.n; ++i) {
+      const int nb = (int)((jobs[first + i].k + 31) / 32);
+      a.F[i] = jobs[first + i].F; a.k[i] = (int)jobs[first + i].k;
+      a.begin[i + 1] = a.begin[i] + nb * (nb - 1) / 2;
+    }
+    if (a.begin[a.n]) k_mirror_lower<<<(unsigned)a.begin[a.n], 256, 0, s>>>(a);
+  }
   return cudaGetLastError();
 }
 
@@ -441,9 +458,17 @@ cudaError_t plain_adam(float* W, float* M, float* V, const void* G, int g_is_bf1
   return cudaGetLastError();
 }
 
-cudaError_t split_bf16(const float* X, __nv_bfloat16* hi, __nv_bfloat16* lo, int64_t numel,
-                       cudaStream_t s) {
-  k_split_bf16<<<grid_for((numel + 3) / 4), kThreads, 0, s>>>(X, hi, lo, numel);
+cudaError_t split_bf16(const SplitJob* jobs, int n, cudaStream_t s) {
+  for (int first = 0; first < n; first += kElemGroup) {
+    SplitArgs a;
+    a.n = std::min(kElemGroup, n - first);
+    a.begin[0] = 0;
+    for (int i = 0; i < a.n; ++i) {
+      a.j[i] = jobs[first + i];
+      a.begin[i + 1] = a.begin[i] + grid_for((a.j[i].numel + 3) / 4);
+    }
+    k_split_bf16<<<(unsigned)a.begin[a.n], kThreads, 0, s>>>(a);
+  }
   return cudaGetLastError();
 }
 

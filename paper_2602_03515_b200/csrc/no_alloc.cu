@@ -71,7 +71,11 @@ extern "C" br_status br_power_static(void* cuda_stream, const float* F, float* Q
   // The array keeps whatever the previous call left.  Only the flag has to start at zero; every
   // other word is written by this call before it is read.
   if (cudaMemsetAsync(flag, 0, sizeof(int), s) != cudaSuccess) return BR_ERR_CUDA;
-  if (sdgemm(0, k, k, k, 1.0, F, k, Q, k, 0.0, A, k, s) != cudaSuccess) return BR_ERR_CUDA;
-  if (orth_whole(A, k, work, nullptr, nullptr, Q, nullptr, nullptr, flag, nullptr, s) != cudaSuccess) return BR_ERR_CUDA;
+  OrthJob job = {};
+  job.A = A; job.k = k; job.F = F; job.Qprev = Q; job.Qout = Q;
+  orth_job_work(&job, work);
+  if (product_group(&job, 1, s) != cudaSuccess) return BR_ERR_CUDA;
+  job.F = nullptr; job.Qprev = nullptr;                  // (a deficient product is reported, not completed)
+  if (orth_group(&job, 1, flag, s) != cudaSuccess) return BR_ERR_CUDA;
   return BR_OK;
 }

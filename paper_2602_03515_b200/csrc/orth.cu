@@ -4,7 +4,7 @@
 // Cholesky-QR) is a chain of hundreds of short dependent steps: Gram matrix, Cholesky factor and its
 // inverse, panel update, projection coefficients, projection.  As launches of their own they cost more
 // in launch gaps than in work: at order 384, 248 launches of which 44 did something, 950 us a basis.
-// Here one cluster of up to 16 CTAs walks the whole chain of a range of columns in one launch, and the
+// Here one cluster of up to 16 CTAs walks the whole chain of a basis, or of a range of its columns, in one launch, and the
 // steps are separated by the cluster's hardware barrier; the second sweep and the completion of a
 // rank-deficient product are branches instead of cancelled launches.  Measured, one basis alone: order 64
 // 32 us, 384 240 us, 1024 1.3 ms, 1536 3.9 ms; stand-alone Power() at order 384 1368 -> 267 us.
@@ -185,53 +185,101 @@ __device__ __forceinline__ void each_entry(double (&acc)[16], int I, int J, FN f
   }
 }
 
-// C = alpha op(X) Y + beta C, X fp32, Y fp32 or fp64, widened while they are staged through registers: one
-// 64 x 64 tile per CTA, for every product of a refresh with an fp32 operand.  A refresh from the momentum (two such
-// products), ms, with tiles of 128 x 128 on one CTA per SM and now: 2048 x 2048 7.8 and 4.2, 4096 x 4096 27.2 and 20.9,
-// 2560 x 6912 16.1 and 11.4, factorisation included.
+// acc += sum over kk < K of x(i, kk) y(kk, j) on one tile, i < I, j < J, with X fp32 and Y fp32 or fp64, widened while
+// they are staged through registers: x(i, kk) = X[kk * lda + i] (TRANS) or X[i * lda + kk], y(kk, j) = Y[kk * ldb + j].
+// Two stages of loads are in flight; the tile ends behind a barrier, so the stages' memory is free again.
+template <bool TRANS, typename TB>
+__device__ __forceinline__ void product_tile(double (&acc)[16], const float* X, int64_t lda, int I, const TB* Y, int64_t ldb, int J, int K) {
+  const int t = threadIdx.x;
+  float ra[2][4];
+  TB rb[2][4];
+  auto load = [&](int k0, float (&a)[4], TB (&b)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = TRANS ? (t & 63) : (t >> 4) + 16 * q, ka = k0 + (TRANS ? (t >> 6) + 4 * q : (t & 15));
+      const int j = t & 63, kb = k0 + (t >> 6) + 4 * q;
+      a[q] = (i < I && ka < K) ? X[TRANS ? (int64_t)ka * lda + i : (int64_t)i * lda + ka] : 0.f;
+      b[q] = (j < J && kb < K) ? Y[(int64_t)kb * ldb + j] : (TB)0;
+    }
+  };
+  auto store = [&](int buf, const float (&a)[4], const TB (&b)[4]) {
+    double* As = sm + oStage + buf * (kOper + kOperB);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      As[TRANS ? ((t >> 6) + 4 * q) * kLdK + (t & 63) : ((t >> 4) + 16 * q) * kLdI + (t & 15)] = (double)a[q];
+      As[kOper + ((t >> 6) + 4 * q) * kLdK + (t & 63)] = (double)b[q];
+    }
+  };
+  const int nk = (K + kKs - 1) / kKs;
+  load(0, ra[0], rb[0]);
+  load(kKs, ra[1], rb[1]);
+  store(0, ra[0], rb[0]);
+  __syncthreads();
+  for (int s = 0; s < nk; s += 2) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      if (u && s + 1 >= nk) break;
+      load((s + u + 2) * kKs, ra[u], rb[u]);
+      const double* st = sm + oStage + u * (kOper + kOperB);
+      mma_stage<TRANS, false, false>(acc, st, st + kOper, I);
+      store(1 - u, ra[1 - u], rb[1 - u]);
+      __syncthreads();
+    }
+  }
+}
+constexpr int kProductSmem = 2 * (kOper + kOperB) * (int)sizeof(double);
+
+// C = alpha op(X) Y + beta C: one 64 x 64 tile per CTA, for the products of a refresh with an fp32 operand.  A refresh
+// from the momentum (two such products), ms, with tiles of 128 x 128 on one CTA per SM and with these: 2048 x 2048 7.8 and
+// 4.2, 4096 x 4096 27.2 and 20.9, 2560 x 6912 16.1 and 11.4, factorisation included.
 template <bool TRANS, typename TB>
 __global__ void __launch_bounds__(kT, 2)
 k_product64(int M, int N, int K, double alpha, const float* __restrict__ X, int64_t lda, const TB* __restrict__ Y, int64_t ldb,
             double beta, double* __restrict__ C, int64_t ldc) {
-  const int t = threadIdx.x, m0 = (int)blockIdx.y * 64, n0 = (int)blockIdx.x * 64;
+  const int m0 = (int)blockIdx.y * 64, n0 = (int)blockIdx.x * 64;
   double acc[16];
-  float ra[4];
-  TB rb[4];
   clear(acc);
-  auto load = [&](int k0) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = m0 + (TRANS ? (t & 63) : (t >> 4) + 16 * q), ka = k0 + (TRANS ? (t >> 6) + 4 * q : (t & 15));
-      const int j = n0 + (t & 63), kb = k0 + (t >> 6) + 4 * q;
-      ra[q] = (i < M && ka < K) ? X[TRANS ? (int64_t)ka * lda + i : (int64_t)i * lda + ka] : 0.f;
-      rb[q] = (j < N && kb < K) ? Y[(int64_t)kb * ldb + j] : (TB)0;
-    }
-  };
-  auto store = [&](int buf) {
-    double* As = sm + oStage + buf * (kOper + kOperB);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      As[TRANS ? ((t >> 6) + 4 * q) * kLdK + (t & 63) : ((t >> 4) + 16 * q) * kLdI + (t & 15)] = (double)ra[q];
-      As[kOper + ((t >> 6) + 4 * q) * kLdK + (t & 63)] = (double)rb[q];
-    }
-  };
-  const int nk = (K + kKs - 1) / kKs;
-  load(0);
-  store(0);
-  __syncthreads();
-  for (int s = 0; s < nk; ++s) {
-    if (s + 1 < nk) load((s + 1) * kKs);
-    const double* st = sm + oStage + (s & 1) * (kOper + kOperB);
-    mma_stage<TRANS, false, false>(acc, st, st + kOper, M - m0);
-    if (s + 1 < nk) store((s + 1) & 1);
-    __syncthreads();
-  }
+  product_tile<TRANS>(acc, X + (TRANS ? m0 : (int64_t)m0 * lda), lda, M - m0, Y + n0, ldb, N - n0, K);
   each_entry(acc, M - m0, N - n0, [&](int i, int j, double v) {
     double* c = C + (int64_t)(m0 + i) * ldc + n0 + j;
     v *= alpha;
     *c = beta != 0.0 ? fma(beta, *c, v) : v;
   });
 }
+
+// A = F Q (fp32 in, fp64 out, k x k) for several bases in one launch, one tile per cluster of 1 to 8 CTAs that share its
+// contraction: the partial sums are added through distributed shared memory in the order of the ranges.  One of order 384
+// 15.4 us; 24 us as 36 CTAs with the whole contraction each.
+template <int NJ> struct ProductGroup { const float *F[NJ], *Q[NJ]; double* A[NJ]; int k[NJ], tile0[NJ + 1], n; };
+template <int NJ>
+__global__ void __launch_bounds__(kT, 2) k_product_group(const __grid_constant__ ProductGroup<NJ> g) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int zs = (int)cl.num_blocks(), z = (int)cl.block_rank(), tile = (int)blockIdx.x / zs;
+  int p = 0;
+  while (p + 1 < g.n && g.tile0[p + 1] <= tile) ++p;
+  const int k = g.k[p], nt = (k + 63) / 64, m0 = (tile - g.tile0[p]) / nt * 64, n0 = (tile - g.tile0[p]) % nt * 64;
+  const int kc = ((k + zs - 1) / zs + kKs - 1) / kKs * kKs, k0 = min(k, z * kc), K = min(kc, k - k0);
+  const int I = min(64, k - m0), J = min(64, k - n0);
+  double* const C = g.A[p] + (int64_t)m0 * k + n0;
+  double acc[16];
+  clear(acc);
+  product_tile<false>(acc, g.F[p] + (int64_t)m0 * k + k0, k, I, g.Q[p] + (int64_t)k0 * k + n0, k, J, K);
+  if (zs == 1) {
+    each_entry(acc, I, J, [&](int i, int j, double v) { C[(int64_t)i * k + j] = v; });
+    return;
+  }
+  each_entry(acc, 64, 64, [&](int i, int j, double v) { sm[i * kLdP + j] = v; });
+  cluster_sync();
+  const int rows = 64 / zs;
+  for (int e = threadIdx.x; e < rows * 64; e += kT) {
+    const int i = z * rows + (e >> 6), j = e & 63;
+    double s = 0.0;
+    for (int q = 0; q < zs; ++q) s += cl.map_shared_rank(sm, q)[i * kLdP + j];
+    if (i < I && j < J) C[(int64_t)i * k + j] = s;
+  }
+  cluster_sync();                              // no CTA leaves while another may still read its partial sums
+}
+static_assert(64 * kLdP * (int)sizeof(double) <= kProductSmem, "the partial sums borrow the stages");
 
 // C = alpha op(X) op(Y) + beta C in fp64, one 64 x 64 tile and a range of the contraction per CTA (split over
 // blockIdx.z: partial sums, added by a second kernel).
@@ -271,7 +319,7 @@ template <typename TB>
 cudaError_t launch_product(int ta, int64_t M, int64_t N, int64_t K, double alpha, const float* A, int64_t lda, const TB* B,
                            int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t s) {
   const dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64));
-  const size_t bytes = 2 * (kOper + kOperB) * sizeof(double);
+  const size_t bytes = kProductSmem;
   if (ta)
     k_product64<true, TB><<<grid, kT, bytes, s>>>((int)M, (int)N, (int)K, alpha, A, lda, B, ldb, beta, C, ldc);
   else
@@ -279,18 +327,17 @@ cudaError_t launch_product(int ta, int64_t M, int64_t N, int64_t K, double alpha
   return cudaGetLastError();
 }
 
-struct OrthArgs {
-  double* A; int64_t k;          // k x k, row-major; columns [j0, j0 + w) are orthonormalised
+struct PartArgs {                // columns [j0, j0 + w) of one sweep over the k x k matrix A, row-major
+  double* A; int64_t k;
   int j0, w;
-  int whole;                     // 1: the complete factorisation (both sweeps, rank decision, completion, outputs)
-  int first;                     // part: this is the first sweep (watch the column norms)
-  double ill_ratio;              // part, first: squared-norm ratio below which the second sweep has to run
-  const double* norm0;           // part, first: squared norms of the columns before any projection
-  double *C, *normp, *rdiag;     // projection coefficients; 2 x cluster x k partial norms (whole); squared diagonal of R
-  double* Acopy; const float* Qprev;   // whole: buffer for a second copy of A, and the basis for its completion (both or none)
-  float* Qout; __nv_bfloat16 *Qh, *Ql; // whole: the result in fp32 and as a bf16 pair (optional)
-  int* status; int* flags; int* cond_out; const int* skip;
+  int first;                     // this is the first sweep (watch the column norms)
+  double ill_ratio;              // first: squared-norm ratio below which the second sweep has to run
+  const double* norm0;           // first: squared norms of the columns before any projection
+  double *C, *rdiag;             // projection coefficients; squared diagonal of R
+  int* status; int* flags; const int* skip;
 };
+// The complete factorisations of several products: both sweeps, rank decision, completion, outputs.
+template <int NJ> struct OrthGroup { OrthJob j[NJ]; int* status; };
 
 struct Ctx {
   int64_t k;
@@ -621,31 +668,51 @@ __device__ __forceinline__ SweepNotes sweep64(const Ctx& q, double* C, int j0, i
   return notes;
 }
 
-template <bool VEC>
-__global__ void __launch_bounds__(kT, 2) k_orth_cluster(OrthArgs a) {
-  if (a.skip && *a.skip) return;               // uniform: a device-side flag cancels the whole launch
+__device__ __forceinline__ Ctx context(double* A, int64_t k) {
   Ctx q;
-  q.k = a.k; q.A = a.A;
-  q.cs = (int)gridDim.x; q.rank = (int)blockIdx.x;
-  const int k = (int)a.k, rc = ((k + q.cs - 1) / q.cs + 7) / 8 * 8;
-  q.r0 = min(k, q.rank * rc); q.r1 = min(k, q.r0 + rc);
-  const int t = threadIdx.x;
+  q.k = k; q.A = A;
+  q.cs = (int)cg::this_cluster().num_blocks(); q.rank = (int)cg::this_cluster().block_rank();
+  const int rc = (((int)k + q.cs - 1) / q.cs + 7) / 8 * 8;
+  q.r0 = min((int)k, q.rank * rc); q.r1 = min((int)k, q.r0 + rc);
+  return q;
+}
 
-  if (!a.whole) {
-    const SweepNotes n = sweep64<VEC>(q, a.C, a.j0, a.w, a.first != 0, a.ill_ratio, a.norm0, 1, a.rdiag, false);
-    if (q.rank == 0 && t == 0) {
-      if (n.clamped) { atomicMax(a.status, (int)BR_WARN_RANK_DEFICIENT); a.flags[3] = 1; }
-      if (a.first && n.ill) a.flags[1] = 0;
-      if (a.first && n.tc_bad) a.flags[2] = 0;
-    }
-    cluster_sync();                              // no CTA leaves while another may still read its shared memory
-    return;
+template <bool VEC>
+__global__ void __launch_bounds__(kT, 2) k_orth_part(PartArgs a) {
+  if (a.skip && *a.skip) return;               // uniform: a device-side flag cancels the whole launch
+  const Ctx q = context(a.A, a.k);
+  const SweepNotes n = sweep64<VEC>(q, a.C, a.j0, a.w, a.first != 0, a.ill_ratio, a.norm0, 1, a.rdiag, false);
+  if (q.rank == 0 && threadIdx.x == 0) {
+    if (n.clamped) { atomicMax(a.status, (int)BR_WARN_RANK_DEFICIENT); a.flags[3] = 1; }
+    if (a.first && n.ill) a.flags[1] = 0;
+    if (a.first && n.tc_bad) a.flags[2] = 0;
   }
+  cluster_sync();                              // no CTA leaves while another may still read its shared memory
+}
 
+// own rows of A <- own rows of F Qprev (a deficient product once more, before it is completed)
+__device__ __noinline__ void own_product(const Ctx q, const float* F, const float* Q) {
+  const int k = (int)q.k;
+  for (int r = q.r0; r < q.r1; r += 64)
+    for (int c = 0; c < k; c += 64) {
+      double acc[16];
+      clear(acc);
+      product_tile<false>(acc, F + (int64_t)r * k, k, min(64, q.r1 - r), Q + c, k, min(64, k - c), k);
+      each_entry(acc, min(64, q.r1 - r), min(64, k - c), [&](int i, int j, double v) { q.A[(int64_t)(r + i) * k + c + j] = v; });
+    }
+  __syncthreads();
+}
+
+template <bool VEC>
+__device__ __forceinline__ void orth_whole_cluster(const OrthJob& a, int* status) {
+  const Ctx q = context(a.A, a.k);
+  const int k = (int)a.k, t = threadIdx.x;
   bool clamped = false, tc_bad = false, deficient = false;
-  const bool fix = a.Acopy != nullptr && a.Qprev != nullptr;
+  const bool fix = a.Qprev != nullptr && (a.Acopy != nullptr || a.F != nullptr) && !a.complete;
   for (int attempt = 0; attempt < 2; ++attempt) {
     double* normp = a.normp + (int64_t)attempt * q.cs * k;
+    if (attempt && !a.complete && a.F) own_product(q, a.F, a.Qprev);
+    const double* from = attempt && a.Acopy && !a.complete ? a.Acopy : q.A;
     for (int j = t; j < k; j += kT) {
       double s = 0.0;
       if (!attempt) {
@@ -656,7 +723,7 @@ __global__ void __launch_bounds__(kT, 2) k_orth_cluster(OrthArgs a) {
           for (int u = 0; u < 8; ++u) v[u] = r + u < q.r1 ? __ldcg(q.A + (int64_t)(r + u) * k + j) : 0.0;
 #pragma unroll
           for (int u = 0; u < 8; ++u) {
-            if (fix && r + u < q.r1) a.Acopy[(int64_t)(r + u) * k + j] = v[u];
+            if (fix && a.Acopy && r + u < q.r1) a.Acopy[(int64_t)(r + u) * k + j] = v[u];
             s = fma(v[u], v[u], s);
           }
         }
@@ -667,7 +734,7 @@ __global__ void __launch_bounds__(kT, 2) k_orth_cluster(OrthArgs a) {
         const double d = n2 > 0.0 ? kOrthCompletion * sqrt(n2) : 1.0;
         for (int r = q.r0; r < q.r1; ++r) {
           const int64_t i = (int64_t)r * k + j;
-          const double v = fma(d, (double)a.Qprev[i], __ldcg(a.Acopy + i));
+          const double v = fma(d, (double)a.Qprev[i], __ldcg(from + i));
           q.A[i] = v;
           s = fma(v, v, s);
         }
@@ -675,10 +742,11 @@ __global__ void __launch_bounds__(kT, 2) k_orth_cluster(OrthArgs a) {
       normp[(int64_t)q.rank * k + j] = s;
     }
     cluster_sync();
+    if (a.complete && !attempt) continue;        // known to be short of rank: completed before the first sweep
     double* const rdiag = fix && !attempt ? a.rdiag : nullptr;
     SweepNotes n = sweep64<VEC>(q, a.C, 0, k, true, kOrthIllRatio, normp, q.cs, rdiag, true);
     clamped |= n.clamped;
-    if (!attempt) tc_bad = n.tc_bad;
+    if (!attempt || a.complete) tc_bad = n.tc_bad;
     if (n.ill) {
       n = sweep64<VEC>(q, a.C, 0, k, false, 0.0, nullptr, 0, rdiag, false);
       clamped |= n.clamped;
@@ -722,11 +790,17 @@ __global__ void __launch_bounds__(kT, 2) k_orth_cluster(OrthArgs a) {
     }
   }
   if (q.rank == 0 && t == 0) {
-    if (clamped || deficient) atomicMax(a.status, (int)BR_WARN_RANK_DEFICIENT);
+    if (clamped || deficient || a.complete) atomicMax(status, (int)BR_WARN_RANK_DEFICIENT);
     // bit 0: no column shrank below 1e-3 of its length; bit 1: numerically rank-deficient
     if (a.cond_out) *a.cond_out = (tc_bad ? 0 : 1) | (clamped || deficient ? 2 : 0);
   }
   cluster_sync();
+}
+template <int NJ>
+__global__ void __launch_bounds__(kT, 2) k_orth_group(const __grid_constant__ OrthGroup<NJ> g) {
+  const OrthJob& a = g.j[blockIdx.x / cg::this_cluster().num_blocks()];
+  // 16-byte copies need even dimensions throughout (the buffers start on 256-byte boundaries)
+  if (a.k % 2 == 0) orth_whole_cluster<true>(a, g.status); else orth_whole_cluster<false>(a, g.status);
 }
 
 // Largest cluster the device schedules for this kernel (16 needs the non-portable size), per device.
@@ -738,7 +812,9 @@ int max_cluster() {
   std::lock_guard<std::mutex> lock(mu);
   if (cap[dev]) return cap[dev];
   int best = kMaxCluster;
-  for (auto kernel : {k_orth_cluster<false>, k_orth_cluster<true>}) {
+  const void* const kernels[] = {(const void*)k_orth_part<false>, (const void*)k_orth_part<true>, (const void*)k_orth_group<1>,
+                                 (const void*)k_orth_group<kOrthGroup>};
+  for (const void* kernel : kernels) {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) { cudaGetLastError(); return 0; }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
@@ -761,18 +837,16 @@ int cluster_for(int64_t k) {
   return cs;
 }
 
-cudaError_t launch(const OrthArgs& a, cudaStream_t s) {
-  const int cap = max_cluster();
-  if (cap == 0) return cudaErrorInvalidConfiguration;
-  const int cs = std::min(cap, cluster_for(a.k));
+// One cluster of `cs` CTAs for each of n jobs.
+template <typename KERNEL, typename ARGS>
+cudaError_t launch(KERNEL kernel, const ARGS& a, int cs, int n, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)cs); cfg.blockDim = dim3(kT); cfg.dynamicSmemBytes = kSmemBytes; cfg.stream = s;
+  cfg.gridDim = dim3((unsigned)(cs * n)); cfg.blockDim = dim3(kT); cfg.dynamicSmemBytes = kSmemBytes; cfg.stream = s;
   cfg.attrs = at; cfg.numAttrs = 1;
-  // 16-byte copies need even dimensions throughout (the buffers start on 256-byte boundaries)
-  return cudaLaunchKernelEx(&cfg, (a.k % 2 == 0) ? k_orth_cluster<true> : k_orth_cluster<false>, a);
+  return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
 inline int64_t pad32(int64_t doubles) { return (doubles + 31) / 32 * 32; }
@@ -783,25 +857,74 @@ int64_t coef_doubles(int64_t k) { return pad32(std::max<int64_t>(((k + 1) / 2) *
 }  // namespace
 
 size_t orth_work_doubles(int64_t k) {
-  return (size_t)(coef_doubles(k) + pad32(2 * cluster_for(k) * k) + pad32(k));
+  return (size_t)(coef_doubles(k) + pad32(2 * kMaxCluster * k) + pad32(k));
+}
+void orth_job_work(OrthJob* j, double* work) {
+  j->C = work; j->normp = j->C + coef_doubles(j->k); j->rdiag = j->normp + pad32(2 * kMaxCluster * j->k);
 }
 
-cudaError_t orth_whole(double* A, int64_t k, double* work, double* Acopy, const float* Qprev,
-                       float* Qout, __nv_bfloat16* Qh, __nv_bfloat16* Ql, int* status, int* cond_out, cudaStream_t s) {
-  OrthArgs a = {};
-  a.A = A; a.k = k; a.j0 = 0; a.w = (int)k; a.whole = 1;
-  a.C = work; a.normp = a.C + coef_doubles(k); a.rdiag = a.normp + pad32(2 * cluster_for(k) * k);
-  a.Acopy = Acopy; a.Qprev = Qprev; a.Qout = Qout; a.Qh = Qh; a.Ql = Ql;
-  a.status = status; a.cond_out = cond_out;
-  return launch(a, s);
+template <int NJ>
+static cudaError_t orth_launch(const OrthJob* jobs, int n, int cs, int* status, cudaStream_t s) {
+  OrthGroup<NJ> g;
+  for (int i = 0; i < n; ++i) g.j[i] = jobs[i];
+  g.status = status;
+  return launch(k_orth_group<NJ>, g, cs, n, s);
+}
+cudaError_t orth_group(const OrthJob* jobs, int n, int* status, cudaStream_t s) {
+  const int cap = max_cluster();
+  if (cap == 0) return cudaErrorInvalidConfiguration;
+  int64_t k = 1;
+  for (int i = 0; i < n; ++i) k = std::max(k, jobs[i].k);
+  const int cs = std::min(cap, cluster_for(k));
+  for (int i = 0; i < n; i += kOrthGroup) {
+    const int m = std::min(kOrthGroup, n - i);
+    const cudaError_t e = m == 1 ? orth_launch<1>(jobs + i, 1, cs, status, s) : orth_launch<kOrthGroup>(jobs + i, m, cs, status, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t orth_part(double* A, int64_t k, int64_t j0, int64_t w, double* C, int first, double ill_ratio, const double* norm0,
                       double* rdiag, int* status, int* flags, const int* skip, cudaStream_t s) {
-  OrthArgs a = {};
+  const int cap = max_cluster();
+  if (cap == 0) return cudaErrorInvalidConfiguration;
+  PartArgs a = {};
   a.A = A; a.k = k; a.j0 = (int)j0; a.w = (int)w; a.first = first; a.ill_ratio = ill_ratio; a.norm0 = norm0;
   a.C = C; a.rdiag = rdiag; a.status = status; a.flags = flags; a.skip = skip;
-  return launch(a, s);
+  const int cs = std::min(cap, cluster_for(k));
+  return k % 2 == 0 ? launch(k_orth_part<true>, a, cs, 1, s) : launch(k_orth_part<false>, a, cs, 1, s);
+}
+
+template <int NJ>
+static cudaError_t product_launch(const OrthJob* jobs, int n, int zs, cudaStream_t s) {
+  ProductGroup<NJ> g;
+  g.n = n;
+  g.tile0[0] = 0;
+  for (int i = 0; i < n; ++i) {
+    const int nt = (int)((jobs[i].k + 63) / 64);
+    g.F[i] = jobs[i].F; g.Q[i] = jobs[i].Qprev; g.A[i] = jobs[i].A; g.k[i] = (int)jobs[i].k;
+    g.tile0[i + 1] = g.tile0[i] + nt * nt;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)zs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)(g.tile0[n] * zs)); cfg.blockDim = dim3(kT); cfg.dynamicSmemBytes = kProductSmem; cfg.stream = s;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_product_group<NJ>, g);
+}
+cudaError_t product_group(const OrthJob* jobs, int n, cudaStream_t s) {
+  for (int i = 0; i < n; i += kOrthGroup) {
+    const int m = std::min(kOrthGroup, n - i);
+    int64_t tiles = 0, k = 0;
+    for (int q = i; q < i + m; ++q) { const int64_t nt = (jobs[q].k + 63) / 64; tiles += nt * nt; k = std::max(k, jobs[q].k); }
+    // fewer tiles than two CTAs per SM can hold: share their contractions, down to three stages each
+    int zs = 1;
+    while (zs < 8 && 2 * zs * tiles <= 296 && 2 * zs * 3 * kKs <= k) zs *= 2;
+    const cudaError_t e = m == 1 ? product_launch<1>(jobs + i, 1, zs, s) : product_launch<kOrthGroup>(jobs + i, m, zs, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t product64(int ta, int64_t M, int64_t N, int64_t K, double alpha, const float* A, int64_t lda, const float* B,

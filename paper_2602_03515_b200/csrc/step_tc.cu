@@ -247,14 +247,17 @@ void destroy(RxPlans& r) {
 
 }  // namespace
 
-int complete_factors(Layer& L, cudaStream_t s, cudaError_t* e) {
-  *e = cudaSuccess;
-  if (!L.lower_stale) return 0;
-  int n = 0;
-  if (L.L) { if ((*e = mirror_lower(L.L, L.d.m, s)) != cudaSuccess) return -1; ++n; }
-  if (L.R) { if ((*e = mirror_lower(L.R, L.d.n, s)) != cudaSuccess) return -1; ++n; }
-  L.lower_stale = false;
-  return n;
+int complete_factors(Layer* const* layers, int n, cudaStream_t s, cudaError_t* e) {
+  std::vector<MirrorJob> jobs;
+  for (int i = 0; i < n; ++i) {
+    const Layer& L = *layers[i];
+    if (!L.lower_stale) continue;
+    if (L.L) jobs.push_back({L.L, L.d.m});
+    if (L.R) jobs.push_back({L.R, L.d.n});
+  }
+  if ((*e = mirror_lower(jobs.data(), (int)jobs.size(), s)) != cudaSuccess) return -1;
+  for (int i = 0; i < n; ++i) layers[i]->lower_stale = false;
+  return ((int)jobs.size() + kElemGroup - 1) / kElemGroup;
 }
 
 struct TcStep {
@@ -393,13 +396,15 @@ struct Launcher {
 // One direction of the re-expression for the layers at the given positions of chunk c.
 int reexpress_chunk(Chunk& c, std::vector<Layer>& layers, const std::vector<int>& slots, bool forward,
                     Launcher& lz) {
+  std::vector<SplitJob> jobs;
   for (int j : slots) {
     const Layer& L = layers[c.ids[j]];
-    if (lz.stats->inject()) return lz.fail("split_bf16", cudaErrorLaunchFailure);
-    cudaError_t e = split_bf16(L.M, c.scr[j].B[0], c.scr[j].B[1], L.d.m * L.d.n, lz.s);
-    if (e != cudaSuccess) return lz.fail("split_bf16", e);
-    lz.stats->launches += 1;
+    jobs.push_back({L.M, c.scr[j].B[0], c.scr[j].B[1], L.d.m * L.d.n});
   }
+  if (lz.stats->inject()) return lz.fail("split_bf16", cudaErrorLaunchFailure);
+  cudaError_t e = split_bf16(jobs.data(), (int)jobs.size(), lz.s);
+  if (e != cudaSuccess) return lz.fail("split_bf16", e);
+  lz.stats->launches += ((int)jobs.size() + kElemGroup - 1) / kElemGroup;
   int rc;
   if (slots.size() == c.ids.size()) {
     if ((rc = lz.run_rx(forward ? c.rx.fwd1 : c.rx.back1, "re-expression, first side"))) return rc;

@@ -32,7 +32,7 @@ void rotated_sides(int64_t m, int64_t n, int geom, bool* left, bool* right);
 
 // Brings the lower block triangles of L and R up to date if they lag behind.  Returns the number of launches, or -1
 // with the error in *e.
-int complete_factors(Layer& L, cudaStream_t s, cudaError_t* e);
+int complete_factors(Layer* const* layers, int n, cudaStream_t s, cudaError_t* e);
 
 struct TcStep;
 struct TcStepCallbacks {

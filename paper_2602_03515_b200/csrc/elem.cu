@@ -306,10 +306,9 @@ __global__ void __launch_bounds__(kThreads) k_clip_final(const double* __restric
   *out = (nrm > (double)clip) ? (float)((double)clip / nrm) : 1.0f;
 }
 
-// Copies (a call's gradients into the ring) that run beside the contraction launches: one CTA of 256 threads and 40
-// registers per SM is what an SM has room for next to one of those (it leaves 11.7 of 64 thousand registers and 1.9 KB of shared
-// memory, of which every CTA takes one; two copy CTAs on an SM would keep the next contraction launch off it until they are
-// done).  One cudaMemcpyAsync per gradient takes 2.7 us each at the sizes of a d = 384 layer, 43 us a step, and finds no room there.
+// Copies (a call's gradients into the ring) that run beside the last contraction launches of a step: one CTA of 256 threads and
+// 40 registers per SM is what fits next to one of those.  One cudaMemcpyAsync per gradient takes 2.7 us each at the sizes of a
+// d = 384 layer, 43 us a step.
 constexpr int kCopyThreads = 256, kCopyLoads = 4;
 struct CopyArgs { CopyJob j[kElemGroup]; long long begin[kElemGroup + 1]; int n; };     // begin: in 16-byte pieces
 __global__ void __launch_bounds__(kCopyThreads, 6) k_ring_copy(const __grid_constant__ CopyArgs a) {

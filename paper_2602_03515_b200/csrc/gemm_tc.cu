@@ -81,8 +81,15 @@ constexpr int SH_STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
 static_assert(SH_STAGES * SH_STAGE_BYTES == STAGES * STAGE_BYTES, "both forms use the same operand area");
 constexpr int EPI_WARPS = 8;
 constexpr int EPI_BYTES = EPI_WARPS * 32 * 32 * 4;   // one 32 x 32 fp32 block per epilogue warp
-constexpr int OPERAND_BYTES = STAGES * STAGE_BYTES;                   // 192 KiB of operand stages in every form
+constexpr int OPERAND_BYTES = STAGES * STAGE_BYTES;                   // 192 KiB of operand stages in the shared-operand form
+// 160 KiB in the others: five stages are as fast as six, and the plain form leaves 34 KB of shared memory.  With a limit of 128
+// registers (launch bounds of 512 threads; no rotated Adam, whose problems always sum operand pairs) it also leaves a
+// quarter of each sub-partition's registers: the copies of the gradients into the ring run beside the last two phases of a step.
+// At 168 registers three warps fill a sub-partition, and the copies kept the weight-write launch waiting (four blocks of
+// d = 2560: 21.4 ms a step instead of 20.1).
+constexpr int PLAIN_OPERAND_BYTES = 160 * 1024;
 constexpr int SMEM_BYTES = OPERAND_BYTES + EPI_BYTES + 1024;          // + slack to align the tiles to 1 KiB
+constexpr int SMEM_BYTES_PLAIN = PLAIN_OPERAND_BYTES + EPI_BYTES + 1024;
 constexpr int MAX_STAGES = 6;
 // Per-form geometry.  PAIR: the CTA pair owns a 256-row tile, each CTA stages 128 columns of B.
 template <bool SHARED, bool PAIR>
@@ -91,14 +98,15 @@ struct Form {
   static constexpr int BNC = PAIR ? BN / 2 : BN;                // result columns whose B rows this CTA stages
   static constexpr int BB = BNC * BK * 2;                       // bytes of one staged B tile
   static constexpr int STAGE = SHARED ? 2 * A_BYTES + 2 * BB : A_BYTES + BB;
-  static constexpr int NST = OPERAND_BYTES / STAGE;             // 4 / 2 unpaired, 6 / 3 paired
-  static_assert(NST <= MAX_STAGES && NST * STAGE == OPERAND_BYTES, "stages fill the operand area");
+  static constexpr int OPERANDS = SHARED ? OPERAND_BYTES : PLAIN_OPERAND_BYTES;
+  static constexpr int NST = OPERANDS / STAGE;                  // 3 / 2 unpaired, 5 / 3 paired
+  static_assert(NST <= MAX_STAGES, "barriers");
 };
 constexpr int TMEM_COLS = 512;
 constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS; // warp 0: TMA, warp 1: MMA, warps 2..9: epilogue (two per lane quadrant)
-// folded form: 160 KiB of operand stages, and two blocks of 32 x 32 floats for each of its eight epilogue warps
-constexpr int FOLD_OPERAND_BYTES = 160 * 1024, FOLD_BLOCK = 32 * 32;
-constexpr int SMEM_BYTES_FOLD = FOLD_OPERAND_BYTES + 8 * 2 * FOLD_BLOCK * 4 + 1024;
+// folded form: two blocks of 32 x 32 floats for each of its eight epilogue warps
+constexpr int FOLD_BLOCK = 32 * 32;
+constexpr int SMEM_BYTES_FOLD = PLAIN_OPERAND_BYTES + EPI_WARPS * 2 * FOLD_BLOCK * 4 + 1024;
 constexpr int MAX_PAIRS = 3;
 // Fixed part of a tile's cost in the schedule (see make_schedule), plain and folded form.  Steady steps with 0 and 0, 6 and
 // 24, 12 and 24, 6 and 0, 6 and 48: one block of d = 1024 620, 587, 587, 610, 586 us; four of d = 384 392, 382, 390, 389,
@@ -416,11 +424,11 @@ __device__ __forceinline__ TileInfo locate_tile(const DevProblem* probs, int n_p
 // The kernel
 // ---------------------------------------------------------------------------------------------
 template <bool SHARED, bool PAIR, bool FOLD = false>
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+__global__ void __launch_bounds__(SHARED || FOLD ? NUM_THREADS : 512, 1)
 k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int total_tiles, const int* __restrict__ schedule,
           long long calls, int tau, float dyn_alpha, float dyn_beta, int* status) {
   using F = Form<SHARED, PAIR>;
-  constexpr int NST = FOLD ? FOLD_OPERAND_BYTES / F::STAGE : F::NST;      // folded: 5 paired, 3 unpaired
+  constexpr int NST = F::NST;
   constexpr int TM = F::TM;
   extern __shared__ uint8_t smem_raw[];
   __shared__ alignas(8) uint64_t bars[2 * MAX_STAGES + 4];
@@ -443,7 +451,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
     return SHARED ? tiles_base + (uint32_t)s * F::STAGE + 2u * A_BYTES + (uint32_t)i * F::BB
                   : tiles_base + (uint32_t)NST * A_BYTES + (uint32_t)s * F::BB;
   };
-  float* epi_tiles = reinterpret_cast<float*>(smem_raw + ((tiles_base - smem_u32(smem_raw)) + (uint32_t)(FOLD ? FOLD_OPERAND_BYTES : OPERAND_BYTES)));
+  float* epi_tiles = reinterpret_cast<float*>(smem_raw + ((tiles_base - smem_u32(smem_raw)) + (uint32_t)F::OPERANDS));
   const uint32_t bar0 = smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
@@ -817,7 +825,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
         __syncwarp();
       };
       auto turned = [&](int it) { return *reinterpret_cast<const float4*>(piece(4 * it + sub_r, lane & 7)); };
-      if (epi == EPI_ROTATED_ADAM) {
+      if (SHARED && epi == EPI_ROTATED_ADAM) {
         const float b1 = p->beta1, ob1 = 1.0f - p->beta1;
         float* const pv = p->D + at_d;                 // V~
         float* const pm = p->D2 + at_d;                // M~
@@ -1241,8 +1249,8 @@ TcPlan* tc_plan_create(const TcProblem* problems, int n, int device, cudaStream_
     d.D = q.D; d.ldd = q.ldd; d.Dh = q.Dh; d.Dl = q.Dl; d.ldh = q.ldh; d.D2 = q.D2;
     const bool need_D = q.epilogue != EPI_SPLIT_BF16;
     const bool need_H = q.epilogue == EPI_SPLIT_BF16 || q.epilogue == EPI_ROTATED_ADAM;
-    if (q.epilogue == EPI_ROTATED_ADAM && (!q.D2 || (reinterpret_cast<uintptr_t>(q.D2) & 15)))
-      return fail("tensor-core problem: second in/out pointer missing or misaligned");
+    if (q.epilogue == EPI_ROTATED_ADAM && (!shared || !q.D2 || (reinterpret_cast<uintptr_t>(q.D2) & 15)))
+      return fail("tensor-core problem: rotated Adam without operand pairs, or its second in/out pointer missing or misaligned");
     if ((need_D && (!q.D || (q.ldd % 4) || (reinterpret_cast<uintptr_t>(q.D) & 15))) ||
         (need_H && (!q.Dh || (q.ldh % 8) || (reinterpret_cast<uintptr_t>(q.Dh) & 15))) ||
         (q.Dl && (reinterpret_cast<uintptr_t>(q.Dl) & 15)))
@@ -1308,7 +1316,7 @@ cudaError_t launch_range(TcPlan* p, int first, int count, long long calls, int t
   const int tiles = t1 - t0;
   TcKernel kernel = kernel_of(p->shared, p->pair, p->fold);
   // per-device attribute: set again when another device is current (cheap, idempotent)
-  const int smem_bytes = p->fold ? SMEM_BYTES_FOLD : SMEM_BYTES;
+  const int smem_bytes = p->fold ? SMEM_BYTES_FOLD : p->shared ? SMEM_BYTES : SMEM_BYTES_PLAIN;
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];

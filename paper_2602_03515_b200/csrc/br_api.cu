@@ -121,6 +121,9 @@ struct br_handle {
   // share their SMs with another run half as long again, so no estimate of the lanes' loads was right.)
   char* pool = nullptr;
   size_t pool_bytes = 0;
+  // What the pool has behind that for the digits of the products of the larger ones (oz.cu), besides the work areas of
+  // the factorisations; 0: those products run on the fp64 unit.
+  size_t oz_bytes = 0;
   struct Side { cudaStream_t stream = nullptr; cudaEvent_t done = nullptr; };
   Side group_side[2];                     // beside the handle's stream (created when there is a pool)
   bool use_graphs = true;                 // cleared when a capture fails (BR_REFRESH_GRAPHS=0 switches it off)
@@ -205,6 +208,8 @@ inline int64_t z_slice(int64_t k, int64_t other) {
 
 constexpr size_t kPoolOfLargest = 12, kPoolCompact = 3;
 constexpr int64_t kSmallGroup = 128;
+// From here on a power product takes less time in digits on the int8 tensor cores than on the fp64 unit.
+constexpr int64_t kOzMinOrder = 1024;
 // A side whose refresh is part of the grouped launches, and what it needs of the pool.
 inline bool grouped_side(const Layer& L, int64_t k) { return L.d.src == BR_SRC_SECOND && qr_one_launch(k); }
 inline size_t pool_need(int64_t k) {
@@ -215,7 +220,8 @@ inline size_t pool_need(int64_t k) {
 void layout(br_handle* h, Bump& b, Sizes* sz) {
   const br_hparams& hp = h->hp;
   if (hp.flags & BR_FLAG_DEBUG_CANARY) { b.guard = kAlign; b.guards = &h->guard_offsets; h->guard_offsets.clear(); }
-  size_t simt_max = 0, simt_total = 0, max_k = 0, max_z = 0, n_sides = 0, pool_sum = 0, pool_max = 0;
+  size_t simt_max = 0, simt_total = 0, max_k = 0, max_z = 0, n_sides = 0, pool_sum = 0, pool_max = 0, n_pool = 0;
+  int64_t pool_k = 0;
   for (Layer& L : h->layers) {
     const size_t mn = (size_t)L.d.m * L.d.n;
     L.M = b.take<float>(mn);
@@ -241,7 +247,7 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
       if (!L.use_tc) { simt_max = std::max(simt_max, simt_need(L)); simt_total += simt_need(L); }
       for (int64_t k : {L.left ? L.d.m : (int64_t)0, L.right ? L.d.n : (int64_t)0}) {
         if (!k) continue;
-        if (grouped_side(L, k)) { pool_sum += pool_need(k); pool_max = std::max(pool_max, pool_need(k)); }
+        if (grouped_side(L, k)) { pool_sum += pool_need(k); pool_max = std::max(pool_max, pool_need(k)); pool_k = std::max(pool_k, k); ++n_pool; }
         else { max_k = std::max(max_k, (size_t)k); ++n_sides; }
       }
       if (!second)
@@ -255,7 +261,16 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
   }
   // the pool: every grouped basis at once, up to twelve of the largest (three in the compact layout)
   h->pool_bytes = std::min(pool_sum, (h->compact ? kPoolCompact : kPoolOfLargest) * pool_max);
-  if (h->pool_bytes) h->pool = b.take<char>(h->pool_bytes);
+  // Digits of two products of the largest order, or of one, as far as pool and digits together stay below eight buffers
+  // for that order with a product and its copy each.
+  h->oz_bytes = 0;
+  if (!h->compact && pool_k >= kOzMinOrder && oz_eligible(pool_k, pool_k, pool_k)) {
+    const size_t one = oz_scratch_bytes(pool_k, pool_k, pool_k);
+    const size_t lanes = std::min<size_t>(n_pool, 8) * (pool_max + align_up(sizeof(double) * (size_t)pool_k * (size_t)pool_k));
+    const size_t room = lanes > h->pool_bytes ? lanes - h->pool_bytes : 0;
+    h->oz_bytes = std::min<size_t>(room / one, 2) * one;
+  }
+  if (h->pool_bytes) h->pool = b.take<char>(h->pool_bytes + h->oz_bytes);
   h->n_lanes = 1;
   h->tcq_bytes = 0;
   for (const Layer& L : h->layers) {
@@ -537,8 +552,9 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
 
 struct GroupSide { int layer; bool left; int64_t k; };
 
-// The grouped refreshes `v` (longest first) on one stream, as many at a time as `bytes` of the pool hold.
-br_status refresh_group(br_handle* h, const GroupSide* v, int n, char* pool, size_t bytes, cudaStream_t s) {
+// The grouped refreshes `v` (longest first) on one stream, as many at a time as `bytes` of the pool hold; behind them are
+// oz_bytes for digits.
+br_status refresh_group(br_handle* h, const GroupSide* v, int n, char* pool, size_t bytes, size_t oz_bytes, cudaStream_t s) {
   std::vector<OrthJob> jobs;
   for (int first = 0; first < n; first += (int)jobs.size()) {
     jobs.clear();
@@ -558,14 +574,30 @@ br_status refresh_group(br_handle* h, const GroupSide* v, int n, char* pool, siz
       j.complete = L.n_accum < (k + other - 1) / other;        // (see refresh_side)
       jobs.push_back(j);
     }
+    // the products, then the work areas, which the digits may overwrite: they are done when the factorisations begin
+    char* const digits = pool + used;
+    const size_t digit_bytes = bytes - used + oz_bytes;
     for (OrthJob& j : jobs) {
       orth_job_work(&j, reinterpret_cast<double*>(pool + used));
       used += align_up(sizeof(double) * orth_work_doubles(j.k));
     }
+    // (longest first: the products in digits are the front of the list)
+    std::vector<OzProduct> oz;
+    for (const OrthJob& j : jobs)
+      if (oz_bytes && j.k >= kOzMinOrder) oz.push_back({j.F, j.Qprev, j.A, j.k, j.k, j.k});
+    const int n_oz = (int)oz.size(), n_rest = (int)jobs.size() - n_oz;
     for (int it = 0; it < h->hp.power_iters; ++it) {
-      BR_CUDA(h, product_group(jobs.data(), (int)jobs.size(), s));
+      if (n_oz) {
+        int launches = 0;
+        BR_CUDA(h, oz_product_group(oz.data(), n_oz, digits, digit_bytes, h->d_status, s, &launches));
+        count(h, launches);
+      }
+      if (n_rest) {
+        BR_CUDA(h, product_group(jobs.data() + n_oz, n_rest, s));
+        count(h, (n_rest + kOrthGroup - 1) / kOrthGroup);
+      }
       BR_CUDA(h, orth_group(jobs.data(), (int)jobs.size(), h->d_status, s));
-      count(h, 2 * (((int)jobs.size() + kOrthGroup - 1) / kOrthGroup));
+      count(h, ((int)jobs.size() + kOrthGroup - 1) / kOrthGroup);
       for (const OrthJob& j : jobs) h->stats.gemm_flops += 4.0 * j.k * j.k * j.k;
     }
   }
@@ -637,12 +669,12 @@ br_status refresh_layers(br_handle* h, const int* ids, int n_ids) {
   }
   const int n_grouped = (int)grouped.size();
   const bool apart = n_large > 0 && n_large < n_grouped && need <= h->pool_bytes;
-  struct Batch { int first, n; char* pool; size_t bytes; br_handle::Side* side; };
+  struct Batch { int first, n; char* pool; size_t bytes, oz_bytes; br_handle::Side* side; };
   std::vector<Batch> batches;
   if (n_grouped) {
     const size_t small = apart ? need - need_large : 0;
-    batches.push_back({0, apart ? n_large : n_grouped, h->pool + small, h->pool_bytes - small, jobs.empty() ? nullptr : &h->group_side[0]});
-    if (apart) batches.push_back({n_large, n_grouped - n_large, h->pool, small, &h->group_side[1]});
+    batches.push_back({0, apart ? n_large : n_grouped, h->pool + small, h->pool_bytes - small, h->oz_bytes, jobs.empty() ? nullptr : &h->group_side[0]});
+    if (apart) batches.push_back({n_large, n_grouped - n_large, h->pool, small, 0, &h->group_side[1]});
   }
   const double f0 = h->stats.gemm_flops;
   const int span = h->stats.prof.begin(PROF_REFRESH, h->stream);
@@ -656,7 +688,7 @@ br_status refresh_layers(br_handle* h, const int* ids, int n_ids) {
   for (auto& v : per_lane) longest = std::max(longest, v.size());
   br_status failed = BR_OK;
   for (const Batch& bt : batches)
-    if (failed == BR_OK) failed = refresh_group(h, grouped.data() + bt.first, bt.n, bt.pool, bt.bytes, bt.side ? bt.side->stream : h->stream);
+    if (failed == BR_OK) failed = refresh_group(h, grouped.data() + bt.first, bt.n, bt.pool, bt.bytes, bt.oz_bytes, bt.side ? bt.side->stream : h->stream);
   for (size_t r = 0; r < longest && failed == BR_OK; ++r)
     for (int i = 0; i < nl && failed == BR_OK; ++i) {
       if (r >= per_lane[i].size()) continue;

@@ -231,6 +231,17 @@ cudaError_t product64(int ta, int64_t M, int64_t N, int64_t K, double alpha, con
                       int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t s);
 
 // ---------------------------------------------------------------------------------------------
+// fp64-accurate products of fp32 matrices on the int8 tensor cores (oz.cu)
+// ---------------------------------------------------------------------------------------------
+// C (M x N, fp64) = X (M x K) Y (K x N), all row-major and contiguous
+struct OzProduct { const float *X, *Y; double* C; int64_t M, N, K; };
+bool oz_eligible(int64_t M, int64_t N, int64_t K);
+size_t oz_scratch_bytes(int64_t M, int64_t N, int64_t K);
+// As many products at a time as the scratch (256-byte aligned) holds, which must be one at least.
+cudaError_t oz_product_group(const OzProduct* v, int n, char* scratch, size_t bytes, int* status, cudaStream_t s, int* launches);
+void* tensor_map_encoder();            // cuTensorMapEncodeTiled, or null
+
+// ---------------------------------------------------------------------------------------------
 // QR with positive diagonal in fp64 (qr.cu).  A (k x k, row-major, ld = k) is overwritten by
 // its Q factor.  work: at least qr_work_doubles(k) doubles.  status: device int, set to
 // BR_WARN_RANK_DEFICIENT when a pivot underflows.  Returns the number of launches in *launches.

@@ -117,13 +117,13 @@ cudaError_t widen_bf16(const __nv_bfloat16* X, float* out, int64_t numel, cudaSt
 // out(double) <- in(float) ; out(float) <- in(double)
 cudaError_t f64_to_f32(const double* X, float* out, int64_t numel, cudaStream_t s);
 cudaError_t f32_to_f64(const float* X, double* out, int64_t numel, cudaStream_t s);
-// Three-term bf16 split (all 24 bits of the fp32 rounding of x) of a rows x cols block of a strided
-// fp64 matrix, or of a contiguous fp32 array, into compact planes; A (fp64, strided) -= D (fp32, compact).
-cudaError_t split3_f64(const double* X, int64_t ld, int64_t rows, int64_t cols, __nv_bfloat16* p1,
-                       __nv_bfloat16* p2, __nv_bfloat16* p3, cudaStream_t s);
-cudaError_t split3_f32(const float* X, int64_t numel, __nv_bfloat16* p1, __nv_bfloat16* p2, __nv_bfloat16* p3,
+// Three-term bf16 split (all 24 bits of the fp32 rounding of x) of a rows x cols block of a strided fp64 matrix into compact
+// planes (p1 not null), after A -= D (fp32, compact) on it (D not null).  cols a multiple of 4, rows on 16-byte boundaries.
+cudaError_t sub_split3(double* A, int64_t ld, int64_t rows, int64_t cols, const float* D, __nv_bfloat16* p1, __nv_bfloat16* p2,
+                       __nv_bfloat16* p3, cudaStream_t s);
+// The same split of the sum of `parts` contiguous fp32 arrays that follow one another.
+cudaError_t split3_f32(const float* X, int64_t numel, int parts, __nv_bfloat16* p1, __nv_bfloat16* p2, __nv_bfloat16* p3,
                        cudaStream_t s);
-cudaError_t sub_f32_from_f64(double* A, int64_t ld, int64_t rows, int64_t cols, const float* D, cudaStream_t s);
 // out <- beta1 M + (1-beta1) G (out-of-place form of Alg. 1 (momentum update))
 cudaError_t ema_out(float* out, const float* M, const void* G, int g_is_bf16, int64_t numel, float beta1,
                     const float* gscale, cudaStream_t s);
@@ -262,7 +262,7 @@ int64_t qr_tc_order(const QrTc* t);
 // work: the QR work area of this order (used for the column norms).
 cudaError_t qr_complete_columns(double* A, const float* Q, int64_t k, double* work, int* status, cudaStream_t s);
 // *out (fp32, k x k, owned by t) = Frest U on the tensor cores (three-term bf16 splits, six products)
-cudaError_t qr_tc_power(QrTc* t, const double* Frest, const double* U, int* status, cudaStream_t s, const float** out);
+cudaError_t qr_tc_power(QrTc* t, double* Frest, double* U, int* status, cudaStream_t s, const float** out);
 cudaError_t qr_tc_project(QrTc* t, int node, double* A, int64_t k, int64_t jp, int64_t wp, int64_t jt,
                           int64_t wt, int* status, cudaStream_t s);
 // tc: null, or the plans for this order: the first sweep then projects on the tensor cores (ask for it

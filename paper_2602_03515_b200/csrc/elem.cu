@@ -348,32 +348,49 @@ __device__ __forceinline__ void split3(float f, __nv_bfloat16& p1, __nv_bfloat16
   p1 = __float2bfloat16_rn(h1); p2 = __float2bfloat16_rn(h2); p3 = __float2bfloat16_rn(r2);
 }
 
-// X: rows x cols block of a row-major fp64 matrix with leading dimension ld -> three compact
-// (ld = cols) bf16 planes
+// Four columns per thread (widths are multiples of 8 and rows start on 16-byte boundaries), 32-bit index arithmetic.
+// SUB: A -= D first (D fp32, compact); SPLIT: the three planes (compact).  Both in one pass between the two passes of a projection.
+struct alignas(8) bf16x4 { __nv_bfloat16 v[4]; };
+__device__ __forceinline__ void split3x4(const float (&x)[4], int64_t i, __nv_bfloat16* p1, __nv_bfloat16* p2, __nv_bfloat16* p3) {
+  bf16x4 a, b, c;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) split3(x[u], a.v[u], b.v[u], c.v[u]);
+  *reinterpret_cast<bf16x4*>(p1 + i) = a;
+  *reinterpret_cast<bf16x4*>(p2 + i) = b;
+  *reinterpret_cast<bf16x4*>(p3 + i) = c;
+}
+template <bool SUB, bool SPLIT>
 __global__ void __launch_bounds__(kThreads)
-k_split3_f64(const double* __restrict__ X, int64_t ld, int64_t rows, int64_t cols, __nv_bfloat16* __restrict__ p1,
-             __nv_bfloat16* __restrict__ p2, __nv_bfloat16* __restrict__ p3) {
-  const int64_t total = rows * cols;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / cols, c = i - r * cols;
-    split3((float)X[r * ld + c], p1[i], p2[i], p3[i]);
+k_sub_split3(double* __restrict__ A, int64_t ld, unsigned groups, unsigned per_row, const float* __restrict__ D,
+             __nv_bfloat16* __restrict__ p1, __nv_bfloat16* __restrict__ p2, __nv_bfloat16* __restrict__ p3) {
+  for (unsigned g = blockIdx.x * kThreads + threadIdx.x; g < groups; g += gridDim.x * kThreads) {
+    const unsigned r = g / per_row, c = 4 * (g - r * per_row);
+    double2* const at = reinterpret_cast<double2*>(A + (int64_t)r * ld + c);
+    double2 lo = at[0], hi = at[1];
+    if (SUB) {
+      const float4 d = *reinterpret_cast<const float4*>(D + 4 * (int64_t)g);
+      lo.x -= (double)d.x; lo.y -= (double)d.y; hi.x -= (double)d.z; hi.y -= (double)d.w;
+      at[0] = lo; at[1] = hi;
+    }
+    if (SPLIT) {
+      const float x[4] = {(float)lo.x, (float)lo.y, (float)hi.x, (float)hi.y};
+      split3x4(x, 4 * (int64_t)g, p1, p2, p3);
+    }
   }
 }
-
+// the sum of `parts` compact arrays (4 * groups entries each) into planes; summed in fp64
 __global__ void __launch_bounds__(kThreads)
-k_split3_f32(const float* __restrict__ X, int64_t numel, __nv_bfloat16* __restrict__ p1,
+k_split3_f32(const float* __restrict__ X, unsigned groups, int parts, __nv_bfloat16* __restrict__ p1,
              __nv_bfloat16* __restrict__ p2, __nv_bfloat16* __restrict__ p3) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < numel; i += (int64_t)gridDim.x * blockDim.x)
-    split3(X[i], p1[i], p2[i], p3[i]);
-}
-
-// A (fp64, leading dimension ld) -= D (fp32, compact rows x cols)
-__global__ void __launch_bounds__(kThreads)
-k_sub_f32_from_f64(double* __restrict__ A, int64_t ld, int64_t rows, int64_t cols, const float* __restrict__ D) {
-  const int64_t total = rows * cols;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / cols, c = i - r * cols;
-    A[r * ld + c] -= (double)D[i];
+  for (unsigned g = blockIdx.x * kThreads + threadIdx.x; g < groups; g += gridDim.x * kThreads) {
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+    for (int z = 0; z < parts; ++z) {
+      const float4 v = *reinterpret_cast<const float4*>(X + 4 * ((int64_t)z * groups + g));
+      s[0] += (double)v.x; s[1] += (double)v.y; s[2] += (double)v.z; s[3] += (double)v.w;
+    }
+    const float x[4] = {(float)s[0], (float)s[1], (float)s[2], (float)s[3]};
+    split3x4(x, 4 * (int64_t)g, p1, p2, p3);
   }
 }
 
@@ -503,20 +520,20 @@ cudaError_t clip_factor(const void* const* grads, const int64_t* numel, const in
   return cudaGetLastError();
 }
 
-cudaError_t split3_f64(const double* X, int64_t ld, int64_t rows, int64_t cols, __nv_bfloat16* p1,
-                       __nv_bfloat16* p2, __nv_bfloat16* p3, cudaStream_t s) {
-  k_split3_f64<<<grid_for(rows * cols), kThreads, 0, s>>>(X, ld, rows, cols, p1, p2, p3);
+cudaError_t sub_split3(double* A, int64_t ld, int64_t rows, int64_t cols, const float* D, __nv_bfloat16* p1, __nv_bfloat16* p2,
+                       __nv_bfloat16* p3, cudaStream_t s) {
+  if (cols % 4 || ld % 2 || rows * cols / 4 > 0xffffffffll - (1 << 22)) return cudaErrorInvalidValue;
+  const unsigned groups = (unsigned)(rows * cols / 4), per_row = (unsigned)(cols / 4);
+  const int grid = grid_for(groups);
+  if (D && p1) k_sub_split3<true, true><<<grid, kThreads, 0, s>>>(A, ld, groups, per_row, D, p1, p2, p3);
+  else if (D) k_sub_split3<true, false><<<grid, kThreads, 0, s>>>(A, ld, groups, per_row, D, p1, p2, p3);
+  else k_sub_split3<false, true><<<grid, kThreads, 0, s>>>(A, ld, groups, per_row, D, p1, p2, p3);
   return cudaGetLastError();
 }
-
-cudaError_t split3_f32(const float* X, int64_t numel, __nv_bfloat16* p1, __nv_bfloat16* p2, __nv_bfloat16* p3,
+cudaError_t split3_f32(const float* X, int64_t numel, int parts, __nv_bfloat16* p1, __nv_bfloat16* p2, __nv_bfloat16* p3,
                        cudaStream_t s) {
-  k_split3_f32<<<grid_for(numel), kThreads, 0, s>>>(X, numel, p1, p2, p3);
-  return cudaGetLastError();
-}
-
-cudaError_t sub_f32_from_f64(double* A, int64_t ld, int64_t rows, int64_t cols, const float* D, cudaStream_t s) {
-  k_sub_f32_from_f64<<<grid_for(rows * cols), kThreads, 0, s>>>(A, ld, rows, cols, D);
+  if (numel % 4 || numel / 4 > 0xffffffffll - (1 << 22)) return cudaErrorInvalidValue;
+  k_split3_f32<<<grid_for(numel / 4), kThreads, 0, s>>>(X, (unsigned)(numel / 4), parts, p1, p2, p3);
   return cudaGetLastError();
 }
 

@@ -164,15 +164,16 @@ void enumerate_nodes(int64_t j0, int64_t w, int64_t b, std::vector<ProjNode>* ou
 
 }  // namespace
 
-// Plans and scratch of the tensor-core projections for one order k.  Problem 2 i of either plan is
-// the coefficient product of node i, problem 2 i + 1 its update product; plan `lead` holds the
-// products of the two leading bf16 terms (hi*hi + mid*hi + hi*mid), plan `tail` the next three.
+// Plans and scratch of the tensor-core projections for one order k.  Problems first[i] .. first[i] + parts[i] - 1 of either
+// plan are the coefficient product of node i, a range of its contraction each, the next one its update product; plan
+// `lead` holds the products of the two leading bf16 terms (hi*hi + mid*hi + hi*mid), plan `tail` the next three.
 struct QrTc {
   int64_t k = 0;
   std::vector<ProjNode> nodes;
+  std::vector<int> first, parts;
   TcPlan *lead = nullptr, *tail = nullptr;
   __nv_bfloat16 *Q[3] = {}, *A[3] = {}, *C[3] = {};
-  float *Cf = nullptr, *Df = nullptr;
+  float* Df = nullptr;         // results: the parts of a coefficient product, an update product, the power product
   int power_index = -1;       // problem index (in both plans) of the deflated power product
 };
 
@@ -188,7 +189,7 @@ size_t qr_tc_scratch_bytes(int64_t k) {
   if (!qr_tc_eligible(k)) return 0;
   const size_t h = (size_t)tc_hmax(k), kk = (size_t)k;
   // operand planes and the fp32 result hold a whole k x k matrix (the deflated power product)
-  return 6 * al256(kk * kk * 2) + al256(h * h * 4) + 3 * al256(h * h * 2) + al256(kk * kk * 4);
+  return 6 * al256(kk * kk * 2) + 3 * al256(h * h * 2) + al256(kk * kk * 4);
 }
 
 void qr_tc_destroy(QrTc* t) {
@@ -209,23 +210,32 @@ QrTc* qr_tc_create(int64_t k, char* scratch, int device, cudaStream_t s, const c
   auto take = [&](size_t bytes) { char* p = scratch + off; off += al256(bytes); return p; };
   for (int i = 0; i < 3; ++i) t->Q[i] = reinterpret_cast<__nv_bfloat16*>(take(kk * kk * 2));
   for (int i = 0; i < 3; ++i) t->A[i] = reinterpret_cast<__nv_bfloat16*>(take(kk * kk * 2));
-  t->Cf = reinterpret_cast<float*>(take(h * h * 4));
   for (int i = 0; i < 3; ++i) t->C[i] = reinterpret_cast<__nv_bfloat16*>(take(h * h * 2));
   t->Df = reinterpret_cast<float*>(take(kk * kk * 4));
   enumerate_nodes(0, k, 128, &t->nodes);
   std::vector<TcProblem> lead, tail;
   auto opnd = [](const void* p, int64_t ld, int mn) { TcOperand o; o.ptr = p; o.ld = ld; o.mn_major = mn; return o; };
   for (const ProjNode& nd : t->nodes) {
-    // coefficients C = Q^T A_r (contraction over the k rows: both operands MN-major)
-    TcProblem c; c.Md = nd.wp; c.Nd = nd.wt; c.K = k; c.n_pairs = 3;
-    c.epilogue = EPI_AXPBY_F32; c.alpha = 1.f; c.D = t->Cf; c.ldd = nd.wt;
-    TcProblem c2 = c;
+    // Coefficients C = Q^T A_r (contraction over the k rows: both operands MN-major), the contraction in as many ranges
+    // as fill the GPU (512 x 512 of order 4096: four tiles, 72 us on eight SMs), of 256 rows at least; the ranges of
+    // a product are added when it is split into terms.
     const int ia[6] = {0, 1, 0, 2, 0, 1}, ib[6] = {0, 0, 1, 0, 2, 1};      // term pairs, leading three first
-    for (int p = 0; p < 3; ++p) {
-      c.A[p] = opnd(t->Q[ia[p]], nd.wp, 1); c.B[p] = opnd(t->A[ib[p]], nd.wt, 1);
-      c2.A[p] = opnd(t->Q[ia[3 + p]], nd.wp, 1); c2.B[p] = opnd(t->A[ib[3 + p]], nd.wt, 1);
+    const int64_t tiles = cdiv(nd.wp, 256) * cdiv(nd.wt, 256);
+    const int64_t want = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(74 / tiles, k / 256), k * k / (nd.wp * nd.wt)));
+    const int64_t range = cdiv(cdiv(k, want), 64) * 64;
+    t->first.push_back((int)lead.size());
+    t->parts.push_back((int)cdiv(k, range));
+    for (int64_t k0 = 0; k0 < k; k0 += range) {
+      TcProblem c; c.Md = nd.wp; c.Nd = nd.wt; c.K = std::min(range, k - k0); c.n_pairs = 3;
+      c.epilogue = EPI_AXPBY_F32; c.alpha = 1.f; c.D = t->Df + k0 / range * nd.wp * nd.wt; c.ldd = nd.wt;
+      TcProblem c2 = c;
+      for (int p = 0; p < 3; ++p) {
+        c.A[p] = opnd(t->Q[ia[p]] + k0 * nd.wp, nd.wp, 1); c.B[p] = opnd(t->A[ib[p]] + k0 * nd.wt, nd.wt, 1);
+        c2.A[p] = opnd(t->Q[ia[3 + p]] + k0 * nd.wp, nd.wp, 1); c2.B[p] = opnd(t->A[ib[3 + p]] + k0 * nd.wt, nd.wt, 1);
+      }
+      c.beta = 0.f; c2.beta = 1.f;
+      lead.push_back(c); tail.push_back(c2);
     }
-    c.beta = 0.f; c2.beta = 1.f;
     // update D = Q C (Q K-major, C MN-major)
     TcProblem d; d.Md = k; d.Nd = nd.wt; d.K = nd.wp; d.n_pairs = 3;
     d.epilogue = EPI_AXPBY_F32; d.alpha = 1.f; d.D = t->Df; d.ldd = nd.wt;
@@ -235,8 +245,7 @@ QrTc* qr_tc_create(int64_t k, char* scratch, int device, cudaStream_t s, const c
       d2.A[p] = opnd(t->Q[ia[3 + p]], nd.wp, 0); d2.B[p] = opnd(t->C[ib[3 + p]], nd.wt, 1);
     }
     d.beta = 0.f; d2.beta = 1.f;
-    lead.push_back(c); lead.push_back(d);
-    tail.push_back(c2); tail.push_back(d2);
+    lead.push_back(d); tail.push_back(d2);
   }
   {
     // the power product of the deflated factor: D = F_rest U, F_rest (k x k) K-major, U MN-major
@@ -273,7 +282,10 @@ cudaError_t qr_tc_project(QrTc* t, int node, double* A, int64_t k, int64_t jp, i
   const ProjNode& nd = t->nodes[node];
   if (nd.jp != jp || nd.wp != wp || nd.jt != jt || nd.wt != wt || t->k != k) return cudaErrorInvalidValue;
   cudaError_t e;
-  if ((e = split3_f64(A + jp, k, k, wp, t->Q[0], t->Q[1], t->Q[2], s)) != cudaSuccess) return e;
+  const int at = t->first[node], parts = t->parts[node];
+  auto run = [&](TcPlan* p, int first, int n) { return tc_plan_launch_range(p, first, n, 1, 0, 1.f, 0.f, status, s); };
+  if ((e = sub_split3(A + jp, k, k, wp, nullptr, t->Q[0], t->Q[1], t->Q[2], s)) != cudaSuccess) return e;
+  if ((e = sub_split3(A + jt, k, k, wt, nullptr, t->A[0], t->A[1], t->A[2], s)) != cudaSuccess) return e;
   // Twice: whatever error the coefficients of the first pass have leaves that much of span(Q_l) in
   // the column, measured against its length BEFORE the projection; the second pass sees the shrunken
   // column and leaves ~1e-7 of its length AFTER the projection.  Because the second pass removes what
@@ -283,24 +295,23 @@ cudaError_t qr_tc_project(QrTc* t, int node, double* A, int64_t k, int64_t jp, i
   // are a small difference of large terms), update with the leading three (C is ~2^-16 of the column
   // by then).  18 products instead of 24.
   for (int pass = 0; pass < 2; ++pass) {
-    if ((e = split3_f64(A + jt, k, k, wt, t->A[0], t->A[1], t->A[2], s)) != cudaSuccess) return e;
-    if ((e = tc_plan_launch_range(t->lead, 2 * node, 1, 1, 0, 1.f, 0.f, status, s)) != cudaSuccess) return e;
-    if (pass == 1 && (e = tc_plan_launch_range(t->tail, 2 * node, 1, 1, 0, 1.f, 0.f, status, s)) != cudaSuccess) return e;
-    if ((e = split3_f32(t->Cf, wp * wt, t->C[0], t->C[1], t->C[2], s)) != cudaSuccess) return e;
-    if ((e = tc_plan_launch_range(t->lead, 2 * node + 1, 1, 1, 0, 1.f, 0.f, status, s)) != cudaSuccess) return e;
-    if (pass == 0 && (e = tc_plan_launch_range(t->tail, 2 * node + 1, 1, 1, 0, 1.f, 0.f, status, s)) != cudaSuccess) return e;
-    if ((e = sub_f32_from_f64(A + jt, k, k, wt, t->Df, s)) != cudaSuccess) return e;
+    if ((e = run(t->lead, at, parts)) != cudaSuccess) return e;
+    if (pass == 1 && (e = run(t->tail, at, parts)) != cudaSuccess) return e;
+    if ((e = split3_f32(t->Df, wp * wt, parts, t->C[0], t->C[1], t->C[2], s)) != cudaSuccess) return e;
+    if ((e = run(t->lead, at + parts, 1)) != cudaSuccess) return e;
+    if (pass == 0 && (e = run(t->tail, at + parts, 1)) != cudaSuccess) return e;
+    if ((e = sub_split3(A + jt, k, k, wt, t->Df, pass ? nullptr : t->A[0], t->A[1], t->A[2], s)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
 // D (fp32, k x k, returned in *out) = Frest U with both operands split into three bf16 terms and the
 // six leading products accumulated in fp32.  Frest and U are fp64, row-major with leading dimension k.
-cudaError_t qr_tc_power(QrTc* t, const double* Frest, const double* U, int* status, cudaStream_t s, const float** out) {
+cudaError_t qr_tc_power(QrTc* t, double* Frest, double* U, int* status, cudaStream_t s, const float** out) {
   const int64_t k = t->k;
   cudaError_t e;
-  if ((e = split3_f64(Frest, k, k, k, t->Q[0], t->Q[1], t->Q[2], s)) != cudaSuccess) return e;
-  if ((e = split3_f64(U, k, k, k, t->A[0], t->A[1], t->A[2], s)) != cudaSuccess) return e;
+  if ((e = sub_split3(Frest, k, k, k, nullptr, t->Q[0], t->Q[1], t->Q[2], s)) != cudaSuccess) return e;
+  if ((e = sub_split3(U, k, k, k, nullptr, t->A[0], t->A[1], t->A[2], s)) != cudaSuccess) return e;
   if ((e = tc_plan_launch_range(t->lead, t->power_index, 1, 1, 0, 1.f, 0.f, status, s)) != cudaSuccess) return e;
   if ((e = tc_plan_launch_range(t->tail, t->power_index, 1, 1, 0, 1.f, 0.f, status, s)) != cudaSuccess) return e;
   *out = t->Df;
@@ -332,7 +343,7 @@ void project(Sweep& q, int64_t jp, int64_t wp, int64_t jt, int64_t wt) {
   const int64_t k = q.k;
   if (q.tc && q.first && tc_node(wp, wt)) {
     q.err = qr_tc_project(q.tc, q.node++, q.A, k, jp, wp, jt, wt, q.status, q.s);
-    q.launches += 13;
+    q.launches += 12;
     return;
   }
   // fewer tiles of 64 x 64 than two per SM: split the contraction until there are four

@@ -154,9 +154,9 @@ typedef enum {
 } br_buf;
 
 /* Bytes of device memory br_create requests for these layers (state, ring, operand shadows and
- * scratch).  If that request is refused and a layout with fewer concurrent refresh lanes is smaller,
- * br_create asks once more, for that one (a refresh takes longer; fp32 layers are grouped into other
- * launches, which may round differently).  Host only.  App. H's
+ * scratch).  If that request is refused and a layout with fewer concurrent refreshes is smaller,
+ * br_create asks once more, for that one (a refresh takes longer; fp32 layers and power products are grouped into
+ * other launches, which may round differently).  Host only.  App. H's
  * table is overhead_bytes: rotation matrices plus factor buffers in fp32, summed over layers (either
  * out pointer may be NULL). */
 BR_API br_status br_state_bytes(const br_layer_desc* layers, int n_layers, const br_hparams* hp,

@@ -127,9 +127,9 @@ struct br_handle {
   struct Side { cudaStream_t stream = nullptr; cudaEvent_t done = nullptr; };
   Side group_side[2];                     // beside the handle's stream (created when there is a pool)
   bool use_graphs = true;                 // cleared when a capture fails (BR_REFRESH_GRAPHS=0 switches it off)
-  // Eight streams in all, the default number of hardware queues.  When the largest order is one that a single
-  // cluster factorises, every lane holds it: a cluster leaves 132 SMs to the others (ten steps and the 32 bases of a d = 384 decoder:
-  // 27.2 -> 16.2 ms against three full-size lanes).  From order 2048 on three lanes do, whose products fill the GPU, and
+  // Lanes serve the orders from 1600 on and, below, the bases of S = 1st layers.  Eight streams in all, the default number of
+  // hardware queues.  When the largest order is one that a single cluster factorises, every lane holds it (a cluster leaves 132
+  // SMs to the others).  From order 2048 on three lanes do, whose products fill the GPU, and
   // between the two six (sixteen bases of order 1792: 24.0 ms on three lanes, 19.6 on four, 17.6 on six); the others hold
   // only the small orders (at most 1/sqrt(2) of the largest, S = 2nd).
   static constexpr int kBigLanes = 3;       // default number of full-size lanes from order 2048 on (BR_REFRESH_LANES: 1..6)
@@ -208,7 +208,9 @@ inline int64_t z_slice(int64_t k, int64_t other) {
 
 constexpr size_t kPoolOfLargest = 12, kPoolCompact = 3;
 constexpr int64_t kSmallGroup = 128;
-// From here on a power product takes less time in digits on the int8 tensor cores than on the fp64 unit.
+// From here on a power product takes less time in digits on the int8 tensor cores than on the fp64 unit (splitting included, us, four
+// bases: order 512 97 and 55, 640 127 and 107, 768 144 and 155, 896 267 and 262, 1024 285 and 387, 1280 500 and 726; eight of
+// 1536 1421 and 2333).
 constexpr int64_t kOzMinOrder = 1024;
 // A side whose refresh is part of the grouped launches, and what it needs of the pool.
 inline bool grouped_side(const Layer& L, int64_t k) { return L.d.src == BR_SRC_SECOND && qr_one_launch(k); }

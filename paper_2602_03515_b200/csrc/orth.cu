@@ -7,7 +7,7 @@
 // Here one cluster of up to 16 CTAs walks the whole chain of a basis, or of a range of its columns, in one launch, and the
 // steps are separated by the cluster's hardware barrier; the second sweep and the completion of a
 // rank-deficient product are branches instead of cancelled launches.  Measured, one basis alone: order 64
-// 32 us, 384 240 us, 1024 1.3 ms, 1536 3.9 ms; stand-alone Power() at order 384 1368 -> 267 us.
+// 31 us, 384 205 us, 1024 1.26 ms, 1536 3.6 ms; stand-alone Power() at order 384 1368 -> 233 us.
 //
 //  * Rows of A are dealt to the CTAs in contiguous chunks.  A CTA computes its rows' share of a panel's
 //    Gram matrix and applies R^-1 and the projections to its own rows only, so these steps need no

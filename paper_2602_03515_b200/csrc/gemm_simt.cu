@@ -16,7 +16,8 @@
 // tile's step is the shortest), 64 x 64 up to a few waves, 128 x 128 (8 x 8 per thread, half the shared-memory
 // reads per multiply-add) above.  With at most four tiles of 32 x 32 per SM a step is bound by the latency of
 // its loads, and four groups of 64 threads take a quarter of the contraction each: the dual launch of the four
-// ragged layers 54 -> 30 us, the others 30 -> 16 us.
+// ragged layers 54 -> 30 us, the others 30 -> 16 us.  The orientations of the operands are compile-time values (four bodies a
+// kernel): factors and first sides of those layers 36.7 -> 26 us, back rotation 11 -> 8.7, weight write 21 -> 16.5.
 #include "br_internal.h"
 
 namespace br {
@@ -31,49 +32,69 @@ struct GroupArgs {
   int n;
 };
 
+// A thread's share of an operand tile of BX rows (columns) by BK steps of the contraction.  T: the tile index is the
+// contiguous one, x(i, kk) = X[kk * ld + i]; otherwise x(i, kk) = X[i * ld + kk].  Everything that does not change from stage to
+// stage is worked out once (with the orientation a runtime value and the address formed per entry, index arithmetic
+// was half of all instructions).
+template <bool T, int BX, int NT>
+struct Operand {
+  static constexpr int L = BX * BK / NT, DI = T ? 0 : NT / BK, DK = T ? NT / BX : 0;
+  static_assert(NT % BX == 0 && NT % BK == 0, "a thread's entries differ in one index only");
+  const float* at;
+  int64_t step, next;
+  int i, k;
+  unsigned rows;                        // bit u: entry u lies inside the matrix
+  __device__ __forceinline__ Operand(const float* X, int64_t ld, int t, int x0, int extent, int kbeg) {
+    i = T ? t % BX : t / BK; k = T ? t / BX : t % BK;
+    at = X + (T ? (int64_t)(kbeg + k) * ld + x0 + i : (int64_t)(x0 + i) * ld + kbeg + k);
+    step = T ? DK * ld : DI * ld; next = T ? BK * ld : BK;
+    rows = 0;
+#pragma unroll
+    for (int u = 0; u < L; ++u) rows |= (unsigned)(x0 + i + u * DI < extent) << u;
+  }
+  __device__ __forceinline__ void fetch(float (&v)[L], int left) {      // left: steps of the contraction from here on
+#pragma unroll
+    for (int u = 0; u < L; ++u) v[u] = ((rows >> u) & 1) && k + u * DK < left ? at[u * step] : 0.f;
+    at += next;
+  }
+  template <typename S> __device__ __forceinline__ void put(S& s, const float (&v)[L]) const {
+#pragma unroll
+    for (int u = 0; u < L; ++u) s[k + u * DK][i + u * DI] = v[u];
+  }
+};
+
+template <int BM, int BN, bool DUAL, int KS> struct Area {
+  static constexpr int FA = BK * (BM + 4), FB = BK * (BN + 4);
+  __align__(16) float v[KS][(DUAL ? 2 : 1) * (FA + FB)];
+};
+
 // KS groups of NT threads share one tile's contraction (a range of it each) and add up their sums at the end.
-template <int BM, int BN, int TM, int TN, bool DUAL, int KS>
-__global__ void __launch_bounds__(KS * (BM / TM) * (BN / TN))
-k_simt_group(const __grid_constant__ GroupArgs ga) {
+template <int BM, int BN, int TM, int TN, bool DUAL, int KS, bool TA, bool TB>
+__device__ __forceinline__ void simt_tile(const SimtProblem& p, int tile, Area<BM, BN, DUAL, KS>& area_) {
   constexpr int NT = (BM / TM) * (BN / TN), NP = DUAL ? 2 : 1;
-  constexpr int LA = BM * BK / NT, LB = BN * BK / NT, FA = BK * (BM + 4), FB = BK * (BN + 4);
+  constexpr int FA = Area<BM, BN, DUAL, KS>::FA, FB = Area<BM, BN, DUAL, KS>::FB;
   static_assert(KS == 1 || (TM == 4 && TN == 4 && KS == TM && NP * TM * NT * 4 <= NP * (FA + FB)), "partial sums fit the operand area");
-  __shared__ __align__(16) float area[KS][NP * (FA + FB)];
+  auto& area = area_.v;
   const int group = KS == 1 ? 0 : (int)threadIdx.x / NT;
   float(*As)[BK][BM + 4] = reinterpret_cast<float(*)[BK][BM + 4]>(area[group]);
   float(*Bs)[BK][BN + 4] = reinterpret_cast<float(*)[BK][BN + 4]>(area[group] + NP * FA);
   auto sync = [&] {      // the groups run at their own pace
     if (KS == 1) __syncthreads(); else asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(NT) : "memory");
   };
-  int pi = 0;
-  while (pi + 1 < ga.n && (int)blockIdx.x >= ga.tile_begin[pi + 1]) ++pi;
-  const SimtProblem& p = ga.p[pi];
-  const int tiles_n = (p.N + BN - 1) / BN, tile = (int)blockIdx.x - ga.tile_begin[pi];
+  const int tiles_n = (p.N + BN - 1) / BN;
   const int m0 = tile / tiles_n * BM, n0 = tile % tiles_n * BN;
   const int M = p.M, N = p.N;
   const int kc = KS == 1 ? p.K : (p.K + KS * BK - 1) / (KS * BK) * BK, kbeg = min(p.K, group * kc), K = min(p.K, kbeg + kc);
   const int t = threadIdx.x % NT, tx = t % (BN / TN), ty = t / (BN / TN);
 
-  float ra[NP][LA], rb[NP][LB];
-  auto fetch = [&](int k0) {
-#pragma unroll
-    for (int u = 0; u < LA; ++u) {
-      const int idx = t + u * NT;
-      const int i = p.ta ? idx % BM : idx / BK, kk = p.ta ? idx / BM : idx % BK;
-      const bool ok = m0 + i < M && k0 + kk < K;
-      const int64_t at = p.ta ? (int64_t)(k0 + kk) * p.lda + m0 + i : (int64_t)(m0 + i) * p.lda + k0 + kk;
-#pragma unroll
-      for (int z = 0; z < NP; ++z) ra[z][u] = ok ? p.A[z][at] : 0.f;
-    }
-#pragma unroll
-    for (int u = 0; u < LB; ++u) {
-      const int idx = t + u * NT;
-      const int j = p.tb ? idx / BK : idx % BN, kk = p.tb ? idx % BK : idx / BN;
-      const bool ok = n0 + j < N && k0 + kk < K;
-      const int64_t at = p.tb ? (int64_t)(n0 + j) * p.ldb + k0 + kk : (int64_t)(k0 + kk) * p.ldb + n0 + j;
-#pragma unroll
-      for (int z = 0; z < NP; ++z) rb[z][u] = ok ? p.B[z][at] : 0.f;
-    }
+  typedef Operand<TA, BM, NT> OpA;
+  typedef Operand<!TB, BN, NT> OpB;
+  OpA a0(p.A[0], p.lda, t, m0, M, kbeg), a1(p.A[NP - 1], p.lda, t, m0, M, kbeg);
+  OpB b0(p.B[0], p.ldb, t, n0, N, kbeg), b1(p.B[NP - 1], p.ldb, t, n0, N, kbeg);
+  float ra[NP][OpA::L], rb[NP][OpB::L];
+  auto fetch = [&](int left) {
+    a0.fetch(ra[0], left); b0.fetch(rb[0], left);
+    if (DUAL) { a1.fetch(ra[NP - 1], left); b1.fetch(rb[NP - 1], left); }
   };
   float acc[NP][TM][TN];
 #pragma unroll
@@ -84,24 +105,12 @@ k_simt_group(const __grid_constant__ GroupArgs ga) {
       for (int j = 0; j < TN; ++j) acc[z][i][j] = 0.f;
   // thread rows ty * 4 + i % 4 (+ BM / 2 for i >= 4), columns likewise: 16-byte reads, neighbours adjacent
   auto sub = [](int base, int i, int half) { return (i < 4 ? 0 : half) + base * 4 + (i & 3); };
-  if (kbeg < K) fetch(kbeg);
+  if (kbeg < K) fetch(K - kbeg);
   for (int k0 = kbeg; k0 < K; k0 += BK) {
-#pragma unroll
-    for (int u = 0; u < LA; ++u) {
-      const int idx = t + u * NT;
-      const int i = p.ta ? idx % BM : idx / BK, kk = p.ta ? idx / BM : idx % BK;
-#pragma unroll
-      for (int z = 0; z < NP; ++z) As[z][kk][i] = ra[z][u];
-    }
-#pragma unroll
-    for (int u = 0; u < LB; ++u) {
-      const int idx = t + u * NT;
-      const int j = p.tb ? idx / BK : idx % BN, kk = p.tb ? idx % BK : idx / BN;
-#pragma unroll
-      for (int z = 0; z < NP; ++z) Bs[z][kk][j] = rb[z][u];
-    }
+    a0.put(As[0], ra[0]); b0.put(Bs[0], rb[0]);
+    if (DUAL) { a1.put(As[NP - 1], ra[NP - 1]); b1.put(Bs[NP - 1], rb[NP - 1]); }
     sync();
-    if (k0 + BK < K) fetch(k0 + BK);
+    if (k0 + BK < K) fetch(K - k0 - BK);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk)
 #pragma unroll
@@ -157,6 +166,21 @@ k_simt_group(const __grid_constant__ GroupArgs ga) {
         p.C[at] = v;
       }
     }
+  }
+}
+
+template <int BM, int BN, int TM, int TN, bool DUAL, int KS>
+__global__ void __launch_bounds__(KS * (BM / TM) * (BN / TN))
+k_simt_group(const __grid_constant__ GroupArgs ga) {
+  __shared__ Area<BM, BN, DUAL, KS> area;
+  int pi = 0;
+  while (pi + 1 < ga.n && (int)blockIdx.x >= ga.tile_begin[pi + 1]) ++pi;
+  const SimtProblem& p = ga.p[pi];
+  const int tile = (int)blockIdx.x - ga.tile_begin[pi];
+  if (p.ta) {
+    if (p.tb) simt_tile<BM, BN, TM, TN, DUAL, KS, true, true>(p, tile, area); else simt_tile<BM, BN, TM, TN, DUAL, KS, true, false>(p, tile, area);
+  } else {
+    if (p.tb) simt_tile<BM, BN, TM, TN, DUAL, KS, false, true>(p, tile, area); else simt_tile<BM, BN, TM, TN, DUAL, KS, false, false>(p, tile, area);
   }
 }
 

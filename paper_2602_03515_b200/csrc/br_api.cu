@@ -1040,8 +1040,8 @@ br_status br_create(br_handle** out, const br_layer_desc* layers, int n_layers, 
     if ((e = cudaEventCreateWithFlags(&g.done, cudaEventDisableTiming)) != cudaSuccess) return fail("cudaEventCreate", e);
   }
   if ((e = cudaEventCreateWithFlags(&h->ev_begin, cudaEventDisableTiming)) != cudaSuccess) return fail("cudaEventCreate", e);
-  // The side stream of a step has the highest priority: the CTAs of a launch that waits for SMs behind a running one (the
-  // next phase of the step) would otherwise keep back those of the copies, which fit beside the running ones.
+  // The side stream of a step has the highest priority, so that the copies' CTAs take their places beside the running phase before
+  // the next one is dispatched.
   int least = 0, greatest = 0;
   if ((e = cudaDeviceGetStreamPriorityRange(&least, &greatest)) != cudaSuccess) return fail("cudaDeviceGetStreamPriorityRange", e);
   if ((e = cudaStreamCreateWithPriority(&h->copy_stream, cudaStreamNonBlocking, greatest)) != cudaSuccess) return fail("cudaStreamCreate", e);

@@ -344,10 +344,6 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
       asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
   }
-  // Up to here nothing of the launches before was touched: a launch may begin while the last CTAs of the one before it
-  // are still working (programmatic dependent launch), and its CTAs find their set-up done when those have finished.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // an earlier launch failed: nothing to do
   if (threadIdx.x == 0) dead_word = (*reinterpret_cast<volatile int*>(status) < 0) ? 1u : 0u;
   tc_fence_before();
@@ -1180,9 +1176,8 @@ void tc_plan_destroy(TcPlan* p) {
 
 double tc_plan_flops(const TcPlan* p) { return p ? p->flops : 0.0; }
 
-namespace {
-cudaError_t launch_range(TcPlan* p, int first, int count, long long calls, int tau, float dyn_alpha, float dyn_beta, int* status_word,
-                         cudaStream_t s, bool overlap) {
+cudaError_t tc_plan_launch_range(TcPlan* p, int first, int count, long long calls, int tau, float dyn_alpha,
+                                 float dyn_beta, int* status_word, cudaStream_t s) {
   if (first < 0 || count < 1 || first + count > p->n) return cudaErrorInvalidValue;
   const int t0 = p->tile_begin[first], t1 = p->tile_begin[first + count];
   const int tiles = t1 - t0;
@@ -1191,20 +1186,14 @@ cudaError_t launch_range(TcPlan* p, int first, int count, long long calls, int t
   const int smem_bytes = p->fold ? SMEM_BYTES_FOLD : p->shared ? SMEM_BYTES : SMEM_BYTES_PLAIN;
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   const bool whole = first == 0 && count == p->n;
-  cfg.attrs = attr;
-  if (overlap) {
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = 1;
-  }
   if (p->pair) {
     const int units = whole ? p->units : tiles < p->max_pairs ? tiles : p->max_pairs;
     cfg.gridDim = dim3(2u * (unsigned)units);
-    cudaLaunchAttribute& a = attr[cfg.numAttrs++];
-    a.id = cudaLaunchAttributeClusterDimension;
-    a.val.clusterDim.x = 2; a.val.clusterDim.y = 1; a.val.clusterDim.z = 1;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
   } else {
     cfg.gridDim = dim3((unsigned)(whole ? p->units : tiles < p->sm_count ? tiles : p->sm_count));
   }
@@ -1216,17 +1205,9 @@ cudaError_t launch_range(TcPlan* p, int first, int count, long long calls, int t
                             dyn_beta, status_word);
 }
 
-}  // namespace
-
-cudaError_t tc_plan_launch_range(TcPlan* p, int first, int count, long long calls, int tau, float dyn_alpha,
-                                 float dyn_beta, int* status_word, cudaStream_t s) {
-  return launch_range(p, first, count, calls, tau, dyn_alpha, dyn_beta, status_word, s, false);
-}
-
-// The phases of a step follow one another on the stream: each launch's set-up overlaps the tail of the one before.
 cudaError_t tc_plan_launch(TcPlan* p, long long calls, int tau, float dyn_alpha, float dyn_beta,
                            int* status_word, cudaStream_t s) {
-  return launch_range(p, 0, p->n, calls, tau, dyn_alpha, dyn_beta, status_word, s, true);
+  return tc_plan_launch_range(p, 0, p->n, calls, tau, dyn_alpha, dyn_beta, status_word, s);
 }
 
 cudaError_t tc_wait_probe(uint64_t limit_ns, int* status_word, cudaStream_t s) {

@@ -208,9 +208,9 @@ inline int64_t z_slice(int64_t k, int64_t other) {
 
 constexpr size_t kPoolOfLargest = 12, kPoolCompact = 3;
 constexpr int64_t kSmallGroup = 128;
-// From here on a power product takes less time in digits on the int8 tensor cores than on the fp64 unit (splitting included, us, four
-// bases: order 512 97 and 55, 640 127 and 107, 768 144 and 155, 896 267 and 262, 1024 285 and 387, 1280 500 and 726; eight of
-// 1536 1421 and 2333).
+// From here on a power product takes less time in digits on the int8 tensor cores than on the fp64 unit.  Refreshes, us, in digits and on
+// the fp64 unit: four bases of order 512 453 and 398, 640 680 and 647, 768 900 and 887, 896 1265 and 1255, 1024 1560 and 1640,
+// 1280 2994 and 3250, 1536 4405 and 4950; eight of 1024 2468 and 2658, 1152 3797 and 4075, 1536 6985 and 8085; two of 1024 1430 and 1458.
 constexpr int64_t kOzMinOrder = 1024;
 // A side whose refresh is part of the grouped launches, and what it needs of the pool.
 inline bool grouped_side(const Layer& L, int64_t k) { return L.d.src == BR_SRC_SECOND && qr_one_launch(k); }
@@ -586,7 +586,7 @@ br_status refresh_group(br_handle* h, const GroupSide* v, int n, char* pool, siz
     // (longest first: the products in digits are the front of the list)
     std::vector<OzProduct> oz;
     for (const OrthJob& j : jobs)
-      if (oz_bytes && j.k >= kOzMinOrder) oz.push_back({j.F, j.Qprev, j.A, j.k, j.k, j.k});
+      if (oz_bytes && j.k >= kOzMinOrder) oz.push_back({j.F, j.Qprev, j.A, j.k, j.k, j.k, j.F, j.k + 1});
     const int n_oz = (int)oz.size(), n_rest = (int)jobs.size() - n_oz;
     for (int it = 0; it < h->hp.power_iters; ++it) {
       if (n_oz) {

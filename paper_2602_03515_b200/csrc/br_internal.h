@@ -233,8 +233,9 @@ cudaError_t product64(int ta, int64_t M, int64_t N, int64_t K, double alpha, con
 // ---------------------------------------------------------------------------------------------
 // fp64-accurate products of fp32 matrices on the int8 tensor cores (oz.cu)
 // ---------------------------------------------------------------------------------------------
-// C (M x N, fp64) = X (M x K) Y (K x N), all row-major and contiguous
-struct OzProduct { const float *X, *Y; double* C; int64_t M, N, K; };
+// C (M x N, fp64) = X (M x K) Y (K x N), all row-major and contiguous.  diag (or null): the diagonal of a positive semidefinite matrix
+// that bounds the entries of X, |x_ik| <= sqrt(d_i d_k), `stride` apart; the columns of X are balanced by it.
+struct OzProduct { const float *X, *Y; double* C; int64_t M, N, K; const float* diag; int64_t stride; };
 bool oz_eligible(int64_t M, int64_t N, int64_t K);
 size_t oz_scratch_bytes(int64_t M, int64_t N, int64_t K);
 // As many products at a time as the scratch (256-byte aligned) holds, which must be one at least.

@@ -2,8 +2,8 @@
 through a refresh: orders that no tile divides, rows of very different size, and what is not finite.
 
 The factors are graded: eigenvalues from 1 down to 1e-6, and a basis that is close to their eigenvectors, so that the trailing
-columns of F Q are what is left of a cancellation a million times their size.  An error of 2^-50 of the scale of a
-row and a column (what the digits leave out) is then 1e-9 of such a column, below the rounding of the basis to fp32 (6e-8); single
+columns of F Q are what is left of a cancellation a million times their size.  What the digits leave out, at most 2^-59 times the order of
+the largest entries of a row and a column, 2^-48, is then 4e-9 of such a column, below the rounding of the basis to fp32 (6e-8); single
 precision anywhere in the product would leave 6e-2.  Reference: LAPACK QR of the float64 product; asserted as in
 test_gpu_orth_cluster.py, 1.2e-7."""
 import numpy as np

@@ -372,6 +372,18 @@ void init_layers(br_handle* h, const br_layer_desc* layers, int n_layers) {
 
 inline void count(br_handle* h, int n = 1) { h->stats.launches += n; }
 
+// The handle's stream waits for an internal one that a call forked from it, whatever became of the call (`st`): nothing of it
+// is still running there once the handle's stream has passed this point.
+br_status join_stream(br_handle* h, cudaStream_t side, cudaEvent_t done, const char* what, br_status st) {
+  cudaError_t e = h->stats.inject() ? cudaErrorLaunchFailure : cudaEventRecord(done, side);
+  if (e == cudaSuccess) e = h->stats.inject() ? cudaErrorLaunchFailure : cudaStreamWaitEvent(h->stream, done, 0);
+  if (e == cudaSuccess) return st;
+  cudaStreamSynchronize(side);                         // no event to wait for: wait here
+  if (st < 0) return st;
+  h->err = format("joining %s failed: %s", what, cudaGetErrorString(e));
+  return BR_ERR_CUDA;
+}
+
 const void* ring_slot_ptr(const Layer& L, int64_t slot) {
   return L.ring + (size_t)slot * L.slot_stride;
 }
@@ -699,20 +711,10 @@ br_status refresh_layers(br_handle* h, const int* ids, int n_ids) {
     }
   // the lanes forked from the handle's stream: join them again whatever happened above, so that
   // nothing of this call is still running on an internal stream once the handle's stream has passed it
-  auto join = [&](cudaStream_t side, cudaEvent_t done) {
-    cudaError_t je = h->stats.inject() ? cudaErrorLaunchFailure : cudaEventRecord(done, side);
-    if (je == cudaSuccess) je = h->stats.inject() ? cudaErrorLaunchFailure : cudaStreamWaitEvent(h->stream, done, 0);
-    if (je == cudaSuccess) return;
-    cudaStreamSynchronize(side);                       // no event to wait for: wait here
-    if (failed == BR_OK) {
-      h->err = format("joining a refresh lane failed: %s", cudaGetErrorString(je));
-      failed = BR_ERR_CUDA;
-    }
-  };
   if (!jobs.empty())
-    for (int i = 1; i < nl; ++i) join(h->lanes[i].stream, h->lanes[i].done);
+    for (int i = 1; i < nl; ++i) failed = join_stream(h, h->lanes[i].stream, h->lanes[i].done, "a refresh lane", failed);
   for (const Batch& bt : batches)
-    if (bt.side) join(bt.side->stream, bt.side->done);
+    if (bt.side) failed = join_stream(h, bt.side->stream, bt.side->done, "a grouped refresh", failed);
   if (failed != BR_OK) return failed;
   h->stats.prof.end(span, h->stream, h->stats.gemm_flops - f0);
   BR_CUDA(h, cudaMemcpyAsync(h->h_cond, h->d_cond, sizeof(int) * h->cond_known.size(), cudaMemcpyDeviceToHost, h->stream));
@@ -1197,16 +1199,19 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
       BR_CUDA(h, cudaEventRecord(h->ev_consumed, h->stream));
       BR_CUDA(h, cudaStreamWaitEvent(ss, h->ev_consumed, 0));
     }
-    BR_CUDA(h, small_step(small.data(), (int)small.size(), hp.lr, hp.beta1, hp.beta2, hp.eps, hp.weight_decay,
-                          hp.beta_factor < 0.f ? hp.beta2 : hp.beta_factor, ss));
-    count(h, ((int)small.size() + 23) / 24);
+    const bool tiny = std::all_of(small.begin(), small.end(), tiny_step_eligible);    // (among larger ones they go along with those)
+    for (size_t at = 0; at < small.size() && st == BR_OK; at += kSmallJobs) {
+      const int n = (int)std::min<size_t>(kSmallJobs, small.size() - at);
+      const cudaError_t e = h->stats.inject() ? cudaErrorLaunchFailure
+                                              : small_step(small.data() + at, n, tiny, hp.lr, hp.beta1, hp.beta2, hp.eps, hp.weight_decay,
+                                                           hp.beta_factor < 0.f ? hp.beta2 : hp.beta_factor, ss);
+      if (e == cudaSuccess) { count(h); continue; }
+      h->err = format("update of the small matrices failed: %s", cudaGetErrorString(e));
+      st = BR_ERR_CUDA;
+    }
   }
-  if (!simt_ids.empty()) st = update_layers_simt(h, simt_ids, G, GS);
-  if (beside) {
-    // (also on a failed step: the side stream must not outlive the caller's view of this call)
-    cudaEventRecord(h->ev_copied, h->copy_stream);
-    cudaStreamWaitEvent(h->stream, h->ev_copied, 0);
-  }
+  if (!simt_ids.empty() && st == BR_OK) st = update_layers_simt(h, simt_ids, G, GS);
+  if (beside) st = join_stream(h, h->copy_stream, h->ev_copied, "the side stream", st);
   if (st != BR_OK) return st;
   if (h->tc) {
     struct StepCtx { br_handle* h; const void* const* grads; std::vector<char>* stored; bool copied; };
@@ -1237,15 +1242,12 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
     };
     const char* terr = nullptr;
     int rc = tc_step_run(h->tc, h->layers, G, h->calls, tau, hp, h->d_status, h->stream, &h->stats, cb, &terr);
-    if (sc.copied) {
-      // (also on a failed step: the side stream must not outlive the caller's view of this call)
-      cudaEventRecord(h->ev_copied, h->copy_stream);
-      cudaStreamWaitEvent(h->stream, h->ev_copied, 0);
-    }
+    if (sc.copied) st = join_stream(h, h->copy_stream, h->ev_copied, "the side stream", rc ? BR_ERR_CUDA : BR_OK);
     if (rc != 0) {
       if (terr) h->err = terr; else if (h->err.empty()) h->err = "tensor-core step failed";
       return rc < 0 ? (br_status)rc : BR_ERR_CUDA;
     }
+    if (st != BR_OK) return st;
   }
   // ---- store g_c in the ring (after every reader of the slot it may overwrite) --------------
   std::vector<CopyJob> copies;

@@ -139,7 +139,10 @@ struct SmallJob {
   float *M, *V2, *U, *V, *L, *R, *W;
   const void* grad; void* ring;            // this call's gradient, and the slot it is stored in (or null), which may be G
 };
-cudaError_t small_step(const SmallJob* jobs, int n, float lr, float beta1, float beta2, float eps, float weight_decay,
+// One launch for at most kSmallJobs matrices; tiny: all of the call's matrices are tiny_step_eligible.
+constexpr int kSmallJobs = 24;               // by value: 3 KB of launch parameters
+bool tiny_step_eligible(const SmallJob& j);
+cudaError_t small_step(const SmallJob* jobs, int n, bool tiny, float lr, float beta1, float beta2, float eps, float weight_decay,
                        float beta_factor, cudaStream_t s);
 
 // Debug canaries (BR_FLAG_DEBUG_CANARY): n guards of 256 bytes at byte offsets offs[] (DEVICE array) of the slab.

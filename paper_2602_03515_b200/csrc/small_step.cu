@@ -25,9 +25,8 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kMaxSmem = 220 * 1024;
-constexpr int kMaxJobs = 24;              // by value: 3 KB of launch parameters
 
-// NJ: 1 or kMaxJobs (3 KB of parameters make a launch longer on the host)
+// NJ: 1 or kSmallJobs (3 KB of parameters make a launch longer on the host)
 template <int NJ> struct SmallGroup { SmallJob j[NJ]; float lr, beta1, beta2, eps, decay, beta_factor; };
 
 __host__ __device__ inline int up4(int x) { return (x + 3) & ~3; }
@@ -434,20 +433,16 @@ cudaError_t launch(const SmallJob* jobs, int n, float lr, float beta1, float bet
 }
 }  // namespace
 
-cudaError_t small_step(const SmallJob* jobs, int n, float lr, float beta1, float beta2, float eps, float weight_decay,
+bool tiny_step_eligible(const SmallJob& j) { return tiny_eligible(j); }
+
+cudaError_t small_step(const SmallJob* jobs, int n, bool tiny, float lr, float beta1, float beta2, float eps, float weight_decay,
                        float beta_factor, cudaStream_t s) {
-  cudaError_t e = cudaSuccess;
-  const bool tiny = std::all_of(jobs, jobs + n, tiny_eligible);      // (among larger ones they go along in the launch of those)
-  for (int at = 0; at < n && e == cudaSuccess; at += kMaxJobs) {
-    const int cnt = n - at < kMaxJobs ? n - at : kMaxJobs;
-    if (tiny)
-      e = cnt == 1 ? launch_tiny<1>(jobs + at, 1, lr, beta1, beta2, eps, weight_decay, beta_factor, s)
-                   : launch_tiny<kMaxJobs>(jobs + at, cnt, lr, beta1, beta2, eps, weight_decay, beta_factor, s);
-    else
-      e = cnt == 1 ? launch<1>(jobs + at, 1, lr, beta1, beta2, eps, weight_decay, beta_factor, s)
-                   : launch<kMaxJobs>(jobs + at, cnt, lr, beta1, beta2, eps, weight_decay, beta_factor, s);
-  }
-  return e;
+  if (n < 1 || n > kSmallJobs) return cudaErrorInvalidValue;
+  if (tiny)
+    return n == 1 ? launch_tiny<1>(jobs, 1, lr, beta1, beta2, eps, weight_decay, beta_factor, s)
+                  : launch_tiny<kSmallJobs>(jobs, n, lr, beta1, beta2, eps, weight_decay, beta_factor, s);
+  return n == 1 ? launch<1>(jobs, 1, lr, beta1, beta2, eps, weight_decay, beta_factor, s)
+                : launch<kSmallJobs>(jobs, n, lr, beta1, beta2, eps, weight_decay, beta_factor, s);
 }
 
 }  // namespace br

@@ -161,6 +161,51 @@ def test_failed_enqueue_leaves_the_integer_state_untouched(prec):
     torch.cuda.synchronize()
 
 
+def test_side_stream_is_joined_whatever_failed():
+    """A call on more small fp32 matrices than one launch takes, beside a larger one: wherever it fails (the second launch of the
+    small ones, the larger one's, the join itself), the handle's stream has passed everything the call put on its side stream
+    when it goes on.  A delay on the handle's stream in front of the call holds back all of its work, so that a copy of the weights
+    enqueued behind the call would overtake an update that is not joined."""
+    import torch
+    import paper_2602_03515_b200 as br
+    specs = [LayerSpec("s%d" % i, 64, 32, GEOM_BI, SRC_SECOND, 1) for i in range(30)] + [LayerSpec("L", 200, 130, GEOM_BI, SRC_SECOND, 1)]
+    errors = []
+    for countdown in range(20):
+        ws = [torch.randn(s.m, s.n, device="cuda") * 0.02 for s in specs]
+        opt = br.BasisRotation(specs, ws, grad_dtype="f32", gemm_prec=br.BR_GEMM_FP32, freq=100)
+        grads = [torch.randn(s.m, s.n, device="cuda") * 0.01 for s in specs]
+        try:
+            for _ in range(2):
+                opt.step(grads, 1)
+            assert opt.sync_status() == br.BR_OK
+            before = [w.clone() for w in ws]
+            c_before = [opt.counters(i) for i in range(len(specs))]
+            torch.cuda.synchronize()
+            torch.cuda._sleep(4_000_000)                 # about 2 ms
+            br.br_debug_inject(opt.handle, br.BR_INJECT_LAUNCH_FAILURE, countdown)
+            try:
+                opt.step(grads, 1)
+                failed = False
+            except br.BrError as e:
+                assert e.status == br.BR_ERR_CUDA
+                errors.append(str(e))
+                failed = True
+            br.br_debug_inject(opt.handle, br.BR_INJECT_NONE, 0)
+            behind = [w.clone() for w in ws]
+            torch.cuda.synchronize()
+            assert all(torch.equal(a, w) for a, w in zip(behind, ws)), countdown
+            if failed:
+                assert [opt.counters(i) for i in range(len(specs))] == c_before
+            else:
+                assert not any(torch.equal(a, w) for a, w in zip(before, ws))
+                break
+        finally:
+            opt.close()
+    assert not failed
+    # the first launch of the small matrices went out, the second did not; and a failed join is an error
+    assert sum("small matrices" in e for e in errors) == 2 and sum("joining the side stream" in e for e in errors) == 2, errors
+
+
 def test_failed_enqueue_inside_forced_refresh():
     import torch
     import paper_2602_03515_b200 as br

@@ -1192,7 +1192,8 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
   }
   // the small matrices beside the grouped launches of the others, where there are any (the update of four ragged layers,
   // one of them small: 146 -> 133 us)
-  const bool beside = !small.empty() && !simt_ids.empty();
+  static const bool side_stream = !(std::getenv("BR_RING_SIDE_STREAM") && std::getenv("BR_RING_SIDE_STREAM")[0] == '0');
+  const bool beside = side_stream && !small.empty() && !simt_ids.empty();
   if (!small.empty()) {
     cudaStream_t ss = beside ? h->copy_stream : h->stream;
     if (beside) {
@@ -1221,8 +1222,7 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
     cb.refresh = [](void* ctx, const int* ids, int n) -> int {
       return (int)refresh_layers(static_cast<StepCtx*>(ctx)->h, ids, n);
     };
-    static const bool side_copies = !(std::getenv("BR_RING_SIDE_STREAM") && std::getenv("BR_RING_SIDE_STREAM")[0] == '0');
-    if (side_copies) cb.consumed = [](void* ctx, const int* ids, int n) -> int {
+    if (side_stream) cb.consumed = [](void* ctx, const int* ids, int n) -> int {
       StepCtx* c = static_cast<StepCtx*>(ctx);
       br_handle* h = c->h;
       BR_CUDA(h, cudaEventRecord(h->ev_consumed, h->stream));

@@ -42,3 +42,34 @@ def test_refresh_without_tensor_cores():
 
 def test_refresh_with_tensor_cores_from_order_1024():
     _run({"BR_QR_TC_MIN_ORDER": "1024"}, ["tests/test_gpu_full_size.py::test_refresh_order_1024_against_oracle_power"])
+
+
+def test_steps_without_the_side_stream():
+    """BR_RING_SIDE_STREAM=0 keeps a step on the handle's stream: ring copies, and small matrices beside larger ones.  The fault
+    injection counts the CUDA calls of a step: none of them records an event or waits for one."""
+    _run({"BR_RING_SIDE_STREAM": "0"}, ["tests/test_gpu_parity_bf16.py", "-k", "not checkpoint"])
+    code = """if True:
+        import torch
+        import paper_2602_03515_b200 as br
+        from workloads import LayerSpec
+        errors = []
+        for prec, dt, shapes in ((br.BR_GEMM_FP32, torch.float32, [(64, 32), (200, 130)]), (br.BR_GEMM_BF16, torch.bfloat16, [(128, 136)])):
+            specs = [LayerSpec("w%d" % i, m, n, br.BR_GEOM_BILATERAL, br.BR_SRC_SECOND, 1) for i, (m, n) in enumerate(shapes)]
+            for countdown in range(60):
+                opt = br.BasisRotation(specs, [torch.zeros(m, n, device="cuda") for m, n in shapes], gemm_prec=prec, freq=100,
+                                       grad_dtype="f32" if dt == torch.float32 else "bf16")
+                g = [(0.01 * torch.randn(m, n, device="cuda")).to(dt) for m, n in shapes]
+                opt.step(g, 1)
+                br.br_debug_inject(opt.handle, br.BR_INJECT_LAUNCH_FAILURE, countdown)
+                try:
+                    opt.step(g, 1)
+                    break
+                except br.BrError as e:
+                    errors.append(str(e))
+                finally:
+                    br.br_debug_inject(opt.handle, br.BR_INJECT_NONE, 0)
+                    opt.close()
+        assert len(errors) > 8 and not any("Event" in e or "join" in e for e in errors), errors
+    """
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, BR_RING_SIDE_STREAM="0"), capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]

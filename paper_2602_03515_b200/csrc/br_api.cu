@@ -1238,6 +1238,7 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
       if (copies.empty()) return (int)BR_OK;
       c->copied = true;
       BR_CUDA(h, ring_copy(copies.data(), (int)copies.size(), true, h->copy_stream));
+      count(h, ((int)copies.size() + kElemGroup - 1) / kElemGroup);
       return (int)BR_OK;
     };
     const char* terr = nullptr;
@@ -1259,7 +1260,12 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
     if (bytes >= kCopyAlone) BR_CUDA(h, cudaMemcpyAsync(slot, grads[i], bytes, cudaMemcpyDeviceToDevice, h->stream));
     else copies.push_back({grads[i], slot, bytes});
   }
-  if (!copies.empty()) BR_CUDA(h, ring_copy(copies.data(), (int)copies.size(), false, h->stream));
+  if (copies.size() == 1) {
+    BR_CUDA(h, cudaMemcpyAsync(copies[0].dst, copies[0].src, copies[0].bytes, cudaMemcpyDeviceToDevice, h->stream));
+  } else if (!copies.empty()) {
+    BR_CUDA(h, ring_copy(copies.data(), (int)copies.size(), false, h->stream));
+    count(h, ((int)copies.size() + kElemGroup - 1) / kElemGroup);
+  }
   return any ? BR_OK : BR_WARMUP;
 }
 

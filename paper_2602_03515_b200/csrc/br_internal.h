@@ -100,7 +100,7 @@ cudaError_t plain_adam(float* W, float* M, float* V, const void* G, int g_is_bf1
 
 // Matrices of one launch at most (by value).
 constexpr int kElemGroup = 64;
-// dst <- src (an even number of bytes; dst on a 16-byte boundary); beside: one CTA per SM, next to contraction launches
+// dst <- src (an even number of bytes, both on 16-byte boundaries); beside: one CTA per SM, next to contraction launches
 struct CopyJob { const void* src; void* dst; size_t bytes; };
 cudaError_t ring_copy(const CopyJob* jobs, int n, bool beside, cudaStream_t s);
 // F[j][i] <- F[i][j] for the 32 x 32 blocks (j, i) strictly below the diagonal of the k x k matrix F.

@@ -326,10 +326,10 @@ __global__ void __launch_bounds__(kCopyThreads, 6) k_ring_copy(const __grid_cons
       const CopyJob& j = a.j[job];
       const size_t off = (size_t)(at - a.begin[job]) * 16;
       const char* s = static_cast<const char*>(j.src) + off;
-      if (reinterpret_cast<uintptr_t>(s) % 16 == 0 && off + 16 <= j.bytes) {
+      if (off + 16 <= j.bytes) {
         v[u] = __ldg(reinterpret_cast<const uint4*>(s));
         d[u] = reinterpret_cast<uint4*>(static_cast<char*>(j.dst) + off);
-      } else {                                 // (gradients are 2-byte aligned at least; the slots are 256-byte aligned)
+      } else {                                 // the last piece (gradients start on 16-byte boundaries, slots on 256-byte ones)
         for (size_t b = off; b < off + 16 && b < j.bytes; b += 2)
           *reinterpret_cast<uint16_t*>(static_cast<char*>(j.dst) + b) = *reinterpret_cast<const uint16_t*>(static_cast<const char*>(j.src) + b);
       }

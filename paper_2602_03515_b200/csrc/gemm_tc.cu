@@ -65,6 +65,7 @@
 #include <vector>
 
 #include "br_internal.h"
+#include "over_sqrt.h"
 #include "tc_ptx.h"
 
 namespace br {
@@ -222,13 +223,6 @@ __device__ __forceinline__ uint32_t make_idesc(int a_mn, int b_mn, int rows = BM
   d |= (uint32_t)(BN >> 3) << 17;
   d |= (uint32_t)(rows >> 4) << 24;
   return d;
-}
-
-// 1 / sqrt(x): the hardware's approximation and one Newton step, without the branches that sqrtf and a division take
-// for their special cases (an approximation of 0 or infinity stands as it is).
-__device__ __forceinline__ float inv_sqrt(float x) {
-  const float r = rsqrtf(x), n = fmaf(0.5f * r, fmaf(-(x * r), r, 1.0f), r);
-  return x > 0.0f && x < __int_as_float(0x7f800000) ? n : r;
 }
 
 __device__ __forceinline__ uint32_t pack2_bf16(float a, float b) {
@@ -725,8 +719,8 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
               *reinterpret_cast<float4*>(dm + it * step_d) = m;
               *reinterpret_cast<float4*>(dv + it * step_d) = q;
               uint2 o;
-              o.x = pack2_bf16(m.x * inv_sqrt(q.x + eps), m.y * inv_sqrt(q.y + eps));
-              o.y = pack2_bf16(m.z * inv_sqrt(q.z + eps), m.w * inv_sqrt(q.w + eps));
+              o.x = pack2_bf16(over_sqrt(m.x, q.x + eps), over_sqrt(m.y, q.y + eps));
+              o.y = pack2_bf16(over_sqrt(m.z, q.z + eps), over_sqrt(m.w, q.w + eps));
               *reinterpret_cast<uint2*>(xh + it * step_h) = o;
             }
             if (it < n_next) {

@@ -7,7 +7,7 @@
 // Here one cluster of up to 16 CTAs walks the whole chain of a basis, or of a range of its columns, in one launch, and the
 // steps are separated by the cluster's hardware barrier; the second sweep and the completion of a
 // rank-deficient product are branches instead of cancelled launches.  Measured, one basis alone: order 64
-// 31 us, 384 205 us, 1024 1.26 ms, 1536 3.6 ms; stand-alone Power() at order 384 1368 -> 233 us.
+// 32 us, 384 214 us, 1024 1.28 ms, 1536 3.6 ms; stand-alone Power() at order 384 1368 -> 242 us.
 //
 //  * Rows of A are dealt to the CTAs in contiguous chunks.  A CTA computes its rows' share of a panel's
 //    Gram matrix and applies R^-1 and the projections to its own rows only, so these steps need no
@@ -355,23 +355,13 @@ struct Ctx {
 // next diagonal block and factors it in registers (every lane the same: no shuffles, 8 dependent square
 // roots), while the other warps update the rest, all of a warp's blocks at once (a block row to a warp took as long as two
 // factorisations).  Two barriers a block instead of one a pivot: 27 us with a barrier a pivot and the matrix in registers,
-// 20 us with two pivots a barrier, 13.3 us with a block row to a warp and CUDA's rsqrt().
+// 20 us with two pivots a barrier, 13.3 us with a block row to a warp.
 // (Multiplying block row c by an explicit R_cc^-T instead loses the factorisation of a panel with a condition
 // number of 1e6, such as a completed rank-deficient product has: its error, 1e-16 times the condition number,
 // swamps pivots of 1e-12.  Substitution is backward stable like the unblocked elimination.)
 // The pivots end up at oPiv, the Gram diagonal at oDiag0.
 constexpr int oZ = oStage, oX = oZ + 64 * kLdK, oD = oX + 8 * kLdK;      // (in the operand stages)
 static_assert(64 * kLdK + 8 * kLdK + 8 * 8 + 8 <= kStageD, "the factorisation borrows the operand stages");
-
-// 1 / sqrt(x) of a positive normal number: the hardware's approximation y (relative error 1e-6) and the third-order
-// iteration y (1 + e / 2 + 3 e^2 / 8), e = 1 - x y^2, four dependent operations: 49 cycles, rsqrt() 61 (the square roots are the
-// chain's critical path).  Largest relative error over 1e-260 .. 1e260: 2.2e-16.
-__device__ __forceinline__ double inv_sqrt(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-(x * y), y, 1.0);
-  return fma(y * e, fma(e, 0.375, 0.5), y);
-}
 
 // The blocks that step c updates with block row c - 1, its own diagonal block excepted: rows i >= c, columns j > i, j = i
 // and (the identity's part) j < c.  Entries beyond the count are valid blocks whose result is dropped.
@@ -399,7 +389,7 @@ __device__ __forceinline__ void factor8(const double* Z, int c) {
 #pragma unroll
   for (int p = 0; p < 8; ++p) {
     piv[p] = u[p][p] > fl[p] ? u[p][p] : fl[p];
-    inv[p] = inv_sqrt(piv[p]);
+    inv[p] = rsqrt(piv[p]);
 #pragma unroll
     for (int j = p + 1; j < 8; ++j) u[p][j] *= inv[p];
 #pragma unroll

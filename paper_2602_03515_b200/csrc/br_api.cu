@@ -194,8 +194,11 @@ struct Bump {
 inline size_t simt_need(const Layer& L) { return 4 * (((size_t)L.d.m * L.d.n + 63) / 64 * 64); }
 constexpr size_t kSimtScratch = 16u << 20;
 
-// A gradient of this size is copied by itself (164 MB: 52 us, 64 in the grouped kernel).
-constexpr size_t kCopyAlone = 4u << 20;
+// From these sizes on a gradient is copied by itself instead of in a launch with the others: beside the contraction launches, where the
+// grouped kernel keeps SMs and power from them (steps of one layer set of d = 768, the largest 3.5 MB, 319.7 us by itself and 320.9; of d = 1024,
+// 6.3 MB, 504.5 and 508.3; d = 1536 1159 and 1166; four of d = 384, 0.9 MB at most, 364 and 342), and behind a step (plain layers, us: 4 of 8 MB 106.7
+// and 96.6, 2 of 32 MB 172.6 and 172.0, 48 MB and six of 0.5 159 and 156.5, 2 of 64 MB 331 and 337, 2 of 160 MB 806 and 820).
+constexpr size_t kCopyAloneBeside = 4u << 20, kCopyAlone = 64u << 20;
 
 // S = 1st: the half product of a refresh (M^T U, or M V) is formed in equal slices of the unrotated dimension, each
 // at most 128 MiB of fp64 in every lane.  (Whole, it was 393 MB a lane for an embedding of 32000 x 1536.  Slices of half
@@ -1231,8 +1234,14 @@ br_status step_enqueue(br_handle* h, const void* const* grads, int tau) {
       for (int j = 0; j < n; ++j) {
         Layer& L = h->layers[ids[j]];
         if (L.ring_slots <= 0 || (*c->stored)[ids[j]]) continue;
-        copies.push_back({c->grads[ids[j]], const_cast<void*>(ring_slot_ptr(L, (h->calls - 1) % L.ring_slots)),
-                          (size_t)L.d.m * L.d.n * dtype_size(L.d.grad_dtype)});
+        void* const slot = const_cast<void*>(ring_slot_ptr(L, (h->calls - 1) % L.ring_slots));
+        const size_t bytes = (size_t)L.d.m * L.d.n * dtype_size(L.d.grad_dtype);
+        if (bytes >= kCopyAloneBeside) {
+          c->copied = true;
+          BR_CUDA(h, cudaMemcpyAsync(slot, c->grads[ids[j]], bytes, cudaMemcpyDeviceToDevice, h->copy_stream));
+        } else {
+          copies.push_back({c->grads[ids[j]], slot, bytes});
+        }
         (*c->stored)[ids[j]] = 1;
       }
       if (copies.empty()) return (int)BR_OK;

@@ -1,5 +1,5 @@
 """Gradients into the ring: several in one launch of the library's kernel, more than a launch takes, sizes that no 16-byte piece
-divides, large ones by themselves; and the launch count, which has the kernel in it."""
+divides, large ones among small ones; and the launch count, which has the kernel in it."""
 import pytest
 
 from workloads import LayerSpec
@@ -36,7 +36,7 @@ def _run(shapes, dtype, geom, prec, calls=3):
 
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_many_and_ragged(dtype):
-    """Sizes around the 16-byte pieces (bf16: 2 to 34 bytes), seventy gradients (two launches), one of 4 MiB or more by itself."""
+    """Sizes around the 16-byte pieces (bf16: 2 to 34 bytes), seventy-one gradients (two launches), one of more than 4 MiB."""
     shapes = [(1, k) for k in (1, 2, 3, 7, 8, 9, 15, 16, 17)] + [(37, 53), (5, 1999)] + [(13, 17)] * 59 + [(1100, 1999)]
     launches = _run(shapes, dtype, GEOM_NONE, "BR_GEMM_FP32")
     assert launches == [2, 2, 2 + len(shapes)]            # copies; the third call updates every matrix too
@@ -47,6 +47,7 @@ def test_one_gradient_is_a_plain_copy():
 
 
 def test_beside_the_contractions():
-    """Tensor-core layers: 66 gradients, two launches, by themselves in the first calls and on the side stream of an update."""
-    with_delay = _run([(16, 24)] * 66, "bf16", GEOM_BI, "BR_GEMM_BF16")
-    assert with_delay[:2] == [2, 2] and with_delay[2] > 2
+    """Tensor-core layers: 66 small gradients, two launches, by themselves in the first calls and on the side stream of an update, where
+    one of 4 MiB or more is copied by itself."""
+    launches = _run([(16, 24)] * 66 + [(1536, 1400)], "bf16", GEOM_BI, "BR_GEMM_BF16")
+    assert launches[:2] == [2, 2] and launches[2] > 2

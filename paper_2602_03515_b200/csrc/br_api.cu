@@ -209,6 +209,7 @@ inline int64_t z_slice(int64_t k, int64_t other) {
   return std::min(std::min(rows, other), ((other + slices - 1) / slices + 63) / 64 * 64);      // (whole tiles)
 }
 
+// Bases of the largest order that the pool holds at least; in the compact layout three, or one beside the lanes of other orders.
 constexpr size_t kPoolOfLargest = 12, kPoolCompact = 3;
 constexpr int64_t kSmallGroup = 128;
 // From here on a power product takes less time in digits on the int8 tensor cores than on the fp64 unit.  Refreshes, us, in digits and on
@@ -218,7 +219,7 @@ constexpr int64_t kOzMinOrder = 1024;
 // A side whose refresh is part of the grouped launches, and what it needs of the pool.
 inline bool grouped_side(const Layer& L, int64_t k) { return L.d.src == BR_SRC_SECOND && qr_one_launch(k); }
 inline size_t pool_need(int64_t k) {
-  return align_up(sizeof(double) * (size_t)k * (size_t)k) + align_up(sizeof(double) * orth_work_doubles(k));
+  return align_up(sizeof(double) * (size_t)k * (size_t)k) + align_up(sizeof(double) * orth_work_doubles(k, true));
 }
 
 // Lays out every buffer of the handle in one slab.  With base == nullptr only sizes are computed.
@@ -264,8 +265,7 @@ void layout(br_handle* h, Bump& b, Sizes* sz) {
     h->simt_floats = h->compact ? simt_max : std::max(simt_max, std::min(simt_total, kSimtScratch));
     h->simt_scratch = b.take<float>(h->simt_floats);
   }
-  // the pool: every grouped basis at once, up to twelve of the largest (three in the compact layout)
-  h->pool_bytes = std::min(pool_sum, (h->compact ? kPoolCompact : kPoolOfLargest) * pool_max);
+  h->pool_bytes = std::min(pool_sum, (!h->compact ? kPoolOfLargest : max_k ? 1 : kPoolCompact) * pool_max);
   // Digits of two products of the largest order, or of one, as far as pool and digits together stay below eight buffers
   // for that order with a product and its copy each.
   h->oz_bytes = 0;
@@ -547,7 +547,7 @@ br_status refresh_side(br_handle* h, Layer& L, bool left_side, br_handle::Lane& 
       OrthJob job = {};
       job.A = ln.rA; job.k = k; job.Acopy = ln.rF; job.Qprev = Q; job.complete = complete ? 1 : 0;
       job.Qout = Q; job.Qh = left_side ? L.Uh : L.Vh; job.Ql = left_side ? L.Ul : L.Vl; job.cond_out = h->d_cond + ci;
-      orth_job_work(&job, ln.rWork);
+      orth_job_work(&job, ln.rWork, false);
       BR_CUDA(h, orth_group(&job, 1, h->d_status, s));
       count(h); h->stats.gemm_flops += 2.0 * k * k * k;
       continue;
@@ -595,8 +595,8 @@ br_status refresh_group(br_handle* h, const GroupSide* v, int n, char* pool, siz
     char* const digits = pool + used;
     const size_t digit_bytes = bytes - used + oz_bytes;
     for (OrthJob& j : jobs) {
-      orth_job_work(&j, reinterpret_cast<double*>(pool + used));
-      used += align_up(sizeof(double) * orth_work_doubles(j.k));
+      orth_job_work(&j, reinterpret_cast<double*>(pool + used), true);
+      used += align_up(sizeof(double) * orth_work_doubles(j.k, true));
     }
     // (longest first: the products in digits are the front of the list)
     std::vector<OzProduct> oz;

@@ -214,8 +214,9 @@ struct OrthJob {
   int complete;
 };
 constexpr int kOrthGroup = 32;        // jobs of one launch at most (by value: 3.4 KB of launch parameters)
-size_t orth_work_doubles(int64_t k);
-void orth_job_work(OrthJob* j, double* work);
+// `grouped`: beside other orders (a launch's clusters are sized for its largest one)
+size_t orth_work_doubles(int64_t k, bool grouped);
+void orth_job_work(OrthJob* j, double* work, bool grouped);
 cudaError_t orth_group(const OrthJob* jobs, int n, int* status, cudaStream_t s);
 // A <- F Qprev of every job (fp32 operands, fp64 sums)
 cudaError_t product_group(const OrthJob* jobs, int n, cudaStream_t s);

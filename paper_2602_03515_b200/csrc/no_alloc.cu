@@ -73,7 +73,7 @@ extern "C" br_status br_power_static(void* cuda_stream, const float* F, float* Q
   if (cudaMemsetAsync(flag, 0, sizeof(int), s) != cudaSuccess) return BR_ERR_CUDA;
   OrthJob job = {};
   job.A = A; job.k = k; job.F = F; job.Qprev = Q; job.Qout = Q;
-  orth_job_work(&job, work);
+  orth_job_work(&job, work, false);
   if (product_group(&job, 1, s) != cudaSuccess) return BR_ERR_CUDA;
   job.F = nullptr; job.Qprev = nullptr;                  // (a deficient product is reported, not completed)
   if (orth_group(&job, 1, flag, s) != cudaSuccess) return BR_ERR_CUDA;

@@ -846,11 +846,10 @@ int64_t coef_doubles(int64_t k) { return pad32(std::max<int64_t>(((k + 1) / 2) *
 
 }  // namespace
 
-size_t orth_work_doubles(int64_t k) {
-  return (size_t)(coef_doubles(k) + pad32(2 * kMaxCluster * k) + pad32(k));
-}
-void orth_job_work(OrthJob* j, double* work) {
-  j->C = work; j->normp = j->C + coef_doubles(j->k); j->rdiag = j->normp + pad32(2 * kMaxCluster * j->k);
+static int64_t norm_doubles(int64_t k, bool grouped) { return pad32(2 * (grouped ? kMaxCluster : cluster_for(k)) * k); }
+size_t orth_work_doubles(int64_t k, bool grouped) { return (size_t)(coef_doubles(k) + norm_doubles(k, grouped) + pad32(k)); }
+void orth_job_work(OrthJob* j, double* work, bool grouped) {
+  j->C = work; j->normp = j->C + coef_doubles(j->k); j->rdiag = j->normp + norm_doubles(j->k, grouped);
 }
 
 template <int NJ>

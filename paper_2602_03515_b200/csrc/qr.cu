@@ -430,7 +430,7 @@ bool qr_one_launch(int64_t k) { return k < std::min(kOneLaunchEnd, tc_min_order(
 
 size_t qr_work_doubles(int64_t k) {
   const int64_t norms = (kNormChunks + 1) * k + 64;        // complete_columns
-  if (qr_one_launch(k)) return (size_t)std::max<int64_t>((int64_t)orth_work_doubles(k), norms);
+  if (qr_one_launch(k)) return (size_t)std::max<int64_t>((int64_t)orth_work_doubles(k, false), norms);
   return (size_t)(64 + pad32(k) + pad32(((k + 1) / 2) * ((k + 1) / 2)) + pad32(proj_part_doubles(k)) + pad32(k));
 }
 

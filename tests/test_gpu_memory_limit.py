@@ -30,12 +30,12 @@ class _Limited:
         self.struct = B.BrAllocator(self.cb[0], self.cb[1], None)
 
 
-def _create(br, weights, limit, geom):
-    specs = [LayerSpec("w", m, n, geom, SRC_SECOND, 1) for m, n in SHAPES[:len(weights)]]
-    descs = [br.BrLayerDesc(m=s.m, n=s.n, geom=s.geom, src=s.src, grad_dtype=br.BR_F32, tau_max=1, freq=0, reserved=0,
+def _create(br, weights, limit, geom, shapes=SHAPES, dtype=0):
+    specs = [LayerSpec("w", m, n, geom, SRC_SECOND, 1) for m, n in shapes[:len(weights)]]
+    descs = [br.BrLayerDesc(m=s.m, n=s.n, geom=s.geom, src=s.src, grad_dtype=dtype, tau_max=1, freq=0, reserved=0,
                             weight=w.data_ptr()) for s, w in zip(specs, weights)]
     hp = br.BrHparams(lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0.0, beta_factor=-1.0, freq=3, power_iters=1,
-                      accum=0, gemm_prec=br.BR_GEMM_FP32, flags=0, clip_norm=0.0, scratch_limit_bytes=0)
+                      accum=0, gemm_prec=br.BR_GEMM_BF16 if dtype else br.BR_GEMM_FP32, flags=0, clip_norm=0.0, scratch_limit_bytes=0)
     a = _Limited(limit)
     try:
         return a, br.br_state_bytes(descs, hp)[0], br.br_create(descs, hp, 0, 0, a.struct)
@@ -82,3 +82,25 @@ def test_no_second_request_where_nothing_is_smaller():
     assert len(a.asked) == 1 and not a.blocks
     a, usual, e = _create(br, W, 1 << 60, GEOM_UNI)
     br.br_destroy(e)
+
+
+@pytest.mark.parametrize("d,blocks,limit", [(456, 3, 807 << 20), (528, 2, 1091 << 20)])
+def test_smaller_layout_beside_lanes(d, blocks, limit):
+    """Orders on both sides of 1600: lanes for the ones above, a pool for the others.  The smaller layout fits where three lanes that
+    hold every order do (791 and 1077 MiB)."""
+    import torch
+    import paper_2602_03515_b200 as br
+    shapes = [(d, 3 * d), (d, d), (d, 4 * d), (4 * d, d)] * blocks
+    W = [0.02 * torch.randn(m, n, device="cuda") for m, n in shapes]
+    G = [(0.01 * torch.randn(m, n, device="cuda")).bfloat16() for m, n in shapes]
+    before = [w.clone() for w in W]
+    torch.cuda.synchronize()
+    a, usual, h = _create(br, W, limit, GEOM_BI, shapes, br.BR_BF16)
+    assert not isinstance(h, Exception), (h, a.asked)
+    try:
+        assert len(a.asked) == 2 and a.asked[1] <= limit < a.asked[0]
+        for _ in range(7):
+            br.br_step(h, [g.data_ptr() for g in G], 1)
+        assert br.br_sync_status(h) >= 0 and all(torch.isfinite(w).all() and not torch.equal(w, b) for w, b in zip(W, before))
+    finally:
+        br.br_destroy(h)

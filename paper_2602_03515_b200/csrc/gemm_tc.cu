@@ -51,8 +51,8 @@
 // for the chunks of a tile of K = 2560.
 //
 // Every wait on an mbarrier is bounded: when a wait gives up the CTA raises an abort flag,
-// records BR_ERR_TIMEOUT in the status word, leaves its loops, frees its tensor memory and
-// returns; later launches return at once while the status word is negative.
+// records BR_ERR_TIMEOUT in the status word, leaves its loops, outlasts its copies in flight, frees its
+// tensor memory and returns; later launches return at once while the status word is negative.
 #include <cuda.h>
 
 #include <cstdlib>
@@ -417,6 +417,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
         }
         if (!ok) break;
       }
+      outlast_copies(abort_flag);
     }
   } else if (warp == 1) {
     // ======================= MMA issuer =======================

@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_gemm(const __grid_constant__
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
   if (!dead_word) {
     if (warp == 0) {
-      if (lane == 0)
+      if (lane == 0) {
         for (int kb = 0; kb < nk; ++kb) {
           const int s = kb % kStages;
           if (!mbar_wait(empty(s), ((kb / kStages) & 1) ^ 1, abort_flag, g.status)) break;
@@ -249,6 +249,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_gemm(const __grid_constant__
           tma_load_3d(base + s * kStage, &p.a, full(s), kb * kBK, m0, 0);
           tma_load_3d(base + s * kStage + kS * kPlaneA, &p.b, full(s), kb * kBK, n0, 0);
         }
+        outlast_copies(abort_flag);
+      }
     } else if (warp == 1) {
       if (lane == 0) {
         // signed 8-bit operands, 32-bit integer accumulators, 128 x 64, both operands K-major

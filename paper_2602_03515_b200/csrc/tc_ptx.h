@@ -96,6 +96,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   return true;
 }
 
+// After a wait has given up: the copies that this CTA (or its pair) still has in flight write to its shared memory, and no barrier tells any
+// more when the last one has landed.  A copy takes microseconds; this waits for a millisecond, at most.
+__device__ __forceinline__ void outlast_copies(volatile int* abort_flag) {
+  if (!*abort_flag) return;
+  const uint64_t t0 = global_timer_ns();
+  for (int i = 0; i < 1000000 && global_timer_ns() - t0 < 1000000ull; ++i) {}
+}
+
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
                                             int x, int y, int z) {
   asm volatile(

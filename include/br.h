@@ -184,7 +184,8 @@ BR_API br_status br_set_lr(br_handle* h, float lr);
  * layer has t == 0 (its factor is all zero).
  * Bases are refreshed several at a time on internal streams that fork from and join the
  * handle's stream inside the call (the same happens for the periodic refresh inside br_step, which
- * also stores the call's gradients through an internal stream that joins before it returns).  The
+ * also stores the call's gradients, and updates small fp32 matrices beside larger ones, through an internal stream that joins
+ * before it returns; BR_RING_SIDE_STREAM=0 in the environment keeps both on the handle's stream).  The
  * launch chain of a basis of order 1600 or more is captured into a CUDA graph the first time its
  * (order, form) occurs and replayed afterwards (plain launches if that capture fails).  Neither this call nor br_step may be
  * issued while the handle's stream is being captured by the caller: both read conditioning notes of

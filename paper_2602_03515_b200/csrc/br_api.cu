@@ -210,7 +210,12 @@ inline int64_t z_slice(int64_t k, int64_t other) {
 }
 
 // Bases of the largest order that the pool holds at least; in the compact layout three, or one beside the lanes of other orders.
+// Refreshes with 6, 8, 12 and 20, ms: 24 bases of order 384 1.10, 1.00, 0.73, 0.88; of 768 3.96, 4.19, 3.13, 3.44; of 1024 6.96, 7.44, 5.75, 6.57;
+// 40 of 512 3.05, 2.76, 2.22, 2.05; 16 of 1536 14.0, 14.0, 12.2, 13.6.
 constexpr size_t kPoolOfLargest = 12, kPoolCompact = 3;
+// Orders up to this one are launched by themselves beside larger ones.  It hardly matters: with 32, 64, 128 and 256 four bases of order 512
+// and eight of 96 418, 419, 420, 417 us, two of 1024 and sixteen of 128 1445, 1447, 1473, 1472, of 64 1437, 1423, 1426, 1423; orders 37 to 515
+// 523, 521, 524, 512.
 constexpr int64_t kSmallGroup = 128;
 // From here on a power product takes less time in digits on the int8 tensor cores than on the fp64 unit.  Refreshes, us, in digits and on
 // the fp64 unit: four bases of order 512 453 and 398, 640 680 and 647, 768 900 and 887, 896 1265 and 1255, 1024 1560 and 1640,

@@ -74,25 +74,22 @@ namespace {
 
 constexpr int BM = 128, BN = 256, BK = 64;       // tile (elements); BK*2 bytes = one 128-byte swizzle row
 constexpr int UMMA_K = 16;
-constexpr int STAGES = 4;
 constexpr int A_BYTES = BM * BK * 2;             // 16 KiB
-constexpr int B_BYTES = BN * BK * 2;             // 32 KiB
-constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-constexpr int SH_STAGES = 2;                     // shared-operand form: two stages of 2 A tiles + 2 B tiles
-constexpr int SH_STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
-static_assert(SH_STAGES * SH_STAGE_BYTES == STAGES * STAGE_BYTES, "both forms use the same operand area");
+// Steps with four epilogue warps of 256 columns each: one block of d = 1024 745 us instead of 602, four of d = 384 402 and 324, one of
+// d = 2048 with its embedding 4.05 and 3.59 ms, four of d = 2560 22.1 and 20.4 ms.
 constexpr int EPI_WARPS = 8;
 constexpr int EPI_BYTES = EPI_WARPS * 32 * 32 * 4;   // one 32 x 32 fp32 block per epilogue warp
-constexpr int OPERAND_BYTES = STAGES * STAGE_BYTES;                   // 192 KiB of operand stages in the shared-operand form
-// 160 KiB in the others: five stages are as fast as six, and the plain form leaves 34 KB of shared memory.  With a limit of 128
-// registers (launch bounds of 512 threads; no rotated Adam, whose problems always sum operand pairs) it also leaves a
+constexpr int OPERAND_BYTES = 192 * 1024;            // operand stages in the shared-operand form
+// 160 KiB in the others.  A sixth stage in the plain form: four blocks of d = 2560 0.7 % shorter, four of d = 384 1.1 % longer, one of d = 2048
+// 0.6 % longer; unpaired, three stages against four: d = 1024 0.9 % longer, d = 384 1.0 % shorter, d = 2048 the same.  With a limit of 128
+// registers (launch bounds of 512 threads; no rotated Adam, whose problems always sum operand pairs) the plain form also leaves a
 // quarter of each sub-partition's registers: the copies of the gradients into the ring run beside the last two phases of a step.
 // At 168 registers three warps fill a sub-partition, and the copies kept the weight-write launch waiting (four blocks of
 // d = 2560: 21.4 ms a step instead of 20.1).
 constexpr int PLAIN_OPERAND_BYTES = 160 * 1024;
 constexpr int SMEM_BYTES = OPERAND_BYTES + EPI_BYTES + 1024;          // + slack to align the tiles to 1 KiB
 constexpr int SMEM_BYTES_PLAIN = PLAIN_OPERAND_BYTES + EPI_BYTES + 1024;
-constexpr int MAX_STAGES = 6;
+constexpr int MAX_STAGES = 5;
 // Per-form geometry.  PAIR: the CTA pair owns a 256-row tile, each CTA stages 128 columns of B.
 template <bool SHARED, bool PAIR>
 struct Form {
@@ -110,9 +107,9 @@ constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS; // warp 0: TMA, warp 1: MMA, wa
 constexpr int FOLD_BLOCK = 32 * 32;
 constexpr int SMEM_BYTES_FOLD = PLAIN_OPERAND_BYTES + EPI_WARPS * 2 * FOLD_BLOCK * 4 + 1024;
 constexpr int MAX_PAIRS = 3;
-// Fixed part of a tile's cost in the schedule (see make_schedule), plain and folded form.  Steady steps with 0 and 0, 6 and
-// 24, 12 and 24, 6 and 0, 6 and 48: one block of d = 1024 620, 587, 587, 610, 586 us; four of d = 384 392, 382, 390, 389,
-// 382 us; one of d = 2048 with its embedding 3.08, 3.01, 3.02, 3.07, 3.05 ms.
+// Fixed part of a tile's cost in the schedule (see make_schedule), plain and folded form.  Steady steps with 6 and 24, 3 and 24, 12 and 24,
+// 6 and 12, 6 and 48: one block of d = 1024 602 to 604 us, four of d = 384 324 to 325 us, one of d = 2048 with its embedding 3.58 to 3.60 ms, four
+// of d = 2560 20.3 to 20.5 ms, in no order (0 and 0, with an epilogue of four warps: 2 to 6 % longer).
 constexpr int kTileCost = 6, kFoldTileCost = 24;
 // Tile rasterisation: a group of row-blocks (or, transposed, of column-blocks) is swept across the
 // other dimension, so that the group's operand panel stays in L2 while the other operand streams

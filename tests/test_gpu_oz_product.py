@@ -59,7 +59,7 @@ def test_graded_factor(k):
 
 def test_rows_of_different_size():
     """Rows and columns whose sizes span a factor of 900, from a basis far from the eigenvectors: the errors of the product,
-    2^-50 of the size of its row and column, reach the result times the condition number of the column-scaled product."""
+    at most 2^-48 of the size of its row and column, reach the result times the condition number of the column-scaled product."""
     rng = np.random.default_rng(7)
     F, Q = _graded(1090, rng, spread=30.0)
     got, _ = _refresh([F, F], [Q, Q])

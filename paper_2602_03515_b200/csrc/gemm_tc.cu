@@ -368,10 +368,13 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
         const TileInfo ti = locate_tile<TM>(probs, n_probs, tile_at(wi), calls, tau);
         if (!ti.active) continue;
         const DevProblem* p = ti.p;
-        const int nkb = (p->K + BK - 1) / BK;
+        // (copies: the barriers' memory clobbers would have every use in the loops read the problem again, out of L2 since
+        // the operand stages leave three KB of L1; the first-side launch of four d = 2560 blocks 4.75 -> 4.5 ms)
+        const int nkb = (p->K + BK - 1) / BK, nA = p->nA, nB = p->nB, n_pairs = p->n_pairs;
+        const int a_mn = p->a_mn, b_mn = p->b_mn, a_ring = p->a_ring_mask, b_ring = p->b_ring_mask;
         bool ok = true;
         auto load_a = [&](uint32_t dst, const CUtensorMap* ma, int k0, int za, uint32_t bar) {
-          if (p->a_mn) {
+          if (a_mn) {
 #pragma unroll
             for (int j = 0; j < BM / 64; ++j) load(dst + j * (BK * 128), ma, bar, ti.m0 + row_off + 64 * j, k0, za);
           } else {
@@ -379,7 +382,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
           }
         };
         auto load_b = [&](uint32_t dst, const CUtensorMap* mb, int k0, int zb, uint32_t bar) {
-          if (p->b_mn) {
+          if (b_mn) {
 #pragma unroll
             for (int j = 0; j < F::BNC / 64; ++j) load(dst + j * (BK * 128), mb, bar, ti.n0 + col_off + 64 * j, k0, zb);
           } else {
@@ -391,17 +394,15 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
           for (int kb = 0; kb < nkb; ++kb) {
             if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, status)) { ok = false; break; }
             const uint32_t fb = PAIR ? map_to_cta(full_bar(stage), 0) : full_bar(stage);
-            if (rank == 0) mbar_expect_tx(full_bar(stage), copies * (uint32_t)(p->nA * A_BYTES + p->nB * F::BB));
-            for (int i = 0; i < p->nA; ++i)
-              load_a(sA(stage, i), &p->mapA[i], kb * BK, ((p->a_ring_mask >> i) & 1) ? ti.z : 0, fb);
-            for (int i = 0; i < p->nB; ++i)
-              load_b(sB(stage, i), &p->mapB[i], kb * BK, ((p->b_ring_mask >> i) & 1) ? ti.z : 0, fb);
+            if (rank == 0) mbar_expect_tx(full_bar(stage), copies * (uint32_t)(nA * A_BYTES + nB * F::BB));
+            for (int i = 0; i < nA; ++i) load_a(sA(stage, i), &p->mapA[i], kb * BK, ((a_ring >> i) & 1) ? ti.z : 0, fb);
+            for (int i = 0; i < nB; ++i) load_b(sB(stage, i), &p->mapB[i], kb * BK, ((b_ring >> i) & 1) ? ti.z : 0, fb);
             if (++stage == NST) { stage = 0; phase ^= 1u; }
           }
         } else {
-          for (int pr = 0; pr < p->n_pairs && ok; ++pr) {
-            const int za = ((p->a_ring_mask >> pr) & 1) ? ti.z : 0;
-            const int zb = ((p->b_ring_mask >> pr) & 1) ? ti.z : 0;
+          for (int pr = 0; pr < n_pairs && ok; ++pr) {
+            const int za = ((a_ring >> pr) & 1) ? ti.z : 0;
+            const int zb = ((b_ring >> pr) & 1) ? ti.z : 0;
             for (int kb = 0; kb < nkb; ++kb) {
               if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, status)) { ok = false; break; }
               const uint32_t fb = PAIR ? map_to_cta(full_bar(stage), 0) : full_bar(stage);
@@ -432,6 +433,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
         if (!ti.active) continue;
         const DevProblem* p = ti.p;
         const int nkb = (p->K + BK - 1) / BK;
+        const int combos = p->combos, fold_kb = p->fold_kb;      // (copies: see the producer)
         const uint32_t idesc = make_idesc(p->a_mn, p->b_mn, TM);
         // K-major: advance 32 bytes per 16-element k step inside the swizzle row;
         // MN-major: 16 k rows = two 8-row groups of 1024 bytes.
@@ -441,13 +443,13 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
           // chunks of fold_kb k-blocks, each accumulated from zero, alternately in the two buffers, and
           // handed to the epilogue warps, which add it to the running sum in their registers
           bool ok = true;
-          for (int kb0 = 0; kb0 < nkb && ok; kb0 += p->fold_kb) {
+          for (int kb0 = 0; kb0 < nkb && ok; kb0 += fold_kb) {
             const int buf = (int)(fold_seq & 1u);
             if (!mbar_wait<PAIR>(tempty_bar(buf), ((fold_seq >> 1) & 1u) ^ 1u, abort_flag, status)) { ok = false; break; }
             tc_fence_after();
             const uint32_t d_chunk = tmem_base + (uint32_t)buf * BN;
             uint32_t accumulate = 0;
-            const int kb1 = min(nkb, kb0 + p->fold_kb);
+            const int kb1 = min(nkb, kb0 + fold_kb);
             for (int kb = kb0; kb < kb1; ++kb) {
               if (!mbar_wait(full_bar(stage), phase, abort_flag, status)) { ok = false; break; }
               tc_fence_after();
@@ -479,13 +481,13 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
         uint32_t accumulate = 0;
         bool ok = true;
         const int n_steps = SHARED ? nkb : p->n_pairs * nkb;
-        const int n_combo = SHARED ? (p->combos >> 8) : 1;
+        const int n_combo = SHARED ? (combos >> 8) : 1;
         for (int it = 0; it < n_steps; ++it) {
           if (!mbar_wait(full_bar(stage), phase, abort_flag, status)) { ok = false; break; }
           tc_fence_after();
           for (int c = 0; c < n_combo; ++c) {
-            const int ai = SHARED ? ((p->combos >> (2 * c)) & 1) : 0;
-            const int bi = SHARED ? ((p->combos >> (2 * c + 1)) & 1) : 0;
+            const int ai = SHARED ? ((combos >> (2 * c)) & 1) : 0;
+            const int bi = SHARED ? ((combos >> (2 * c + 1)) & 1) : 0;
             const uint64_t adesc = make_smem_desc(sA(stage, ai), a_lbo, 1024);
             const uint64_t bdesc = make_smem_desc(sB(stage, bi), b_lbo, 1024);
 #pragma unroll
@@ -558,7 +560,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
       if constexpr (FOLD) {
         // ---- folded form: this warp owns 32 rows (its lane quadrant) x 128 columns (its half) ----
         float* const fbuf = epi_tiles + (warp - 2) * (2 * FOLD_BLOCK);
-        const int nkb = (p->K + BK - 1) / BK;
+        const int nkb = (p->K + BK - 1) / BK, fold_kb = p->fold_kb;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * 128);
         // which of the four 32-column blocks are written at all (uniform across the warp)
         uint32_t need = 0;
@@ -597,7 +599,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
         // block at a time (the other warp of the quadrant covers the load latency).
         uint32_t sum[4][32];
         bool ok = true;
-        for (int kb0 = 0; kb0 < nkb; kb0 += p->fold_kb) {
+        for (int kb0 = 0; kb0 < nkb; kb0 += fold_kb) {
           const int buf = (int)(fold_seq & 1u);
           if (!mbar_wait(tfull_bar(buf), (fold_seq >> 1) & 1u, abort_flag, status)) { ok = false; break; }
           tc_fence_after();

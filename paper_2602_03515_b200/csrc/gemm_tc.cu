@@ -233,11 +233,12 @@ struct TileInfo {
   bool active;
 };
 
-// tile index -> problem (binary search over tile_begin) and block coordinates
+// tile index -> problem (`problem`, or where that is negative by a binary search over tile_begin) and block coordinates
 template <int TM>
-__device__ __forceinline__ TileInfo locate_tile(const DevProblem* probs, int n_probs, int tile,
+__device__ __forceinline__ TileInfo locate_tile(const DevProblem* probs, int n_probs, int tile, int problem,
                                                 long long calls, int tau) {
-  int lo = 0, hi = n_probs - 1;
+  int lo = problem, hi = problem;
+  if (problem < 0) { lo = 0; hi = n_probs - 1; }
   while (lo < hi) {
     int mid = (lo + hi + 1) >> 1;
     if (probs[mid].tile_begin <= tile) lo = mid; else hi = mid - 1;
@@ -348,11 +349,14 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
   }
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
-  // this unit's tiles: entries [walk_begin, walk_end) of the schedule's list behind its n_units + 1 offsets, or,
-  // without a schedule, every n_units-th tile of the range.  A dead pair finds an empty list in every role.
+  // this unit's tiles: entries [walk_begin, walk_end) of the schedule's list behind its n_units + 1 offsets, with their problems
+  // in a second list behind that, or, without a schedule, every n_units-th tile of the range.  A dead pair finds an empty list in every role.
   const int walk_begin = schedule ? schedule[unit] : first_tile + unit, walk_step = schedule ? 1 : n_units;
   const int walk_end = dead ? walk_begin : schedule ? schedule[unit + 1] : total_tiles;
-  auto tile_at = [&](int i) { return schedule ? schedule[n_units + 1 + i] : i; };
+  auto tile_at = [&](int i) {
+    const int* at = schedule + n_units + 1 + i;
+    return locate_tile<TM>(probs, n_probs, schedule ? at[0] : i, schedule ? at[total_tiles] : -1, calls, tau);
+  };
 
   if (warp == 0) {
     // ======================= TMA producer =======================
@@ -365,7 +369,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
         if (PAIR) tma_load_3d_pair(dst, map, bar, x, y, z); else tma_load_3d(dst, map, bar, x, y, z);
       };
       for (int wi = walk_begin; wi < walk_end && !*abort_flag; wi += walk_step) {
-        const TileInfo ti = locate_tile<TM>(probs, n_probs, tile_at(wi), calls, tau);
+        const TileInfo ti = tile_at(wi);
         if (!ti.active) continue;
         const DevProblem* p = ti.p;
         // (copies: the barriers' memory clobbers would have every use in the loops read the problem again, out of L2 since
@@ -429,7 +433,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
         if (PAIR) { umma_commit_pair(bar); umma_commit_pair(map_to_cta(bar, 1)); } else { umma_commit(bar); }
       };
       for (int wi = walk_begin; wi < walk_end && !*abort_flag; wi += walk_step) {
-        const TileInfo ti = locate_tile<TM>(probs, n_probs, tile_at(wi), calls, tau);
+        const TileInfo ti = tile_at(wi);
         if (!ti.active) continue;
         const DevProblem* p = ti.p;
         const int nkb = (p->K + BK - 1) / BK;
@@ -530,7 +534,7 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
     int acc = 0; uint32_t acc_phase = 0;
     uint32_t fold_seq = 0;
     for (int wi = walk_begin; wi < walk_end && !*abort_flag; wi += walk_step) {
-      const TileInfo ti = locate_tile<TM>(probs, n_probs, tile_at(wi), calls, tau);
+      const TileInfo ti = tile_at(wi);
       if (!ti.active) continue;
       const DevProblem* p = ti.p;
       float alpha = p->dyn_scalars ? dyn_alpha : p->alpha;
@@ -923,31 +927,33 @@ int pair_capacity(bool shared) {
 // its embedding: 55 tiles of 500 k-blocks behind 1739 of 40 to 108) or has few tiles per unit.  Tiles of equal
 // length keep their order, so that neighbours in the walk still run at the same time and share operands in L2.
 // A tile costs its k-blocks plus `fixed` (the part of its epilogue that the next tile's main loop does not
-// cover, in k-blocks).  Layout: units + 1 offsets, then the tiles.
+// cover, in k-blocks).  Layout: units + 1 offsets, then the tiles, then their problems.
 std::vector<int> make_schedule(const std::vector<DevProblem>& probs, int total, int units, int fixed) {
-  struct Tile { int cost, index; };
+  struct Tile { int cost, index, problem; };
   std::vector<Tile> tiles;
   tiles.reserve((size_t)total);
-  for (const DevProblem& d : probs)
-    for (int i = 0; i < d.tile_count; ++i) tiles.push_back({d.n_pairs * ((d.K + BK - 1) / BK) + fixed, d.tile_begin + i});
+  for (size_t p = 0; p < probs.size(); ++p)
+    for (int i = 0; i < probs[p].tile_count; ++i)
+      tiles.push_back({probs[p].n_pairs * ((probs[p].K + BK - 1) / BK) + fixed, probs[p].tile_begin + i, (int)p});
   std::stable_sort(tiles.begin(), tiles.end(), [](const Tile& a, const Tile& b) { return a.cost > b.cost; });
   typedef std::pair<long long, int> Load;                     // (work so far, unit)
   std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
   for (int u = 0; u < units; ++u) heap.push({0, u});
-  std::vector<std::vector<int>> list((size_t)units);
+  std::vector<std::vector<Tile>> list((size_t)units);
   for (const Tile& t : tiles) {
     Load l = heap.top();
     heap.pop();
-    list[(size_t)l.second].push_back(t.index);
+    list[(size_t)l.second].push_back(t);
     l.first += t.cost;
     heap.push(l);
   }
   std::vector<int> out;
-  out.reserve((size_t)(units + 1 + total));
+  out.reserve((size_t)(units + 1 + 2 * total));
   int at = 0;
   for (int u = 0; u < units; ++u) { out.push_back(at); at += (int)list[(size_t)u].size(); }
   out.push_back(at);
-  for (const auto& l : list) out.insert(out.end(), l.begin(), l.end());
+  for (const auto& l : list) for (const Tile& t : l) out.push_back(t.index);
+  for (const auto& l : list) for (const Tile& t : l) out.push_back(t.problem);
   return out;
 }
 

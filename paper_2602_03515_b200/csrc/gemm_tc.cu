@@ -65,7 +65,6 @@
 #include <vector>
 
 #include "br_internal.h"
-#include "over_sqrt.h"
 #include "tc_ptx.h"
 
 namespace br {
@@ -723,8 +722,8 @@ k_tc_gemm(const DevProblem* __restrict__ probs, int n_probs, int first_tile, int
               *reinterpret_cast<float4*>(dm + it * step_d) = m;
               *reinterpret_cast<float4*>(dv + it * step_d) = q;
               uint2 o;
-              o.x = pack2_bf16(over_sqrt(m.x, q.x + eps), over_sqrt(m.y, q.y + eps));
-              o.y = pack2_bf16(over_sqrt(m.z, q.z + eps), over_sqrt(m.w, q.w + eps));
+              o.x = pack2_bf16(m.x / sqrtf(q.x + eps), m.y / sqrtf(q.y + eps));
+              o.y = pack2_bf16(m.z / sqrtf(q.z + eps), m.w / sqrtf(q.w + eps));
               *reinterpret_cast<uint2*>(xh + it * step_h) = o;
             }
             if (it < n_next) {

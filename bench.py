@@ -25,9 +25,9 @@ sys.path.insert(0, ROOT)
 from workloads import get_workload  # noqa: E402
 from workloads.configs import GEOM_BI, GEOM_NONE, GEOM_UNI, SRC_SECOND  # noqa: E402
 
-# profiles/k_tc_gemm_c5_1layer.md: 10.89e9 B of DRAM traffic for the five launches of one step, which
+# profiles/k_tc_gemm_c5_1layer.md: 10.62e9 B of DRAM traffic for the five launches of one step, which
 # execute 6.395e12 flop
-NCU_DRAM_BYTES_PER_EXECUTED_FLOP = 10.89e9 / 6.395e12
+NCU_DRAM_BYTES_PER_EXECUTED_FLOP = 10.62e9 / 6.395e12
 
 METRIC = "rotated_adam_params_per_sec"
 UNIT = "params/s"
@@ -573,7 +573,7 @@ def main():
         ref_flops = sum((2.0 + 8.0 / 3.0) * float(k) ** 3 for k in orders)
         ref_tflops = ref_flops / (refresh_ms / 1e3) / 1e12
         fp64_peak = 148 * 64 * 2 * 1.965e9 / 1e12       # 148 SMs x 64 fp64 FMA per clock (mma.sync.m8n8k4.f64) x 2 x 1.965 GHz
-        roofline_refresh = {"bound": "fp64 matrix unit / tensor", "kernel": "k_orth_cluster + k_dgemm64 + k_tc_gemm (three-term bf16 splits)",
+        roofline_refresh = {"bound": "fp64 matrix unit / tensor", "kernel": "k_orth_group / k_orth_part + k_dgemm64 + k_tc_gemm (three-term bf16 splits)",
                             "bases": len(orders), "algorithmic_flops": ref_flops, "achieved": ref_tflops, "unit": "TFLOP/s",
                             "peak_fp64_unit": fp64_peak, "frac_of_fp64_unit": ref_tflops / fp64_peak,
                             "peak_bf16_split6": peaks["tf_sustained"] / 6.0, "frac_of_bf16_split6": ref_tflops / (peaks["tf_sustained"] / 6.0),
